@@ -50,6 +50,8 @@ struct FmmDev {
     unsigned long long *upq;               // upward pass: next unclaimed leaf box, CTAs past the end
     int64_t *split;                        // leaf boxes with long near lists (any order) and their
     int32_t *nsplit;                       // count, filled by the tree build
+    int32_t *ffbad;                        // per problem: 1 if the split FP32 forms (split.cuh) are not
+                                           // allowed; written with the secular roots, read by zhat and b
     int64_t cap_f;                         // capacity of the FMM problem list
     int ncol, nfield;                      // workspace widths
     unsigned long long *flops;             // algorithmic FP64 work of the far fields and of the
@@ -62,6 +64,7 @@ struct FmmPlan {
     int64_t cap_boxes = 0, cap_leaves = 0, cap_f = 0;
     int lmax = 0;                          // upper bound on tree levels
     int nb0max = 0;                        // upper bound on leaf boxes per problem
+    int64_t total = 0;                     // extent of the row-indexed arrays
     int box = 0;                           // indices per leaf box (32 or 64) of this plan
     bool on = false;                       // some problem may take the FMM path
     std::vector<void *> bufs;

@@ -996,6 +996,36 @@ __global__ void __launch_bounds__(128) k_fmm_down(FmmDev pl, const int32_t *__re
     }
 }
 
+// Split parts of the kept poles and weights of the FMM problems (split.cuh);
+// pl.ffbad says which problems' scale and gaps do not allow them
+struct FfDev {
+    const ff_f4 *d;
+    const ff_f2 *w;
+};
+
+__global__ void k_ff_prep(int64_t nprob, const int64_t *__restrict__ off, int64_t total,
+                          const int32_t *__restrict__ fslot, R1Out o, ff_f4 *__restrict__ fd,
+                          ff_f2 *__restrict__ fw, int32_t *__restrict__ bad)
+{
+    for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < total;
+         x += (int64_t)gridDim.x * blockDim.x) {
+        if (x < off[0] || x >= off[nprob]) continue;
+        const int64_t p = sdc_upper_index(off, nprob, x);
+        if (fslot[p] < 0) continue;
+        const int64_t b0 = off[p];
+        const int m = o.mk[p], j = (int)(x - b0);
+        if (j >= m) continue;
+        const FfScale s = ff_scale(o.dk[b0], o.dk[b0 + m - 1], o.wsum[p]);
+        if (!s.ok || o.unshifted || (j + 1 < m && !ff_gap_ok(o.dk[x], o.dk[x + 1], s.kk))) {
+            bad[p] = 1;
+            continue;
+        }
+        const double z = o.zk[x];
+        fd[x] = ff_pole(o.dk[x], s);
+        fw[x] = ff_weight(z * z, s.kw);
+    }
+}
+
 // ---------------------------------------------------------------------------
 // Secular roots of the FMM problems, one warp per leaf box: with boxes of 64
 // a lane takes the next root of the box when its root has converged (the
@@ -1007,12 +1037,15 @@ __global__ void __launch_bounds__(128) k_fmm_down(FmmDev pl, const int32_t *__re
 // root of each problem (outside the tree) is solved by k_secular_last.
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(64)
-k_secular_fmm(FmmDev pl, const int64_t *__restrict__ off, R1Out o, double stop_c, int max_iter,
+k_secular_fmm(FmmDev pl, FfDev ff, const int64_t *__restrict__ off, R1Out o, double stop_c, int max_iter,
               unsigned long long *terms)
 {
-    __shared__ double sd[2][SPLIT_NEAR * B], sw[2][SPLIT_NEAR * B];
+    __shared__ __align__(16) unsigned char stage[2][SPLIT_NEAR * B * (sizeof(ff_f4) + sizeof(ff_f2))];
     const unsigned FULL = 0xffffffffu;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    ff_f4 *const fd = (ff_f4 *)stage[warp];              // near poles: split parts, or FP64 (the general form)
+    ff_f2 *const fw = (ff_f2 *)(fd + SPLIT_NEAR * B);
+    double *const sd = (double *)stage[warp], *const sw = sd + SPLIT_NEAR * B;
     const int64_t nleaf = pl.leaf_base[pl.nprob];
     for (int64_t gl = (int64_t)blockIdx.x * 2 + warp; gl < nleaf; gl += (int64_t)gridDim.x * 2) {
         const int64_t p = sdc_upper_index(pl.leaf_base, pl.nprob, gl);
@@ -1034,6 +1067,8 @@ k_secular_fmm(FmmDev pl, const int64_t *__restrict__ off, R1Out o, double stop_c
         const int nnr = pl.nnear[g];
         const int nn = near_len(nnr, (m + B - 1) / B);
         if (nnr < 0 || nnr >= SPLIT_NEAR) continue;     // long near list: k_secular_fmm_split
+        const bool ok = pl.ffbad[p] == 0;
+        const FfScale fs = ff_scale(dk[0], dk[m - 1], W);
         int near_terms = 0;
         __syncwarp();
         for (int i = 0; i < nn; i++) {
@@ -1041,9 +1076,14 @@ k_secular_fmm(FmmDev pl, const int64_t *__restrict__ off, R1Out o, double stop_c
             const int cnt = min(B, m - j0);
             near_terms += cnt;
             for (int jj = lane; jj < cnt; jj += 32) {
-                sd[warp][i * B + jj] = dk[j0 + jj];
-                const double z = zk[j0 + jj];
-                sw[warp][i * B + jj] = z * z;
+                if (ok) {
+                    fd[i * B + jj] = ff.d[b0 + j0 + jj];
+                    fw[i * B + jj] = ff.w[b0 + j0 + jj];
+                } else {
+                    sd[i * B + jj] = dk[j0 + jj];
+                    const double z = zk[j0 + jj];
+                    sw[i * B + jj] = z * z;
+                }
             }
         }
         __syncwarp();
@@ -1061,6 +1101,16 @@ k_secular_fmm(FmmDev pl, const int64_t *__restrict__ off, R1Out o, double stop_c
             const unsigned amask = __ballot_sync(FULL, act);
             if (terms && lane == 0) atomicAdd(terms, (unsigned long long)__popc(amask) * (unsigned long long)near_terms);
             Acc A = {0.0, 0.0, 0.0, 0.0};
+            FfAcc S = {};
+            const ff_f4 x = ff_point(R.dK, R.y, fs);
+            for (int i = 0; i < nn; i++) {
+                const int j0 = near_box_chk(pl, g, nnr, i, (m + B - 1) / B, o.status) * B;
+                const int cnt = min(B, m - j0);
+                if (ok)      ff_sweep(fd + i * B, fw + i * B, 0, cnt, j0, kk, kwlo, kwhi, x, S);
+                else if (p0) sweep<false>(sd + i * B, sw + i * B, 0, cnt, j0, kk, kwlo, kwhi, R.dK, R.y, A);
+                else         sweep<true>(sd + i * B, sw + i * B, 0, cnt, j0, kk, kwlo, kwhi, R.dK, R.y, A);
+            }
+            if (ok) A = ff_collect(S, R, fs.kk, fs.kw);
             if (act) {
                 // far field at the plain position x = d_K + y (local shifting)
                 const double uu = ((R.dK + R.y) - cT) * ihT;
@@ -1073,17 +1123,10 @@ k_secular_fmm(FmmDev pl, const int64_t *__restrict__ off, R1Out o, double stop_c
                     t = fma(u2, c1, cf[2 * P + n] - c2); c2 = c1; c1 = t;
                     t = fma(u2, e1, cf[3 * P + n] - e2); e2 = e1; e1 = t;
                 }
-                A.psi = fma(uu, a1, cf[0] - a2);
-                A.phi = fma(uu, b1, cf[P] - b2);
-                A.dpsi = fma(uu, c1, cf[2 * P] - c2);
-                A.dphi = fma(uu, e1, cf[3 * P] - e2);
-            }
-            for (int i = 0; i < nn; i++) {
-                const int j0 = near_box_chk(pl, g, nnr, i, (m + B - 1) / B, o.status) * B;
-                const int cnt = min(B, m - j0);
-                const double *bd = sd[warp] + i * B, *bw = sw[warp] + i * B;
-                if (p0) sweep<false>(bd, bw, 0, cnt, j0, kk, kwlo, kwhi, R.dK, R.y, A);
-                else    sweep<true>(bd, bw, 0, cnt, j0, kk, kwlo, kwhi, R.dK, R.y, A);
+                A.psi += fma(uu, a1, cf[0] - a2);
+                A.phi += fma(uu, b1, cf[P] - b2);
+                A.dpsi += fma(uu, c1, cf[2 * P] - c2);
+                A.dphi += fma(uu, e1, cf[3 * P] - e2);
             }
             bool fin = false;
             if (act && R.update(A, tol, max_iter, o.status)) {
@@ -1133,7 +1176,7 @@ k_secular_fmm(FmmDev pl, const int64_t *__restrict__ off, R1Out o, double stop_c
 constexpr int TAIL_LANES = 4;
 
 __global__ void __launch_bounds__(128)
-k_secular_tail(FmmDev pl, const int64_t *__restrict__ off, R1Out o, double stop_c, int max_iter,
+k_secular_tail(FmmDev pl, FfDev ff, const int64_t *__restrict__ off, R1Out o, double stop_c, int max_iter,
                unsigned long long *terms)
 {
     const unsigned FULL = 0xffffffffu;
@@ -1145,6 +1188,8 @@ k_secular_tail(FmmDev pl, const int64_t *__restrict__ off, R1Out o, double stop_
     R.dK = 0.0; R.y = 1.0; R.phase = 1; R.k = 0;
     int64_t b0 = 0, g = 0, gl = 0;
     int m = 1, nnr = 0, nn = 0;
+    bool ok = false;
+    FfScale fs = {};
     unsigned nterm = 0;
     double cT = 0.0, ihT = 1.0, tol = 0.0;
     while (true) {
@@ -1174,6 +1219,8 @@ k_secular_tail(FmmDev pl, const int64_t *__restrict__ off, R1Out o, double stop_
                 box_ch(pl.blo[g], pl.bhi[g], cT, hT);
                 ihT = 1.0 / hT;
                 tol = stop_c * (double)m * SDC_EPS;
+                ok = pl.ffbad[p] == 0;
+                fs = ff_scale(o.dk[b0], o.dk[b0 + m - 1], o.wsum[p]);
                 act = true;
             } else {
                 dry = true;
@@ -1185,7 +1232,24 @@ k_secular_tail(FmmDev pl, const int64_t *__restrict__ off, R1Out o, double stop_
             if (lane == 0) atomicAdd(terms, (unsigned long long)nt);
         }
         Acc A = {0.0, 0.0, 0.0, 0.0};
-        if (act) {
+        if (act && ok) {
+            FfAcc S = {};
+            const ff_f4 x = ff_point(R.dK, R.y, fs);
+            for (int i = 0; i < nn; i++) {
+                const int j0 = near_box_chk(pl, g, nnr, i, (m + B - 1) / B, o.status) * B;
+                const int cnt = min(B, m - j0);
+                const ff_f4 *dd = ff.d + b0 + j0;
+                const ff_f2 *ww = ff.w + b0 + j0;
+#pragma unroll 4
+                for (int jj = part; jj < cnt; jj += TAIL_LANES) {
+                    float pp, ppl, qq;
+                    ff_term(dd[jj], ww[jj], x, pp, ppl, qq);
+                    ff_select(S, pp, ppl, qq, j0 + jj, R.k);
+                }
+                ff_close(S);
+            }
+            A = ff_collect(S, R, fs.kk, fs.kw, part == 0);
+        } else if (act) {
             for (int i = 0; i < nn; i++) {
                 const int j0 = near_box_chk(pl, g, nnr, i, (m + B - 1) / B, o.status) * B;
                 const int cnt = min(B, m - j0);
@@ -1244,13 +1308,16 @@ k_secular_tail(FmmDev pl, const int64_t *__restrict__ off, R1Out o, double stop_
 // run in groups of 32.
 template <int SPW>
 __global__ void __launch_bounds__(SPW * 32)
-k_secular_fmm_split(FmmDev pl, const int64_t *__restrict__ off, R1Out o, double stop_c, int max_iter,
+k_secular_fmm_split(FmmDev pl, FfDev ff, const int64_t *__restrict__ off, R1Out o, double stop_c, int max_iter,
                     unsigned long long *terms)
 {
-    __shared__ double sd[SPW][B], sw[SPW][B];
+    __shared__ __align__(16) unsigned char stage[SPW][B * (sizeof(ff_f4) + sizeof(ff_f2))];
     __shared__ double red[SPW][4][32];
     const unsigned FULL = 0xffffffffu;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    ff_f4 *const fd = (ff_f4 *)stage[warp];
+    ff_f2 *const fw = (ff_f2 *)(fd + B);
+    double *const sd = (double *)stage[warp], *const sw = sd + B;
     const int nsplit = *pl.nsplit;
     for (int u = blockIdx.x; u < nsplit; u += gridDim.x) {
         const int64_t gl = pl.split[u];                  // a leaf box with a long near list
@@ -1271,6 +1338,8 @@ k_secular_fmm_split(FmmDev pl, const int64_t *__restrict__ off, R1Out o, double 
         box_ch(pl.blo[g], pl.bhi[g], cT, hT);
         const double ihT = 1.0 / hT;
         const double *cf = pl.coef + gl * pl.nfield * P;
+        const bool ok = pl.ffbad[p] == 0;
+        const FfScale fs = ff_scale(dk[0], dk[m - 1], W);
         int near_terms = 0;
         if (terms)
             for (int i = 0; i < nn; i++) near_terms += min(B, m - near_box(pl, g, nnr, i) * B);
@@ -1289,26 +1358,35 @@ k_secular_fmm_split(FmmDev pl, const int64_t *__restrict__ off, R1Out o, double 
                 if (terms && warp == 0 && lane == 0)
                     atomicAdd(terms, (unsigned long long)__popc(amask) * (unsigned long long)near_terms);
                 Acc A = {0.0, 0.0, 0.0, 0.0};
-                if (warp == 0 && act) {
-                    const double uu = ((R.dK + R.y) - cT) * ihT;
-                    A.psi = clenshaw(cf, uu);
-                    A.phi = clenshaw(cf + P, uu);
-                    A.dpsi = clenshaw(cf + 2 * P, uu);
-                    A.dphi = clenshaw(cf + 3 * P, uu);
-                }
+                FfAcc fa = {};
+                const ff_f4 x = ff_point(R.dK, R.y, fs);
                 for (int i = warp; i < nn; i += SPW) {
                     const int S = near_box_chk(pl, g, nnr, i, (m + B - 1) / B, o.status);
                     const int j0 = S * B;
                     const int cnt = min(B, m - j0);
                     __syncwarp();
                     for (int jj = lane; jj < cnt; jj += 32) {
-                        sd[warp][jj] = dk[j0 + jj];
-                        const double z = zk[j0 + jj];
-                        sw[warp][jj] = z * z;
+                        if (ok) {
+                            fd[jj] = ff.d[b0 + j0 + jj];
+                            fw[jj] = ff.w[b0 + j0 + jj];
+                        } else {
+                            sd[jj] = dk[j0 + jj];
+                            const double z = zk[j0 + jj];
+                            sw[jj] = z * z;
+                        }
                     }
                     __syncwarp();
-                    if (p0) sweep<false>(sd[warp], sw[warp], 0, cnt, j0, kk, kwlo, kwhi, R.dK, R.y, A);
-                    else    sweep<true>(sd[warp], sw[warp], 0, cnt, j0, kk, kwlo, kwhi, R.dK, R.y, A);
+                    if (ok)      ff_sweep(fd, fw, 0, cnt, j0, kk, kwlo, kwhi, x, fa);
+                    else if (p0) sweep<false>(sd, sw, 0, cnt, j0, kk, kwlo, kwhi, R.dK, R.y, A);
+                    else         sweep<true>(sd, sw, 0, cnt, j0, kk, kwlo, kwhi, R.dK, R.y, A);
+                }
+                if (ok) A = ff_collect(fa, R, fs.kk, fs.kw, warp == 0);
+                if (warp == 0 && act) {
+                    const double uu = ((R.dK + R.y) - cT) * ihT;
+                    A.psi += clenshaw(cf, uu);
+                    A.phi += clenshaw(cf + P, uu);
+                    A.dpsi += clenshaw(cf + 2 * P, uu);
+                    A.dphi += clenshaw(cf + 3 * P, uu);
                 }
                 red[warp][0][lane] = A.psi;
                 red[warp][1][lane] = A.phi;
@@ -1511,7 +1589,9 @@ struct Prod {
 // lambda_j, -1 at d_j).  One CTA of B threads per leaf box, one target each.
 __global__ void __launch_bounds__(B) k_lowner_fmm(FmmDev pl, const int64_t *__restrict__ off, R1Out o)
 {
-    __shared__ double sd[B], so[B], se[B];
+    __shared__ __align__(16) double stage[4 * B];
+    double *const sd = stage, *const so = stage + B, *const se = stage + 2 * B;    // FP64 products
+    ff_w4 *const wd = (ff_w4 *)stage, *const wl = wd + B;                         // integer products
     const int tid = threadIdx.x;
     const int64_t nleaf = pl.leaf_base[pl.nprob];
     for (int64_t gl = blockIdx.x; gl < nleaf; gl += gridDim.x) {
@@ -1526,7 +1606,12 @@ __global__ void __launch_bounds__(B) k_lowner_fmm(FmmDev pl, const int64_t *__re
         const bool act = i < m;
         const double di = act ? dk[i] : 0.0;
         Prod pr;
-        if (act) {
+        FfProd fn = {1ull << 63, 0}, fd = {1ull << 63, 0};
+        const bool ok = pl.ffbad[p] == 0;
+        const FfScale fs = ff_scale(dk[0], dk[m - 1], o.wsum[p]);
+        const ff_w4 d4 = ff_words4(ff_fixed(di, fs.kk) - fs.ref);
+        const ff_u96 dw = {d4.lo, d4.mid, d4.hi};
+        if (act && !ok) {
             const double num = (dorg[m - 1] - di) + eta[m - 1];
             const double den = (i == m - 1) ? 1.0 : dk[m - 1] - di;
             pr.mul(num, den);
@@ -1540,15 +1625,33 @@ __global__ void __launch_bounds__(B) k_lowner_fmm(FmmDev pl, const int64_t *__re
             const int cnt = min(B, (m - 1) - j0);
             nsrc += max(cnt, 0);
             __syncthreads();
-            if (tid < cnt) { sd[tid] = dk[j0 + tid]; so[tid] = dorg[j0 + tid]; se[tid] = eta[j0 + tid]; }
+            if (tid < cnt) {
+                if (ok) {
+                    wd[tid] = ff_words4(ff_fixed(dk[j0 + tid], fs.kk) - fs.ref);
+                    wl[tid] = ff_words4(ff_fixed(dorg[j0 + tid], fs.kk) + ff_fixed(eta[j0 + tid], fs.kk) - fs.ref);
+                } else {
+                    sd[tid] = dk[j0 + tid];
+                    so[tid] = dorg[j0 + tid];
+                    se[tid] = eta[j0 + tid];
+                }
+            }
             __syncthreads();
-            if (act) {
+            if (ok) {
+                ff_prod_sweep(wd, wl, cnt, j0, i, dw, fn, fd);
+            } else if (act) {
                 for (int jj = 0; jj < cnt; jj++) {
                     const double num = (so[jj] - di) + se[jj];
                     const double den = (j0 + jj == i) ? 1.0 : sd[jj] - di;
                     pr.mul(num, den);
                 }
             }
+        }
+        if (act && ok) {
+            // near factors outside the integer products, then those
+            lowner_edges(dk, dorg, eta, di, i, m, pr.pn, pr.pd, pr.ex);
+            pr.pn *= (double)fn.m;
+            pr.pd *= (double)fd.m;
+            pr.ex += fn.e - fd.e;
         }
         if (act) {
             double cT, hT;
@@ -1574,7 +1677,9 @@ __global__ void __launch_bounds__(B) k_lowner_fmm(FmmDev pl, const int64_t *__re
 // k_fmm_lastsum combines the boxes (so no single CTA walks all m sources).
 __global__ void __launch_bounds__(B) k_bnorm_fmm(FmmDev pl, const int64_t *__restrict__ off, R1Out o)
 {
-    __shared__ double sd[B], sv[B];
+    __shared__ __align__(16) double stage[4 * B];
+    double *const sd = stage, *const sv = stage + B;                // FP64 sums
+    ff_f4 *const fd = (ff_f4 *)stage, *const fv = fd + B;           // three-float sums
     __shared__ double red[B];
     const int tid = threadIdx.x;
     const int64_t nleaf = pl.leaf_base[pl.nprob];
@@ -1594,6 +1699,13 @@ __global__ void __launch_bounds__(B) k_bnorm_fmm(FmmDev pl, const int64_t *__res
             box_ch(pl.blo[g], pl.bhi[g], cT, hT);
             s = clenshaw(pl.coef + gl * pl.nfield * P, ((dK + e) - cT) / hT);
         }
+        const bool ok = pl.ffbad[p] == 0;
+        const FfScale fs = ff_scale(o.dk[b0], o.dk[b0 + m - 1], o.wsum[p]);
+        const int kv = fs.kw >> 1;
+        const int K = act ? o.org[b0 + j] : -1;
+        const ff_f4 x = ff_point(dK, e, fs);
+        const double sc = ok ? ff_pow2(-kv) : 1.0;
+        ff_t3 s3 = {0.0f, 0.0f, 0.0f};
         const int nnr = pl.nnear[g];
         const int nn = near_len(nnr, (m + B - 1) / B);
         int64_t nsrc = 0;
@@ -1603,15 +1715,30 @@ __global__ void __launch_bounds__(B) k_bnorm_fmm(FmmDev pl, const int64_t *__res
             const int cnt = min(B, m - i0);
             nsrc += max(cnt, 0);
             __syncthreads();
-            if (tid < cnt) { sd[tid] = o.dk[b0 + i0 + tid]; sv[tid] = o.vhat[b0 + i0 + tid]; }
+            if (tid < cnt) {
+                if (ok) {
+                    const ff_t3 t = ff_split3(o.vhat[b0 + i0 + tid] * sc);
+                    fd[tid] = ff_pole(o.dk[b0 + i0 + tid], fs);
+                    fv[tid] = {t.a, t.b, t.c, 0.0f};
+                } else {
+                    sd[tid] = o.dk[b0 + i0 + tid];
+                    sv[tid] = o.vhat[b0 + i0 + tid];
+                }
+            }
             __syncthreads();
-            if (act) {
+            if (ok) {
+                ff_sqr_sweep(fd, fv, cnt, i0, K, x, s3);
+            } else if (act) {
                 for (int ii = 0; ii < cnt; ii++) {
                     const double r = rcp_nr2((sd[ii] - dK) - e);
                     const double vr = sv[ii] * r;
                     s = fma(vr, vr, s);
                 }
             }
+        }
+        if (act && ok) {
+            const double vr = o.vhat[b0 + K] * rcp_nr2(-e);         // the origin's term
+            s = fma(vr, vr, fma(ff_join3(s3), ff_pow2(2 * (kv + fs.kk)), s));
         }
         if (act) o.bnorm[b0 + j] = 1.0 / sqrt(s);
         // this box's sources in the sum for the last target
@@ -1846,6 +1973,9 @@ k_cauchyN_fmm(FmmDev pl, FactorView f, const double *__restrict__ X, int64_t ldx
 }
 
 unsigned fmm_grid() { return (unsigned)(sdc_num_sms() * 8); }
+// zhat and b: CTAs of one or two warps whose chains of FP32 operations wait on
+// their own latency; 32 warps per SM
+unsigned near_grid() { return (unsigned)(sdc_num_sms() * (1024 / B)); }
 
 // As many CTAs of kernel K as the GPU holds at once (threads per CTA, static
 // shared memory only), from the occupancy calculator, once per device: the
@@ -1940,6 +2070,7 @@ superdc_status plan(FmmPlan &pl, int64_t nprob, const int64_t *off, int64_t tota
 {
     pl = FmmPlan();
     pl.box = B;
+    pl.total = total;
     if (nprob <= 0) return SUPERDC_OK;
     if (used) SDC_CHECK(cudaMemsetAsync(used, 0, (size_t)nprob * sizeof(int32_t), st));
     if (min_m <= 0) return SUPERDC_OK;
@@ -1997,6 +2128,7 @@ superdc_status plan(FmmPlan &pl, int64_t nprob, const int64_t *off, int64_t tota
     SDC_CHECK(al(&d.upcnt, pl.cap_boxes));
     SDC_CHECK(cudaMemsetAsync(d.upcnt, 0, (size_t)pl.cap_boxes * sizeof(int32_t), st));
     SDC_CHECK(al(&d.upq, 2));
+    SDC_CHECK(al(&d.ffbad, nprob));
     SDC_CHECK(al(&d.split, pl.cap_leaves));
     SDC_CHECK(al(&d.nsplit, 1));
     SDC_CHECK(cudaMemsetAsync(d.upq, 0, 2 * sizeof(unsigned long long), st));
@@ -2037,15 +2169,26 @@ superdc_status secular(const FmmPlan &pl, const int64_t *off, const R1Out &o, do
     if (!pl.on) return SUPERDC_OK;
     far_field<M_SEC, K_SEC>(pl, src_from_r1(off, o), 1, 1, st);      // keeps the kernel matrices
     const unsigned gl = (unsigned)std::max<int64_t>(1, std::min<int64_t>(pl.cap_f, (int64_t)sdc_num_sms() * 2));
+    ff_f4 *fd = nullptr;
+    ff_f2 *fw = nullptr;
+    SdcScratch sc(st);
+    SDC_CHECK(sc.get(&fd, (size_t)pl.total));
+    SDC_CHECK(sc.get(&fw, (size_t)pl.total));
+    SDC_CHECK(cudaMemsetAsync(pl.dv.ffbad, 0, (size_t)pl.dv.nprob * sizeof(int32_t), st));
+    const unsigned gp = (unsigned)std::max<int64_t>(1, std::min<int64_t>((pl.total + 255) / 256,
+                                                                         (int64_t)sdc_num_sms() * 8));
+    PROF_LAUNCH("fmm_secular", st, k_ff_prep<<<gp, 256, 0, st>>>(pl.dv.nprob, off, pl.total, pl.dv.fslot, o, fd, fw,
+                                                                 pl.dv.ffbad));
+    const FfDev ff = {fd, fw};
     unsigned long long *terms = prof_counter("fmm_secular_terms");
     unsigned long long *lterms = prof_counter("fmm_secular_last_terms");
     PROF_LAUNCH("fmm_secular_last", st, k_secular_last<<<gl, SL_T, 0, st>>>(pl.dv, off, o, stop_c, max_iter,
                                                                              lterms));
-    PROF_LAUNCH("fmm_secular", st, k_secular_fmm<<<fmm_grid(), 64, 0, st>>>(pl.dv, off, o, stop_c, max_iter,
+    PROF_LAUNCH("fmm_secular", st, k_secular_fmm<<<fmm_grid(), 64, 0, st>>>(pl.dv, ff, off, o, stop_c, max_iter,
                                                                              terms));
     PROF_LAUNCH("fmm_secular", st, k_secular_tail<<<(unsigned)(sdc_num_sms() * 4), 128, 0, st>>>(
-                                       pl.dv, off, o, stop_c, max_iter, terms));
-    PROF_LAUNCH("fmm_secular", st, (k_secular_fmm_split<8><<<fmm_grid(), 256, 0, st>>>(pl.dv, off, o, stop_c,
+                                       pl.dv, ff, off, o, stop_c, max_iter, terms));
+    PROF_LAUNCH("fmm_secular", st, (k_secular_fmm_split<8><<<fmm_grid(), 256, 0, st>>>(pl.dv, ff, off, o, stop_c,
                                                                                       max_iter, terms)));
     SDC_CHECK(cudaGetLastError());
     return SUPERDC_OK;
@@ -2055,7 +2198,7 @@ superdc_status lowner(const FmmPlan &pl, const int64_t *off, const R1Out &o, cud
 {
     if (!pl.on) return SUPERDC_OK;
     far_field<M_LOW, K_LOG>(pl, src_from_r1(off, o), 1, 2, st);      // reads them
-    PROF_LAUNCH("fmm_lowner", st, k_lowner_fmm<<<fmm_grid(), B, 0, st>>>(pl.dv, off, o));
+    PROF_LAUNCH("fmm_lowner", st, k_lowner_fmm<<<near_grid(), B, 0, st>>>(pl.dv, off, o));
     SDC_CHECK(cudaGetLastError());
     return SUPERDC_OK;
 }
@@ -2064,7 +2207,7 @@ superdc_status bnorm(const FmmPlan &pl, const int64_t *off, const R1Out &o, cuda
 {
     if (!pl.on) return SUPERDC_OK;
     far_field<M_BN, K_2>(pl, src_from_r1(off, o), 1, 2, st);
-    PROF_LAUNCH("fmm_bnorm", st, k_bnorm_fmm<<<fmm_grid(), B, 0, st>>>(pl.dv, off, o));
+    PROF_LAUNCH("fmm_bnorm", st, k_bnorm_fmm<<<near_grid(), B, 0, st>>>(pl.dv, off, o));
     PROF_LAUNCH("fmm_bnorm", st, k_fmm_lastsum<0><<<lastsum_grid(pl, 1), 128, 0, st>>>(
                                      pl.dv, off, o.mk, o.bnorm, nullptr, nullptr, nullptr, 0, 0, 1));
     SDC_CHECK(cudaGetLastError());

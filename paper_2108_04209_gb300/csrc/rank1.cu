@@ -32,7 +32,7 @@
 
 namespace {
 
-constexpr int SEC_CHUNK = 2048;   // poles staged per shared-memory chunk
+constexpr int SEC_CHUNK = 1024;   // poles staged per shared-memory chunk (24 bytes each)
 constexpr int DEFL_BIG = 128;     // problems larger than this deflate with a whole CTA
 
 
@@ -496,8 +496,11 @@ k_secular(const int64_t *__restrict__ off, const int4 *__restrict__ units,
           const int *__restrict__ nunits, int *__restrict__ counter,
           R1Out o, double stop_c, int max_iter)
 {
-    __shared__ double sd[SEC_CHUNK];
-    __shared__ double sw[SEC_CHUNK];
+    // staged poles and weights: split parts (ok), or FP64 (the general form)
+    __shared__ __align__(16) unsigned char stage[SEC_CHUNK * (sizeof(ff_f4) + sizeof(ff_f2))];
+    ff_f4 *const fd = (ff_f4 *)stage;
+    ff_f2 *const fw = (ff_f2 *)(fd + SEC_CHUNK);
+    double *const sd = (double *)stage, *const sw = sd + SEC_CHUNK;
     __shared__ double red[SPLIT ? NW : 1][4][32];
     __shared__ double s_dK[SPLIT ? 32 : 1], s_y[SPLIT ? 32 : 1];
     __shared__ int s_ph[SPLIT ? 32 : 1], s_fin[SPLIT ? 32 : 1];
@@ -518,9 +521,16 @@ k_secular(const int64_t *__restrict__ off, const int4 *__restrict__ units,
         const double *dk = o.dk + b0, *zk = o.zk + b0;
         const double W = o.wsum[p];
         const double tol = stop_c * (double)m * SDC_EPS;
-        const int len = U.z - U.y;
+        // split FP32 sweeps where the problem's scale allows; its last root (right
+        // of every pole, outside the fixed-point range) then runs on its own
+        const FfScale fs = ff_scale(dk[0], dk[m - 1], W);
+        bool okt = fs.ok && !o.unshifted && m >= 2;
+        for (int j = threadIdx.x; okt && j + 1 < m; j += NW * 32) okt = ff_gap_ok(dk[j], dk[j + 1], fs.kk);
+        const bool ok = __syncthreads_and(okt);
+        const int uend = ok ? min(U.z, m - 1) : U.z;
+        const int len = uend - U.y;
         const int wbeg = SPLIT ? U.y : U.y + (int)(((int64_t)len * warp) / NW);
-        const int wend = SPLIT ? U.z : U.y + (int)(((int64_t)len * (warp + 1)) / NW);
+        const int wend = SPLIT ? uend : U.y + (int)(((int64_t)len * (warp + 1)) / NW);
         int k = wbeg + lane;
         bool act = k < wend;
         int next = wbeg + 32;
@@ -528,13 +538,19 @@ k_secular(const int64_t *__restrict__ off, const int4 *__restrict__ units,
         R.dK = 0.0; R.y = 1.0; R.phase = 1;     // defined values for lanes that stay idle
         if (act) R.init(dk, zk, k, m, W, o.unshifted != 0);
         const bool single = (m <= SEC_CHUNK);
-        if (single) {
-            for (int j = threadIdx.x; j < m; j += NW * 32) {
-                sd[j] = dk[j];
-                double zj = zk[j];
-                sw[j] = zj * zj;
+        auto stage_chunk = [&](int c0, int cn) {
+            for (int j = threadIdx.x; j < cn; j += NW * 32) {
+                const double zj = zk[c0 + j];
+                if (ok) {
+                    fd[j] = ff_pole(dk[c0 + j], fs);
+                    fw[j] = ff_weight(zj * zj, fs.kw);
+                } else {
+                    sd[j] = dk[c0 + j];
+                    sw[j] = zj * zj;
+                }
             }
-        }
+        };
+        if (single) stage_chunk(0, m);
         __syncthreads();
         const bool lockstep = SPLIT || !single;
         while (lockstep ? __syncthreads_or(act) : __any_sync(FULL, act)) {
@@ -544,24 +560,24 @@ k_secular(const int64_t *__restrict__ off, const int4 *__restrict__ units,
             const bool p0 = __all_sync(FULL, !act || R.phase == 0);
             const bool any = __any_sync(FULL, act);
             Acc A = {0.0, 0.0, 0.0, 0.0};
+            FfAcc S = {};
+            const ff_f4 x = ff_point(R.dK, R.y, fs);
             for (int c0 = 0; c0 < m; c0 += SEC_CHUNK) {
                 const int cn = min(SEC_CHUNK, m - c0);
                 if (!single) {
                     __syncthreads();
-                    for (int j = threadIdx.x; j < cn; j += NW * 32) {
-                        sd[j] = dk[c0 + j];
-                        double zj = zk[c0 + j];
-                        sw[j] = zj * zj;
-                    }
+                    stage_chunk(c0, cn);
                     __syncthreads();
                 }
                 const int j0 = SPLIT ? (int)(((int64_t)cn * warp) / NW) : 0;
                 const int j1 = SPLIT ? (int)(((int64_t)cn * (warp + 1)) / NW) : cn;
                 if (any) {
-                    if (p0) sweep<false>(sd, sw, j0, j1, c0, kk, kwlo, kwhi, R.dK, R.y, A);
-                    else    sweep<true>(sd, sw, j0, j1, c0, kk, kwlo, kwhi, R.dK, R.y, A);
+                    if (ok)      ff_sweep(fd, fw, j0, j1, c0, kk, kwlo, kwhi, x, S);
+                    else if (p0) sweep<false>(sd, sw, j0, j1, c0, kk, kwlo, kwhi, R.dK, R.y, A);
+                    else         sweep<true>(sd, sw, j0, j1, c0, kk, kwlo, kwhi, R.dK, R.y, A);
                 }
             }
+            if (ok) A = ff_collect(S, R, fs.kk, fs.kw, !SPLIT || warp == 0);
             bool fin = false;
             if (SPLIT) {
                 // the warps hold the same roots: warp 0 alone reduces the partial
@@ -621,6 +637,16 @@ k_secular(const int64_t *__restrict__ off, const int4 *__restrict__ units,
             }
             next += __popc(mask);
         }
+        if (ok && U.z == m && warp == NW - 1) {
+            last_root_warp(dk, zk, m, W, tol, max_iter, o.status, R);
+            if (lane == 0) {
+                o.org[b0 + m - 1] = R.K;
+                o.eta[b0 + m - 1] = R.y;
+                o.dorg[b0 + m - 1] = R.dK;
+                o.lamk[b0 + m - 1] = R.dK + R.y;
+                if (o.sweeps) o.sweeps[b0 + m - 1] = R.nsw;
+            }
+        }
     }
 }
 
@@ -636,6 +662,7 @@ k_lowner(int64_t nprob, const int64_t *__restrict__ off, const int64_t *__restri
          const int32_t *__restrict__ fslot, unsigned long long *__restrict__ queue)
 {
     __shared__ int64_t s_tile;
+    __shared__ ff_w4 sd[TR], sl[TR];
     const int64_t ntiles = tile_off[nprob];
     for (int64_t it = blockIdx.x;; it += gridDim.x) {
         int64_t tile = it;
@@ -651,27 +678,54 @@ k_lowner(int64_t nprob, const int64_t *__restrict__ off, const int64_t *__restri
         const int64_t b0 = off[p];
         const int m = o.mk[p];
         const int i = (int)(tile - tile_off[p]) * TR + threadIdx.x;
-        if (i >= m) continue;
         const double *dk = o.dk + b0, *dorg = o.dorg + b0, *eta = o.eta + b0;
-        const double di = dk[i];
-        // numerator and denominator products kept apart (one division per
-        // entry instead of one per factor); every 8 factors both are brought
-        // back to [1/2, 1) by exponent arithmetic, the exponents summed in ex
-        double pn = (dorg[m - 1] - di) + eta[m - 1];
-        double pd = 1.0;
+        const FfScale fs = ff_scale(dk[0], dk[m - 1], o.wsum[p]);
+        bool okt = fs.ok && !o.unshifted && m >= 2;
+        for (int j = threadIdx.x; okt && j + 1 < m; j += TR) okt = ff_gap_ok(dk[j], dk[j + 1], fs.kk);
+        const bool ok = __syncthreads_and(okt);
+        const double di = i < m ? dk[i] : 0.0;
+        double pn = 1.0, pd = 1.0;
         int ex = 0;
-        for (int j = 0; j < m - 1; j++) {
-            double num = (dorg[j] - di) + eta[j];
-            double den = ((j < i) ? dk[j] : dk[j + 1]) - di;
-            pn *= num;
-            pd *= den;
-            if ((j & 7) == 7) {
-                int hn = __double2hiint(pn), hd = __double2hiint(pd);
-                int en = (hn >> 20) & 0x7FF, ed = (hd >> 20) & 0x7FF;
-                if (en != 0 && ed != 0 && en != 0x7FF && ed != 0x7FF) {
-                    ex += en - ed;
-                    pn = __hiloint2double((hn & 0x800FFFFF) | (1022 << 20), __double2loint(pn));
-                    pd = __hiloint2double((hd & 0x800FFFFF) | (1022 << 20), __double2loint(pd));
+        if (ok) {
+            // integer products (split.cuh); the two eigenvalues next to d_i and
+            // the last one (outside the positions' range) in FP64
+            FfProd num = {1ull << 63, 0}, den = {1ull << 63, 0};
+            const ff_w4 d4 = ff_words4(ff_fixed(di, fs.kk) - fs.ref);
+            const ff_u96 dw = {d4.lo, d4.mid, d4.hi};
+            for (int c0 = 0; c0 < m - 1; c0 += TR) {
+                const int cn = min(TR, m - 1 - c0), j = c0 + threadIdx.x;
+                __syncthreads();
+                if (threadIdx.x < cn) {
+                    sd[threadIdx.x] = ff_words4(ff_fixed(dk[j], fs.kk) - fs.ref);
+                    sl[threadIdx.x] = ff_words4(ff_fixed(dorg[j], fs.kk) + ff_fixed(eta[j], fs.kk) - fs.ref);
+                }
+                __syncthreads();
+                ff_prod_sweep(sd, sl, cn, c0, i, dw, num, den);
+            }
+            if (i >= m) continue;
+            lowner_edges(dk, dorg, eta, di, i, m, pn, pd, ex);
+            pn *= (double)num.m;
+            pd *= (double)den.m;
+            ex += num.e - den.e;
+        } else {
+            if (i >= m) continue;
+            // numerator and denominator products kept apart (one division per
+            // entry instead of one per factor); every 8 factors both are brought
+            // back to [1/2, 1) by exponent arithmetic, the exponents summed in ex
+            pn = (dorg[m - 1] - di) + eta[m - 1];
+            for (int j = 0; j < m - 1; j++) {
+                double num = (dorg[j] - di) + eta[j];
+                double den = ((j < i) ? dk[j] : dk[j + 1]) - di;
+                pn *= num;
+                pd *= den;
+                if ((j & 7) == 7) {
+                    int hn = __double2hiint(pn), hd = __double2hiint(pd);
+                    int en = (hn >> 20) & 0x7FF, ed = (hd >> 20) & 0x7FF;
+                    if (en != 0 && ed != 0 && en != 0x7FF && ed != 0x7FF) {
+                        ex += en - ed;
+                        pn = __hiloint2double((hn & 0x800FFFFF) | (1022 << 20), __double2loint(pn));
+                        pd = __hiloint2double((hd & 0x800FFFFF) | (1022 << 20), __double2loint(pd));
+                    }
                 }
             }
         }
@@ -694,6 +748,8 @@ k_bnorm(int64_t nprob, const int64_t *__restrict__ off, const int64_t *__restric
          const int32_t *__restrict__ fslot, unsigned long long *__restrict__ queue)
 {
     __shared__ int64_t s_tile;
+    __shared__ ff_f4 sd[TR], sv[TR];
+    __shared__ double red[TR / 32];
     const int64_t ntiles = tile_off[nprob];
     for (int64_t it = blockIdx.x;; it += gridDim.x) {
         int64_t tile = it;
@@ -709,9 +765,54 @@ k_bnorm(int64_t nprob, const int64_t *__restrict__ off, const int64_t *__restric
         const int64_t b0 = off[p];
         const int m = o.mk[p];
         const int j = (int)(tile - tile_off[p]) * TR + threadIdx.x;
-        if (j >= m) continue;
         const double *dk = o.dk + b0, *v = o.vhat + b0;
-        const double dK = o.dorg[b0 + j], e = o.eta[b0 + j];
+        const FfScale fs = ff_scale(dk[0], dk[m - 1], o.wsum[p]);
+        bool okt = fs.ok && !o.unshifted && m >= 2;
+        for (int i = threadIdx.x; okt && i + 1 < m; i += TR) okt = ff_gap_ok(dk[i], dk[i + 1], fs.kk);
+        const bool ok = __syncthreads_and(okt);
+        const double dK = j < m ? o.dorg[b0 + j] : 0.0, e = j < m ? o.eta[b0 + j] : 1.0;
+        if (ok) {
+            // three-float sums (split.cuh); the origin's term in FP64, the last
+            // eigenvalue (outside the positions' range) by the whole CTA in FP64
+            ff_t3 S = {0.0f, 0.0f, 0.0f};
+            const int K = j < m ? o.org[b0 + j] : -1;
+            const ff_f4 x = ff_point(dK, e, fs);
+            const int kv = fs.kw >> 1;
+            const double sc = ff_pow2(-kv);
+            for (int c0 = 0; c0 < m; c0 += TR) {
+                const int cn = min(TR, m - c0);
+                __syncthreads();
+                if (threadIdx.x < cn) {
+                    const ff_t3 t = ff_split3(v[c0 + threadIdx.x] * sc);
+                    sd[threadIdx.x] = ff_pole(dk[c0 + threadIdx.x], fs);
+                    sv[threadIdx.x] = {t.a, t.b, t.c, 0.0f};
+                }
+                __syncthreads();
+                ff_sqr_sweep(sd, sv, cn, c0, K, x, S);
+            }
+            if (j < m - 1) {
+                const double r = v[K] * rcp_nr2(-e);
+                o.bnorm[b0 + j] = 1.0 / sqrt(fma(r, r, ff_join3(S) * ff_pow2(2 * (kv + fs.kk))));
+            }
+            if (m - 1 - (int)(tile - tile_off[p]) * TR < TR) {
+                const double dl = o.dorg[b0 + m - 1], el = o.eta[b0 + m - 1];
+                double s = 0.0;
+                for (int i = threadIdx.x; i < m; i += TR) {
+                    const double vr = v[i] * rcp_nr2((dk[i] - dl) - el);
+                    s = fma(vr, vr, s);
+                }
+                for (int sh = 16; sh > 0; sh >>= 1) s += __shfl_xor_sync(0xffffffffu, s, sh);
+                if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+                __syncthreads();
+                if (threadIdx.x == 0) {
+                    s = 0.0;
+                    for (int w = 0; w < TR / 32; w++) s += red[w];
+                    o.bnorm[b0 + m - 1] = 1.0 / sqrt(s);
+                }
+            }
+            continue;
+        }
+        if (j >= m) continue;
         double s = 0.0;
         for (int i = 0; i < m; i++) {
             double t = (dk[i] - dK) - e;

@@ -5,6 +5,7 @@
 // and the per-root iteration state (Algorithm 2, stopping test eq. (4.12)).
 #pragma once
 #include "common.cuh"
+#include "split.cuh"
 
 namespace {
 
@@ -229,5 +230,83 @@ struct Root {
         return false;
     }
 };
+
+// sums of a root from its split sweep and the terms of the two poles next to it
+// in FP64 (two Newton steps: one step's bias, of one sign for every term, would
+// not cancel against the split ones).  own: false in the warps that leave the
+// two terms to another.
+__device__ __forceinline__ Acc ff_collect(const FfAcc &S, const Root &R, int kk, int kw, bool own = true)
+{
+    const double c1 = ff_pow2(kk + kw), c2 = ff_pow2(2 * kk + kw);
+    double a0 = 0.0, a1 = 0.0, b0 = 0.0, b1 = 0.0;
+    if (own) {
+        const double r0 = rcp_nr2((R.d0 - R.dK) - R.y), r1 = rcp_nr2((R.d1 - R.dK) - R.y);
+        a0 = R.w0 * r0;
+        a1 = R.w1 * r1;
+        b0 = a0 * r0;
+        b1 = a1 * r1;
+    }
+    Acc A;
+    A.psi = fma((double)S.psi, c1, a0);
+    A.phi = (fma((double)S.s, c1, fma((double)S.sl, c1, a0)) + a1) - A.psi;
+    A.dpsi = fma((double)S.dpsi, c2, b0);
+    A.dphi = fma((double)S.dphi, c2, b1);
+    return A;
+}
+
+// The last root of a problem (right of every pole), by one warp: the lanes
+// split the poles, every lane holds the same iterate.
+__device__ __forceinline__ void last_root_warp(const double *__restrict__ dk, const double *__restrict__ zk, int m,
+                                               double W, double tol, int max_iter, int32_t *status, Root &R)
+{
+    const int lane = threadIdx.x & 31;
+    R.init(dk, zk, m - 1, m, W);
+    for (bool fin = false; !fin;) {
+        Acc A = {0.0, 0.0, 0.0, 0.0};
+        for (int j = lane; j < m; j += 32) {
+            const double r = rcp_nr1(shifted_t(dk[j], R.dK, R.y));
+            const double z = zk[j];
+            const double a = (z * z) * r;
+            A.psi += a;
+            A.dpsi = fma(a, r, A.dpsi);
+        }
+        for (int sh = 16; sh > 0; sh >>= 1) {
+            A.psi += __shfl_xor_sync(0xffffffffu, A.psi, sh);
+            A.dpsi += __shfl_xor_sync(0xffffffffu, A.dpsi, sh);
+        }
+        fin = R.update(A, tol, max_iter, lane == 0 ? status : nullptr);
+    }
+}
+
+// p 2^ex *= f, p kept in [1/2, 1) (zero, subnormal and non-finite products pass through)
+__device__ __forceinline__ void exp_mul(double &p, int &ex, double f)
+{
+    p *= f;
+    const int h = __double2hiint(p), e = (h >> 20) & 0x7FF;
+    if (e != 0 && e != 0x7FF) {
+        ex += e - 1022;
+        p = __hiloint2double((h & 0x800FFFFF) | (1022 << 20), __double2loint(p));
+    }
+}
+
+// The factors of zhat_i that the integer products leave out: the eigenvalues
+// next to d_i (j = i - 1, i) with their poles, and the last one (j = m - 1).
+// pn / pd 2^ex is multiplied by them.
+__device__ __forceinline__ void lowner_edges(const double *__restrict__ dk, const double *__restrict__ dorg,
+                                             const double *__restrict__ eta, double di, int i, int m, double &pn,
+                                             double &pd, int &ex)
+{
+    int xd = 0;
+    exp_mul(pn, ex, (dorg[m - 1] - di) + eta[m - 1]);
+    if (i < m - 1) {
+        exp_mul(pn, ex, (dorg[i] - di) + eta[i]);
+        exp_mul(pd, xd, dk[m - 1] - di);
+    }
+    if (i > 0) {
+        exp_mul(pn, ex, (dorg[i - 1] - di) + eta[i - 1]);
+        exp_mul(pd, xd, dk[i - 1] - di);
+    }
+    ex -= xd;
+}
 
 }  // namespace
