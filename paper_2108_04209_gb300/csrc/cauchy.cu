@@ -298,7 +298,7 @@ superdc_status run(const FactorView &f, int64_t total, double *Xmut, const doubl
         // boxes of 32 halve the near field; with many columns the translations
         // (P^2 per column and box pair) dominate and boxes of 64 halve those
         superdc_status fs = fmm_plan(fp, f.nprob, f.off, total, f.max_m, f.mk, f.dk, f.fmm_min_m, w, w, nullptr,
-                                     box, 0, st);
+                                     box, false, st);
         if (fs != SUPERDC_OK) { fmm_free(fp, st); return fs; }
     }
     const FmmPlan &pl = use_shared ? *shared : fp;

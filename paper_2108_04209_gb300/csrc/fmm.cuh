@@ -9,6 +9,7 @@
 #pragma once
 #include <vector>
 #include "common.cuh"
+#include "split.cuh"
 #include "rank1.cuh"
 #include "cauchy.cuh"
 
@@ -40,9 +41,11 @@ struct FmmDev {
                                            // the sums for the last eigenvalue (outside the tree)
     FmmTail *tail;                         // roots left to the tail pass (capacity: every kept root)
     unsigned int *ntail;                   // their count, then the tail pass's next unclaimed entry
-    double *kmat;                          // per box, its first kslots interaction pairs: the P x P
-    int kslots;                            // matrix 1/(s_q2 - t_q) of nodes (M2L kernel, shared by
-                                           // the far fields built on one plan)
+    // plans of a rank-one step (FP32-split far fields, split.cuh): positions and weights of every box's
+    // Chebyshev nodes, and the first 64 candidates of its interaction list as a bit mask
+    ff_f4 *npos;
+    ff_f2 *nwt;
+    unsigned long long *amask;
     const int64_t *lev_off;                // per level: prefix of the FMM problems' box counts
     const int64_t *top_off;                // the same per level counted from each problem's top box
     int32_t *upcnt;                        // per box: children whose moments are done in the current
@@ -76,11 +79,10 @@ struct FmmPlan {
 // used (may be NULL): per problem 1 if it takes the FMM path, else 0.
 // box: indices per leaf box, 32 or 64 (smaller boxes halve the near field,
 // larger ones halve the number of box pairs whose expansions are translated).
-// kslots: M2L kernel matrices kept per box for the later far fields of the
-// same plan (0: none).
+// step: the plan serves the sums of a rank-one step (secular, zhat, b).
 superdc_status fmm_plan(FmmPlan &pl, int64_t nprob, const int64_t *off, int64_t total, int64_t max_m,
                         const int32_t *mk, const double *dk, int min_m, int ncol, int nfield, int32_t *used,
-                        int box, int kslots, cudaStream_t st);
+                        int box, bool step, cudaStream_t st);
 void fmm_free(FmmPlan &pl, cudaStream_t st);
 
 // Roots of the FMM problems (same outputs as the direct secular kernel).

@@ -370,6 +370,7 @@ struct SrcArgs {
     const int64_t *off;
     const int32_t *mk;
     const double *dk, *zk, *vhat, *bnorm, *dorg, *eta;
+    const double *wsum;                  // one-column modes: scale of the split node weights
     const int32_t *src, *pinv;
     const double *X;
     int64_t ldx;
@@ -385,7 +386,7 @@ constexpr int UP_ROWS = (B > 2 * P) ? B : 2 * P;   // rows of the staging arrays
 
 template <int MODE, int WW>
 __device__ __forceinline__ void leaf_moments(const FmmDev &pl, const SrcArgs &a, int64_t p, int64_t gl, int64_t g,
-                                             int Tb, int nw, double (*Tt)[P + 1], double (*Wt)[WW + 1],
+                                             int Tb, int nw, int kw, double (*Tt)[P + 1], double (*Wt)[WW + 1],
                                              double (*Ms)[WW + 1], const double *Tx)
 {
     const int tid = threadIdx.x;
@@ -462,6 +463,7 @@ __device__ __forceinline__ void leaf_moments(const FmmDev &pl, const SrcArgs &a,
         double s = Ms[0][q];
         for (int n = 1; n < P; n++) s = fma(Tx[qn * P + n], Ms[n][q], s);     // Tx holds 2 T_n
         pl.W[(g * P + qn) * pl.ncol + q] = s * (1.0 / P);
+        if (WW == 1) pl.nwt[g * P + qn] = ff_weight(s * (1.0 / P), kw);       // for k_fmm_far
     }
     // Chebyshev recurrence per source, moments, moments -> node weights
     const int64_t cnt = max(0, min(B, jend - Tb * B));
@@ -536,7 +538,7 @@ __global__ void k_fmm_levoff(const int32_t *__restrict__ mk, const int32_t *__re
 // through L2 (ld.global.cg): the sibling's were written by another CTA of the
 // same launch, which published them before its arrival count.
 template <int WW>
-__device__ __forceinline__ void m2m_box(const FmmDev &pl, int64_t p, int nb0, int l, int b, int64_t g, int nw,
+__device__ __forceinline__ void m2m_box(const FmmDev &pl, int64_t p, int nb0, int l, int b, int64_t g, int nw, int kw,
                                         double (*Tv)[P + 1], double (*Wc)[WW + 1], double (*Ms)[WW + 1],
                                         const double *Tx, const double *xq)
 {
@@ -587,6 +589,7 @@ __device__ __forceinline__ void m2m_box(const FmmDev &pl, int64_t p, int nb0, in
         double s = Ms[0][q];
         for (int n = 1; n < P; n++) s = fma(Tx[qn * P + n], Ms[n][q], s);     // Tx holds 2 T_n
         pl.W[(g * P + qn) * pl.ncol + q] = s * (1.0 / P);
+        if (WW == 1) pl.nwt[g * P + qn] = ff_weight(s * (1.0 / P), kw);       // for k_fmm_far
     }
     // children's node positions, the children's weights into moments, moments -> weights
     fl_add(pl, (int64_t)nch * 2 * P * (P - 2) + (int64_t)nch * 2 * P * P * nw + 2 * P * P * nw);
@@ -640,7 +643,8 @@ __global__ void __launch_bounds__(up_threads<MODE>()) k_fmm_up(FmmDev pl, SrcArg
         if (pl.fslot[p] < 0) continue;
         const int Tb = (int)(gl - pl.leaf_base[p]);
         const int64_t g = pl.box_base[p] + Tb;
-        leaf_moments<MODE, WW>(pl, a, p, gl, g, Tb, nw, Tt, Wt, Ms, Tx);
+        const int kw = (MODE == M_SEC || MODE == M_BN) ? ff_exp(a.wsum[p]) - 1022 : 0;
+        leaf_moments<MODE, WW>(pl, a, p, gl, g, Tb, nw, kw, Tt, Wt, Ms, Tx);
         const int nb0 = (a.mk[p] + B - 1) / B;
         const int L = lev_count(nb0);
         int l = 0, b = Tb;
@@ -658,43 +662,353 @@ __global__ void __launch_bounds__(up_threads<MODE>()) k_fmm_up(FmmDev pl, SrcArg
             __syncthreads();
             if (!last) break;
             __threadfence();
-            m2m_box<WW>(pl, p, nb0, l + 1, bp, gp, nw, Tt, Wt, Ms, Tx, xq);
+            m2m_box<WW>(pl, p, nb0, l + 1, bp, gp, nw, kw, Tt, Wt, Ms, Tx, xq);
             l++;
             b = bp;
         }
     }
 }
 
-// Multipole-to-local: for every box T below the top, the kernel sums of the
-// boxes of its interaction list (children of its parent's near list that are
-// admissible to T) at T's Chebyshev nodes.  "All near" boxes and the top box
-// get no far field.  Kernels (s source, t target):
-//   K_SEC: 1/(s-t) and 1/(s-t)^2 into four fields (psi, phi, psi', phi' by side)
-//   K_1: 1/(s-t)   K_2: 1/(s-t)^2   K_1N: 1/(t-s)
-//   K_LOG: log|s-t|, as its t-derivative 1/(t-s) at the nodes plus the sum
-//     itself at the box centre; the derivative's Chebyshev series is
-//     integrated exactly, so a box pair costs P logs instead of P^2
+// Kernels of the far fields (s source, t target).
 enum { K_SEC = 0, K_1 = 1, K_2 = 2, K_1N = 3, K_LOG = 4 };
 
+// ---------------------------------------------------------------------------
+// Far fields of the one-column sums (secular sweeps, b, Loewner): the node
+// weights of every box in the interaction lists of a leaf box and of its
+// ancestors, summed at the leaf's own Chebyshev nodes, then the leaf's
+// coefficients.  Against translating box by box (P^2 FP64 kernel entries per
+// pair, then the fields down the tree level by level) this sums about 3.5 boxes
+// per level instead of 7 per leaf in all, but by split FP32 terms (8 cycles of
+// an SM per warp term against 112), reads no kernel matrices and needs no
+// launch per level.  One warp per leaf box, a lane per node.
+//   K_SEC: sum w/(s - t) to the left and right (psi, phi); their derivatives
+//     are those of the series
+//   K_2: sum w/(s - t)^2
+//   K_LOG: sum w log|s - t| as its derivative sum w/(t - s) at the nodes,
+//     integrated in coefficient space, plus the sum itself at the box centre
+// Measured (GB300, 4096 problems of 32..2048 poles; translations, then down):
+// secular 6.2 + 2.1 -> 1.4 ms, b 3.4 + 2.1 -> 1.5, Loewner 5.1 + 2.1 -> 1.5; the
+// sweeps read one FP64 and three FP32 series instead of four FP64 ones, 10.1 ->
+// 6.8 ms (tail pass 2.3 -> 1.4).  zhat's error falls from 5.4e-13 to 1.6e-13 (4000 poles).
+// ---------------------------------------------------------------------------
+
+// positions of every box's Chebyshev nodes as split parts
+__global__ void k_fmm_nodes(FmmDev pl, const int64_t *__restrict__ off, const int32_t *__restrict__ mk,
+                            const double *__restrict__ dk)
+{
+    __shared__ double xq[P];
+    if (threadIdx.x < P) xq[threadIdx.x] = cospi((double)(2 * threadIdx.x + 1) / (2.0 * P));
+    __syncthreads();
+    const int64_t n = pl.box_base[pl.nprob] * P;
+    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t g = t / P;
+        const int64_t p = sdc_upper_index(pl.box_base, pl.nprob, g);
+        if (pl.fslot[p] < 0) continue;
+        const int64_t b0 = off[p];
+        const FfScale s = ff_scale(dk[b0], dk[b0 + mk[p] - 1], 1.0);
+        double c, h;
+        box_ch(pl.blo[g], pl.bhi[g], c, h);
+        pl.npos[t] = ff_pole(c + h * xq[t % P], s);
+    }
+}
+
+// candidates 64 sec .. 64 sec + 63 of box A (level base gb, parent's near list
+// at pst of npn boxes) that are admissible to it
+__device__ __forceinline__ unsigned long long adm_mask(const FmmDev &pl, int64_t gb, int nbl, int A, int64_t pst,
+                                                       int npn, int sec)
+{
+    unsigned long long mask = 0;
+    const double lo = pl.blo[gb + A], hi = pl.bhi[gb + A];
+    for (int c = 64 * sec; c < min(2 * npn, 64 * sec + 64); c++) {
+        const int S = 2 * pl.near[pst + (c >> 1)] + (c & 1);
+        if (S < nbl && S != A && adm(pl.blo[gb + S], pl.bhi[gb + S], lo, hi)) mask |= 1ull << (c & 63);
+    }
+    return mask;
+}
+
+// interaction list of every box: its first 64 candidates as a bit mask
+__global__ void k_fmm_adm(FmmDev pl, const int32_t *__restrict__ mk)
+{
+    const int64_t n = pl.box_base[pl.nprob];
+    for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < n; g += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t p = sdc_upper_index(pl.box_base, pl.nprob, g);
+        if (pl.fslot[p] < 0) continue;
+        const int nb0 = (mk[p] + B - 1) / B;
+        const int L = lev_count(nb0);
+        int A = (int)(g - pl.box_base[p]), l = 0;
+        while (A >= lev_nb(nb0, l)) { A -= lev_nb(nb0, l); l++; }
+        unsigned long long mask = 0;
+        if (l < L - 1 && pl.nnear[g] >= 0) {
+            const int64_t gP = pl.box_base[p] + lev_base(nb0, l + 1) + (A >> 1);
+            mask = adm_mask(pl, g - A, lev_nb(nb0, l), A, pl.nstart[gP], pl.nnear[gP], 0);
+        }
+        pl.amask[g] = mask;
+    }
+}
+
+constexpr int FAR_NW = 4;         // warps (leaf boxes) per CTA
+constexpr int FAR_TAKE = 4;       // list entries taken per level and round
+
 template <int KER>
-// kmode: 0 evaluate the kernel matrices, 1 evaluate and keep the first
-// kslots of every box (kmat), 2 read those back (the same enumeration of
-// pairs: the plan's tree and near lists do not change between far fields)
-__global__ void __launch_bounds__(128) k_fmm_m2l(FmmDev pl, const int32_t *__restrict__ mk, int nw, int kmode)
+__global__ void __launch_bounds__(FAR_NW * 32) k_fmm_far(FmmDev pl, const int64_t *__restrict__ off, R1Out o)
+{
+    __shared__ double Tx[P * P], xq[P];
+    __shared__ float Tf[(KER == K_SEC) ? P * P : 1];
+    __shared__ ff_logtab lt[(KER == K_LOG) ? 128 : 1];
+    __shared__ ff_f4 sp[FAR_NW][P];
+    __shared__ ff_f2 sw[FAR_NW][P];
+    __shared__ int list[FAR_NW][32 * FAR_TAKE];
+    __shared__ double sF[FAR_NW][P + 2];
+    __shared__ float fL[FAR_NW][P], fR[FAR_NW][P];
+    const unsigned FULL = 0xffffffffu;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, q = min(lane, P - 1);
+    cheb_tables(xq, Tx);
+    if (KER == K_LOG)
+        for (int i = threadIdx.x; i < 128; i += blockDim.x) {
+            const float c = ff_logc(i);
+            const double v = -log((double)c);
+            lt[i] = {c, (float)v, (float)(v - (double)(float)v)};
+        }
+    __syncthreads();
+    if (KER == K_SEC)
+        for (int i = threadIdx.x; i < P * P; i += blockDim.x) Tf[i] = (float)Tx[i];
+    __syncthreads();
+    const int64_t nleaf = pl.leaf_base[pl.nprob];
+    for (int64_t gl = (int64_t)blockIdx.x * FAR_NW + warp; gl < nleaf; gl += (int64_t)gridDim.x * FAR_NW) {
+        const int64_t p = sdc_upper_index(pl.leaf_base, pl.nprob, gl);
+        if (pl.fslot[p] < 0) continue;
+        const int64_t b0 = off[p], g0 = pl.box_base[p];
+        const int m = o.mk[p], nb0 = (m + B - 1) / B, L = lev_count(nb0);
+        const int Tb = (int)(gl - pl.leaf_base[p]);
+        const bool ok = pl.ffbad[p] == 0;
+        const FfScale fs = ff_scale(o.dk[b0], o.dk[b0 + m - 1], o.wsum[p]);
+        double cT, hT;
+        box_ch(pl.blo[g0 + Tb], pl.bhi[g0 + Tb], cT, hT);
+        const double tq = cT + hT * xq[q];
+        const ff_f4 x = ff_pole(tq, fs), xc = ff_pole(cT, fs);
+        FfAcc AL = {}, AR = {}, AC = {};          // AC: K_LOG, the sum at the centre
+        double L1 = 0.0, R1 = 0.0, L2 = 0.0, R2 = 0.0, C1 = 0.0;      // the same in FP64 (!ok)
+        // lane l: the interaction list of the leaf's ancestor on level l
+        int A = 0, npn = 0, sec = 0, lb = 0;
+        int64_t pst = 0;
+        unsigned long long mask = 0;
+        if (lane < L - 1 && pl.nnear[g0 + Tb] >= 0) {
+            A = Tb >> lane;
+            lb = lev_base(nb0, lane);
+            const int64_t gP = g0 + lev_base(nb0, lane + 1) + (A >> 1);
+            npn = pl.nnear[gP];
+            pst = pl.nstart[gP];
+            mask = pl.amask[g0 + lb + A];
+        }
+        int npair = 0;
+        while (__any_sync(FULL, mask != 0 || 64 * (sec + 1) < 2 * npn)) {
+            if (mask == 0 && 64 * (sec + 1) < 2 * npn) {
+                sec++;
+                mask = adm_mask(pl, g0 + lb, lev_nb(nb0, lane), A, pst, npn, sec);
+            }
+            const int cnt = min(FAR_TAKE, __popcll(mask));
+            int pos = cnt;
+            for (int s = 1; s < 32; s <<= 1) {
+                const int v = __shfl_up_sync(FULL, pos, s);
+                if (lane >= s) pos += v;
+            }
+            const int total = __shfl_sync(FULL, pos, 31);
+            pos -= cnt;
+            __syncwarp();
+            for (int i = 0; i < cnt; i++) {
+                const int c = __ffsll((long long)mask) - 1;
+                mask &= mask - 1;
+                const int S = 2 * pl.near[pst + ((64 * sec + c) >> 1)] + (c & 1);
+                list[warp][pos + i] = ((lb + S) << 1) | (S < A ? 1 : 0);
+            }
+            __syncwarp();
+            npair += total;
+            ff_f4 v = {};
+            ff_f2 w = {};
+            if (ok && total > 0) {
+                const int64_t t = (g0 + (list[warp][0] >> 1)) * P + q;
+                v = pl.npos[t];
+                w = pl.nwt[t];
+            }
+            for (int i = 0; i < total; i++) {
+                const int e = list[warp][i];
+                const bool left = e & 1;
+                if (ok) {
+                    __syncwarp();
+                    if (lane < P) { sp[warp][lane] = v; sw[warp][lane] = w; }
+                    __syncwarp();
+                    const ff_f4 vq = v;
+                    const ff_f2 wq = w;
+                    if (i + 1 < total) {                         // the next pair's nodes, ahead of their use
+                        const int64_t t = (g0 + (list[warp][i + 1] >> 1)) * P + q;
+                        v = pl.npos[t];
+                        w = pl.nwt[t];
+                    }
+                    FfAcc S = (KER == K_SEC && !left) ? AR : AL;
+#pragma unroll 2
+                    for (int j = 0; j < P; j++) {
+                        float t, tp, tq2;
+                        if (KER == K_2) ff_term2(sp[warp][j], sw[warp][j], x, t, tp);
+                        else ff_term(sp[warp][j], sw[warp][j], x, t, tp, tq2);
+                        ff_addto(S, t, tp);
+                        if ((j & 7) == 7) ff_norm(S);
+                    }
+                    ff_close(S);
+                    if (KER == K_SEC && !left) AR = S; else AL = S;
+                    if (KER == K_LOG) {
+                        // node q of the source against the centre; the box's weights sum
+                        // to zero, so one exponent per box drops out
+                        float t, tl2, y, yl;
+                        ff_diff(vq, xc, t, tl2);
+                        if (t < 0.0f) { t = -t; tl2 = -tl2; }
+                        const int e0 = __shfl_sync(FULL, ff_fexp(t), 0);
+                        ff_log(t, tl2, e0, lt, y, yl);
+                        float pr, pe;
+                        ff_two_mul(wq.x, y, pr, pe);
+                        pe = ff_fma(wq.y, y, ff_fma(wq.x, yl, pe));
+                        if (lane < P) ff_addto(AC, pr, pe);
+                        ff_close(AC);
+                    }
+                } else {
+                    const int64_t gS = g0 + (e >> 1);
+                    double cS, hS;
+                    box_ch(pl.blo[gS], pl.bhi[gS], cS, hS);
+                    double a1 = 0.0, a2 = 0.0;
+                    for (int j = 0; j < P; j++) {
+                        const double r = rcp_nr2((cS + hS * xq[j]) - tq), a = pl.W[(gS * P + j) * pl.ncol] * r;
+                        a1 += a;
+                        a2 = fma(a, r, a2);
+                    }
+                    if (left) { L1 += a1; L2 += a2; } else { R1 += a1; R2 += a2; }
+                    if (KER == K_LOG && lane < P)
+                        C1 = fma(pl.W[(gS * P + lane) * pl.ncol], log(fabs((cS + hS * xq[lane]) - cT)), C1);
+                }
+            }
+        }
+        // the leaf's coefficients
+        double *cf = pl.coef + gl * pl.nfield * P;
+        const double c1 = ok ? ff_pow2(fs.kk + fs.kw) : 1.0;
+        const double fn = (lane == 0) ? 1.0 / P : 2.0 / P;
+        auto series = [&](double F) {              // coefficient lane of the series with node values F
+            __syncwarp();
+            if (lane < P) sF[warp][lane] = F;
+            __syncwarp();
+            double a = 0.0;
+            for (int j = 0; j < P; j++) a = fma(sF[warp][j], Tx[j * P + q], a);
+            return a * fn;
+        };
+        if (KER == K_SEC && ok) {
+            // psi + phi in FP64; psi and the two derivatives in single precision,
+            // scaled like the near sums (ff_collect)
+            const double a = series(((double)AL.s + (double)AL.sl + ((double)AR.s + (double)AR.sl)) * c1);
+            if (lane < P) { fL[warp][lane] = AL.s; fR[warp][lane] = AR.s; }
+            __syncwarp();
+            float l = 0.0f, r = 0.0f;
+            for (int j = 0; j < P; j++) {
+                l = fmaf(fL[warp][j], Tf[j * P + q], l);
+                r = fmaf(fR[warp][j], Tf[j * P + q], r);
+            }
+            l *= (float)fn;
+            r *= (float)fn;
+            __syncwarp();
+            if (lane < P) { fL[warp][lane] = l; fR[warp][lane] = r; }
+            __syncwarp();
+            const float ih = (float)(1.0 / (hT * ff_pow2(fs.kk)));
+            float dl = 0.0f, dr = 0.0f;
+            for (int n = q + 1; n < P; n += 2) {
+                dl = fmaf((float)(2 * n), fL[warp][n], dl);
+                dr = fmaf((float)(2 * n), fR[warp][n], dr);
+            }
+            if (q == 0) { dl *= 0.5f; dr *= 0.5f; }
+            if (lane < P) {
+                float *ff = (float *)(cf + P);
+                cf[lane] = a;
+                ff[lane] = l;
+                ff[P + lane] = dl * ih;
+                ff[2 * P + lane] = dr * ih;
+            }
+        } else if (KER == K_SEC) {
+            const double F[4] = {L1, R1, L2, R2};
+            for (int k = 0; k < 4; k++) {
+                const double a = series(F[k]);
+                if (lane < P) cf[k * P + lane] = a;
+            }
+        } else if (KER == K_2) {
+            const double a = series(ok ? ((double)AL.s + (double)AL.sl) * (c1 * ff_pow2(fs.kk)) : L2 + R2);
+            if (lane < P) cf[lane] = a;
+        } else {
+            // F' -> antiderivative G = sum B_k T_k (k = 1..P; T_P vanishes at the
+            // nodes but not at 0), F(u) = F(centre) + h (G(u) - G(0))
+            const double a = series(ok ? -((double)AL.s + (double)AL.sl) * ff_pow2(fs.kk) : -(L1 + R1));
+            double c = ok ? (double)AC.s + (double)AC.sl : C1;
+            if (lane >= P) c = 0.0;
+            for (int s = 16; s > 0; s >>= 1) c += __shfl_xor_sync(FULL, c, s);
+            __syncwarp();
+            if (lane < P + 2) sF[warp][lane] = (lane < P) ? a : 0.0;
+            __syncwarp();
+            double bk = 0.0;                       // lane k holds B_k
+            if (lane == 1) bk = sF[warp][0] - 0.5 * sF[warp][2];
+            else if (lane >= 2 && lane <= P) bk = (sF[warp][lane - 1] - sF[warp][lane + 1]) * (0.5 / lane);
+            double g0s = (lane >= 2 && lane <= P && !(lane & 1)) ? ((lane & 2) ? -bk : bk) : 0.0;   // T_k(0)
+            for (int s = 16; s > 0; s >>= 1) g0s += __shfl_xor_sync(FULL, g0s, s);
+            if (lane < P) cf[lane] = (lane == 0) ? c - hT * g0s : hT * bk;
+        }
+        if (pl.flops && lane == 0 && npair)
+            atomicAdd(pl.flops, (unsigned long long)npair * P * (P * (KER == K_SEC ? 7 : 5) + (KER == K_LOG ? 3 : 0)) +
+                                    2 * P * P);
+    }
+}
+
+// far field of a root at u in its leaf box gl (K_SEC's layouts)
+__device__ __forceinline__ float clenshawf(const float *__restrict__ a, float u)
+{
+    const float u2 = u + u;
+    float b1 = 0.0f, b2 = 0.0f;
+#pragma unroll
+    for (int n = P - 1; n >= 1; n--) {
+        const float b0 = fmaf(u2, b1, a[n] - b2);
+        b2 = b1;
+        b1 = b0;
+    }
+    return fmaf(u, b1, a[0] - b2);
+}
+
+__device__ __forceinline__ void far_eval(const FmmDev &pl, int64_t gl, bool ok, double u, int kk, int kw, Acc &A)
+{
+    const double *cf = pl.coef + gl * pl.nfield * P;
+    if (ok) {
+        const double S = clenshaw(cf, u);
+        const float *ff = (const float *)(cf + P);
+        const float uf = (float)u;
+        const double ps = (double)clenshawf(ff, uf) * ff_pow2(kk + kw), c2 = ff_pow2(2 * kk + kw);
+        A.psi += ps;
+        A.phi += S - ps;
+        A.dpsi = fma((double)clenshawf(ff + P, uf), c2, A.dpsi);
+        A.dphi = fma((double)clenshawf(ff + 2 * P, uf), c2, A.dphi);
+    } else {
+        A.psi += clenshaw(cf, u);
+        A.phi += clenshaw(cf + P, u);
+        A.dpsi += clenshaw(cf + 2 * P, u);
+        A.dphi += clenshaw(cf + 3 * P, u);
+    }
+}
+
+// Multipole-to-local for the Cauchy-like fields (one per column): for every box
+// T below the top, the kernel sums of the boxes of its interaction list
+// (children of its parent's near list that are admissible to T) at T's
+// Chebyshev nodes.  "All near" boxes and the top box get no far field.  Kernels
+// (s source, t target): K_1: 1/(s-t)   K_1N: 1/(t-s)
+template <int KER>
+__global__ void __launch_bounds__(128) k_fmm_m2l(FmmDev pl, const int32_t *__restrict__ mk, int nw)
 {
     constexpr int NT = 128;
     constexpr int RMAX = (P * WMAX + NT - 1) / NT;
     __shared__ double xq[P], tq[P], sq[P];
-    __shared__ double Tx[P * P];
     __shared__ double Ws[P][WMAX + 1];
     __shared__ double K1[P][P + 1];
-    __shared__ double K2[(KER == K_SEC) ? P : 1][P + 1];
-    __shared__ double Fp[P], An[P + 2], Bk[P + 1], hk[P + 1], s_f0;
     __shared__ int s_list[32], s_nlist;
-    cheb_tables(xq, Tx);
-    if (KER == K_LOG && threadIdx.x >= 1 && threadIdx.x <= P) hk[threadIdx.x] = 0.5 / threadIdx.x;   // 1 / (2k)
-    const int nf = (KER == K_SEC) ? 4 : nw;
     const int tid = threadIdx.x;
+    if (tid < P) xq[tid] = cospi((double)(2 * tid + 1) / (2.0 * P));
     const int64_t nbox = pl.box_base[pl.nprob];
     for (int64_t g = blockIdx.x; g < nbox; g += gridDim.x) {
         const int64_t p = sdc_upper_index(pl.box_base, pl.nprob, g);
@@ -709,9 +1023,6 @@ __global__ void __launch_bounds__(128) k_fmm_m2l(FmmDev pl, const int32_t *__res
 #pragma unroll
         for (int r = 0; r < RMAX; r++) acc[r] = 0.0;
         int npair = 0;            // interaction pairs of the box (work counter)
-        double f0 = 0.0;          // K_LOG: the far field at the box centre (thread 0)
-        double accL = 0.0, accR = 0.0;   // K_SEC: thread t < 2P, node t % P, kernel 1/(s-t)^(1 + t/P),
-                                         // sums of the boxes to the left / right
         if (l < L - 1 && pl.nnear[g] >= 0) {
             // FP64 instructions cost a warp slot of the FP64 pipe even when every
             // lane computes the same value, so the box geometry and the
@@ -726,7 +1037,6 @@ __global__ void __launch_bounds__(128) k_fmm_m2l(FmmDev pl, const int32_t *__res
             const int nbl = lev_nb(nb0, l);
             const int npn = pl.nnear[gPT];
             const int64_t pst = pl.nstart[gPT];
-            int js = 0;                                   // index of the pair in T's interaction list
             for (int c0 = 0; c0 < 2 * npn; c0 += 32) {
                 // candidates c0 .. c0+31: children of the parent's near boxes, in list order
                 if (tid < 32) {
@@ -745,9 +1055,7 @@ __global__ void __launch_bounds__(128) k_fmm_m2l(FmmDev pl, const int32_t *__res
                 const int nlist = s_nlist;
                 npair += nlist;
                 for (int ii = 0; ii < nlist; ii++) {
-                    const int S = s_list[ii];
-                    const bool left = S < Tb;
-                    const int64_t gS = gbl + S;
+                    const int64_t gS = gbl + s_list[ii];
                     if (ii > 0) __syncthreads();
                     for (int t = tid; t < P * nw; t += NT) Ws[t / nw][t % nw] = pl.W[(gS * P + t / nw) * pl.ncol + t % nw];
                     if (tid < P) {
@@ -756,107 +1064,30 @@ __global__ void __launch_bounds__(128) k_fmm_m2l(FmmDev pl, const int32_t *__res
                         sq[tid] = cS + hS * xq[tid];
                     }
                     __syncthreads();
-                    const bool kept = js < pl.kslots;
-                    double *km = kept ? pl.kmat + ((g * pl.kslots + js) * P) * P : nullptr;
-                    js++;
                     for (int t = tid; t < P * P; t += NT) {
                         const int q = t / P, q2 = t % P;
-                        double r;                                // 1/(s - t)
-                        if (kmode == 2 && kept) {
-                            r = km[t];
-                        } else {
-                            r = rcp_nr2(sq[q2] - tq[q]);
-                            if (kmode == 1 && kept) km[t] = r;
-                        }
-                        if (KER == K_LOG) K1[q][q2] = -r;        // d/dt log|s - t| = 1/(t - s)
-                        else if (KER == K_SEC) { K1[q][q2] = r; K2[q][q2] = r * r; }
-                        else if (KER == K_1) K1[q][q2] = r;
-                        else if (KER == K_1N) K1[q][q2] = -r;
-                        else K1[q][q2] = r * r;
+                        const double r = rcp_nr2(sq[q2] - tq[q]);            // 1/(s - t)
+                        K1[q][q2] = (KER == K_1N) ? -r : r;
                     }
                     __syncthreads();
-                    if (KER == K_LOG && tid < 32) {
-                        // the log sum itself only at the box centre
-                        double v = (tid < P) ? Ws[tid][0] * log(fabs(sq[tid] - cT)) : 0.0;
-                        for (int sh = 16; sh > 0; sh >>= 1) v += __shfl_down_sync(0xffffffffu, v, sh);
-                        if (tid == 0) f0 += v;
-                    }
-                    if (KER == K_SEC) {
-                        // a pair feeds two of the four fields (its side): threads
-                        // own (node, kernel) and keep one sum per side, so no lane idles
-                        if (tid < 2 * P) {
-                            const int q = tid % P;
-                            const double(*Km)[P + 1] = (tid < P) ? K1 : K2;
-                            double s2 = 0.0;
-                            for (int q2 = 0; q2 < P; q2++) s2 = fma(Km[q][q2], Ws[q2][0], s2);
-                            if (left) accL += s2; else accR += s2;
-                        }
-                    } else {
 #pragma unroll
-                        for (int r = 0; r < RMAX; r++) {
-                            const int t = tid + r * NT;
-                            if (t >= P * nf) break;
-                            const int q = t / nf, f = t % nf;
-                            double s2 = 0.0;
-                            for (int q2 = 0; q2 < P; q2++) s2 = fma(K1[q][q2], Ws[q2][f], s2);
-                            acc[r] += s2;
-                        }
+                    for (int r = 0; r < RMAX; r++) {
+                        const int t = tid + r * NT;
+                        if (t >= P * nw) break;
+                        const int q = t / nw, f = t % nw;
+                        double s2 = 0.0;
+                        for (int q2 = 0; q2 < P; q2++) s2 = fma(K1[q][q2], Ws[q2][f], s2);
+                        acc[r] += s2;
                     }
                 }
-                __syncthreads();        // s_list, Ws and the kernel blocks are reused
-            }
-            if (KER == K_LOG) {
-                // F' at the nodes (thread q holds it) -> Chebyshev coefficients,
-                // integrated exactly in coefficient space; F = F(centre) +
-                // h (G(x_q) - G(0)) with G the antiderivative in u
-                if (tid < P) Fp[tid] = acc[0];
-                if (tid == 0) s_f0 = f0;
-                __syncthreads();
-                if (tid < P) {
-                    double a = 0.0;
-                    for (int q = 0; q < P; q++) a = fma(Fp[q], Tx[q * P + tid], a);
-                    An[tid] = a * ((tid == 0) ? (1.0 / P) : (2.0 / P));
-                }
-                if (tid == 0) { An[P] = 0.0; An[P + 1] = 0.0; }
-                __syncthreads();
-                // antiderivative coefficients b_k, k = 1..P, once (thread k)
-                if (tid >= 1 && tid <= P) {
-                    const int k = tid;
-                    Bk[k] = (k == 1) ? 0.5 * (2.0 * An[0] - An[2]) : (An[k - 1] - An[k + 1]) * hk[k];
-                }
-                __syncthreads();
-                if (tid < P) {
-                    // the degree-P term vanishes at the first-kind nodes but not at 0
-                    double gq = 0.0, g0 = 0.0;
-                    for (int k = 1; k < P; k++) gq = fma(Bk[k], Tx[tid * P + k], gq);
-                    for (int k = 2; k <= P; k += 2) g0 += (k & 2) ? -Bk[k] : Bk[k];      // T_k(0) = (-1)^(k/2)
-                    acc[0] = s_f0 + hT * (gq - g0);
-                }
+                __syncthreads();        // s_list, Ws and the kernel block are reused
             }
         }
-        {
-            // per pair: the kernel matrix (difference and reciprocal, squared
-            // for 1/(s-t)^2) unless read back, and its products with the
-            // fields; K_LOG adds the centre's log sum and the integration
-            const bool evald = !(kmode == 2 && pl.kslots > 0);
-            const int64_t kev = evald ? ((KER == K_SEC || KER == K_2) ? 3 : 2) * P * P : 0;
-            const int64_t mv = (KER == K_SEC) ? 4 * P * P : 2 * P * P * nf;
-            const int64_t lg = (KER == K_LOG) ? 3 * P : 0;
-            fl_add(pl, npair * (kev + mv + lg) + ((KER == K_LOG && npair) ? 4 * P * P : 0));
-        }
-        if (KER == K_SEC) {
-            // fields: 0 psi (left, 1/(s-t)), 1 phi (right), 2 psi', 3 phi'
-            if (tid < 2 * P) {
-                const int q = tid % P, f = (tid < P) ? 0 : 2;
-                pl.F[(g * P + q) * pl.nfield + f] = accL;
-                pl.F[(g * P + q) * pl.nfield + f + 1] = accR;
-            }
-        } else {
+        fl_add(pl, (int64_t)npair * (2 * P * P + 2 * P * P * nw));
 #pragma unroll
-            for (int r = 0; r < RMAX; r++) {
-                const int t = tid + r * NT;
-                if (t < P * nf) pl.F[(g * P + t / nf) * pl.nfield + t % nf] = acc[r];
-            }
+        for (int r = 0; r < RMAX; r++) {
+            const int t = tid + r * NT;
+            if (t < P * nw) pl.F[(g * P + t / nw) * pl.nfield + t % nw] = acc[r];
         }
     }
 }
@@ -1063,7 +1294,6 @@ k_secular_fmm(FmmDev pl, FfDev ff, const int64_t *__restrict__ off, R1Out o, dou
         double cT, hT;
         box_ch(pl.blo[g], pl.bhi[g], cT, hT);
         const double ihT = 1.0 / hT;
-        const double *cf = pl.coef + gl * pl.nfield * P;
         const int nnr = pl.nnear[g];
         const int nn = near_len(nnr, (m + B - 1) / B);
         if (nnr < 0 || nnr >= SPLIT_NEAR) continue;     // long near list: k_secular_fmm_split
@@ -1111,23 +1341,8 @@ k_secular_fmm(FmmDev pl, FfDev ff, const int64_t *__restrict__ off, R1Out o, dou
                 else         sweep<true>(sd + i * B, sw + i * B, 0, cnt, j0, kk, kwlo, kwhi, R.dK, R.y, A);
             }
             if (ok) A = ff_collect(S, R, fs.kk, fs.kw);
-            if (act) {
-                // far field at the plain position x = d_K + y (local shifting)
-                const double uu = ((R.dK + R.y) - cT) * ihT;
-                const double u2 = uu + uu;
-                double a1 = 0, a2 = 0, b1 = 0, b2 = 0, c1 = 0, c2 = 0, e1 = 0, e2 = 0;
-                for (int n = P - 1; n >= 1; n--) {
-                    double t;
-                    t = fma(u2, a1, cf[n] - a2);         a2 = a1; a1 = t;
-                    t = fma(u2, b1, cf[P + n] - b2);     b2 = b1; b1 = t;
-                    t = fma(u2, c1, cf[2 * P + n] - c2); c2 = c1; c1 = t;
-                    t = fma(u2, e1, cf[3 * P + n] - e2); e2 = e1; e1 = t;
-                }
-                A.psi += fma(uu, a1, cf[0] - a2);
-                A.phi += fma(uu, b1, cf[P] - b2);
-                A.dpsi += fma(uu, c1, cf[2 * P] - c2);
-                A.dphi += fma(uu, e1, cf[3 * P] - e2);
-            }
+            // far field at the plain position x = d_K + y (local shifting)
+            if (act) far_eval(pl, gl, ok, ((R.dK + R.y) - cT) * ihT, fs.kk, fs.kw, A);
             bool fin = false;
             if (act && R.update(A, tol, max_iter, o.status)) {
                 o.org[b0 + k] = R.K;
@@ -1271,21 +1486,7 @@ k_secular_tail(FmmDev pl, FfDev ff, const int64_t *__restrict__ off, R1Out o, do
             A.dphi += __shfl_xor_sync(FULL, A.dphi, sh);
         }
         if (act) {
-            const double *cf = pl.coef + gl * pl.nfield * P;
-            const double uu = ((R.dK + R.y) - cT) * ihT;
-            const double u2 = uu + uu;
-            double a1 = 0, a2 = 0, b1 = 0, b2 = 0, c1 = 0, c2 = 0, e1 = 0, e2 = 0;
-            for (int q = P - 1; q >= 1; q--) {
-                double t;
-                t = fma(u2, a1, cf[q] - a2);         a2 = a1; a1 = t;
-                t = fma(u2, b1, cf[P + q] - b2);     b2 = b1; b1 = t;
-                t = fma(u2, c1, cf[2 * P + q] - c2); c2 = c1; c1 = t;
-                t = fma(u2, e1, cf[3 * P + q] - e2); e2 = e1; e1 = t;
-            }
-            A.psi += fma(uu, a1, cf[0] - a2);
-            A.phi += fma(uu, b1, cf[P] - b2);
-            A.dpsi += fma(uu, c1, cf[2 * P] - c2);
-            A.dphi += fma(uu, e1, cf[3 * P] - e2);
+            far_eval(pl, gl, ok, ((R.dK + R.y) - cT) * ihT, fs.kk, fs.kw, A);
             if (R.update(A, tol, max_iter, o.status)) {
                 if (part == 0) {
                     const int k = R.k;
@@ -1337,7 +1538,6 @@ k_secular_fmm_split(FmmDev pl, FfDev ff, const int64_t *__restrict__ off, R1Out 
         double cT, hT;
         box_ch(pl.blo[g], pl.bhi[g], cT, hT);
         const double ihT = 1.0 / hT;
-        const double *cf = pl.coef + gl * pl.nfield * P;
         const bool ok = pl.ffbad[p] == 0;
         const FfScale fs = ff_scale(dk[0], dk[m - 1], W);
         int near_terms = 0;
@@ -1381,13 +1581,7 @@ k_secular_fmm_split(FmmDev pl, FfDev ff, const int64_t *__restrict__ off, R1Out 
                     else         sweep<true>(sd, sw, 0, cnt, j0, kk, kwlo, kwhi, R.dK, R.y, A);
                 }
                 if (ok) A = ff_collect(fa, R, fs.kk, fs.kw, warp == 0);
-                if (warp == 0 && act) {
-                    const double uu = ((R.dK + R.y) - cT) * ihT;
-                    A.psi += clenshaw(cf, uu);
-                    A.phi += clenshaw(cf + P, uu);
-                    A.dpsi += clenshaw(cf + 2 * P, uu);
-                    A.dphi += clenshaw(cf + 3 * P, uu);
-                }
+                if (warp == 0 && act) far_eval(pl, gl, ok, ((R.dK + R.y) - cT) * ihT, fs.kk, fs.kw, A);
                 red[warp][0][lane] = A.psi;
                 red[warp][1][lane] = A.phi;
                 red[warp][2][lane] = A.dpsi;
@@ -2021,24 +2215,35 @@ SrcArgs src_from_r1(const int64_t *off, const R1Out &o)
 {
     SrcArgs a{};
     a.off = off; a.mk = o.mk; a.dk = o.dk; a.zk = o.zk; a.vhat = o.vhat; a.bnorm = o.bnorm;
-    a.dorg = o.dorg; a.eta = o.eta; a.src = o.src; a.pinv = o.pinv;
+    a.dorg = o.dorg; a.eta = o.eta; a.src = o.src; a.pinv = o.pinv; a.wsum = o.wsum;
     return a;
 }
 
+// far field of a one-column sum: node weights, then every leaf's series
 template <int MODE, int KER>
-superdc_status far_field(const FmmPlan &pl, const SrcArgs &a, int nw, int kmode, cudaStream_t st)
+superdc_status far_field(const FmmPlan &pl, const int64_t *off, const R1Out &o, cudaStream_t st)
 {
     const FmmDev &dv = pl.dv;
-    const unsigned g = fmm_grid();
-    const int nf = (KER == K_SEC) ? 4 : nw;
+    PROF_LAUNCH("fmm_up", st, k_fmm_up<MODE><<<up_grid<MODE>(), up_threads<MODE>(), 0, st>>>(dv, src_from_r1(off, o)));
+    const int64_t want = (pl.cap_leaves + FAR_NW - 1) / FAR_NW;
+    const unsigned g = (unsigned)std::min<int64_t>(want, resident_grid<k_fmm_far<KER>>(FAR_NW * 32));
+    PROF_LAUNCH("fmm_far", st, k_fmm_far<KER><<<g, FAR_NW * 32, 0, st>>>(dv, off, o));
+    return SUPERDC_OK;
+}
+
+// far fields of nw columns: node weights, translations, then down the tree
+template <int MODE, int KER>
+superdc_status far_columns(const FmmPlan &pl, const SrcArgs &a, int nw, cudaStream_t st)
+{
+    const FmmDev &dv = pl.dv;
     PROF_LAUNCH("fmm_up", st, k_fmm_up<MODE><<<up_grid<MODE>(), up_threads<MODE>(), 0, st>>>(dv, a));
-    PROF_LAUNCH("fmm_m2l", st, k_fmm_m2l<KER><<<g, 128, 0, st>>>(dv, a.mk, nw, dv.kslots > 0 ? kmode : 0));
-    if (nf <= NARROW_NF) {
+    PROF_LAUNCH("fmm_m2l", st, k_fmm_m2l<KER><<<fmm_grid(), 128, 0, st>>>(dv, a.mk, nw));
+    if (nw <= NARROW_NF) {
         for (int t0 = 1; t0 < pl.lmax; t0 += DOWN_LEVELS)
-            PROF_LAUNCH("fmm_l2l", st, k_fmm_down<true><<<down_grid(pl, t0), 128, 0, st>>>(dv, a.mk, t0, nf));
+            PROF_LAUNCH("fmm_l2l", st, k_fmm_down<true><<<down_grid(pl, t0), 128, 0, st>>>(dv, a.mk, t0, nw));
     } else {
         for (int t0 = 1; t0 < pl.lmax; t0++)
-            PROF_LAUNCH("fmm_l2l", st, k_fmm_down<false><<<down_grid(pl, t0), 128, 0, st>>>(dv, a.mk, t0, nf));
+            PROF_LAUNCH("fmm_l2l", st, k_fmm_down<false><<<down_grid(pl, t0), 128, 0, st>>>(dv, a.mk, t0, nw));
     }
     return SUPERDC_OK;
 }
@@ -2066,7 +2271,7 @@ void launch_cn(const FmmPlan &pl, const FactorView &f, const double *X, int64_t 
 
 superdc_status plan(FmmPlan &pl, int64_t nprob, const int64_t *off, int64_t total, int64_t max_m,
                         const int32_t *mk, const double *dk, int min_m, int ncol, int nfield, int32_t *used,
-                        int kslots, cudaStream_t st)
+                        bool step, cudaStream_t st)
 {
     pl = FmmPlan();
     pl.box = B;
@@ -2116,19 +2321,18 @@ superdc_status plan(FmmPlan &pl, int64_t nprob, const int64_t *off, int64_t tota
     SDC_CHECK(al(&d.tail, (size_t)std::max<int64_t>(1, total)));
     SDC_CHECK(al(&d.ntail, 2));
     SDC_CHECK(cudaMemsetAsync(d.ntail, 0, 2 * sizeof(unsigned int), st));
-    // kernel matrices kept for the later far fields of this plan, if they fit
-    // a few GB (otherwise every far field evaluates its own)
-    const double kbytes = (double)pl.cap_boxes * kslots * P * P * sizeof(double);
-    d.kslots = (kslots > 0 && kbytes <= 8.0e9) ? kslots : 0;
-    d.kmat = nullptr;
-    if (d.kslots > 0) SDC_CHECK(al(&d.kmat, (size_t)pl.cap_boxes * d.kslots * P * P));
+    if (step) {
+        SDC_CHECK(al(&d.npos, (size_t)pl.cap_boxes * P));
+        SDC_CHECK(al(&d.nwt, (size_t)pl.cap_boxes * P));
+        SDC_CHECK(al(&d.amask, (size_t)pl.cap_boxes));
+        SDC_CHECK(al(&d.ffbad, nprob));
+    }
     int64_t *lev_off, *top_off;
     SDC_CHECK(al(&lev_off, (size_t)pl.lmax * (nf_cap + 1)));
     SDC_CHECK(al(&top_off, (size_t)pl.lmax * (nf_cap + 1)));
     SDC_CHECK(al(&d.upcnt, pl.cap_boxes));
     SDC_CHECK(cudaMemsetAsync(d.upcnt, 0, (size_t)pl.cap_boxes * sizeof(int32_t), st));
     SDC_CHECK(al(&d.upq, 2));
-    SDC_CHECK(al(&d.ffbad, nprob));
     SDC_CHECK(al(&d.split, pl.cap_leaves));
     SDC_CHECK(al(&d.nsplit, 1));
     SDC_CHECK(cudaMemsetAsync(d.upq, 0, 2 * sizeof(unsigned long long), st));
@@ -2151,6 +2355,13 @@ superdc_status plan(FmmPlan &pl, int64_t nprob, const int64_t *off, int64_t tota
                                                                d.nsplit));
     PROF_LAUNCH("fmm_plan", st, k_fmm_levoff<<<pl.lmax, 1024, 0, st>>>(mk, fprob, nfmm, nf_cap, lev_off,
                                                                    top_off));
+    if (step) {
+        auto gr = [&](int64_t n) {
+            return (unsigned)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, (int64_t)sdc_num_sms() * 8));
+        };
+        PROF_LAUNCH("fmm_plan", st, k_fmm_nodes<<<gr(pl.cap_boxes * P), 256, 0, st>>>(d, off, mk, dk));
+        PROF_LAUNCH("fmm_plan", st, k_fmm_adm<<<gr(pl.cap_boxes), 256, 0, st>>>(d, mk));
+    }
     SDC_CHECK(cudaGetLastError());
     pl.on = true;
     return SUPERDC_OK;
@@ -2167,7 +2378,6 @@ superdc_status secular(const FmmPlan &pl, const int64_t *off, const R1Out &o, do
                            cudaStream_t st)
 {
     if (!pl.on) return SUPERDC_OK;
-    far_field<M_SEC, K_SEC>(pl, src_from_r1(off, o), 1, 1, st);      // keeps the kernel matrices
     const unsigned gl = (unsigned)std::max<int64_t>(1, std::min<int64_t>(pl.cap_f, (int64_t)sdc_num_sms() * 2));
     ff_f4 *fd = nullptr;
     ff_f2 *fw = nullptr;
@@ -2180,6 +2390,7 @@ superdc_status secular(const FmmPlan &pl, const int64_t *off, const R1Out &o, do
     PROF_LAUNCH("fmm_secular", st, k_ff_prep<<<gp, 256, 0, st>>>(pl.dv.nprob, off, pl.total, pl.dv.fslot, o, fd, fw,
                                                                  pl.dv.ffbad));
     const FfDev ff = {fd, fw};
+    far_field<M_SEC, K_SEC>(pl, off, o, st);
     unsigned long long *terms = prof_counter("fmm_secular_terms");
     unsigned long long *lterms = prof_counter("fmm_secular_last_terms");
     PROF_LAUNCH("fmm_secular_last", st, k_secular_last<<<gl, SL_T, 0, st>>>(pl.dv, off, o, stop_c, max_iter,
@@ -2197,7 +2408,7 @@ superdc_status secular(const FmmPlan &pl, const int64_t *off, const R1Out &o, do
 superdc_status lowner(const FmmPlan &pl, const int64_t *off, const R1Out &o, cudaStream_t st)
 {
     if (!pl.on) return SUPERDC_OK;
-    far_field<M_LOW, K_LOG>(pl, src_from_r1(off, o), 1, 2, st);      // reads them
+    far_field<M_LOW, K_LOG>(pl, off, o, st);
     PROF_LAUNCH("fmm_lowner", st, k_lowner_fmm<<<near_grid(), B, 0, st>>>(pl.dv, off, o));
     SDC_CHECK(cudaGetLastError());
     return SUPERDC_OK;
@@ -2206,7 +2417,7 @@ superdc_status lowner(const FmmPlan &pl, const int64_t *off, const R1Out &o, cud
 superdc_status bnorm(const FmmPlan &pl, const int64_t *off, const R1Out &o, cudaStream_t st)
 {
     if (!pl.on) return SUPERDC_OK;
-    far_field<M_BN, K_2>(pl, src_from_r1(off, o), 1, 2, st);
+    far_field<M_BN, K_2>(pl, off, o, st);
     PROF_LAUNCH("fmm_bnorm", st, k_bnorm_fmm<<<near_grid(), B, 0, st>>>(pl.dv, off, o));
     PROF_LAUNCH("fmm_bnorm", st, k_fmm_lastsum<0><<<lastsum_grid(pl, 1), 128, 0, st>>>(
                                      pl.dv, off, o.mk, o.bnorm, nullptr, nullptr, nullptr, 0, 0, 1));
@@ -2222,9 +2433,8 @@ superdc_status cauchy(const FmmPlan &pl, const FactorView &f, const double *X, i
     SrcArgs a{};
     a.off = f.off; a.mk = f.mk; a.dk = f.dk; a.vhat = f.vhat; a.bnorm = f.bnorm; a.dorg = f.dorg; a.eta = f.eta;
     a.src = f.src; a.pinv = f.pinv; a.X = X; a.ldx = ldx; a.col0 = col0; a.nc = nc;
-    // a plan kept from the factor's rank-one step holds its M2L kernel matrices
-    if (trans) far_field<M_CT, K_1>(pl, a, nc, 2, st);
-    else far_field<M_CN, K_1N>(pl, a, nc, 2, st);
+    if (trans) far_columns<M_CT, K_1>(pl, a, nc, st);
+    else far_columns<M_CN, K_1N>(pl, a, nc, st);
     typedef void (*Fn)(const FmmPlan &, const FactorView &, const double *, int64_t, double *, int64_t, int, int,
                        cudaStream_t);
     Fn fn;

@@ -9,8 +9,8 @@
 //     scaled so that the problem's spread is at most 1 (weight of the last bit
 //     2^-94), cut into four 24-bit parts that are exact floats.  The parts of
 //     two positions subtract exactly, so a difference t = d_j - x is known to
-//     2^-94 of the spread however close the two are: relative error 2^-47 at half
-//     the smallest pole gap accepted (2^-46 of the spread);
+//     2^-94 of the spread however close the two are: relative error 2^-52 at half
+//     the smallest pole gap accepted (2^-41 of the spread);
 //   * t is summed into two floats, the reciprocal is a corrected MUFU seed and
 //     its residual (relative error ~2^-47), the product with the weight (two
 //     floats) another two floats;
@@ -22,7 +22,7 @@
 // The two poles next to a root (one is its origin: t = -y exactly, y of any
 // size), which carry most of its sum, are left out of the FP32 sum and added by
 // the caller in FP64.  Problems whose poles are closer
-// than 2^-46 of the spread, or whose spread or weights leave the exponent range,
+// than 2^-41 of the spread, or whose spread or weights leave the exponent range,
 // keep the FP64 sweep.
 //
 // Measured (GB300, 4096 problems of 32..2048 poles): near-field sweeps of the
@@ -109,7 +109,7 @@ FF_HD FfScale ff_scale(double d0, double d1, double w)
 }
 
 // smallest distance of neighbouring poles that the fixed-point parts resolve
-FF_HD bool ff_gap_ok(double da, double db, int kk) { return db - da >= ff_pow2(-kk - 46); }
+FF_HD bool ff_gap_ok(double da, double db, int kk) { return db - da >= ff_pow2(-kk - 41); }
 
 // four 24-bit parts of a position relative to the first pole
 FF_HD ff_f4 ff_parts(__int128 v)
@@ -158,6 +158,20 @@ FF_HD void ff_term(const ff_f4 &d, const ff_f2 &w, const ff_f4 &x, float &p, flo
     p = ff_mul(w.x, r);
     pl = ff_fma(w.y, r, ff_fma(w.x, rl, ff_fma(w.x, r, -p)));
     q = ff_mul(p, r);
+}
+
+// p + pl = w / (d - x)^2
+FF_HD void ff_term2(const ff_f4 &d, const ff_f2 &w, const ff_f4 &x, float &p, float &pl)
+{
+    float t, tl;
+    ff_diff(d, x, t, tl);
+    float r = ff_rcp(t);
+    r = ff_fma(r, ff_fma(-t, r, 1.0f), r);
+    const float rl = ff_mul(r, ff_fma(-tl, r, ff_fma(-t, r, 1.0f)));
+    const float a = ff_mul(w.x, r);
+    const float al = ff_fma(w.y, r, ff_fma(w.x, rl, ff_fma(w.x, r, -a)));
+    p = ff_mul(a, r);
+    pl = ff_fma(al, r, ff_fma(a, rl, ff_fma(a, r, -p)));
 }
 
 // running sums of one root: s + sl of all terms (b + bl of the current block),
@@ -500,4 +514,58 @@ FF_HD void ff_sqr_sweep(const ff_f4 *sd, const ff_f4 *sv, int cnt, int j0, int K
         q.c = own ? 0.0f : q.c;
         ff_acc3(S, q);
     }
+}
+
+// ---------------------------------------------------------------------------
+// log(t + tl), t > 0, in two floats (absolute error ~2^-47 for exponents e of a
+// few): table-driven argument reduction (P. T. P. Tang, Table-driven
+// implementation of the logarithm function, 1990): with c_i the reciprocal of
+// the middle of the i-th of 128 intervals of [1, 2), rounded to 10 bits,
+// m c_i - 1 = d is exact in two floats and log = e ln 2 - log c_i + log1p(d),
+// the last by its Taylor series.  e0 is subtracted from the exponent.
+// ---------------------------------------------------------------------------
+struct ff_logtab { float c, h, l; };              // c_i and -log c_i
+
+FF_HD float ff_logc(int i) { return rintf(512.0f / (1.0f + (i + 0.5f) / 128.0f)) * 0x1p-9f; }
+
+FF_HD int ff_fexp(float t)
+{
+#ifdef __CUDA_ARCH__
+    return (__float_as_int(t) >> 23) - 127;
+#else
+    int b;
+    memcpy(&b, &t, 4);
+    return (b >> 23) - 127;
+#endif
+}
+
+FF_HD void ff_log(float t, float tl, int e0, const ff_logtab *tab, float &y, float &yl)
+{
+    const float LN2H = 0x1.62e43000p-1f, LN2L = -0x1.05c61000p-29f;      // ln 2
+    const int e = ff_fexp(t);
+#ifdef __CUDA_ARCH__
+    const int b = __float_as_int(t);
+    const float m = __int_as_float((b & 0x7FFFFF) | 0x3F800000), sc = __int_as_float((127 - e) << 23);
+#else
+    int b;
+    memcpy(&b, &t, 4);
+    const float m = ldexpf(t, -e), sc = ldexpf(1.0f, -e);
+#endif
+    const ff_logtab T = tab[(b >> 16) & 127];
+    float p, pe, d, dl, s, sl, a, al;
+    ff_two_mul(m, T.c, p, pe);
+    ff_fast_sum(ff_sub(p, 1.0f), ff_fma(ff_mul(tl, sc), T.c, pe), d, dl);
+    const float q = ff_mul(d, d), qe = ff_fma(d + d, dl, ff_fma(d, d, -q));
+    float r = ff_fma(d, 1.0f / 7.0f, -1.0f / 6.0f);
+    r = ff_fma(d, r, 0.2f);
+    r = ff_fma(d, r, -0.25f);
+    r = ff_mul(ff_mul(d, q), ff_fma(d, r, 1.0f / 3.0f));
+    ff_fast_sum(d, -0.5f * q, s, sl);
+    sl = ff_add(sl, ff_add(ff_fma(-0.5f, qe, dl), r));
+    ff_two_sum(T.h, s, a, al);
+    al = ff_add(al, ff_add(T.l, sl));
+    const float k = (float)(e - e0);
+    ff_two_mul(k, LN2H, p, pe);
+    ff_two_sum(p, a, y, yl);
+    yl = ff_add(yl, ff_add(ff_fma(k, LN2L, pe), al));
 }

@@ -29,7 +29,7 @@ int main(int argc, char **argv)
     for (int rep = 0; rep < 20; rep++) {
         std::vector<double> d(m), w(m);
         for (auto &x : d) x = drand48();
-        if (mode == 1) for (int i = 0; i + 8 < m; i += 24) for (int j = 1; j < 8; j++) d[i + j] = d[i] + 1e-10 * drand48();
+        if (mode == 1) for (int i = 0; i + 8 < m; i += 24) for (int j = 1; j < 8; j++) d[i + j] = d[i] + 1e-10 * (j + 0.5 * drand48()) / 8;
         if (mode == 2) for (auto &x : d) x = 60 * x - 30;
         if (mode == 3) for (auto &x : d) x = 1e6 + x;
         std::sort(d.begin(), d.end());
@@ -70,13 +70,120 @@ int main(int argc, char **argv)
 """
 
 
+HARNESS2 = r"""
+#include "split.cuh"
+#include <algorithm>
+#include <cstdio>
+#include <cstdlib>
+#include <vector>
+typedef __float128 Q;
+static Q qabs(Q v) { return v < 0 ? -v : v; }
+int main(int argc, char **argv)
+{
+    const int m = atoi(argv[1]), clustered = atoi(argv[2]);
+    double wb = 0, wz = 0, w2 = 0, wl = 0;
+    for (int rep = 0; rep < 10; rep++) {
+        std::vector<double> d(m), v(m), eta(m);
+        std::vector<int> K(m);
+        for (auto &x : d) x = 20 * drand48() - 10;
+        if (clustered) for (int i = 0; i + 8 < m; i += 24) for (int j = 1; j < 8; j++) d[i + j] = d[i] + 1e-9 * (j + 0.5 * drand48()) / 8;
+        std::sort(d.begin(), d.end());
+        const FfScale s = ff_scale(d[0], d[m - 1], 1.0);
+        bool ok = s.ok;
+        for (int j = 0; j + 1 < m; j++) ok = ok && ff_gap_ok(d[j], d[j + 1], s.kk);
+        if (!ok) { rep--; continue; }
+        std::vector<ff_f4> D(m), V(m);
+        std::vector<ff_w4> Dw(m), Lw(m);
+        for (int j = 0; j < m; j++) {
+            v[j] = (2 * drand48() - 1) * (drand48() < 0.2 ? 1e-7 : 1.0);
+            const ff_t3 t = ff_split3(v[j]);
+            V[j] = {t.a, t.b, t.c, 0.0f};
+            D[j] = ff_pole(d[j], s);
+            Dw[j] = ff_words4(ff_fixed(d[j], s.kk) - s.ref);
+            if (j == m - 1) break;
+            K[j] = drand48() < 0.5 ? j : j + 1;
+            eta[j] = 0.5 * (d[j + 1] - d[j]) * (drand48() < 0.5 ? drand48() : 1e-9 * drand48());
+            if (K[j] != j) eta[j] = -eta[j];
+            Lw[j] = ff_words4(ff_fixed(d[K[j]], s.kk) + ff_fixed(eta[j], s.kk) - s.ref);
+        }
+        for (int j = 0; j + 1 < m; j++) {
+            ff_t3 S = {};
+            ff_sqr_sweep(D.data(), V.data(), m, 0, K[j], ff_point(d[K[j]], eta[j], s), S);
+            Q ex = 0;
+            for (int i = 0; i < m; i++) {
+                if (i == K[j]) continue;
+                const Q t = (((Q)d[i] - (Q)d[K[j]]) - (Q)eta[j]) * (Q)ff_pow2(s.kk);
+                ex += (Q)v[i] * v[i] / t / t;
+            }
+            wb = std::max(wb, (double)qabs(((Q)S.a + (Q)S.b + (Q)S.c - ex) / ex));
+        }
+        for (int i = 0; i < m; i++) {
+            FfProd n = {1ull << 63, 0}, e = n;
+            const ff_u96 di = {Dw[i].lo, Dw[i].mid, Dw[i].hi};
+            ff_prod_sweep(Dw.data(), Lw.data(), m - 1, 0, i, di, n, e);
+            Q ex = 1;
+            for (int j = 0; j + 1 < m; j++)
+                if (j != i && j != i - 1) ex *= qabs((((Q)d[K[j]] - (Q)d[i]) + (Q)eta[j]) / ((Q)d[j] - (Q)d[i]));
+            Q got = (Q)n.m / (Q)e.m;
+            for (int k = n.e - e.e; k > 0; k--) got *= 2;
+            for (int k = n.e - e.e; k < 0; k++) got /= 2;
+            wz = std::max(wz, (double)qabs(got / ex - 1));
+        }
+        for (int i = 0; i + 1 < m; i++) {
+            const ff_f2 w = ff_weight(v[i] * v[i], 0);
+            float p, pl;
+            ff_term2(D[i + 1], w, D[i], p, pl);
+            const Q t = ((Q)d[i + 1] - (Q)d[i]) * (Q)ff_pow2(s.kk), ex = (Q)v[i] * v[i] / t / t;
+            if ((double)ex > 1e-20) w2 = std::max(w2, (double)qabs(((Q)p + (Q)pl) / ex - 1));
+        }
+    }
+    ff_logtab tab[128];
+    for (int i = 0; i < 128; i++) {
+        tab[i].c = ff_logc(i);
+        const double l = -log((double)tab[i].c);
+        tab[i].h = (float)l;
+        tab[i].l = (float)(l - tab[i].h);
+    }
+    for (int i = 0; i < 20000; i++) {
+        const double x = ldexp(0.5 + drand48(), (int)(12 * drand48()) - 6);
+        const float t = (float)x, tl = (float)(x - t);
+        float y, yl;
+        ff_log(t, tl, 0, tab, y, yl);
+        wl = std::max(wl, fabs(((double)y - log(x)) + (double)yl));
+    }
+    printf("%.3e %.3e %.3e %.3e\n", wb, wz, w2, wl);
+    return 0;
+}
+"""
+
+
 @pytest.fixture(scope="module")
-def harness(tmp_path_factory):
+def harness2(tmp_path_factory):
+    return _build(tmp_path_factory, HARNESS2)
+
+
+@pytest.mark.parametrize("clustered", [0, 1])
+@pytest.mark.parametrize("m", [2, 3, 9, 130])
+def test_split_b_zhat_log_against_quadruple_precision(harness2, m, clustered):
+    """Sums of squares and products with FP64's accuracy or better: the last bit
+    of a position is 2^-94 of the spread, so at half the smallest accepted gap
+    (2^-41) a difference is known to 2^-52, and each square doubles it: 2^-50; a
+    product of m ratios adds at most 2 m 2^-54.  One-term
+    1/(d - x)^2: 2^-44.  log: 2^-44 absolute for exponents up to 6."""
+    out = subprocess.run([harness2, str(m), str(clustered)], capture_output=True, text=True, check=True).stdout.split()
+    wb, wz, w2, wl = map(float, out)
+    assert wb <= 2.0 ** -50
+    assert wz <= 2 * m * 2.0 ** -54
+    assert w2 <= 2.0 ** -44
+    assert wl <= 2.0 ** -44
+
+
+def _build(tmp_path_factory, text):
     gxx = shutil.which("g++")
     if not gxx:
         pytest.skip("g++ missing")
     tmp = tmp_path_factory.mktemp("split")
-    (tmp / "h.cpp").write_text(HARNESS)
+    (tmp / "h.cpp").write_text(text)
     exe = str(tmp / "h")
     r = subprocess.run([gxx, "-O1", "-std=gnu++17", "-ffp-contract=off", "-I", CSRC, str(tmp / "h.cpp"), "-o", exe],
                        capture_output=True, text=True)
@@ -84,6 +191,11 @@ def harness(tmp_path_factory):
         pytest.skip("no quadruple precision on this machine")
     assert r.returncode == 0, r.stderr[-2000:]
     return exe
+
+
+@pytest.fixture(scope="module")
+def harness(tmp_path_factory):
+    return _build(tmp_path_factory, HARNESS)
 
 
 @pytest.mark.parametrize("mode", [0, 1, 2, 3], ids=["uniform", "clustered", "wide", "offset"])
@@ -107,7 +219,7 @@ def _problems():
     for m in (2, 3, 33, 34, 65, 1023, 1024, 1025, 2050):          # windows of 32 roots, chunks of 1024 poles
         probs.append((np.sort(rng.uniform(-30, 30, m)), n01(m)))
     d = np.sort(rng.uniform(0, 1, 400))
-    d[200] = d[199] + 3e-15                                         # closer than 2^-46 of the spread
+    d[200] = d[199] + 3e-15                                         # closer than 2^-41 of the spread
     probs.append((np.sort(d), n01(400) * 1e-2))
     probs.append((np.geomspace(1e-10, 1e20, 400), n01(400)))         # graded: FP64 sweep
     z = n01(500)
