@@ -1,13 +1,11 @@
-// Cauchy-like factor application kernels (direct tiled evaluator).
-//
+// Application of one batched rank-one factor to a block of columns:
 // Transpose (conquering stage, Algorithm 3; superdcmv with transpose,
 // Algorithm 4):   y_j = b_j sum_i vhat_i x_i / ((d_i - d_{K_j}) - eta_j)
 // Forward (superdcmv without transpose):
 //                 y_i = vhat_i sum_j b_j x_j / ((d_i - d_{K_j}) - eta_j)
-// Every entry uses the shifted difference of eq. (4.28).  One reciprocal per
-// (i, j) pair is shared by all columns of the block; the column sums run as
-// FP64 FMAs in registers, the operands of the other side are staged in shared
-// memory in chunks of TI rows.
+// with the shifted differences of eq. (4.28).  The rotations, the deflated
+// slots and the order of the calls are here; the kept rows' products run on
+// the tensor cores (fmm_columns, k_cm_apply).
 #include "common.cuh"
 #include <algorithm>
 #include "cauchy.cuh"
@@ -16,35 +14,7 @@
 
 namespace {
 
-__device__ __forceinline__ float mufu_rcp(float x)
-{
-    float r;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-    return r;
-}
-
-// full-accuracy FP64 reciprocal: MUFU seed on the mantissa, exponent by
-// integer arithmetic, two Newton-Raphson steps (see rank1.cu)
-__device__ __forceinline__ double rcp2(double t)
-{
-    const int hi = __double2hiint(t);
-    const unsigned lo = (unsigned)__double2loint(t);
-    const unsigned sign = (unsigned)hi & 0x80000000u;
-    const int e = (hi >> 20) & 0x7FF;
-    const unsigned mb = (((unsigned)hi & 0xFFFFFu) << 3) | (lo >> 29);
-    const float rm = mufu_rcp(__uint_as_float(0x3F800000u | mb));
-    const unsigned rb = __float_as_uint(rm);
-    const int E = (int)(rb >> 23) - 127 - (e - 1023) + 1023;
-    const unsigned rmant = rb & 0x7FFFFFu;
-    double r = __hiloint2double((int)(sign | ((unsigned)E << 20) | (rmant >> 3)), (int)(rmant << 29));
-    double q = fma(-t, r, 1.0);
-    r = fma(r, q, r);
-    q = fma(-t, r, 1.0);
-    return fma(r, q, r);
-}
-
-constexpr int TJ = 128;   // outputs per CTA (one per thread)
-constexpr int TI = 128;   // staged rows per chunk
+constexpr int TR = 64;    // kept rows per tile of the application kernels
 
 __global__ void k_tiles_c(int64_t nprob, const int32_t *__restrict__ mk, int tr, int64_t *__restrict__ tile_off)
 {
@@ -110,111 +80,6 @@ __global__ void k_givens(FactorView f, int64_t total, double *X, int64_t ldx, in
     }
 }
 
-// y_j = b_j sum_i vhat_i x_{src_i} / ((d_i - d_{K_j}) - eta_j), written at
-// merged position pinv[j]; columns [col0, col0 + NC) (fewer at the tail)
-template <int NC>
-__global__ void __launch_bounds__(TJ)
-k_cauchy_T(FactorView f, const int64_t *__restrict__ tile_off, const double *__restrict__ X, int64_t ldx,
-           double *__restrict__ Y, int64_t ldy, int col0, int ncols, const int32_t *__restrict__ fslot)
-{
-    __shared__ double sd[TI];
-    __shared__ double sx[NC][TI];
-    const int64_t ntiles = tile_off[f.nprob];
-    const int nc = min(NC, ncols - col0);
-    for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-        const int64_t p = sdc_upper_index(tile_off, f.nprob, tile);
-        if (fslot && fslot[p] >= 0) continue;   // FMM problem (uniform per CTA)
-        const int64_t b0 = f.off[p];
-        const int m = f.mk[p];
-        const int j = (int)(tile - tile_off[p]) * TJ + threadIdx.x;
-        const bool act = j < m;
-        const double dK = act ? f.dorg[b0 + j] : 0.0;
-        const double e = act ? f.eta[b0 + j] : 1.0;
-        double acc[NC];
-#pragma unroll
-        for (int q = 0; q < NC; q++) acc[q] = 0.0;
-        for (int i0 = 0; i0 < m; i0 += TI) {
-            const int cn = min(TI, m - i0);
-            __syncthreads();
-            for (int ii = threadIdx.x; ii < cn; ii += TJ) {
-                const int64_t row = b0 + SDC_IDX(f.src[b0 + i0 + ii], f.off[p + 1] - b0, f.status);
-                const double v = f.vhat[b0 + i0 + ii];
-                sd[ii] = f.dk[b0 + i0 + ii];
-#pragma unroll
-                for (int q = 0; q < NC; q++)
-                    sx[q][ii] = (q < nc) ? v * X[row + (int64_t)(col0 + q) * ldx] : 0.0;
-            }
-            __syncthreads();
-            if (act) {
-                for (int ii = 0; ii < cn; ii++) {
-                    const double r = rcp2((sd[ii] - dK) - e);
-#pragma unroll
-                    for (int q = 0; q < NC; q++) acc[q] = fma(sx[q][ii], r, acc[q]);
-                }
-            }
-        }
-        if (act) {
-            const double bj = f.bnorm[b0 + j];
-            const int64_t row = b0 + SDC_IDX(f.pinv[b0 + j], f.off[p + 1] - b0, f.status);
-#pragma unroll
-            for (int q = 0; q < NC; q++)
-                if (q < nc) Y[row + (int64_t)(col0 + q) * ldy] = bj * acc[q];
-        }
-    }
-}
-
-// y_{src_i} = vhat_i sum_j b_j x_{pinv_j} / ((d_i - d_{K_j}) - eta_j)
-template <int NC>
-__global__ void __launch_bounds__(TJ)
-k_cauchy_N(FactorView f, const int64_t *__restrict__ tile_off, const double *__restrict__ X, int64_t ldx,
-           double *__restrict__ Y, int64_t ldy, int col0, int ncols, const int32_t *__restrict__ fslot)
-{
-    __shared__ double sk[TI], se[TI];
-    __shared__ double sx[NC][TI];
-    const int64_t ntiles = tile_off[f.nprob];
-    const int nc = min(NC, ncols - col0);
-    for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-        const int64_t p = sdc_upper_index(tile_off, f.nprob, tile);
-        if (fslot && fslot[p] >= 0) continue;   // FMM problem (uniform per CTA)
-        const int64_t b0 = f.off[p];
-        const int m = f.mk[p];
-        const int i = (int)(tile - tile_off[p]) * TJ + threadIdx.x;
-        const bool act = i < m;
-        const double di = act ? f.dk[b0 + i] : 0.0;
-        double acc[NC];
-#pragma unroll
-        for (int q = 0; q < NC; q++) acc[q] = 0.0;
-        for (int j0 = 0; j0 < m; j0 += TI) {
-            const int cn = min(TI, m - j0);
-            __syncthreads();
-            for (int jj = threadIdx.x; jj < cn; jj += TJ) {
-                const int64_t row = b0 + SDC_IDX(f.pinv[b0 + j0 + jj], f.off[p + 1] - b0, f.status);
-                const double bj = f.bnorm[b0 + j0 + jj];
-                sk[jj] = f.dorg[b0 + j0 + jj];
-                se[jj] = f.eta[b0 + j0 + jj];
-#pragma unroll
-                for (int q = 0; q < NC; q++)
-                    sx[q][jj] = (q < nc) ? bj * X[row + (int64_t)(col0 + q) * ldx] : 0.0;
-            }
-            __syncthreads();
-            if (act) {
-                for (int jj = 0; jj < cn; jj++) {
-                    const double r = rcp2((di - sk[jj]) - se[jj]);
-#pragma unroll
-                    for (int q = 0; q < NC; q++) acc[q] = fma(sx[q][jj], r, acc[q]);
-                }
-            }
-        }
-        if (act) {
-            const double v = f.vhat[b0 + i];
-            const int64_t row = b0 + SDC_IDX(f.src[b0 + i], f.off[p + 1] - b0, f.status);
-#pragma unroll
-            for (int q = 0; q < NC; q++)
-                if (q < nc) Y[row + (int64_t)(col0 + q) * ldy] = v * acc[q];
-        }
-    }
-}
-
 // deflated slots: identity part of the factor
 __global__ void k_defl_copy(FactorView f, int64_t total, const double *__restrict__ X, int64_t ldx,
                             double *__restrict__ Y, int64_t ldy, int ncols, int trans)
@@ -235,46 +100,6 @@ __global__ void k_defl_copy(FactorView f, int64_t total, const double *__restric
     }
 }
 
-template <template <int> class K>
-struct Dummy {};
-
-// the inner loops run all NC columns: even widths up to 20 (the ranks of
-// typical HSS generators) waste at most one FMA per term
-int pick_nc(int c)
-{
-    if (c <= 20) return std::max(2, (c + 1) & ~1);
-    if (c <= 24) return 24;
-    return 32;
-}
-
-template <int NC>
-void launch_T(const FactorView &f, const int64_t *tile_off, const double *X, int64_t ldx, double *Y, int64_t ldy,
-              int col0, int ncols, unsigned grid, const int32_t *fslot, cudaStream_t st)
-{
-    k_cauchy_T<NC><<<grid, TJ, 0, st>>>(f, tile_off, X, ldx, Y, ldy, col0, ncols, fslot);
-}
-
-template <int NC>
-void launch_N(const FactorView &f, const int64_t *tile_off, const double *X, int64_t ldx, double *Y, int64_t ldy,
-              int col0, int ncols, unsigned grid, const int32_t *fslot, cudaStream_t st)
-{
-    k_cauchy_N<NC><<<grid, TJ, 0, st>>>(f, tile_off, X, ldx, Y, ldy, col0, ncols, fslot);
-}
-
-typedef void (*LaunchFn)(const FactorView &, const int64_t *, const double *, int64_t, double *, int64_t, int, int,
-                         unsigned, const int32_t *, cudaStream_t);
-
-LaunchFn pick(bool trans, int nc)
-{
-    switch (nc) {
-#define SDC_NC(W) case W: return trans ? launch_T<W> : launch_N<W>;
-    SDC_NC(2) SDC_NC(4) SDC_NC(6) SDC_NC(8) SDC_NC(10) SDC_NC(12) SDC_NC(14) SDC_NC(16) SDC_NC(18) SDC_NC(20)
-    SDC_NC(24)
-#undef SDC_NC
-    default: return trans ? launch_T<32> : launch_N<32>;
-    }
-}
-
 superdc_status run(const FactorView &f, int64_t total, double *Xmut, const double *X, int64_t ldx, double *Y,
                    int64_t ldy, int ncols, bool trans, cudaStream_t st, const FmmPlan *shared)
 {
@@ -283,34 +108,21 @@ superdc_status run(const FactorView &f, int64_t total, double *Xmut, const doubl
     int64_t *tile_off = nullptr;
     SdcScratch sc(st);
     SDC_CHECK(sc.get(&tile_off, f.nprob + 1));
-    k_tiles_c<<<1, 1024, 0, st>>>(f.nprob, f.mk, TJ, tile_off);
+    k_tiles_c<<<1, 1024, 0, st>>>(f.nprob, f.mk, TR, tile_off);
     const int gthreads = 128;
     if (trans)
         PROF_LAUNCH("givens", st, k_givens<<<(unsigned)(nsm * 8), gthreads, 0, st>>>(f, total, Xmut, ldx, ncols, 0));
-    // problems whose kept size reaches the threshold: triangular FMM
+    // problems whose kept size reaches the threshold have a box tree: the plan
+    // of this factor's rank-one step when one was kept, else a new one
     FmmPlan fp;
     const int w = std::min(32, ncols);
-    const int box = (w <= 24) ? 32 : 64;
-    // the plan of this factor's rank-one step serves when its boxes and widths fit
-    const bool use_shared = shared && shared->on && shared->box == box && shared->dv.ncol >= w &&
-                            shared->dv.nfield >= w;
+    const bool use_shared = shared && shared->on && shared->dv.ncol >= w;
     if (!use_shared) {
-        // boxes of 32 halve the near field; with many columns the translations
-        // (P^2 per column and box pair) dominate and boxes of 64 halve those
-        superdc_status fs = fmm_plan(fp, f.nprob, f.off, total, f.max_m, f.mk, f.dk, f.fmm_min_m, w, w, nullptr,
-                                     box, false, st);
+        superdc_status fs = fmm_plan(fp, f.nprob, f.off, total, f.max_m, f.mk, f.dk, f.fmm_min_m, w, nullptr, false,
+                                     st);
         if (fs != SUPERDC_OK) { fmm_free(fp, st); return fs; }
     }
-    const FmmPlan &pl = use_shared ? *shared : fp;
-    const int32_t *fslot = pl.on ? pl.dv.fslot : nullptr;
-    superdc_status fs = SUPERDC_OK;
-    const unsigned grid = (unsigned)(nsm * 4);
-    for (int c0 = 0; c0 < ncols; c0 += 32) {
-        const int c = min(32, ncols - c0);
-        LaunchFn fn = pick(trans, pick_nc(c));
-        PROF_LAUNCH("cauchy", st, fn(f, tile_off, X, ldx, Y, ldy, c0, ncols, grid, fslot, st));
-        if (fs == SUPERDC_OK) fs = fmm_cauchy(pl, f, X, ldx, Y, ldy, c0, c, trans, st);
-    }
+    const superdc_status fs = fmm_columns(use_shared ? *shared : fp, f, total, tile_off, X, ldx, Y, ldy, ncols, trans, st);
     PROF_LAUNCH("deflcopy", st, k_defl_copy<<<(unsigned)(nsm * 8), 256, 0, st>>>(f, total, X, ldx, Y, ldy, ncols,
                                                                                   trans ? 1 : 0));
     if (!trans)

@@ -36,18 +36,15 @@ struct FmmDev {
     const int32_t *nnear, *near;           // per box: near-list length (< 0: every source direct); list pool
     const int64_t *nstart;                 // per box: start of its near list in the pool
     double *W, *coef;                      // workspace: node weights, leaf coefficients
-    double *F;                             // workspace: far field at every box's nodes
-    double *lastp;                         // workspace: per leaf box (ncol wide), its sources' share of
-                                           // the sums for the last eigenvalue (outside the tree)
+    double *lastp;                         // workspace: per leaf box, its sources' share of the last
+                                           // eigenvalue's b (outside the tree)
     FmmTail *tail;                         // roots left to the tail pass (capacity: every kept root)
     unsigned int *ntail;                   // their count, then the tail pass's next unclaimed entry
-    // plans of a rank-one step (FP32-split far fields, split.cuh): positions and weights of every box's
-    // Chebyshev nodes, and the first 64 candidates of its interaction list as a bit mask
+    // positions (split.cuh) of every box's Chebyshev nodes, their split weights (plans of a rank-one
+    // step), and the first 64 candidates of the box's interaction list as a bit mask
     ff_f4 *npos;
     ff_f2 *nwt;
     unsigned long long *amask;
-    const int64_t *lev_off;                // per level: prefix of the FMM problems' box counts
-    const int64_t *top_off;                // the same per level counted from each problem's top box
     int32_t *upcnt;                        // per box: children whose moments are done in the current
                                            // upward pass (the last one computes the box; reset by it)
     unsigned long long *upq;               // upward pass: next unclaimed leaf box, CTAs past the end
@@ -56,7 +53,7 @@ struct FmmDev {
     int32_t *ffbad;                        // per problem: 1 if the split FP32 forms (split.cuh) are not
                                            // allowed; written with the secular roots, read by zhat and b
     int64_t cap_f;                         // capacity of the FMM problem list
-    int ncol, nfield;                      // workspace widths
+    int ncol;                              // width of the node weights (columns)
     unsigned long long *flops;             // algorithmic FP64 work of the far fields and of the
                                            // zhat / b / Cauchy-like consumers (profiling only; NULL
                                            // otherwise): FMA 2, other operations 1
@@ -68,21 +65,18 @@ struct FmmPlan {
     int lmax = 0;                          // upper bound on tree levels
     int nb0max = 0;                        // upper bound on leaf boxes per problem
     int64_t total = 0;                     // extent of the row-indexed arrays
-    int box = 0;                           // indices per leaf box (32 or 64) of this plan
     bool on = false;                       // some problem may take the FMM path
     std::vector<void *> bufs;
 };
 
 // Decide per problem (kept size mk >= min_m) and build the box trees from the
 // kept poles dk.  max_m: an upper bound on the problem sizes (-1 unknown).
-// ncol / nfield: widths of the moment and coefficient workspaces.
-// used (may be NULL): per problem 1 if it takes the FMM path, else 0.
-// box: indices per leaf box, 32 or 64 (smaller boxes halve the near field,
-// larger ones halve the number of box pairs whose expansions are translated).
-// step: the plan serves the sums of a rank-one step (secular, zhat, b).
+// ncol: width of the node weights.  used (may be NULL): per problem 1 if it
+// takes the FMM path, else 0.  step: the plan serves the sums of a rank-one step
+// (secular, zhat, b).
 superdc_status fmm_plan(FmmPlan &pl, int64_t nprob, const int64_t *off, int64_t total, int64_t max_m,
-                        const int32_t *mk, const double *dk, int min_m, int ncol, int nfield, int32_t *used,
-                        int box, bool step, cudaStream_t st);
+                        const int32_t *mk, const double *dk, int min_m, int ncol, int32_t *used,
+                        bool step, cudaStream_t st);
 void fmm_free(FmmPlan &pl, cudaStream_t st);
 
 // Roots of the FMM problems (same outputs as the direct secular kernel).
@@ -91,10 +85,12 @@ superdc_status fmm_secular(const FmmPlan &pl, const int64_t *off, const R1Out &o
 // zhat (eq. (4.23) via eq. (4.25)) and b (eq. (4.27)) of the FMM problems.
 superdc_status fmm_lowner(const FmmPlan &pl, const int64_t *off, const R1Out &o, cudaStream_t st);
 superdc_status fmm_bnorm(const FmmPlan &pl, const int64_t *off, const R1Out &o, cudaStream_t st);
-// Columns [col0, col0 + nc) of Y = Qhat^T X (trans) or Y = Qhat X for the FMM
-// problems (layouts as cauchy_apply_T / cauchy_apply_N; X already rotated for trans).
-superdc_status fmm_cauchy(const FmmPlan &pl, const FactorView &f, const double *X, int64_t ldx, double *Y,
-                          int64_t ldy, int col0, int nc, bool trans, cudaStream_t st);
+// Y = Qhat^T X (trans; X already rotated) or Y = Qhat X on the kept rows, every
+// problem (with or without a tree), ncols columns; tile_off: prefix of the
+// problems' tiles of 64 kept rows.
+superdc_status fmm_columns(const FmmPlan &pl, const FactorView &f, int64_t total, const int64_t *tile_off,
+                           const double *X, int64_t ldx, double *Y, int64_t ldy, int ncols, bool trans,
+                           cudaStream_t st);
 
 // Library default of the FMM threshold (kept problem size), and the
 // threshold an option value selects (> 0 itself, 0 the default, < 0 off).

@@ -72,7 +72,8 @@ constexpr int B = FMM_BOX;
 constexpr double FMM_KAPPA = 0.75;
 constexpr int SPLIT_NEAR = 512 / B;   // leaf boxes with this many near boxes (512 poles) or more: CTA-split sweeps
 constexpr int TAIL_X = 12;        // k_secular_fmm hands a box's last roots to the tail pass below this many busy lanes
-constexpr int WMAX = 32;          // widest moment / coefficient block (columns)
+constexpr int WMAX = 32;          // widest moment block (columns)
+constexpr int NFIELD = 4;         // series per leaf box (P doubles each)
 
 // ---------------------------------------------------------------------------
 // tree shape of a problem with m kept indices: nb0 = ceil(m / B) leaf boxes,
@@ -470,67 +471,6 @@ __device__ __forceinline__ void leaf_moments(const FmmDev &pl, const SrcArgs &a,
     fl_add(pl, cnt * ((MODE == M_LOW) ? 4 : 2) * (P - 2) + 2 * cnt * P * nw + 2 * P * P * nw);
 }
 
-// Boxes of level l of the FMM problems, enumerated as (FMM problem f, box b)
-// with b below the widest level-l box count nbl_max (host bound); returns
-// false for slots without a box.
-// Box u of level l over all FMM problems (per-level prefix lev_off[l][f]).
-__device__ __forceinline__ bool level_box(const FmmDev &pl, const int32_t *__restrict__ mk, int l, int64_t u,
-                                          int64_t &p, int &nb0, int &b, int64_t &g)
-{
-    const int nf = *pl.nfmm;
-    const int64_t *lo = pl.lev_off + (int64_t)l * (pl.cap_f + 1);
-    const int64_t f = sdc_upper_index(lo, (int64_t)nf, u);
-    b = (int)(u - lo[f]);
-    p = pl.fprob[f];
-    if (pl.fslot[p] < 0) return false;
-    nb0 = (mk[p] + B - 1) / B;
-    if (l >= lev_count(nb0) || b >= lev_nb(nb0, l)) return false;
-    g = pl.box_base[p] + lev_base(nb0, l) + b;
-    return true;
-}
-
-// per-level prefix of the box counts of the FMM problems (one CTA per level):
-// lev_off by absolute level (leaves 0), top_off by level counted from each
-// problem's top box (top 0)
-__device__ __forceinline__ int levoff_count(int nb0, int l, bool top)
-{
-    const int L = lev_count(nb0);
-    if (l >= L) return 0;
-    return lev_nb(nb0, top ? L - 1 - l : l);
-}
-
-__global__ void k_fmm_levoff(const int32_t *__restrict__ mk, const int32_t *__restrict__ fprob,
-                             const int32_t *__restrict__ nfmm, int64_t cap_f, int64_t *__restrict__ lev_off,
-                             int64_t *__restrict__ top_off)
-{
-    __shared__ int64_t part[1024];
-    const int l = blockIdx.x;
-    const int nf = *nfmm;
-    const int T = blockDim.x;
-    const int per = (nf + T - 1) / T;
-    const int beg = min(nf, (int)threadIdx.x * per), end = min(nf, beg + per);
-    for (int pass = 0; pass < 2; pass++) {
-        const bool top = pass == 1;
-        int64_t *out = (top ? top_off : lev_off) + (int64_t)l * (cap_f + 1);
-        int64_t sum = 0;
-        for (int f = beg; f < end; f++) sum += levoff_count((mk[fprob[f]] + B - 1) / B, l, top);
-        __syncthreads();
-        part[threadIdx.x] = sum;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            int64_t acc = 0;
-            for (int i = 0; i < T; i++) { const int64_t v = part[i]; part[i] = acc; acc += v; }
-            out[nf] = acc;
-        }
-        __syncthreads();
-        int64_t acc = part[threadIdx.x];
-        for (int f = beg; f < end; f++) {
-            out[f] = acc;
-            acc += levoff_count((mk[fprob[f]] + B - 1) / B, l, top);
-        }
-    }
-}
-
 // moments of box g (level l >= 1, index b) from its children's node weights:
 // M_n(parent) = sum_children sum_q W_q(child) T_n(alpha x_q + beta), exact
 // because T_n(alpha u + beta) has degree n < P and the children's weights
@@ -708,7 +648,7 @@ __global__ void k_fmm_nodes(FmmDev pl, const int64_t *__restrict__ off, const in
         const FfScale s = ff_scale(dk[b0], dk[b0 + mk[p] - 1], 1.0);
         double c, h;
         box_ch(pl.blo[g], pl.bhi[g], c, h);
-        pl.npos[t] = ff_pole(c + h * xq[t % P], s);
+        pl.npos[t] = ff_point(c, h * xq[t % P], s);         // not rounded to the spacing of c
     }
 }
 
@@ -785,7 +725,7 @@ __global__ void __launch_bounds__(FAR_NW * 32) k_fmm_far(FmmDev pl, const int64_
         double cT, hT;
         box_ch(pl.blo[g0 + Tb], pl.bhi[g0 + Tb], cT, hT);
         const double tq = cT + hT * xq[q];
-        const ff_f4 x = ff_pole(tq, fs), xc = ff_pole(cT, fs);
+        const ff_f4 x = ff_point(cT, hT * xq[q], fs), xc = ff_pole(cT, fs);
         FfAcc AL = {}, AR = {}, AC = {};          // AC: K_LOG, the sum at the centre
         double L1 = 0.0, R1 = 0.0, L2 = 0.0, R2 = 0.0, C1 = 0.0;      // the same in FP64 (!ok)
         // lane l: the interaction list of the leaf's ancestor on level l
@@ -886,7 +826,7 @@ __global__ void __launch_bounds__(FAR_NW * 32) k_fmm_far(FmmDev pl, const int64_
             }
         }
         // the leaf's coefficients
-        double *cf = pl.coef + gl * pl.nfield * P;
+        double *cf = pl.coef + gl * NFIELD * P;
         const double c1 = ok ? ff_pow2(fs.kk + fs.kw) : 1.0;
         const double fn = (lane == 0) ? 1.0 / P : 2.0 / P;
         auto series = [&](double F) {              // coefficient lane of the series with node values F
@@ -975,7 +915,7 @@ __device__ __forceinline__ float clenshawf(const float *__restrict__ a, float u)
 
 __device__ __forceinline__ void far_eval(const FmmDev &pl, int64_t gl, bool ok, double u, int kk, int kw, Acc &A)
 {
-    const double *cf = pl.coef + gl * pl.nfield * P;
+    const double *cf = pl.coef + gl * NFIELD * P;
     if (ok) {
         const double S = clenshaw(cf, u);
         const float *ff = (const float *)(cf + P);
@@ -990,240 +930,6 @@ __device__ __forceinline__ void far_eval(const FmmDev &pl, int64_t gl, bool ok, 
         A.phi += clenshaw(cf + P, u);
         A.dpsi += clenshaw(cf + 2 * P, u);
         A.dphi += clenshaw(cf + 3 * P, u);
-    }
-}
-
-// Multipole-to-local for the Cauchy-like fields (one per column): for every box
-// T below the top, the kernel sums of the boxes of its interaction list
-// (children of its parent's near list that are admissible to T) at T's
-// Chebyshev nodes.  "All near" boxes and the top box get no far field.  Kernels
-// (s source, t target): K_1: 1/(s-t)   K_1N: 1/(t-s)
-template <int KER>
-__global__ void __launch_bounds__(128) k_fmm_m2l(FmmDev pl, const int32_t *__restrict__ mk, int nw)
-{
-    constexpr int NT = 128;
-    constexpr int RMAX = (P * WMAX + NT - 1) / NT;
-    __shared__ double xq[P], tq[P], sq[P];
-    __shared__ double Ws[P][WMAX + 1];
-    __shared__ double K1[P][P + 1];
-    __shared__ int s_list[32], s_nlist;
-    const int tid = threadIdx.x;
-    if (tid < P) xq[tid] = cospi((double)(2 * tid + 1) / (2.0 * P));
-    const int64_t nbox = pl.box_base[pl.nprob];
-    for (int64_t g = blockIdx.x; g < nbox; g += gridDim.x) {
-        const int64_t p = sdc_upper_index(pl.box_base, pl.nprob, g);
-        if (pl.fslot[p] < 0) continue;
-        const int m = mk[p];
-        const int nb0 = (m + B - 1) / B;
-        const int L = lev_count(nb0);
-        int local = (int)(g - pl.box_base[p]), l = 0;
-        while (local >= lev_nb(nb0, l)) { local -= lev_nb(nb0, l); l++; }
-        const int Tb = local;
-        double acc[RMAX];
-#pragma unroll
-        for (int r = 0; r < RMAX; r++) acc[r] = 0.0;
-        int npair = 0;            // interaction pairs of the box (work counter)
-        if (l < L - 1 && pl.nnear[g] >= 0) {
-            // FP64 instructions cost a warp slot of the FP64 pipe even when every
-            // lane computes the same value, so the box geometry and the
-            // admissibility tests run once, in warp 0 (lane-parallel over the
-            // candidates), not in every warp
-            double cT = 0.0, hT = 1.0;
-            if (tid < 32) box_ch(pl.blo[g], pl.bhi[g], cT, hT);
-            __syncthreads();
-            if (tid < P) tq[tid] = cT + hT * xq[tid];
-            const int64_t gbl = pl.box_base[p] + lev_base(nb0, l);
-            const int64_t gPT = pl.box_base[p] + lev_base(nb0, l + 1) + (Tb >> 1);
-            const int nbl = lev_nb(nb0, l);
-            const int npn = pl.nnear[gPT];
-            const int64_t pst = pl.nstart[gPT];
-            for (int c0 = 0; c0 < 2 * npn; c0 += 32) {
-                // candidates c0 .. c0+31: children of the parent's near boxes, in list order
-                if (tid < 32) {
-                    const int c = c0 + tid;
-                    int S = -1;
-                    bool ok = false;
-                    if (c < 2 * npn) {
-                        S = 2 * pl.near[pst + (c >> 1)] + (c & 1);
-                        ok = S < nbl && S != Tb && adm(pl.blo[gbl + S], pl.bhi[gbl + S], pl.blo[g], pl.bhi[g]);
-                    }
-                    const unsigned bal = __ballot_sync(0xffffffffu, ok);
-                    if (ok) s_list[__popc(bal & ((1u << tid) - 1u))] = S;
-                    if (tid == 0) s_nlist = __popc(bal);
-                }
-                __syncthreads();
-                const int nlist = s_nlist;
-                npair += nlist;
-                for (int ii = 0; ii < nlist; ii++) {
-                    const int64_t gS = gbl + s_list[ii];
-                    if (ii > 0) __syncthreads();
-                    for (int t = tid; t < P * nw; t += NT) Ws[t / nw][t % nw] = pl.W[(gS * P + t / nw) * pl.ncol + t % nw];
-                    if (tid < P) {
-                        double cS, hS;
-                        box_ch(pl.blo[gS], pl.bhi[gS], cS, hS);
-                        sq[tid] = cS + hS * xq[tid];
-                    }
-                    __syncthreads();
-                    for (int t = tid; t < P * P; t += NT) {
-                        const int q = t / P, q2 = t % P;
-                        const double r = rcp_nr2(sq[q2] - tq[q]);            // 1/(s - t)
-                        K1[q][q2] = (KER == K_1N) ? -r : r;
-                    }
-                    __syncthreads();
-#pragma unroll
-                    for (int r = 0; r < RMAX; r++) {
-                        const int t = tid + r * NT;
-                        if (t >= P * nw) break;
-                        const int q = t / nw, f = t % nw;
-                        double s2 = 0.0;
-                        for (int q2 = 0; q2 < P; q2++) s2 = fma(K1[q][q2], Ws[q2][f], s2);
-                        acc[r] += s2;
-                    }
-                }
-                __syncthreads();        // s_list, Ws and the kernel block are reused
-            }
-        }
-        fl_add(pl, (int64_t)npair * (2 * P * P + 2 * P * P * nw));
-#pragma unroll
-        for (int r = 0; r < RMAX; r++) {
-            const int t = tid + r * NT;
-            if (t < P * nw) pl.F[(g * P + t / nw) * pl.nfield + t % nw] = acc[r];
-        }
-    }
-}
-
-// Local-to-local for box g (level l, index b, below its problem's top box):
-// add the parent's far field, interpolated at the box's Chebyshev nodes
-// (Chebyshev coefficients of the parent's node values, evaluated at
-// alpha x_q + beta).  On the leaf level the field is converted to Chebyshev
-// coefficients for the targets.  Computed by a group of G threads (a warp, or
-// the whole CTA), tid in [0, G); WF the staged width.
-template <int G>
-__device__ __forceinline__ void grp_sync()
-{
-    if (G == 32) __syncwarp();
-    else __syncthreads();
-}
-
-template <int G, int WF>
-__device__ __forceinline__ void l2l_box(const FmmDev &pl, int64_t p, int nb0, int l, int b, int64_t g, int nf, int tid,
-                                        double (*Fs)[WF + 1], double (*Ac)[WF + 1], double (*Tv)[P + 1],
-                                        const double *Tx, const double *xq)
-{
-    const bool alln = pl.nnear[g] < 0;
-    const int64_t gP = pl.box_base[p] + lev_base(nb0, l + 1) + (b >> 1);
-    grp_sync<G>();
-    if (!alln) {
-        // parent's node values
-        for (int t = tid; t < P * nf; t += G) Fs[t / nf][t % nf] = pl.F[(gP * P + t / nf) * pl.nfield + t % nf];
-        if (tid < P) {
-            double cP, hP, cT, hT;
-            box_ch(pl.blo[gP], pl.bhi[gP], cP, hP);
-            box_ch(pl.blo[g], pl.bhi[g], cT, hT);
-            // the node in the parent's variable as alpha x_q + beta: forming the
-            // node's position c + h x_q first would round it to the spacing of
-            // c, which on a box of one point (h = |c| 1e-15) moves the nodes by
-            // several percent of h; a chain of such boxes then re-evaluates the
-            // field's rounding noise off the nodes at every level (relative
-            // errors up to 1e-7 in zhat of the last pole)
-            const double ihP = rcp_nr2(hP);
-            const double v = fma(hT * ihP, xq[tid], (cT - cP) * ihP);
-            double t0 = 1.0, t1 = v;
-            Tv[tid][0] = 1.0;
-            Tv[tid][1] = v;
-            for (int n = 2; n < P; n++) {
-                const double t2 = 2.0 * v * t1 - t0;
-                Tv[tid][n] = t2;
-                t0 = t1; t1 = t2;
-            }
-        }
-        grp_sync<G>();
-        for (int t = tid; t < P * nf; t += G) {
-            const int n = t / nf, f = t % nf;
-            double s = 0.0;
-            for (int q = 0; q < P; q++) s = fma(Fs[q][f], Tx[q * P + n], s);
-            Ac[n][f] = s * ((n == 0) ? (1.0 / P) : (2.0 / P));
-        }
-        grp_sync<G>();
-        for (int t = tid; t < P * nf; t += G) {
-            const int q = t / nf, f = t % nf;
-            double s = pl.F[(g * P + q) * pl.nfield + f];
-            for (int n = 0; n < P; n++) s = fma(Tv[q][n], Ac[n][f], s);
-            Fs[q][f] = s;     // own row (q, f) only
-        }
-    } else {
-        for (int t = tid; t < P * nf; t += G) Fs[t / nf][t % nf] = 0.0;
-    }
-    grp_sync<G>();
-    // parent's node values -> coefficients -> this box's nodes; on the
-    // leaves the field -> coefficients for the targets
-    if (tid == 0 && pl.flops) {
-        const int64_t v = (alln ? 0 : 2 * P * (P - 2) + 4 * P * P * nf) + ((l == 0) ? 2 * P * P * nf : 0);
-        if (v > 0) atomicAdd(pl.flops, (unsigned long long)v);
-    }
-    if (l > 0) {
-        for (int t = tid; t < P * nf; t += G) pl.F[(g * P + t / nf) * pl.nfield + t % nf] = Fs[t / nf][t % nf];
-    } else {
-        const int64_t gl = pl.leaf_base[p] + b;
-        for (int t = tid; t < P * nf; t += G) {
-            const int n = t / nf, f = t % nf;
-            double s = 0.0;
-            for (int q = 0; q < P; q++) s = fma(Fs[q][f], Tx[q * P + n], s);
-            pl.coef[(gl * pl.nfield + f) * P + n] = s * ((n == 0) ? (1.0 / P) : (2.0 / P));
-        }
-    }
-}
-
-// Downward pass, launched per top-relative level t0 >= 1 (levels counted from
-// each problem's top box, level L-1 of a problem with L levels), one CTA per
-// box of level t0 (the parent is final: done by an earlier launch).
-//   NARROW (fields of at most NARROW_NF columns: secular, b, Loewner): the
-//     CTA also finishes the box's subtree DOWN_LEVELS - 1 levels further
-//     down, level by level, a warp per box (the 1, 2, 4, 8 boxes of the four
-//     levels take 1, 1, 1, 2 rounds of the four warps), so the narrow fields
-//     take a quarter of the launches;
-//   wide fields (the Cauchy-like ones, one field per column): one level per
-//     launch, the whole CTA on one box.
-// Same arithmetic per box either way.
-constexpr int DOWN_LEVELS = 4;
-constexpr int NARROW_NF = 4;
-
-template <bool NARROW>
-__global__ void __launch_bounds__(128) k_fmm_down(FmmDev pl, const int32_t *__restrict__ mk, int t0, int nf)
-{
-    constexpr int WF = NARROW ? NARROW_NF : WMAX;
-    constexpr int NG = NARROW ? 4 : 1;               // box groups per CTA
-    constexpr int G = 128 / NG;
-    __shared__ double xq[P];
-    __shared__ double Tx[P * P];
-    __shared__ double Fs[NG][P][WF + 1];
-    __shared__ double Ac[NG][P][WF + 1];
-    __shared__ double Tv[NG][P][P + 1];
-    cheb_tables(xq, Tx);
-    const int grp = threadIdx.x / G, tid = threadIdx.x % G;
-    const int nf_ = *pl.nfmm;
-    const int64_t *lo = pl.top_off + (int64_t)t0 * (pl.cap_f + 1);
-    const int64_t nu = lo[nf_];
-    for (int64_t u = blockIdx.x; u < nu; u += gridDim.x) {
-        const int64_t f = sdc_upper_index(lo, (int64_t)nf_, u);
-        const int br = (int)(u - lo[f]);
-        const int64_t p = pl.fprob[f];
-        if (pl.fslot[p] < 0) continue;
-        const int nb0 = (mk[p] + B - 1) / B;
-        const int L = lev_count(nb0);
-        const int lr = L - 1 - t0;
-        if (lr < 0 || br >= lev_nb(nb0, lr)) continue;
-        for (int k = 0; k < (NARROW ? DOWN_LEVELS : 1) && lr - k >= 0; k++) {
-            const int l = lr - k;
-            const int b0 = br << k, bend = min(lev_nb(nb0, l), (br + 1) << k);
-            __syncthreads();                   // the parents (previous level) are written
-            for (int bb = b0; bb < bend; bb += NG) {
-                const int b = bb + grp;
-                if (b < bend)
-                    l2l_box<G, WF>(pl, p, nb0, l, b, pl.box_base[p] + lev_base(nb0, l) + b, nf, tid, Fs[grp],
-                                   Ac[grp], Tv[grp], Tx, xq);
-            }
-        }
     }
 }
 
@@ -1850,7 +1556,7 @@ __global__ void __launch_bounds__(B) k_lowner_fmm(FmmDev pl, const int64_t *__re
         if (act) {
             double cT, hT;
             box_ch(pl.blo[g], pl.bhi[g], cT, hT);
-            const double Lf = clenshaw(pl.coef + gl * pl.nfield * P, (di - cT) / hT);
+            const double Lf = clenshaw(pl.coef + gl * NFIELD * P, (di - cT) / hT);
             double prod = pr.pn / pr.pd;
             int ex = pr.ex;
             if (ex & 1) { prod *= 2.0; ex -= 1; }
@@ -1891,7 +1597,7 @@ __global__ void __launch_bounds__(B) k_bnorm_fmm(FmmDev pl, const int64_t *__res
         if (act) {
             double cT, hT;
             box_ch(pl.blo[g], pl.bhi[g], cT, hT);
-            s = clenshaw(pl.coef + gl * pl.nfield * P, ((dK + e) - cT) / hT);
+            s = clenshaw(pl.coef + gl * NFIELD * P, ((dK + e) - cT) / hT);
         }
         const bool ok = pl.ffbad[p] == 0;
         const FfScale fs = ff_scale(o.dk[b0], o.dk[b0 + m - 1], o.wsum[p]);
@@ -1948,7 +1654,7 @@ __global__ void __launch_bounds__(B) k_bnorm_fmm(FmmDev pl, const int64_t *__res
         if (tid == 0) {
             double a = 0.0;
             for (int q = 0; q < B; q++) a += red[q];
-            pl.lastp[gl * pl.ncol] = a;
+            pl.lastp[gl] = a;
         }
         // near terms (6 each, as the direct kernel), Clenshaw, the last target's share
         const int64_t nt = max(0, min(B, (m - 1) - Tb * B)), ns = max(0, min(B, m - Tb * B));
@@ -1956,213 +1662,637 @@ __global__ void __launch_bounds__(B) k_bnorm_fmm(FmmDev pl, const int64_t *__res
     }
 }
 
-// The last eigenvalue's sums from the leaf boxes' shares (lastp), one warp per
-// (FMM problem, column), in a fixed order: lane-strided partial sums, then a
-// butterfly.  MODE 0: b_{m-1} = sum^{-1/2} into bout.  MODE 1: row pinv_{m-1}
-// of Y = Qhat^T X, b_{m-1} (from bnorm) times the sum.
-template <int MODE>
+// The last eigenvalue's b from the leaf boxes' shares (lastp), one warp per FMM
+// problem, in a fixed order: lane-strided partial sums, then a butterfly.
 __global__ void __launch_bounds__(128) k_fmm_lastsum(FmmDev pl, const int64_t *__restrict__ off,
-                                                     const int32_t *__restrict__ mk, double *__restrict__ bout,
-                                                     const double *__restrict__ bnorm,
-                                                     const int32_t *__restrict__ pinv, double *__restrict__ Y,
-                                                     int64_t ldy, int col0, int nc)
+                                                     const int32_t *__restrict__ mk, double *__restrict__ bout)
 {
     const int lane = threadIdx.x & 31;
-    const int64_t nw = (int64_t)(*pl.nfmm) * nc;
+    const int64_t nw = *pl.nfmm;
     for (int64_t w = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < nw;
          w += ((int64_t)gridDim.x * blockDim.x) >> 5) {
-        const int64_t p = pl.fprob[w / nc];
-        const int q = (int)(w % nc);
+        const int64_t p = pl.fprob[w];
         if (pl.fslot[p] < 0) continue;
-        const int64_t l0 = pl.leaf_base[p], l1 = pl.leaf_base[p + 1];
         double a = 0.0;
-        for (int64_t gl = l0 + lane; gl < l1; gl += 32) a += pl.lastp[gl * pl.ncol + q];
+        for (int64_t gl = pl.leaf_base[p] + lane; gl < pl.leaf_base[p + 1]; gl += 32) a += pl.lastp[gl];
         for (int sh = 16; sh > 0; sh >>= 1) a += __shfl_xor_sync(0xffffffffu, a, sh);
-        if (lane == 0) {
-            const int64_t b0 = off[p];
-            const int m = mk[p];
-            if (MODE == 0) bout[b0 + m - 1] = 1.0 / sqrt(a);
-            else Y[b0 + pinv[b0 + m - 1] + (int64_t)(col0 + q) * ldy] = bnorm[b0 + m - 1] * a;
+        if (lane == 0) bout[off[p] + mk[p] - 1] = 1.0 / sqrt(a);
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Cauchy-like applications to blocks of columns on the tensor cores.
+//
+// Y = Qhat^T X or Qhat X is, per tile of 16 targets, a product of a kernel
+// matrix and a block: sources are the poles (eigenvalues) of the near boxes, or
+// every one of a problem without a tree, with the columns as they are, and the
+// Chebyshev nodes of the boxes of the interaction lists of the tile's leaf and
+// its ancestors with the node weights.  In FP64 that is one FMA per entry and
+// column on a pipe that retires 2 per clock.  Here both operands are cut into
+// seven 8-bit digits on fixed grids (Ozaki, Ogita, Oishi, Rump, Error-free
+// transformations of matrix multiplication, 2012), every product of two digit
+// matrices is a bf16 mma whose FP32 sums are exact integers (128 sources of
+// products below 2^14, up to seven per order, stay below 2^24), and the 28
+// products with i + j <= 8 carry the result to 2^-55 of the largest entry
+// times the largest column value.
+//   * Kernel entries come from split positions (three floats, ff_diff3,
+//     ff_rcp3).  Near rows are scaled by the power of two below b_j (|v_i| for
+//     Qhat X): an entry is then at most one in magnitude, as one of an
+//     orthogonal matrix, and the error is that of FP64 in norm.  Far rows
+//     share one power of two per tile that covers every box of the lists.
+//   * The source that may be closer than the positions resolve (the origin of
+//     eta_j) and the last eigenvalue (outside the positions' range) are added
+//     in FP64.
+//   * Problems out of the positions' scale (cm_prep) take FP64 loops.
+// One warp per 16 targets, digit fragments read in mma order from global
+// memory (written once per call by k_cm_slice / k_cm_slicew).
+// ---------------------------------------------------------------------------
+constexpr int CM_D = 7;           // digits
+constexpr int CM_NT = 3;          // column tiles of 8 per pass
+constexpr int CM_TR = 64;         // targets per CTA (4 warps)
+
+__device__ __forceinline__ float pow2f(int e) { return __int_as_float((e + 127) << 23); }      // -126 <= e <= 127
+
+__device__ __forceinline__ int64_t cm_chunk(int64_t b0, int64_t p) { return (b0 >> 4) + p; }   // 16-slot chunks
+
+// digit s (1..7) of y in [-1, 1] on the grid 2^-(8 s - 1), as bf16 bits
+__device__ __forceinline__ void cm_digits(double y, unsigned short *out)
+{
+    long long v = __double2ll_rn(y * 36028797018963968.0);        // 2^55
+#pragma unroll
+    for (int s = 1; s <= CM_D; s++) {
+        const int sh = 8 * (CM_D - s);
+        const long long d = (s < CM_D) ? (v + (1ll << (sh - 1))) >> sh : v;
+        v -= d << sh;
+        out[s - 1] = (unsigned short)(__float_as_uint((float)(int)d * pow2f(1 - 8 * s)) >> 16);
+    }
+}
+
+// positions and factors of the sources, and the problems out of scale
+struct CmDev {
+    ff_f4 *pos, *fac;            // per slot: source position, source factor (three floats)
+    int32_t *bad;                // per problem
+    int32_t *cmax;               // per (problem, column of the call): biased exponent of max |x|
+    int64_t ccols;               // columns of the call (stride of cmax)
+    uint2 *xf;                   // column digits in mma order: [chunk][tile][digit][lane]
+    uint2 *wf0;                  // node weights' digits: nodes 0..15 [box][tile][digit][lane]
+    unsigned *wf1;               //                       nodes 16..21
+    int32_t *eb;                 // per box: exponent of its node weights over the columns' scales
+    double *lastp;               // per (tile of 64, column): partial sums for the last eigenvalue
+};
+
+template <bool TRANS>
+__global__ void k_cm_prep(FactorView f, int64_t total, CmDev c)
+{
+    for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < total;
+         x += (int64_t)gridDim.x * blockDim.x) {
+        if (x < f.off[0] || x >= f.off[f.nprob]) continue;
+        const int64_t p = sdc_upper_index(f.off, f.nprob, x);
+        const int64_t b0 = f.off[p];
+        const int m = f.mk[p], j = (int)(x - b0);
+        if (j >= m) continue;
+        const double *dk = f.dk + b0;
+        const FfScale s = ff_scale(dk[0], dk[m - 1], 1.0);
+        const double dK = f.dorg[x];
+        bool ok = s.ok && m >= 2 && (j + 1 >= m || ff_gap_ok(dk[j], dk[j + 1], s.kk)) &&
+                  (dK == dk[j] || (j + 1 < m && dK == dk[j + 1]));
+        const double v = TRANS ? f.vhat[x] : f.bnorm[x] * ff_pow2(s.ok ? s.kk : 0);
+        const int ev = ff_exp(f.vhat[x]), eb = ff_exp(f.bnorm[x] * ff_pow2(s.ok ? s.kk : 0));
+        ok = ok && ev > 923 && ev < 1113 && eb > 923 && eb < 1113;
+        if (!ok) {
+            c.bad[p] = 1;
+            continue;
+        }
+        const ff_t3 t = ff_split3(v);
+        c.fac[x] = {t.a, t.b, t.c, 0.0f};
+        c.pos[x] = (TRANS || j == m - 1) ? ff_pole(dk[j], s) : ff_point(dK, f.eta[x], s);
+    }
+}
+
+__global__ void k_cm_colmax(FactorView f, int64_t total, const double *__restrict__ X, int64_t ldx, int ncols,
+                            CmDev c)
+{
+    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total * ncols;
+         t += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t x = t % total;
+        const int col = (int)(t / total);
+        int64_t p = -1;
+        int e = 0;
+        if (x >= f.off[0] && x < f.off[f.nprob]) {
+            p = sdc_upper_index(f.off, f.nprob, x);
+            e = ff_exp(X[x + (int64_t)col * ldx]);
+        }
+        // one atomic per run of lanes with the same problem and column
+        const unsigned grp = __match_any_sync(__activemask(), p * ncols + col);
+        const int mx = __reduce_max_sync(grp, e);
+        if (p >= 0 && (int)(threadIdx.x & 31) == __ffs(grp) - 1 && mx > 0) atomicMax(&c.cmax[p * c.ccols + col], mx);
+    }
+}
+
+// 2^-e x with |x| < 2^e for every row of the problem (e from the biased exponent)
+__device__ __forceinline__ int cm_exp(const CmDev &c, int64_t p, int col) { return c.cmax[p * c.ccols + col] - 1022; }
+
+// digits of the columns [col0, col0 + nc) of the kept slots; row: src (TRANS) or pinv
+template <bool TRANS>
+__global__ void k_cm_slice(FactorView f, int64_t nchunk_rows, const double *__restrict__ X, int64_t ldx, int col0,
+                           int nc, int nt, CmDev c)
+{
+    // one thread per (row, column): rows in units of chunks of 16
+    const int64_t n = nchunk_rows * nt * 8;
+    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t row = t % nchunk_rows;            // chunk * 16 + k
+        const int col = (int)(t / nchunk_rows);
+        const int64_t ch = row >> 4;
+        const int k = (int)(row & 15);
+        // problem of the chunk: the last with cm_chunk(off, p) <= ch
+        int64_t lo = 0, hi = f.nprob;
+        while (hi - lo > 1) {
+            const int64_t mid = (lo + hi) >> 1;
+            if (cm_chunk(f.off[mid], mid) <= ch) lo = mid; else hi = mid;
+        }
+        const int64_t b0 = f.off[lo];
+        const int64_t first = cm_chunk(b0, lo);
+        if (ch < first) continue;
+        const int j = (int)((ch - first) * 16 + k), m = f.mk[lo];
+        if ((ch - first) * 16 >= m) continue;
+        unsigned short dg[CM_D] = {0, 0, 0, 0, 0, 0, 0};
+        if (col < nc && j < m && c.bad[lo] == 0) {
+            const int64_t r = b0 + (TRANS ? f.src[b0 + j] : f.pinv[b0 + j]);
+            const int e = cm_exp(c, lo, col0 + col);
+            cm_digits(ldexp(X[r + (int64_t)(col0 + col) * ldx], -e), dg);
+        }
+        // B fragment of m16n8k16: column n = lane / 4, k = 2 (lane % 4) + {0, 1} (+ 8)
+        const int lane = (col & 7) * 4 + ((k & 7) >> 1);
+        unsigned short *dst = (unsigned short *)(c.xf + ((ch * nt + (col >> 3)) * CM_D) * 32 + lane);
+        for (int s = 0; s < CM_D; s++) dst[(int64_t)s * 32 * 4 + ((k >> 3) << 1) + (k & 1)] = dg[s];
+    }
+}
+
+// node weights of one box (a warp per box): exponent over the columns' scales, digits
+__global__ void __launch_bounds__(128) k_cm_slicew(FmmDev pl, int col0, int nc, int nt, CmDev c)
+{
+    const unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const int64_t n = pl.box_base[pl.nprob];
+    for (int64_t g = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; g < n;
+         g += ((int64_t)gridDim.x * blockDim.x) >> 5) {
+        const int64_t p = sdc_upper_index(pl.box_base, pl.nprob, g);
+        if (pl.fslot[p] < 0 || c.bad[p]) continue;
+        int e = -4000;
+        for (int col = 0; col < nc; col++) {
+            const double w = lane < P ? pl.W[(g * P + lane) * pl.ncol + col] : 0.0;
+            const int ex = ff_exp(w);
+            if (ex > 0) e = max(e, ex - 1022 - cm_exp(c, p, col0 + col));
+        }
+        e = __reduce_max_sync(FULL, e);
+        if (lane == 0) c.eb[g] = e;
+        for (int col = 0; col < nt * 8; col++) {
+            unsigned short dg[CM_D] = {0, 0, 0, 0, 0, 0, 0};
+            if (lane < P && col < nc && e > -4000)
+                cm_digits(ldexp(pl.W[(g * P + lane) * pl.ncol + col], -e - cm_exp(c, p, col0 + col)), dg);
+            const int k = lane, ln = (col & 7) * 4 + ((k & 7) >> 1);
+            if (k < 16) {
+                unsigned short *dst = (unsigned short *)(c.wf0 + ((g * nt + (col >> 3)) * CM_D) * 32 + ln);
+                for (int s = 0; s < CM_D; s++) dst[s * 32 * 4 + ((k >> 3) << 1) + (k & 1)] = dg[s];
+            } else if (k < 24) {
+                unsigned short *dst = (unsigned short *)(c.wf1 + ((g * nt + (col >> 3)) * CM_D) * 32 + ln);
+                for (int s = 0; s < CM_D; s++) dst[s * 32 * 2 + (k & 1)] = dg[s];
+            }
         }
     }
 }
 
-// Y = Qhat^T X (columns [col0, col0+nc)) for the FMM problems:
-//   y_{pinv_j} = b_j sum_i vhat_i x_{src_i} / ((d_i - d_{K_j}) - eta_j)
-// The row of the last eigenvalue (outside the tree) is summed directly,
-// spread over the leaf boxes (lastp, then k_fmm_lastsum).
-template <int NC>
-__global__ void __launch_bounds__(B)
-k_cauchyT_fmm(FmmDev pl, FactorView f, const double *__restrict__ X, int64_t ldx, double *__restrict__ Y,
-              int64_t ldy, int col0, int nc)
+__device__ __forceinline__ void cm_mma16(float (&d)[4], const unsigned (&a)[4], uint2 b)
 {
-    __shared__ double sd[B];
-    __shared__ double sx[NC][B + 1];
-    const int tid = threadIdx.x;
-    const int64_t nleaf = pl.leaf_base[pl.nprob];
-    for (int64_t gl = blockIdx.x; gl < nleaf; gl += gridDim.x) {
-        double acc[NC];
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
+                 "{%0,%1,%2,%3};"
+                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b.x), "r"(b.y));
+}
+
+__device__ __forceinline__ void cm_mma8(float (&d)[4], unsigned a0, unsigned a1, unsigned b)
+{
+    asm volatile("mma.sync.aligned.m16n8k8.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5}, {%6}, {%0,%1,%2,%3};"
+                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+                 : "r"(a0), "r"(a1), "r"(b));
+}
+
+// digits of an entry t (three floats, |t| <= 1) as floats on the grids 2^-(8 s - 1)
+__device__ __forceinline__ void cm_cut(const ff_t3 &t, float (&d)[CM_D])
+{
+    float r = t.a;
 #pragma unroll
-        for (int q = 0; q < NC; q++) acc[q] = 0.0;
-        const int64_t p = sdc_upper_index(pl.leaf_base, pl.nprob, gl);
-        if (pl.fslot[p] < 0) continue;
-        const int64_t b0 = f.off[p];
-        const int m = f.mk[p];
-        const int Tb = (int)(gl - pl.leaf_base[p]);
-        const int64_t g = pl.box_base[p] + Tb;
-        const int j = Tb * B + tid;
-        const bool act = j < m - 1;
-        const double dK = act ? f.dorg[b0 + j] : 0.0, e = act ? f.eta[b0 + j] : 1.0;
-        if (act) {
-            double cT, hT;
-            box_ch(pl.blo[g], pl.bhi[g], cT, hT);
-            const double uu = ((dK + e) - cT) / hT;
-            const double *cf = pl.coef + gl * pl.nfield * P;
-#pragma unroll
-            for (int q = 0; q < NC; q++)
-                if (q < nc) acc[q] = clenshaw(cf + q * P, uu);
+    for (int s = 0; s < CM_D; s++) {
+        if (s == 3) {                               // the leading part has 24 bits: bring in the next
+            float e;
+            ff_two_sum(r, t.b, r, e);
+            d[6] = ff_add(e, t.c);
         }
-        const int nnr = pl.nnear[g];
-        const int nn = near_len(nnr, (m + B - 1) / B);
-        int64_t nsrc = 0;
-        for (int s = 0; s < nn; s++) {
-            const int S = SDC_IDX(near_box(pl, g, nnr, s), (m + B - 1) / B, f.status);
-            const int i0 = S * B;
-            const int cnt = min(B, m - i0);
-            nsrc += max(cnt, 0);
-            __syncthreads();
-            if (tid < cnt) {
-                const int i = i0 + tid;
-                sd[tid] = f.dk[b0 + i];
-                const double v = f.vhat[b0 + i];
-                const int64_t row = b0 + f.src[b0 + i];
-#pragma unroll
-                for (int q = 0; q < NC; q++) sx[q][tid] = (q < nc) ? v * X[row + (int64_t)(col0 + q) * ldx] : 0.0;
-            }
-            __syncthreads();
-            if (act) {
-                // two sources per iteration: the next reciprocal's dependent
-                // chain overlaps this one's column FMAs (same order per column)
-#pragma unroll 2
-                for (int ii = 0; ii < cnt; ii++) {
-                    const double r = rcp_nr2((sd[ii] - dK) - e);
-#pragma unroll
-                    for (int q = 0; q < NC; q++) acc[q] = fma(sx[q][ii], r, acc[q]);
-                }
-            }
-        }
-        if (act) {
-            const double bj = f.bnorm[b0 + j];
-            const int64_t row = b0 + f.pinv[b0 + j];
-#pragma unroll
-            for (int q = 0; q < NC; q++)
-                if (q < nc) Y[row + (int64_t)(col0 + q) * ldy] = bj * acc[q];
-        }
-        // this box's sources in the row of the last eigenvalue
-        __syncthreads();
-        if (j < m) {
-            const double r = rcp_nr2((f.dk[b0 + j] - f.dorg[b0 + m - 1]) - f.eta[b0 + m - 1]);
-            const double v = f.vhat[b0 + j] * r;
-            const int64_t row = b0 + f.src[b0 + j];
-#pragma unroll
-            for (int q = 0; q < NC; q++) sx[q][tid] = (q < nc) ? v * X[row + (int64_t)(col0 + q) * ldx] : 0.0;
-        } else {
-#pragma unroll
-            for (int q = 0; q < NC; q++) sx[q][tid] = 0.0;
-        }
-        __syncthreads();
-        for (int q = tid; q < nc; q += B) {
-            double t = 0.0;
-            for (int i = 0; i < B; i++) t += sx[q][i];
-            pl.lastp[gl * pl.ncol + q] = t;
-        }
-        // near terms (difference, reciprocal, one FMA per column), Clenshaw
-        // and the scale by b per column, the last row's share per source
-        const int64_t nt = max(0, min(B, (m - 1) - Tb * B)), ns = max(0, min(B, m - Tb * B));
-        fl_add(pl, nt * (nsrc * (3 + 2 * nc) + (2 * P + 1) * nc) + ns * (4 + 2 * nc));
+        if (s == 6) r = ff_add(r, d[6]);
+        const float M = 1.5f * (float)(1 << 23) * pow2f(-7 - 8 * s);
+        d[s] = ff_sub(ff_add(r, M), M);
+        r = ff_sub(r, d[s]);
     }
 }
 
-// Y = Qhat X (columns [col0, col0+nc)) for the FMM problems:
-//   y_{src_i} = vhat_i sum_j b_j x_{pinv_j} / ((d_i - d_{K_j}) - eta_j)
-template <int NC>
-__global__ void __launch_bounds__(B)
-k_cauchyN_fmm(FmmDev pl, FactorView f, const double *__restrict__ X, int64_t ldx, double *__restrict__ Y,
-              int64_t ldy, int col0, int nc)
+// two neighbouring k of a row: bf16 pair (the digits fit in 8 bits: truncation is exact)
+__device__ __forceinline__ unsigned cm_pack(float lo, float hi)
 {
-    __shared__ double sk[B], se[B];
-    __shared__ double sx[NC][B + 1];
-    const int tid = threadIdx.x;
-    const int64_t nleaf = pl.leaf_base[pl.nprob];
-    for (int64_t gl = blockIdx.x; gl < nleaf; gl += gridDim.x) {
-        const int64_t p = sdc_upper_index(pl.leaf_base, pl.nprob, gl);
-        if (pl.fslot[p] < 0) continue;
+    return __byte_perm(__float_as_uint(lo), __float_as_uint(hi), 0x7632);
+}
+
+// exact sums of the orders i + j = 2..8 -> double (unit entries)
+__device__ __forceinline__ double cm_fold(const float (&a)[CM_D][4], int i)
+{
+    long long hi = (long long)__float2int_rn(a[0][i] * 0x1p14f) << 16;
+    hi += (long long)__float2int_rn(a[1][i] * 0x1p22f) << 8;
+    hi += __float2int_rn(a[2][i] * 0x1p30f);
+    long long lo = (long long)__float2int_rn(a[3][i] * 0x1p38f) << 24;
+    lo += (long long)__float2int_rn(a[4][i] * 0x1p46f) << 16;
+    lo += (long long)__float2int_rn(a[5][i] * 0x1p54f) << 8;
+    lo += __float2int_rn(a[6][i] * 0x1p62f);
+    return fma((double)hi, 0x1p-30, (double)lo * 0x1p-62);
+}
+
+template <int NT, bool TRANS>
+__global__ void __launch_bounds__(128)
+k_cm_apply(FmmDev pl, FactorView f, const int64_t *__restrict__ tile_off, CmDev c, const double *__restrict__ X,
+           int64_t ldx, double *__restrict__ Y, int64_t ldy, int col0, int nc)
+{
+    __shared__ int list[4][32 * FAR_TAKE];
+    const unsigned FULL = 0xffffffffu;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, gr = lane >> 2, gc = lane & 3;
+    const int64_t ntiles = tile_off[f.nprob];
+    for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+        const int64_t p = sdc_upper_index(tile_off, f.nprob, tile);
         const int64_t b0 = f.off[p];
         const int m = f.mk[p];
-        const int Tb = (int)(gl - pl.leaf_base[p]);
-        const int64_t g = pl.box_base[p] + Tb;
-        const int i = Tb * B + tid;
-        const bool act = i < m;
-        const double di = act ? f.dk[b0 + i] : 0.0;
-        double acc[NC];
+        const int t0 = (int)(tile - tile_off[p]) * CM_TR + warp * 16;
+        const int tend = TRANS ? m - 1 : m;              // T: the last target is summed by k_cm_last
+        if (t0 >= tend) continue;
+        const bool tree = pl.fslot && pl.fslot[p] >= 0;
+        const double *dk = f.dk + b0, *dorg = f.dorg + b0, *eta = f.eta + b0;
+        const int nb0 = (m + B - 1) / B, Tb = t0 / B;
+        const int64_t gbx = tree ? pl.box_base[p] : 0;
+        const int nnr = tree ? pl.nnear[gbx + Tb] : -1;
+        const int nn = near_len(nnr, nb0);               // without a tree: every box
+        const int nsrc = TRANS ? m : m - 1;
+        if (c.bad[p]) {
+            // FP64: a row per lane pair, half of the columns each
+            const int r = min(t0 + (lane & 15), tend - 1), h = lane >> 4;
+            const double a0 = TRANS ? dorg[r] : dk[r], a1 = TRANS ? eta[r] : 0.0;
+            double acc[NT * 4] = {};
+            auto add = [&](double t, double s, const double *col, int64_t st) {
+                const double w = s * rcp_nr2(t);
 #pragma unroll
-        for (int q = 0; q < NC; q++) acc[q] = 0.0;
-        if (act) {
-            double cT, hT;
-            box_ch(pl.blo[g], pl.bhi[g], cT, hT);
-            const double uu = (di - cT) / hT;
-            const double *cf = pl.coef + gl * pl.nfield * P;
-#pragma unroll
-            for (int q = 0; q < NC; q++)
-                if (q < nc) acc[q] = clenshaw(cf + q * P, uu);
-            // the last eigenvalue (outside the tree) as a source
-            const int jl = m - 1;
-            const double r = rcp_nr2((di - f.dorg[b0 + jl]) - f.eta[b0 + jl]);
-            const double bl = f.bnorm[b0 + jl] * r;
-            const int64_t row = b0 + f.pinv[b0 + jl];
-#pragma unroll
-            for (int q = 0; q < NC; q++)
-                if (q < nc) acc[q] = fma(bl, X[row + (int64_t)(col0 + q) * ldx], acc[q]);
-        }
-        const int nnr = pl.nnear[g];
-        const int nn = near_len(nnr, (m + B - 1) / B);
-        int64_t nsrc = 0;
-        for (int s = 0; s < nn; s++) {
-            const int S = SDC_IDX(near_box(pl, g, nnr, s), (m + B - 1) / B, f.status);
-            const int j0 = S * B;
-            const int cnt = min(B, (m - 1) - j0);
-            nsrc += max(cnt, 0);
-            __syncthreads();
-            if (tid < cnt) {
-                const int j = j0 + tid;
-                sk[tid] = f.dorg[b0 + j];
-                se[tid] = f.eta[b0 + j];
-                const double bj = f.bnorm[b0 + j];
-                const int64_t row = b0 + f.pinv[b0 + j];
-#pragma unroll
-                for (int q = 0; q < NC; q++) sx[q][tid] = (q < nc) ? bj * X[row + (int64_t)(col0 + q) * ldx] : 0.0;
-            }
-            __syncthreads();
-            if (act) {
-#pragma unroll 2
-                for (int jj = 0; jj < cnt; jj++) {
-                    const double r = rcp_nr2((di - sk[jj]) - se[jj]);
-#pragma unroll
-                    for (int q = 0; q < NC; q++) acc[q] = fma(sx[q][jj], r, acc[q]);
+                for (int q = 0; q < NT * 4; q++)
+                    if (h * NT * 4 + q < nc) acc[q] = fma(w, col[(int64_t)(h * NT * 4 + q) * st], acc[q]);
+            };
+            for (int i = 0; i < nn; i++) {
+                const int j0 = SDC_IDX(near_box(pl, gbx + Tb, nnr, i), nb0, f.status) * B;
+                for (int j = j0; j < min(j0 + B, nsrc); j++) {
+                    if (TRANS) add((dk[j] - a0) - a1, f.vhat[b0 + j], X + b0 + f.src[b0 + j] + (int64_t)col0 * ldx, ldx);
+                    else add((a0 - dorg[j]) - eta[j], f.bnorm[b0 + j], X + b0 + f.pinv[b0 + j] + (int64_t)col0 * ldx, ldx);
                 }
             }
-        }
-        if (act) {
-            const double v = f.vhat[b0 + i];
-            const int64_t row = b0 + f.src[b0 + i];
+            if (!TRANS) add((a0 - dorg[m - 1]) - eta[m - 1], f.bnorm[b0 + m - 1],
+                            X + b0 + f.pinv[b0 + m - 1] + (int64_t)col0 * ldx, ldx);
+            if (tree && nnr >= 0) {
+                const int L = lev_count(nb0);
+                const double x = TRANS ? a0 + a1 : a0;
+                for (int l = 0; l < L - 1; l++) {
+                    const int A = Tb >> l;
+                    const int64_t gl = gbx + lev_base(nb0, l), gP = gbx + lev_base(nb0, l + 1) + (A >> 1);
+                    for (int i = 0; i < 2 * pl.nnear[gP]; i++) {
+                        const int S = 2 * pl.near[pl.nstart[gP] + (i >> 1)] + (i & 1);
+                        if (S >= lev_nb(nb0, l) || S == A ||
+                            !adm(pl.blo[gl + S], pl.bhi[gl + S], pl.blo[gl + A], pl.bhi[gl + A]))
+                            continue;
+                        double cS, hS;
+                        box_ch(pl.blo[gl + S], pl.bhi[gl + S], cS, hS);
+                        for (int q = 0; q < P; q++) {
+                            const double s = cS + hS * cospi((double)(2 * q + 1) / (2.0 * P));
+                            add(TRANS ? s - x : x - s, 1.0, pl.W + ((gl + S) * P + q) * pl.ncol, 1);
+                        }
+                    }
+                }
+            }
+            const int64_t row = b0 + (TRANS ? f.pinv[b0 + r] : f.src[b0 + r]);
+            const double sc = TRANS ? f.bnorm[b0 + r] : f.vhat[b0 + r];
+            if (t0 + (lane & 15) < tend)
 #pragma unroll
-            for (int q = 0; q < NC; q++)
-                if (q < nc) Y[row + (int64_t)(col0 + q) * ldy] = v * acc[q];
+                for (int q = 0; q < NT * 4; q++)
+                    if (h * NT * 4 + q < nc) Y[row + (int64_t)(col0 + h * NT * 4 + q) * ldy] = sc * acc[q];
+            continue;
         }
-        // near terms and the last source (difference, reciprocal, one FMA
-        // per column), Clenshaw and the scale by vhat per column
-        const int64_t nt = max(0, min(B, m - Tb * B));
-        fl_add(pl, nt * ((nsrc + 1) * (3 + 2 * nc) + (2 * P + 1) * nc));
+        const FfScale fs = ff_scale(dk[0], dk[m - 1], 1.0);
+        // the two rows of this lane: positions and the powers of two of their near entries
+        ff_f4 x[2];
+        float rs[2];
+        int skip[2];                                     // T: the origin's index; N: the target (skip, skip - 1)
+#pragma unroll
+        for (int h = 0; h < 2; h++) {
+            const int r = min(t0 + gr + 8 * h, tend - 1);
+            const double sc = TRANS ? f.bnorm[b0 + r] : f.vhat[b0 + r];
+            x[h] = TRANS ? ff_point(dorg[r], eta[r], fs) : ff_pole(dk[r], fs);
+            const int e = ff_exp(sc) - 1023 + (TRANS ? fs.kk : 0);
+            rs[h] = pow2f(max(-126, min(126, e)));
+            skip[h] = TRANS ? (dorg[r] == dk[r] ? r : r + 1) : r;
+        }
+        float acc[NT][CM_D][4];
+        double y[NT][4];
+        auto clear = [&]() {
+#pragma unroll
+            for (int n = 0; n < NT; n++)
+#pragma unroll
+                for (int s = 0; s < CM_D; s++)
+#pragma unroll
+                    for (int i = 0; i < 4; i++) acc[n][s][i] = 0.0f;
+        };
+        clear();
+#pragma unroll
+        for (int n = 0; n < NT; n++)
+#pragma unroll
+            for (int i = 0; i < 4; i++) y[n][i] = 0.0;
+        // ---- far field: the nodes of the interaction lists
+        int ET = -4000, far_src = 0;
+        if (tree && nnr >= 0) {
+            const int L = lev_count(nb0);
+            int A = 0, npn = 0, lb = 0, nbl = 0;
+            int64_t pst = 0;
+            unsigned long long mask = 0;
+            double lo = 0.0, hi = 0.0;
+            if (lane < L - 1) {
+                A = Tb >> lane;
+                lb = lev_base(nb0, lane);
+                nbl = lev_nb(nb0, lane);
+                const int64_t gP = gbx + lev_base(nb0, lane + 1) + (A >> 1);
+                npn = pl.nnear[gP];
+                pst = pl.nstart[gP];
+                lo = pl.blo[gbx + lb + A];
+                hi = pl.bhi[gbx + lb + A];
+                // largest weight over distance of the list
+                for (int sec = 0; sec == 0 || 64 * sec < 2 * npn; sec++) {
+                    unsigned long long mk = sec == 0 ? pl.amask[gbx + lb + A] : adm_mask(pl, gbx + lb, nbl, A, pst, npn, sec);
+                    if (sec == 0) mask = mk;
+                    while (mk) {
+                        const int i = __ffsll((long long)mk) - 1;
+                        mk &= mk - 1;
+                        const int64_t gS = gbx + lb + 2 * pl.near[pst + ((64 * sec + i) >> 1)] + (i & 1);
+                        const double gap = fmax(lo - pl.bhi[gS], pl.blo[gS] - hi);
+                        if (c.eb[gS] > -4000) ET = max(ET, c.eb[gS] - (ff_exp(gap) - 1023 + fs.kk));
+                    }
+                }
+            }
+            ET = __reduce_max_sync(FULL, ET);
+            int sec = 0, nsum = 0;
+            while (ET > -4000 && __any_sync(FULL, mask != 0 || 64 * (sec + 1) < 2 * npn)) {
+                if (mask == 0 && 64 * (sec + 1) < 2 * npn) {
+                    sec++;
+                    mask = adm_mask(pl, gbx + lb, nbl, A, pst, npn, sec);
+                }
+                const int cnt = min(FAR_TAKE, __popcll(mask));
+                int pos = cnt;
+                for (int s = 1; s < 32; s <<= 1) {
+                    const int v = __shfl_up_sync(FULL, pos, s);
+                    if (lane >= s) pos += v;
+                }
+                const int total = __shfl_sync(FULL, pos, 31);
+                pos -= cnt;
+                __syncwarp();
+                for (int i = 0; i < cnt; i++) {
+                    const int b = __ffsll((long long)mask) - 1;
+                    mask &= mask - 1;
+                    list[warp][pos + i] = lb + 2 * pl.near[pst + ((64 * sec + b) >> 1)] + (b & 1);
+                }
+                __syncwarp();
+                far_src += total * P;
+                for (int i = 0; i < total; i++) {
+                    const int64_t gS = gbx + list[warp][i];
+                    const int e = c.eb[gS] - ET;
+                    if (e < -62) continue;               // below the last digit
+                    const float sc = TRANS ? pow2f(e) : -pow2f(e);
+                    const ff_f4 *np = pl.npos + gS * P;
+                    unsigned a[CM_D][4];
+                    // nodes 0..15
+#pragma unroll
+                    for (int kp = 0; kp < 2; kp++) {
+                        const ff_f4 s0 = np[2 * gc + 8 * kp], s1 = np[2 * gc + 8 * kp + 1];
+#pragma unroll
+                        for (int h = 0; h < 2; h++) {
+                            ff_t3 u = ff_rcp3(ff_diff3(s0, x[h])), v = ff_rcp3(ff_diff3(s1, x[h]));
+                            u = {u.a * sc, u.b * sc, u.c * sc};
+                            v = {v.a * sc, v.b * sc, v.c * sc};
+                            float d0[CM_D], d1[CM_D];
+                            cm_cut(u, d0);
+                            cm_cut(v, d1);
+#pragma unroll
+                            for (int s = 0; s < CM_D; s++) a[s][2 * kp + h] = cm_pack(d0[s], d1[s]);
+                        }
+                    }
+#pragma unroll
+                    for (int n = 0; n < NT; n++) {
+                        const uint2 *bf = c.wf0 + ((gS * NT + n) * CM_D) * 32 + lane;
+                        uint2 b[CM_D];
+#pragma unroll
+                        for (int s = 0; s < CM_D; s++) b[s] = bf[s * 32];
+#pragma unroll
+                        for (int i1 = 0; i1 < CM_D; i1++)
+#pragma unroll
+                            for (int j1 = 0; i1 + j1 < CM_D; j1++) cm_mma16(acc[n][i1 + j1], a[i1], b[j1]);
+                    }
+                    // nodes 16..21
+                    {
+                        const bool in = gc < 3;
+                        const ff_f4 s0 = np[in ? 16 + 2 * gc : 0], s1 = np[in ? 17 + 2 * gc : 1];
+#pragma unroll
+                        for (int h = 0; h < 2; h++) {
+                            ff_t3 u = ff_rcp3(ff_diff3(s0, x[h])), v = ff_rcp3(ff_diff3(s1, x[h]));
+                            u = {u.a * sc, u.b * sc, u.c * sc};
+                            v = {v.a * sc, v.b * sc, v.c * sc};
+                            float d0[CM_D], d1[CM_D];
+                            cm_cut(u, d0);
+                            cm_cut(v, d1);
+#pragma unroll
+                            for (int s = 0; s < CM_D; s++) a[s][h] = in ? cm_pack(d0[s], d1[s]) : 0u;
+                        }
+                    }
+#pragma unroll
+                    for (int n = 0; n < NT; n++) {
+                        const unsigned *bf = c.wf1 + ((gS * NT + n) * CM_D) * 32 + lane;
+                        unsigned b[CM_D];
+#pragma unroll
+                        for (int s = 0; s < CM_D; s++) b[s] = bf[s * 32];
+#pragma unroll
+                        for (int i1 = 0; i1 < CM_D; i1++)
+#pragma unroll
+                            for (int j1 = 0; i1 + j1 < CM_D; j1++) cm_mma8(acc[n][i1 + j1], a[i1][0], a[i1][1], b[j1]);
+                    }
+                    if (++nsum == 5) {                   // 110 sources: fold before the sums leave 24 bits
+                        nsum = 0;
+#pragma unroll
+                        for (int n = 0; n < NT; n++)
+#pragma unroll
+                            for (int q = 0; q < 4; q++) y[n][q] += cm_fold(acc[n], q);
+                        clear();
+                    }
+                }
+                __syncwarp();
+            }
+            const double sc = ET > -4000 ? ff_pow2(ET + fs.kk) : 0.0;
+#pragma unroll
+            for (int n = 0; n < NT; n++)
+#pragma unroll
+                for (int q = 0; q < 4; q++) y[n][q] = (y[n][q] + cm_fold(acc[n], q)) * sc;
+            clear();
+        }
+        // ---- near field
+        // near sums carry the row's power of two (and 2^kk by the factors of Qhat X)
+        double ns[2];
+#pragma unroll
+        for (int h = 0; h < 2; h++) ns[h] = TRANS ? ff_pow2(fs.kk) / (double)rs[h] : 1.0 / (double)rs[h];
+        const int64_t ch0 = cm_chunk(b0, p);
+        if (pl.flops && lane == 0)
+            atomicAdd(pl.flops, (unsigned long long)min(16, tend - t0) * (far_src + (int64_t)nn * B) * (3 + 2 * nc));
+        int steps = 0;
+        for (int i = 0; i < 2 * nn; i++) {
+            const int k0 = SDC_IDX(near_box(pl, gbx + Tb, nnr, i >> 1), nb0, f.status) * B + (i & 1) * 16;
+            if (k0 >= nsrc) continue;
+            unsigned a[CM_D][4];
+#pragma unroll
+            for (int kp = 0; kp < 2; kp++) {
+                const int ka = k0 + 2 * gc + 8 * kp, kb = ka + 1;
+                const int64_t ia = b0 + min(ka, nsrc - 1), ib = b0 + min(kb, nsrc - 1);
+                const ff_f4 sa = c.pos[ia], sb = c.pos[ib], fa = c.fac[ia], fb = c.fac[ib];
+                const ff_t3 va = {fa.x, fa.y, fa.z}, vb = {fb.x, fb.y, fb.z};
+#pragma unroll
+                for (int h = 0; h < 2; h++) {
+                    const ff_t3 ta = TRANS ? ff_diff3(sa, x[h]) : ff_diff3(x[h], sa);
+                    const ff_t3 tb = TRANS ? ff_diff3(sb, x[h]) : ff_diff3(x[h], sb);
+                    ff_t3 u = ff_mul3(va, ff_rcp3(ta)), v = ff_mul3(vb, ff_rcp3(tb));
+                    const bool ua = ka < nsrc && (TRANS ? ka != skip[h] : (unsigned)(skip[h] - ka) > 1u);
+                    const bool ub = kb < nsrc && (TRANS ? kb != skip[h] : (unsigned)(skip[h] - kb) > 1u);
+                    u = {ua ? u.a * rs[h] : 0.0f, ua ? u.b * rs[h] : 0.0f, ua ? u.c * rs[h] : 0.0f};
+                    v = {ub ? v.a * rs[h] : 0.0f, ub ? v.b * rs[h] : 0.0f, ub ? v.c * rs[h] : 0.0f};
+                    float d0[CM_D], d1[CM_D];
+                    cm_cut(u, d0);
+                    cm_cut(v, d1);
+#pragma unroll
+                    for (int s = 0; s < CM_D; s++) a[s][2 * kp + h] = cm_pack(d0[s], d1[s]);
+                }
+            }
+#pragma unroll
+            for (int n = 0; n < NT; n++) {
+                const uint2 *bf = c.xf + (((ch0 + (k0 >> 4)) * NT + n) * CM_D) * 32 + lane;
+                uint2 b[CM_D];
+#pragma unroll
+                for (int s = 0; s < CM_D; s++) b[s] = bf[s * 32];
+#pragma unroll
+                for (int i1 = 0; i1 < CM_D; i1++)
+#pragma unroll
+                    for (int j1 = 0; i1 + j1 < CM_D; j1++) cm_mma16(acc[n][i1 + j1], a[i1], b[j1]);
+            }
+            if (++steps == 8) {                          // 128 sources
+                steps = 0;
+#pragma unroll
+                for (int n = 0; n < NT; n++)
+#pragma unroll
+                    for (int q = 0; q < 4; q++) y[n][q] = fma(cm_fold(acc[n], q), ns[q >> 1], y[n][q]);
+                clear();
+            }
+        }
+        // ---- FP64 terms: lane r < 16 has row r's coefficients
+        double g0 = 0.0, g1 = 0.0, g2 = 0.0;
+        int64_t r0 = 0, r1 = 0, r2 = 0;
+        {
+            const int r = min(t0 + (lane & 15), tend - 1);
+            if (TRANS) {
+                const int K = dorg[r] == dk[r] ? r : r + 1;
+                g0 = f.vhat[b0 + K] * rcp_nr2((dk[K] - dorg[r]) - eta[r]);
+                r0 = b0 + f.src[b0 + K];
+            } else {
+                if (r < m - 1) {
+                    g0 = f.bnorm[b0 + r] * rcp_nr2((dk[r] - dorg[r]) - eta[r]);
+                    r0 = b0 + f.pinv[b0 + r];
+                }
+                if (r > 0) {
+                    g1 = f.bnorm[b0 + r - 1] * rcp_nr2((dk[r] - dorg[r - 1]) - eta[r - 1]);
+                    r1 = b0 + f.pinv[b0 + r - 1];
+                }
+                g2 = f.bnorm[b0 + m - 1] * rcp_nr2((dk[r] - dorg[m - 1]) - eta[m - 1]);
+                r2 = b0 + f.pinv[b0 + m - 1];
+            }
+        }
+#pragma unroll
+        for (int h = 0; h < 2; h++) {
+            const int src = gr + 8 * h, r = t0 + src;
+            const double u0 = __shfl_sync(FULL, g0, src), u1 = __shfl_sync(FULL, g1, src), u2 = __shfl_sync(FULL, g2, src);
+            const int64_t q0 = __shfl_sync(FULL, r0, src), q1 = __shfl_sync(FULL, r1, src), q2 = __shfl_sync(FULL, r2, src);
+            if (r >= tend) continue;
+            const double sc = TRANS ? f.bnorm[b0 + r] : f.vhat[b0 + r];
+            const int64_t row = b0 + (TRANS ? f.pinv[b0 + r] : f.src[b0 + r]);
+#pragma unroll
+            for (int n = 0; n < NT; n++)
+#pragma unroll
+                for (int q = 0; q < 2; q++) {
+                    const int col = n * 8 + 2 * gc + q;
+                    if (col >= nc) continue;
+                    const int i = 2 * h + q;
+                    const int cm = c.cmax[p * c.ccols + col0 + col];
+                    double v = fma(cm_fold(acc[n], i), ns[h], y[n][i]);
+                    v = cm >= 0x7FF ? nan("") : ldexp(v, cm - 1022);
+                    const double *xc = X + (int64_t)(col0 + col) * ldx;
+                    v = fma(u0, xc[q0], v);
+                    if (!TRANS) v = fma(u1, xc[q1], fma(u2, xc[q2], v));
+                    Y[row + (int64_t)(col0 + col) * ldy] = sc * v;
+                }
+        }
+    }
+}
+
+// Row of the last eigenvalue of Qhat^T X: the sources of one tile of 64, FP64
+__global__ void __launch_bounds__(64)
+k_cm_last(FactorView f, const int64_t *__restrict__ tile_off, CmDev c, const double *__restrict__ X, int64_t ldx,
+          int col0, int nc)
+{
+    __shared__ double w[CM_TR];
+    __shared__ int64_t row[CM_TR];
+    const int64_t ntiles = tile_off[f.nprob];
+    for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+        const int64_t p = sdc_upper_index(tile_off, f.nprob, tile);
+        const int64_t b0 = f.off[p];
+        const int m = f.mk[p], i = (int)(tile - tile_off[p]) * CM_TR + threadIdx.x;
+        __syncthreads();
+        w[threadIdx.x] = 0.0;
+        row[threadIdx.x] = 0;
+        if (i < m) {
+            w[threadIdx.x] = f.vhat[b0 + i] * rcp_nr2((f.dk[b0 + i] - f.dorg[b0 + m - 1]) - f.eta[b0 + m - 1]);
+            row[threadIdx.x] = b0 + f.src[b0 + i];
+        }
+        __syncthreads();
+        for (int q = threadIdx.x; q < nc; q += CM_TR) {
+            double s = 0.0;
+            for (int k = 0; k < CM_TR; k++)
+                if (w[k] != 0.0) s = fma(w[k], X[row[k] + (int64_t)(col0 + q) * ldx], s);
+            c.lastp[tile * (CM_NT * 8) + q] = s;
+        }
+    }
+}
+
+__global__ void __launch_bounds__(128)
+k_cm_lastsum(FactorView f, const int64_t *__restrict__ tile_off, CmDev c, double *__restrict__ Y, int64_t ldy, int col0,
+             int nc)
+{
+    const int lane = threadIdx.x & 31;
+    for (int64_t u = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; u < f.nprob * nc;
+         u += ((int64_t)gridDim.x * blockDim.x) >> 5) {
+        const int64_t p = u / nc, b0 = f.off[p];
+        const int q = (int)(u % nc), m = f.mk[p];
+        if (m < 1) continue;
+        double a = 0.0;
+        for (int64_t t = tile_off[p] + lane; t < tile_off[p + 1]; t += 32) a += c.lastp[t * (CM_NT * 8) + q];
+        for (int sh = 16; sh > 0; sh >>= 1) a += __shfl_xor_sync(0xffffffffu, a, sh);
+        if (lane == 0) Y[b0 + f.pinv[b0 + m - 1] + (int64_t)(col0 + q) * ldy] = f.bnorm[b0 + m - 1] * a;
     }
 }
 
@@ -2194,21 +2324,10 @@ unsigned resident_grid(int threads)
 template <int MODE>
 unsigned up_grid() { return resident_grid<k_fmm_up<MODE>>(up_threads<MODE>()); }
 
-// one warp per (FMM problem, column) of k_fmm_lastsum, 4 warps per CTA
-unsigned lastsum_grid(const FmmPlan &pl, int nc)
+// one warp per FMM problem of k_fmm_lastsum, 4 warps per CTA
+unsigned lastsum_grid(const FmmPlan &pl)
 {
-    const int64_t w = std::max<int64_t>(1, pl.cap_f) * nc;
-    return (unsigned)std::max<int64_t>(1, std::min<int64_t>((w + 3) / 4, (int64_t)sdc_num_sms() * 8));
-}
-
-// grid of a downward-pass launch: at most one CTA per box that top-relative
-// level t0 can hold (a problem has at most 2^t0 boxes there, and at most its
-// leaf boxes)
-unsigned down_grid(const FmmPlan &pl, int t0)
-{
-    const int64_t per = (t0 >= 30) ? (int64_t)pl.nb0max : std::min<int64_t>(pl.nb0max, (int64_t)1 << t0);
-    const int64_t nb = per * std::max<int64_t>(1, pl.cap_f);
-    return (unsigned)std::max<int64_t>(1, std::min<int64_t>(nb, (int64_t)sdc_num_sms() * 8));
+    return (unsigned)std::max<int64_t>(1, std::min<int64_t>((pl.cap_f + 3) / 4, (int64_t)sdc_num_sms() * 8));
 }
 
 SrcArgs src_from_r1(const int64_t *off, const R1Out &o)
@@ -2231,50 +2350,24 @@ superdc_status far_field(const FmmPlan &pl, const int64_t *off, const R1Out &o, 
     return SUPERDC_OK;
 }
 
-// far fields of nw columns: node weights, translations, then down the tree
-template <int MODE, int KER>
-superdc_status far_columns(const FmmPlan &pl, const SrcArgs &a, int nw, cudaStream_t st)
+template <int NT>
+void launch_apply(bool trans, const FmmDev &dv, const FactorView &f, const int64_t *tile_off, const CmDev &c,
+                  const double *X, int64_t ldx, double *Y, int64_t ldy, int col0, int nc, int64_t tiles, cudaStream_t st)
 {
-    const FmmDev &dv = pl.dv;
-    PROF_LAUNCH("fmm_up", st, k_fmm_up<MODE><<<up_grid<MODE>(), up_threads<MODE>(), 0, st>>>(dv, a));
-    PROF_LAUNCH("fmm_m2l", st, k_fmm_m2l<KER><<<fmm_grid(), 128, 0, st>>>(dv, a.mk, nw));
-    if (nw <= NARROW_NF) {
-        for (int t0 = 1; t0 < pl.lmax; t0 += DOWN_LEVELS)
-            PROF_LAUNCH("fmm_l2l", st, k_fmm_down<true><<<down_grid(pl, t0), 128, 0, st>>>(dv, a.mk, t0, nw));
-    } else {
-        for (int t0 = 1; t0 < pl.lmax; t0++)
-            PROF_LAUNCH("fmm_l2l", st, k_fmm_down<false><<<down_grid(pl, t0), 128, 0, st>>>(dv, a.mk, t0, nw));
-    }
-    return SUPERDC_OK;
-}
-
-// grids: 8 CTAs per SM, or what fits when the column count's accumulators
-// leave room for fewer
-template <int NC>
-void launch_ct(const FmmPlan &pl, const FactorView &f, const double *X, int64_t ldx, double *Y, int64_t ldy, int col0,
-               int nc, cudaStream_t st)
-{
-    const unsigned g = std::min(fmm_grid(), resident_grid<k_cauchyT_fmm<NC>>(B));
-    k_cauchyT_fmm<NC><<<g, B, 0, st>>>(pl.dv, f, X, ldx, Y, ldy, col0, nc);
-}
-
-template <int NC>
-void launch_cn(const FmmPlan &pl, const FactorView &f, const double *X, int64_t ldx, double *Y, int64_t ldy, int col0,
-               int nc, cudaStream_t st)
-{
-    const unsigned g = std::min(fmm_grid(), resident_grid<k_cauchyN_fmm<NC>>(B));
-    k_cauchyN_fmm<NC><<<g, B, 0, st>>>(pl.dv, f, X, ldx, Y, ldy, col0, nc);
+    const int64_t res = trans ? resident_grid<k_cm_apply<NT, true>>(128) : resident_grid<k_cm_apply<NT, false>>(128);
+    const unsigned g = (unsigned)std::max<int64_t>(1, std::min(tiles, res));
+    if (trans) k_cm_apply<NT, true><<<g, 128, 0, st>>>(dv, f, tile_off, c, X, ldx, Y, ldy, col0, nc);
+    else k_cm_apply<NT, false><<<g, 128, 0, st>>>(dv, f, tile_off, c, X, ldx, Y, ldy, col0, nc);
 }
 
 }  // namespace
 
 
 superdc_status plan(FmmPlan &pl, int64_t nprob, const int64_t *off, int64_t total, int64_t max_m,
-                        const int32_t *mk, const double *dk, int min_m, int ncol, int nfield, int32_t *used,
-                        bool step, cudaStream_t st)
+                        const int32_t *mk, const double *dk, int min_m, int ncol, int32_t *used, bool step,
+                    cudaStream_t st)
 {
     pl = FmmPlan();
-    pl.box = B;
     pl.total = total;
     if (nprob <= 0) return SUPERDC_OK;
     if (used) SDC_CHECK(cudaMemsetAsync(used, 0, (size_t)nprob * sizeof(int32_t), st));
@@ -2290,11 +2383,9 @@ superdc_status plan(FmmPlan &pl, int64_t nprob, const int64_t *off, int64_t tota
     pl.nb0max = nb0max;
     pl.lmax = lev_count(nb0max);
     ncol = std::max(1, std::min(ncol, WMAX));
-    nfield = std::max(1, std::min(nfield, WMAX));
     FmmDev &d = pl.dv;
     d.nprob = nprob;
     d.ncol = ncol;
-    d.nfield = nfield;
     auto al = [&](auto **ptr, size_t cnt) -> cudaError_t {
         cudaError_t e = sdc_alloc(ptr, cnt, st);
         if (e == cudaSuccess) pl.bufs.push_back((void *)*ptr);
@@ -2315,29 +2406,23 @@ superdc_status plan(FmmPlan &pl, int64_t nprob, const int64_t *off, int64_t tota
     SDC_CHECK(al(&near, pl.cap_boxes * FMM_NPOOL));
     SDC_CHECK(al(&nstart, pl.cap_boxes));
     SDC_CHECK(al(&d.W, (size_t)pl.cap_boxes * P * ncol));
-    SDC_CHECK(al(&d.coef, (size_t)pl.cap_leaves * nfield * P));
-    SDC_CHECK(al(&d.F, (size_t)pl.cap_boxes * P * nfield));
-    SDC_CHECK(al(&d.lastp, (size_t)pl.cap_leaves * ncol));
-    SDC_CHECK(al(&d.tail, (size_t)std::max<int64_t>(1, total)));
-    SDC_CHECK(al(&d.ntail, 2));
-    SDC_CHECK(cudaMemsetAsync(d.ntail, 0, 2 * sizeof(unsigned int), st));
+    SDC_CHECK(al(&d.npos, (size_t)pl.cap_boxes * P));
+    SDC_CHECK(al(&d.amask, (size_t)pl.cap_boxes));
     if (step) {
-        SDC_CHECK(al(&d.npos, (size_t)pl.cap_boxes * P));
+        SDC_CHECK(al(&d.coef, (size_t)pl.cap_leaves * NFIELD * P));
+        SDC_CHECK(al(&d.lastp, (size_t)pl.cap_leaves));
+        SDC_CHECK(al(&d.tail, (size_t)std::max<int64_t>(1, total)));
+        SDC_CHECK(al(&d.ntail, 2));
+        SDC_CHECK(cudaMemsetAsync(d.ntail, 0, 2 * sizeof(unsigned int), st));
         SDC_CHECK(al(&d.nwt, (size_t)pl.cap_boxes * P));
-        SDC_CHECK(al(&d.amask, (size_t)pl.cap_boxes));
         SDC_CHECK(al(&d.ffbad, nprob));
     }
-    int64_t *lev_off, *top_off;
-    SDC_CHECK(al(&lev_off, (size_t)pl.lmax * (nf_cap + 1)));
-    SDC_CHECK(al(&top_off, (size_t)pl.lmax * (nf_cap + 1)));
     SDC_CHECK(al(&d.upcnt, pl.cap_boxes));
     SDC_CHECK(cudaMemsetAsync(d.upcnt, 0, (size_t)pl.cap_boxes * sizeof(int32_t), st));
     SDC_CHECK(al(&d.upq, 2));
     SDC_CHECK(al(&d.split, pl.cap_leaves));
     SDC_CHECK(al(&d.nsplit, 1));
     SDC_CHECK(cudaMemsetAsync(d.upq, 0, 2 * sizeof(unsigned long long), st));
-    d.lev_off = lev_off;
-    d.top_off = top_off;
     d.cap_f = nf_cap;
 
     d.flops = prof_counter("fmm_flops");
@@ -2353,9 +2438,7 @@ superdc_status plan(FmmPlan &pl, int64_t nprob, const int64_t *off, int64_t tota
     PROF_LAUNCH("fmm_tree", st, k_fmm_tree<<<gt, tt, 0, st>>>(nprob, off, mk, dk, box_base, fslot, blo, bhi,
                                                                nnear, nstart, near, used, leaf_base, d.split,
                                                                d.nsplit));
-    PROF_LAUNCH("fmm_plan", st, k_fmm_levoff<<<pl.lmax, 1024, 0, st>>>(mk, fprob, nfmm, nf_cap, lev_off,
-                                                                   top_off));
-    if (step) {
+    {
         auto gr = [&](int64_t n) {
             return (unsigned)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, (int64_t)sdc_num_sms() * 8));
         };
@@ -2419,37 +2502,61 @@ superdc_status bnorm(const FmmPlan &pl, const int64_t *off, const R1Out &o, cuda
     if (!pl.on) return SUPERDC_OK;
     far_field<M_BN, K_2>(pl, off, o, st);
     PROF_LAUNCH("fmm_bnorm", st, k_bnorm_fmm<<<near_grid(), B, 0, st>>>(pl.dv, off, o));
-    PROF_LAUNCH("fmm_bnorm", st, k_fmm_lastsum<0><<<lastsum_grid(pl, 1), 128, 0, st>>>(
-                                     pl.dv, off, o.mk, o.bnorm, nullptr, nullptr, nullptr, 0, 0, 1));
+    PROF_LAUNCH("fmm_bnorm", st, k_fmm_lastsum<<<lastsum_grid(pl), 128, 0, st>>>(pl.dv, off, o.mk, o.bnorm));
     SDC_CHECK(cudaGetLastError());
     return SUPERDC_OK;
 }
 
-superdc_status cauchy(const FmmPlan &pl, const FactorView &f, const double *X, int64_t ldx, double *Y,
-                          int64_t ldy, int col0, int nc, bool trans, cudaStream_t st)
+superdc_status columns(const FmmPlan &pl, const FactorView &f, int64_t total, const int64_t *tile_off,
+                       const double *X, int64_t ldx, double *Y, int64_t ldy, int ncols, bool trans, cudaStream_t st)
 {
-    if (!pl.on || nc <= 0) return SUPERDC_OK;
-    if (nc > WMAX || nc > pl.dv.ncol || nc > pl.dv.nfield) return SUPERDC_ERR_ARG;
-    SrcArgs a{};
-    a.off = f.off; a.mk = f.mk; a.dk = f.dk; a.vhat = f.vhat; a.bnorm = f.bnorm; a.dorg = f.dorg; a.eta = f.eta;
-    a.src = f.src; a.pinv = f.pinv; a.X = X; a.ldx = ldx; a.col0 = col0; a.nc = nc;
-    if (trans) far_columns<M_CT, K_1>(pl, a, nc, st);
-    else far_columns<M_CN, K_1N>(pl, a, nc, st);
-    typedef void (*Fn)(const FmmPlan &, const FactorView &, const double *, int64_t, double *, int64_t, int, int,
-                       cudaStream_t);
-    Fn fn;
-    // the inner loops run all NC columns: even widths up to 20 (the ranks of
-    // typical HSS generators) waste at most one FMA per term
-#define SDC_FMM_NC(W) else if (nc <= W) fn = trans ? launch_ct<W> : launch_cn<W>;
-    if (false) {}
-    SDC_FMM_NC(2) SDC_FMM_NC(4) SDC_FMM_NC(6) SDC_FMM_NC(8) SDC_FMM_NC(10) SDC_FMM_NC(12)
-    SDC_FMM_NC(14) SDC_FMM_NC(16) SDC_FMM_NC(18) SDC_FMM_NC(20) SDC_FMM_NC(24)
-    else fn = trans ? launch_ct<32> : launch_cn<32>;
-#undef SDC_FMM_NC
-    PROF_LAUNCH("fmm_cauchy", st, fn(pl, f, X, ldx, Y, ldy, col0, nc, st));
-    if (trans)
-        PROF_LAUNCH("fmm_cauchy", st, k_fmm_lastsum<1><<<lastsum_grid(pl, nc), 128, 0, st>>>(
-                                          pl.dv, f.off, f.mk, nullptr, f.bnorm, f.pinv, Y, ldy, col0, nc));
+    const int ntmax = std::min(CM_NT, (ncols + 7) / 8);
+    const int64_t chunks = total / 16 + f.nprob + 1, tiles = total / CM_TR + f.nprob + 1;
+    SdcScratch sc(st);
+    CmDev c{};
+    c.ccols = ncols;
+    SDC_CHECK(sc.get(&c.pos, (size_t)total));
+    SDC_CHECK(sc.get(&c.fac, (size_t)total));
+    SDC_CHECK(sc.get(&c.bad, (size_t)f.nprob));
+    SDC_CHECK(sc.get(&c.cmax, (size_t)f.nprob * ncols));
+    SDC_CHECK(sc.get(&c.xf, (size_t)chunks * ntmax * CM_D * 32));
+    if (trans) SDC_CHECK(sc.get(&c.lastp, (size_t)tiles * CM_NT * 8));
+    if (pl.on) {
+        SDC_CHECK(sc.get(&c.wf0, (size_t)pl.cap_boxes * ntmax * CM_D * 32));
+        SDC_CHECK(sc.get(&c.wf1, (size_t)pl.cap_boxes * ntmax * CM_D * 32));
+        SDC_CHECK(sc.get(&c.eb, (size_t)pl.cap_boxes));
+    }
+    SDC_CHECK(cudaMemsetAsync(c.bad, 0, (size_t)f.nprob * sizeof(int32_t), st));
+    SDC_CHECK(cudaMemsetAsync(c.cmax, 0, (size_t)f.nprob * ncols * sizeof(int32_t), st));
+    auto gr = [&](int64_t n) {
+        return (unsigned)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, (int64_t)sdc_num_sms() * 8));
+    };
+    const int64_t rows = chunks * 16;
+    if (trans) PROF_LAUNCH("cauchy", st, k_cm_prep<true><<<gr(total), 256, 0, st>>>(f, total, c));
+    else PROF_LAUNCH("cauchy", st, k_cm_prep<false><<<gr(total), 256, 0, st>>>(f, total, c));
+    PROF_LAUNCH("cauchy", st, k_cm_colmax<<<gr(total * ncols), 256, 0, st>>>(f, total, X, ldx, ncols, c));
+    FmmDev dv = pl.dv;
+    if (!pl.on) dv = FmmDev{};
+    for (int c0 = 0; c0 < ncols; c0 += CM_NT * 8) {
+        const int nc = std::min(CM_NT * 8, ncols - c0), nt = (nc + 7) / 8;
+        if (trans) PROF_LAUNCH("cauchy", st, k_cm_slice<true><<<gr(rows * nt * 8), 256, 0, st>>>(f, rows, X, ldx, c0, nc, nt, c));
+        else PROF_LAUNCH("cauchy", st, k_cm_slice<false><<<gr(rows * nt * 8), 256, 0, st>>>(f, rows, X, ldx, c0, nc, nt, c));
+        if (pl.on) {
+            SrcArgs a{};
+            a.off = f.off; a.mk = f.mk; a.dk = f.dk; a.vhat = f.vhat; a.bnorm = f.bnorm; a.dorg = f.dorg; a.eta = f.eta;
+            a.src = f.src; a.pinv = f.pinv; a.X = X; a.ldx = ldx; a.col0 = c0; a.nc = nc;
+            if (trans) PROF_LAUNCH("fmm_up", st, k_fmm_up<M_CT><<<up_grid<M_CT>(), up_threads<M_CT>(), 0, st>>>(dv, a));
+            else PROF_LAUNCH("fmm_up", st, k_fmm_up<M_CN><<<up_grid<M_CN>(), up_threads<M_CN>(), 0, st>>>(dv, a));
+            PROF_LAUNCH("fmm_up", st, k_cm_slicew<<<gr(pl.cap_boxes * 32), 128, 0, st>>>(dv, c0, nc, nt, c));
+        }
+        auto fn = (nt == 1) ? launch_apply<1> : (nt == 2) ? launch_apply<2> : launch_apply<3>;
+        PROF_LAUNCH("cauchy", st, fn(trans, dv, f, tile_off, c, X, ldx, Y, ldy, c0, nc, tiles, st));
+        if (trans) {
+            PROF_LAUNCH("cauchy", st, k_cm_last<<<(unsigned)std::min<int64_t>(tiles, (int64_t)sdc_num_sms() * 16), 64, 0,
+                                                 st>>>(f, tile_off, c, X, ldx, c0, nc));
+            PROF_LAUNCH("cauchy", st, k_cm_lastsum<<<gr(f.nprob * nc * 32), 128, 0, st>>>(f, tile_off, c, Y, ldy, c0, nc));
+        }
+    }
     SDC_CHECK(cudaGetLastError());
     return SUPERDC_OK;
 }

@@ -945,10 +945,9 @@ superdc_status r1_run(const R1Args &a_in, cudaStream_t st)
     // path; the direct kernels below skip them
     FmmPlan fp;
     {
-        // boxes of 32: the secular sweeps repeat the near field every iteration
         const int w = a.keep ? std::min(32, a.keep_width) : 0;
         superdc_status fs = fmm_plan(fp, a.nprob, a.off, a.total, a.max_m, a.o.mk, a.o.dk, a.fmm_min_m,
-                                     std::max(1, w), std::max(4, w), a.o.fmm_used, 32, true, st);
+                                     std::max(1, w), a.o.fmm_used, true, st);
         if (fs != SUPERDC_OK) { fmm_free(fp, st); return fs; }
     }
     const int32_t *fslot = fp.on ? fp.dv.fslot : nullptr;
