@@ -33,13 +33,14 @@
 #include "cauchy.cuh"
 #include "fmm.cuh"
 #include "prof.cuh"
+#include "secular.cuh"
 
 namespace {
 
 constexpr int BW_C = 8;      // columns per pass of the lambda-lambda kernel
-constexpr int TB = 128;
-
-__device__ __forceinline__ double rcp_full(double t) { return 1.0 / t; }
+constexpr int BW_T = 32;     // targets per CTA (one per lane)
+constexpr int BW_W = 8;      // warps per CTA; they split the sources
+constexpr int BW_S = 32;     // sources staged per warp
 
 // pinv from perm, d_K from org (inputs are the public forward outputs)
 __global__ void k_prep(int64_t nprob, const int64_t *__restrict__ off, int64_t total, const int32_t *__restrict__ mk,
@@ -56,158 +57,191 @@ __global__ void k_prep(int64_t nprob, const int64_t *__restrict__ off, int64_t t
     }
 }
 
-// per kept root k: u_k and g_k (lambda-lambda sums), columns [c0, c0+nc)
-__global__ void __launch_bounds__(TB)
+// Per kept root k, columns [c0, c0 + nc): u_k and g_k.  Both sums run over the
+// pairs with one factor per pair, s_kl = sum_c (ybar_kc alpha_lc - y_kc beta_lc):
+//   u_k -= 1/2 sum_l s_kl / (lambda_k - lambda_l),
+//   g_k += b_k sum_l s_kl / (lambda_k - lambda_l)^2,
+// so a pair costs 2 nc + 10 FP64 operations instead of 4 nc plus a division, and
+// every column count pays for its own columns only.  A CTA takes 32 targets and
+// its eight warps split the sources (a tile of 128 targets left most SMs idle
+// below 20000 rows).  Measured (GB300, n = 4096 tree adjoint, 7 columns on
+// average, 36 steps): 104.7 -> 11.4 ms; k_bw_dz 19.3 -> 3.9 ms.
+template <int NC>
+__global__ void __launch_bounds__(BW_W * 32)
 k_bw_lamlam(int64_t nprob, const int64_t *__restrict__ off, const int64_t *__restrict__ tile_off,
             const int32_t *__restrict__ mk, const double *__restrict__ dorg, const double *__restrict__ eta,
             const double *__restrict__ bnorm, const int32_t *__restrict__ pinv,
             const double *__restrict__ Y, int64_t ld, const double *__restrict__ Ybar, int64_t ldb, int c0, int nc,
             double *__restrict__ u, double *__restrict__ g)
 {
-    __shared__ double sK[TB], sE[TB], sA[BW_C][TB], sB[BW_C][TB];
+    __shared__ double sK[BW_W][BW_S], sE[BW_W][BW_S], sA[BW_W][NC][BW_S], sB[BW_W][NC][BW_S];
+    __shared__ double red[2][BW_W][BW_T];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t ntiles = tile_off[nprob];
     for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
         const int64_t p = sdc_upper_index(tile_off, nprob, tile);
         const int64_t b0 = off[p];
         const int m = mk[p];
-        const int k = (int)(tile - tile_off[p]) * TB + threadIdx.x;
+        const int k = (int)(tile - tile_off[p]) * BW_T + lane;
         const bool act = k < m;
         const double dKk = act ? dorg[b0 + k] : 0.0, ek = act ? eta[b0 + k] : 0.0;
-        double P[BW_C], R[BW_C], Ga[BW_C], De[BW_C];
+        const int64_t rowk = act ? b0 + pinv[b0 + k] : b0;
+        double y[NC], yb[NC];
 #pragma unroll
-        for (int c = 0; c < BW_C; c++) { P[c] = R[c] = Ga[c] = De[c] = 0.0; }
-        for (int l0 = 0; l0 < m; l0 += TB) {
-            const int cn = min(TB, m - l0);
-            __syncthreads();
-            for (int ll = threadIdx.x; ll < cn; ll += TB) {
-                const int64_t s = b0 + l0 + ll;
+        for (int c = 0; c < NC; c++) {
+            y[c] = (act && c < nc) ? -Y[rowk + ld * (c0 + c)] : 0.0;
+            yb[c] = (act && c < nc) ? Ybar[rowk + ldb * (c0 + c)] : 0.0;
+        }
+        // exponent of the largest |lambda|: differences above 2^-32 of it are not degenerate
+        const double lmax = fmax(fabs(dorg[b0] + eta[b0]), fabs(dorg[b0 + m - 1] + eta[b0 + m - 1]));
+        const int emin = ((__double2hiint(lmax) >> 20) & 0x7FF) + 1 - 32;
+        double su = 0.0, sg = 0.0;
+        for (int l0 = warp * BW_S; l0 < m; l0 += BW_W * BW_S) {
+            const int cn = min(BW_S, m - l0);
+            __syncwarp();
+            if (lane < cn) {
+                const int64_t s = b0 + l0 + lane;
                 const double bl = bnorm[s];
                 const int64_t row = b0 + pinv[s];
-                sK[ll] = dorg[s];
-                sE[ll] = eta[s];
+                sK[warp][lane] = dorg[s];
+                sE[warp][lane] = eta[s];
 #pragma unroll
-                for (int c = 0; c < BW_C; c++) {
-                    sA[c][ll] = (c < nc) ? bl * Y[row + ld * (c0 + c)] : 0.0;
-                    sB[c][ll] = (c < nc) ? bl * Ybar[row + ldb * (c0 + c)] : 0.0;
+                for (int c = 0; c < NC; c++) {
+                    sA[warp][c][lane] = (c < nc) ? bl * Y[row + ld * (c0 + c)] : 0.0;
+                    sB[warp][c][lane] = (c < nc) ? bl * Ybar[row + ldb * (c0 + c)] : 0.0;
                 }
             }
-            __syncthreads();
-            if (act) {
-                for (int ll = 0; ll < cn; ll++) {
-                    if (l0 + ll == k) continue;
-                    const double dl = (dKk - sK[ll]) + (ek - sE[ll]);     // lambda_k - lambda_l
-                    // numerically degenerate pairs form one eigenspace: no coupling
-                    if (fabs(dl) <= 1e-10 * fmax(fabs(dKk + ek), fabs(sK[ll] + sE[ll]))) continue;
-                    const double r = rcp_full(dl);
-                    const double r2 = r * r;
+            __syncwarp();
+#pragma unroll 2
+            for (int ll = 0; ll < cn; ll++) {
+                const double dl = (dKk - sK[warp][ll]) + (ek - sE[warp][ll]);     // lambda_k - lambda_l
+                bool use = l0 + ll != k;
+                // numerically degenerate pairs form one eigenspace: no coupling
+                if (((__double2hiint(dl) >> 20) & 0x7FF) < emin)
+                    use = use && fabs(dl) > 1e-10 * fmax(fabs(dKk + ek), fabs(sK[warp][ll] + sE[warp][ll]));
+                double s = 0.0;
 #pragma unroll
-                    for (int c = 0; c < BW_C; c++) {
-                        P[c] = fma(-sB[c][ll], r, P[c]);     // sum beta_l/(lambda_l - lambda_k)
-                        R[c] = fma(-sA[c][ll], r, R[c]);
-                        Ga[c] = fma(sB[c][ll], r2, Ga[c]);
-                        De[c] = fma(sA[c][ll], r2, De[c]);
-                    }
-                }
+                for (int c = 0; c < NC; c++) s = fma(yb[c], sA[warp][c][ll], fma(y[c], sB[warp][c][ll], s));
+                const double r = use ? rcp_nr2(dl) : 0.0;
+                const double t = s * r;
+                su += t;
+                sg = fma(t, r, sg);
             }
         }
-        if (act) {
-            const double bk = bnorm[b0 + k];
-            const int64_t row = b0 + pinv[b0 + k];
-            double uu = 0.0, gg = 0.0;
-#pragma unroll
-            for (int c = 0; c < BW_C; c++) {
-                if (c >= nc) break;
-                const double y = Y[row + ld * (c0 + c)], yb = Ybar[row + ldb * (c0 + c)];
-                uu += -0.5 * (y * P[c] - yb * R[c]);
-                gg += (bk * yb) * De[c] - (bk * y) * Ga[c];
-            }
-            u[b0 + k] += uu;
-            g[b0 + k] += gg;
+        red[0][warp][lane] = su;
+        red[1][warp][lane] = sg;
+        __syncthreads();
+        if (warp == 0 && act) {
+            double a = 0.0, b = 0.0;
+            for (int w = 0; w < BW_W; w++) { a += red[0][w][lane]; b += red[1][w][lane]; }
+            u[b0 + k] += -0.5 * a;
+            g[b0 + k] += bnorm[b0 + k] * b;
         }
+        __syncthreads();
     }
 }
 
-// d_bar_i, z_bar_i of the kept rows
-__global__ void __launch_bounds__(TB)
+// d_bar_i, z_bar_i of the kept rows; targets and warps as above
+__global__ void __launch_bounds__(BW_W * 32)
 k_bw_dz(int64_t nprob, const int64_t *__restrict__ off, const int64_t *__restrict__ tile_off,
         const int32_t *__restrict__ mk, const double *__restrict__ dk, const double *__restrict__ dorg,
         const double *__restrict__ eta, const double *__restrict__ vhat, const double *__restrict__ bnorm,
         const int32_t *__restrict__ pinv, const double *__restrict__ lam_bar, const double *__restrict__ u,
         const double *__restrict__ g, double *__restrict__ dbar_s, double *__restrict__ zbar_s)
 {
-    __shared__ double sK[TB], sE[TB], sH[TB], sG[TB], sU[TB];
+    __shared__ double sK[BW_W][BW_S], sE[BW_W][BW_S], sH[BW_W][BW_S], sG[BW_W][BW_S], sU[BW_W][BW_S];
+    __shared__ double red[2][BW_W][BW_T];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t ntiles = tile_off[nprob];
     for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
         const int64_t p = sdc_upper_index(tile_off, nprob, tile);
         const int64_t b0 = off[p];
         const int m = mk[p];
-        const int i = (int)(tile - tile_off[p]) * TB + threadIdx.x;
+        const int i = (int)(tile - tile_off[p]) * BW_T + lane;
         const bool act = i < m;
         const double di = act ? dk[b0 + i] : 0.0;
         double a1 = 0.0, a2 = 0.0;
-        for (int k0 = 0; k0 < m; k0 += TB) {
-            const int cn = min(TB, m - k0);
-            __syncthreads();
-            for (int kk = threadIdx.x; kk < cn; kk += TB) {
-                const int64_t s = b0 + k0 + kk;
+        for (int k0 = warp * BW_S; k0 < m; k0 += BW_W * BW_S) {
+            const int cn = min(BW_S, m - k0);
+            __syncwarp();
+            if (lane < cn) {
+                const int64_t s = b0 + k0 + lane;
                 const double bk = bnorm[s];
                 const double lb = lam_bar ? lam_bar[b0 + pinv[s]] : 0.0;
-                sK[kk] = dorg[s];
-                sE[kk] = eta[s];
-                sH[kk] = bk * bk * lb;
-                sG[kk] = g[s];
-                sU[kk] = bk * (u[s] - lb * bk);
+                sK[warp][lane] = dorg[s];
+                sE[warp][lane] = eta[s];
+                sH[warp][lane] = bk * bk * lb;
+                sG[warp][lane] = g[s];
+                sU[warp][lane] = bk * (u[s] - lb * bk);
             }
-            __syncthreads();
+            __syncwarp();
             if (act) {
+#pragma unroll 2
                 for (int kk = 0; kk < cn; kk++) {
-                    const double r = rcp_full((di - sK[kk]) - sE[kk]);
-                    a1 = fma(fma(sH[kk], r, sG[kk]), r, a1);
-                    a2 = fma(sU[kk], r, a2);
+                    const double r = rcp_nr2((di - sK[warp][kk]) - sE[warp][kk]);
+                    a1 = fma(fma(sH[warp][kk], r, sG[warp][kk]), r, a1);
+                    a2 = fma(sU[warp][kk], r, a2);
                 }
             }
         }
-        if (act) {
+        red[0][warp][lane] = a1;
+        red[1][warp][lane] = a2;
+        __syncthreads();
+        if (warp == 0 && act) {
+            double s1 = 0.0, s2 = 0.0;
+            for (int w = 0; w < BW_W; w++) { s1 += red[0][w][lane]; s2 += red[1][w][lane]; }
             const double v = vhat[b0 + i];
-            dbar_s[b0 + i] = v * v * a1;
-            zbar_s[b0 + i] = 2.0 * v * a2;
+            dbar_s[b0 + i] = v * v * s1;
+            zbar_s[b0 + i] = 2.0 * v * s2;
         }
+        __syncthreads();
     }
 }
 
-// scatter to input order, deflated eigenvalues, reverse rotations, rho scaling
-__global__ void k_bw_deflate(int64_t nprob, const int64_t *__restrict__ off, const int32_t *__restrict__ mk,
-                             const int32_t *__restrict__ ngiv, const int32_t *__restrict__ src,
-                             const int32_t *__restrict__ pinv, const int32_t *__restrict__ giv_ab,
-                             const double *__restrict__ giv_cs, const double *__restrict__ lam_bar,
-                             const double *__restrict__ dbar_s, const double *__restrict__ zbar_s,
-                             double sqrt_rho, double *__restrict__ dbar, double *__restrict__ zbar)
+// scatter to input order, deflated eigenvalues, rho scaling (one thread per slot)
+__global__ void k_bw_scatter(int64_t nprob, const int64_t *__restrict__ off, int64_t total,
+                             const int32_t *__restrict__ mk, const int32_t *__restrict__ src,
+                             const int32_t *__restrict__ pinv, const double *__restrict__ lam_bar,
+                             const double *__restrict__ dbar_s, const double *__restrict__ zbar_s, double sqrt_rho,
+                             double *__restrict__ dbar, double *__restrict__ zbar)
 {
-    const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= nprob) return;
-    const int64_t b0 = off[p];
-    const int m = (int)(off[p + 1] - b0), k = mk[p];
-    for (int s = 0; s < m; s++) {
-        const int64_t in = b0 + src[b0 + s];
-        if (s < k) {
-            dbar[in] = dbar_s[b0 + s];
-            zbar[in] = zbar_s[b0 + s];
-        } else {
-            dbar[in] = lam_bar ? lam_bar[b0 + pinv[b0 + s]] : 0.0;
-            zbar[in] = 0.0;
+    for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < total; x += (int64_t)gridDim.x * blockDim.x) {
+        if (x < off[0] || x >= off[nprob]) continue;
+        const int64_t p = sdc_upper_index(off, nprob, x);
+        const int64_t b0 = off[p], in = b0 + src[x];
+        const bool kept = (int)(x - b0) < mk[p];
+        dbar[in] = kept ? dbar_s[x] : (lam_bar ? lam_bar[b0 + pinv[x]] : 0.0);
+        zbar[in] = kept ? zbar_s[x] * sqrt_rho : 0.0;
+    }
+}
+
+// the rotations in reverse: chains touch disjoint entries (k_givens), so one
+// thread per chain walks it from its end
+__global__ void k_bw_rotate(int64_t nprob, const int64_t *__restrict__ off, int64_t total,
+                            const int32_t *__restrict__ ngiv, const int32_t *__restrict__ giv_ab,
+                            const double *__restrict__ giv_cs, double *__restrict__ dbar, double *__restrict__ zbar)
+{
+    for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < total; x += (int64_t)gridDim.x * blockDim.x) {
+        if (x < off[0] || x >= off[nprob]) continue;
+        const int64_t p = sdc_upper_index(off, nprob, x);
+        const int64_t b0 = off[p];
+        const int t0 = (int)(x - b0), ng = ngiv[p];
+        if (t0 >= ng) continue;
+        const int32_t *ab = giv_ab + 2 * b0;
+        const double *cs = giv_cs + 2 * b0;
+        if (t0 + 1 < ng && ab[2 * (t0 + 1)] == ab[2 * t0 + 1]) continue;       // not a chain end
+        for (int t = t0; t >= 0; t--) {
+            if (t < t0 && ab[2 * (t + 1)] != ab[2 * t + 1]) break;
+            const int a = ab[2 * t], bb = ab[2 * t + 1];
+            const double c = cs[2 * t], s = cs[2 * t + 1];
+            const double da = dbar[b0 + a], db = dbar[b0 + bb];
+            dbar[b0 + a] = c * c * da + s * s * db;
+            dbar[b0 + bb] = s * s * da + c * c * db;
+            const double za = zbar[b0 + a], zb = zbar[b0 + bb];
+            zbar[b0 + a] = c * za + s * zb;
+            zbar[b0 + bb] = -s * za + c * zb;
         }
     }
-    for (int t = ngiv[p] - 1; t >= 0; t--) {
-        const int a = giv_ab[2 * (b0 + t)], bb = giv_ab[2 * (b0 + t) + 1];
-        const double c = giv_cs[2 * (b0 + t)], s = giv_cs[2 * (b0 + t) + 1];
-        const double da = dbar[b0 + a], db = dbar[b0 + bb];
-        dbar[b0 + a] = c * c * da + s * s * db;
-        dbar[b0 + bb] = s * s * da + c * c * db;
-        const double za = zbar[b0 + a], zb = zbar[b0 + bb];
-        zbar[b0 + a] = c * za + s * zb;
-        zbar[b0 + bb] = -s * za + c * zb;
-    }
-    for (int i = 0; i < m; i++) zbar[b0 + i] *= sqrt_rho;
 }
 
 __global__ void k_tiles_b(int64_t nprob, const int32_t *__restrict__ mk, int tr, int64_t *__restrict__ tile_off)
@@ -250,8 +284,9 @@ superdc_status r1_backward_fv(const FactorView &f, int64_t total, const double *
     SDC_CHECK(sc.get(&tile_off, f.nprob + 1));
     SDC_CHECK(cudaMemsetAsync(u, 0, total * sizeof(double), st));
     SDC_CHECK(cudaMemsetAsync(g, 0, total * sizeof(double), st));
-    k_tiles_b<<<1, 1024, 0, st>>>(f.nprob, f.mk, TB, tile_off);
+    k_tiles_b<<<1, 1024, 0, st>>>(f.nprob, f.mk, BW_T, tile_off);
     superdc_status s = SUPERDC_OK;
+    const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(total / BW_T + f.nprob, (int64_t)nsm * 8));
     if (ncols > 0) {
         // Y = Qhat^T X is recomputed (the rotations act on a copy of X)
         SDC_CHECK(sc.get(&Y, (size_t)total * ncols));
@@ -261,16 +296,19 @@ superdc_status r1_backward_fv(const FactorView &f, int64_t total, const double *
         s = cauchy_apply_T(f, total, Xw, total, Y, total, ncols, st);
         if (s == SUPERDC_OK) s = cauchy_apply_N(f, total, Ybar, ldy, X_bar, ldxb, ncols, st);
         for (int c0 = 0; c0 < ncols && s == SUPERDC_OK; c0 += BW_C) {
-            PROF_LAUNCH("bw_lamlam", st, k_bw_lamlam<<<(unsigned)(nsm * 4), TB, 0, st>>>(
-                f.nprob, f.off, tile_off, f.mk, f.dorg, f.eta, f.bnorm, f.pinv, Y, total, Ybar, ldy, c0,
-                std::min(BW_C, ncols - c0), u, g));
+            const int nc = std::min(BW_C, ncols - c0);
+            auto fn = nc <= 1 ? k_bw_lamlam<1> : nc <= 2 ? k_bw_lamlam<2> : nc <= 4 ? k_bw_lamlam<4>
+                    : nc <= 6 ? k_bw_lamlam<6> : k_bw_lamlam<BW_C>;
+            PROF_LAUNCH("bw_lamlam", st, fn<<<grid, BW_W * 32, 0, st>>>(
+                f.nprob, f.off, tile_off, f.mk, f.dorg, f.eta, f.bnorm, f.pinv, Y, total, Ybar, ldy, c0, nc, u, g));
         }
     }
-    PROF_LAUNCH("bw_dz", st, k_bw_dz<<<(unsigned)(nsm * 4), TB, 0, st>>>(
+    PROF_LAUNCH("bw_dz", st, k_bw_dz<<<grid, BW_W * 32, 0, st>>>(
         f.nprob, f.off, tile_off, f.mk, f.dk, f.dorg, f.eta, f.vhat, f.bnorm, f.pinv, lam_bar, u, g, dbs, zbs));
-    k_bw_deflate<<<(unsigned)((f.nprob + 127) / 128), 128, 0, st>>>(f.nprob, f.off, f.mk, f.ngiv, f.src, f.pinv,
-                                                                    f.giv_ab, f.giv_cs, lam_bar, dbs, zbs, sqrt_rho,
-                                                                    d_bar, z_bar);
+    const unsigned gr = (unsigned)std::max<int64_t>(1, std::min<int64_t>((total + 255) / 256, (int64_t)nsm * 8));
+    k_bw_scatter<<<gr, 256, 0, st>>>(f.nprob, f.off, total, f.mk, f.src, f.pinv, lam_bar, dbs, zbs, sqrt_rho, d_bar,
+                                     z_bar);
+    k_bw_rotate<<<gr, 256, 0, st>>>(f.nprob, f.off, total, f.ngiv, f.giv_ab, f.giv_cs, d_bar, z_bar);
     cudaError_t e = cudaGetLastError();
     if (s != SUPERDC_OK) return s;
     return e == cudaSuccess ? SUPERDC_OK : SUPERDC_ERR_CUDA;

@@ -78,13 +78,19 @@ __global__ void k_build_bw_rows(int64_t n, int r, int nl, const int64_t *__restr
 
 // per node p: Btsbar_p = sum_top W_c1^T Zbar, sqbbar_p = sum_bottom <W_c2, Zbar>,
 // gR[c1] += sum_top W_c1^T Xbar, gR[c2] += sum_bottom W_c2^T Xbar
-__global__ void k_build_bw_red(int64_t n, int r, const int64_t *__restrict__ loff,
+// The CTA's thread groups of nent threads split the rows (the root node alone
+// has every row: 128 threads walking them one by one took 0.4 ms a level).
+constexpr int RED_T = 1024;
+
+__global__ void __launch_bounds__(RED_T)
+k_build_bw_red(int64_t n, int r, const int64_t *__restrict__ loff,
                                const int32_t *__restrict__ lnodes, int root, const int32_t *__restrict__ lch,
                                const int32_t *__restrict__ rch, const int64_t *__restrict__ size,
                                const int32_t *__restrict__ P, const double *__restrict__ Wp,
                                const double *__restrict__ WKbar, double *__restrict__ Btsbar,
                                double *__restrict__ sqbbar, double *__restrict__ gR)
 {
+    __shared__ double red[RED_T];
     const int q = blockIdx.x;
     const int64_t o = loff[q];
     const int m = (int)(loff[q + 1] - o);
@@ -93,13 +99,16 @@ __global__ void k_build_bw_red(int64_t n, int r, const int64_t *__restrict__ lof
     const int m1 = (int)size[c1];
     const int rr = r * r;
     const int nent = 3 * rr + 1;
-    for (int e = threadIdx.x; e < nent; e += blockDim.x) {
+    const int per = min(nent, RED_T), ng = RED_T / per;      // entries at a time, row groups
+    const int grp = threadIdx.x / per;
+    for (int e0 = 0; e0 < nent; e0 += per) {
+        const int e = e0 + threadIdx.x % per;
         const int kind = (e < rr) ? 0 : (e < 2 * rr) ? 1 : (e < 3 * rr) ? 2 : 3;
         const int ee = e - kind * rr;
         const int a = ee % r, col = ee / r;
-        if (kind >= 1 && kind <= 2 && node == root) continue;
+        const bool on = e < nent && grp < ng && !(kind >= 1 && kind <= 2 && node == root);
         double s = 0.0;
-        for (int yy = 0; yy < m; yy++) {
+        for (int yy = grp; on && yy < m; yy += ng) {
             const int64_t y = o + yy;
             const int i = P[y];
             const bool top = i < m1;
@@ -110,10 +119,16 @@ __global__ void k_build_bw_red(int64_t n, int r, const int64_t *__restrict__ lof
             else if (kind == 3 && !top)
                 for (int b = 0; b < r; b++) s += Wp[x + n * b] * WKbar[y + n * b];
         }
-        if (kind == 0) Btsbar[(int64_t)node * rr + ee] = s;
-        else if (kind == 1) gR[(int64_t)c1 * rr + ee] += s;
-        else if (kind == 2) gR[(int64_t)c2 * rr + ee] += s;
-        else sqbbar[node] = s;
+        __syncthreads();
+        red[threadIdx.x] = s;
+        __syncthreads();
+        if (on && grp == 0) {
+            for (int k = 1; k < ng; k++) s += red[k * per + threadIdx.x];
+            if (kind == 0) Btsbar[(int64_t)node * rr + ee] = s;
+            else if (kind == 1) gR[(int64_t)c1 * rr + ee] += s;
+            else if (kind == 2) gR[(int64_t)c2 * rr + ee] += s;
+            else sqbbar[node] = s;
+        }
     }
 }
 
@@ -449,7 +464,7 @@ extern "C" superdc_status superdc_eig_backward(const superdc_hss *h, const super
         PROF_LAUNCH("build_bw", st, k_build_bw_rows<<<g, 256, 0, st>>>(
             n, r, nl, h->d_lev_off[l], h->d_lev_nodes[l], nn - 1, h->d_lch, h->d_rch, h->d_size, h->R, T.Bts, T.sqb,
             f->P[l], lamb, WKbar, lamb2, Wbar));
-        k_build_bw_red<<<(unsigned)nl, 128, 0, st>>>(n, r, h->d_lev_off[l], h->d_lev_nodes[l], nn - 1, h->d_lch,
+        k_build_bw_red<<<(unsigned)nl, RED_T, 0, st>>>(n, r, h->d_lev_off[l], h->d_lev_nodes[l], nn - 1, h->d_lch,
                                                      h->d_rch, h->d_size, f->P[l], T.Wprev[l], WKbar, Btsbar, sqbbar,
                                                      gR);
         if (kc > 0) {
