@@ -2,10 +2,9 @@
 //
 // For every problem p of a batch (independent problems, or all nodes of one
 // HSS tree level), with poles d ascending and update vector z:
-//   k_deflate   -- Remark 4.1: |z_k| < tau, then the sequential Givens scan
-//                  over the survivors (one thread per problem: each test
-//                  depends on the z produced by the previous rotation);
-//                  compaction into kept / deflated slots.
+//   k_deflate   -- Remark 4.1: |z_k| < tau, then the Givens scan over the
+//                  survivors (in parallel but for chains of consecutive
+//                  rotations); compaction into kept / deflated slots.
 //   k_tiles     -- prefix of root tiles per problem (device-side, so a level
 //                  can be launched without a host round trip).
 //   k_secular   -- Algorithm 2 with the shifted secular equation eq. (4.13):
@@ -33,207 +32,143 @@
 namespace {
 
 constexpr int SEC_CHUNK = 1024;   // poles staged per shared-memory chunk (24 bytes each)
-constexpr int DEFL_BIG = 128;     // problems larger than this deflate with a whole CTA
+constexpr int DEFL_BIG = 128;     // problems larger than this deflate with more than one warp
 
 
 // ---------------------------------------------------------------------------
-// Deflation (Remark 4.1), one thread per problem.
-// ---------------------------------------------------------------------------
-__global__ void k_deflate(int64_t nprob, const int64_t *__restrict__ off,
-                          const double *__restrict__ d, const double *__restrict__ z,
-                          double sqrt_rho, double tau,
-                          double *__restrict__ wd, double *__restrict__ wz, int8_t *__restrict__ kept,
-                          R1Out o)
-{
-    int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= nprob) return;
-    const int64_t b0 = off[p];
-    const int m = (int)(off[p + 1] - b0);
-    if (m > DEFL_BIG) return;            // handled by k_deflate_big
-    bool bad = false;
-    for (int i = 0; i < m; i++) {
-        double di = d[b0 + i], zi = z[b0 + i] * sqrt_rho;
-        if (!isfinite(di) || !isfinite(zi)) bad = true;
-        wd[b0 + i] = di;
-        bool keep = !(fabs(zi) < tau);
-        wz[b0 + i] = keep ? zi : 0.0;
-        kept[b0 + i] = keep ? 1 : 0;
-    }
-    if (bad) sdc_latch(o.status, SUPERDC_DEV_NONFINITE);
-    // Givens scan over the survivors (left to right, candidate a)
-    int ng = 0;
-    int a = -1;
-    for (int bb = 0; bb < m; bb++) {
-        if (!kept[b0 + bb]) continue;
-        if (a >= 0) {
-            // the test and the rotation use explicitly rounded operations (no
-            // fused multiply-add), so decisions and rotated values are
-            // reproducible bit for bit by any IEEE evaluation in this order
-            double za = wz[b0 + a], zb = wz[b0 + bb];
-            double da = wd[b0 + a], db = wd[b0 + bb];
-            double lhs = fabs(__dmul_rn(__dmul_rn(__dsub_rn(da, db), za), zb));
-            double nrm2 = __dadd_rn(__dmul_rn(za, za), __dmul_rn(zb, zb));
-            double rhs = __dmul_rn(nrm2, tau);
-            if (lhs < rhs) {
-                double r = __dsqrt_rn(nrm2);
-                double c = __ddiv_rn(zb, r), s = __ddiv_rn(za, r);
-                double cc = __dmul_rn(c, c), ss = __dmul_rn(s, s);
-                wd[b0 + a] = __dadd_rn(__dmul_rn(cc, da), __dmul_rn(ss, db));
-                wd[b0 + bb] = __dadd_rn(__dmul_rn(ss, da), __dmul_rn(cc, db));
-                wz[b0 + a] = 0.0;
-                wz[b0 + bb] = r;
-                kept[b0 + a] = 0;
-                o.giv_ab[2 * (b0 + ng)] = a;
-                o.giv_ab[2 * (b0 + ng) + 1] = bb;
-                o.giv_cs[2 * (b0 + ng)] = c;
-                o.giv_cs[2 * (b0 + ng) + 1] = s;
-                ng++;
-            }
-        }
-        a = bb;
-    }
-    // compaction: kept slots first (ascending), then deflated sorted by (value, index)
-    int mk = 0;
-    double W = 0.0;
-    for (int i = 0; i < m; i++) {
-        if (!kept[b0 + i]) continue;
-        double zi = wz[b0 + i];
-        o.dk[b0 + mk] = wd[b0 + i];
-        o.zk[b0 + mk] = zi;
-        o.src[b0 + mk] = i;
-        W = __dadd_rn(W, __dmul_rn(zi, zi));
-        mk++;
-    }
-    int nd = 0;
-    for (int i = 0; i < m; i++) {
-        if (kept[b0 + i]) continue;
-        double v = wd[b0 + i];
-        int s = mk + nd;
-        // insertion: shift larger keys right (src increases with i, so ties keep order)
-        while (s > mk && o.dk[b0 + s - 1] > v) {
-            o.dk[b0 + s] = o.dk[b0 + s - 1];
-            o.src[b0 + s] = o.src[b0 + s - 1];
-            s--;
-        }
-        o.dk[b0 + s] = v;
-        o.src[b0 + s] = i;
-        nd++;
-    }
-    for (int s = mk; s < m; s++) {
-        o.zk[b0 + s] = 0.0;
-        o.org[b0 + s] = -1;
-        o.eta[b0 + s] = 0.0;
-        o.dorg[b0 + s] = o.dk[b0 + s];
-        o.vhat[b0 + s] = 0.0;
-        o.bnorm[b0 + s] = 1.0;
-        if (o.sweeps) o.sweeps[b0 + s] = 0;
-    }
-    o.mk[p] = mk;
-    o.ngiv[p] = ng;
-    o.wsum[p] = W;
-}
-
-
-// ---------------------------------------------------------------------------
-// Deflation of large problems, one CTA (DB_T threads) per problem: the
-// |z| < tau mask, the adjacent Givens tests and the compactions run in
-// parallel; only chains of consecutive rotations are walked sequentially.
-// The arithmetic is the same explicitly rounded sequence as k_deflate, so
-// decisions and rotated values agree bit for bit.
+// Deflation (Remark 4.1), one CTA of T threads per problem (one warp up to
+// DEFL_BIG entries).  The |z| < tau mask, the adjacent Givens tests and the
+// compactions run in parallel: every warp takes a contiguous segment in steps of
+// 32 (ballots give the places within a step), and one sum over the warps joins
+// the segments, so a pass costs one barrier instead of one scan per T entries
+// (GB300, one problem of 100003 poles: 0.65 -> 0.3 ms; 64-entry problems were
+// one thread each, 37 us a launch).  Only chains of consecutive rotations are
+// walked sequentially.  All arithmetic is one explicitly rounded sequence (no
+// fused multiply-add), so decisions and rotated values are reproducible bit for
+// bit by any IEEE evaluation in the order of the plain left-to-right scan.
 // ---------------------------------------------------------------------------
 constexpr int DB_T = 512;         // threads per problem; 1024 when a batch has fewer problems than SMs
 constexpr int WALK_CAP = 64;      // speculative steps of one chain before one thread finishes it
 
-// exclusive block scan of one int per thread; returns the prefix, *total = sum
+// sum of cnt over the warps before this one; *total over all (every thread calls)
 template <int T>
-__device__ __forceinline__ int block_exscan(int v, int *sh, int *total)
+__device__ __forceinline__ int seg_base(int cnt, int *sh, int *total)
 {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    int x = v;
-    for (int o = 1; o < 32; o <<= 1) {
-        int y = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= o) x += y;
+    const int warp = threadIdx.x >> 5;
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) sh[warp] = cnt;
+    __syncthreads();
+    int before = 0, all = 0;
+    for (int w = 0; w < T / 32; w++) {
+        const int v = sh[w];
+        before += (w < warp) ? v : 0;
+        all += v;
     }
-    if (lane == 31) sh[warp] = x;
-    __syncthreads();
-    if (warp == 0) {
-        int w = (lane < T / 32) ? sh[lane] : 0;
-        for (int o = 1; o < 32; o <<= 1) {
-            int y = __shfl_up_sync(0xffffffffu, w, o);
-            if (lane >= o) w += y;
-        }
-        sh[lane] = w;   // inclusive warp totals
-    }
-    __syncthreads();
-    const int before = (warp > 0) ? sh[warp - 1] : 0;
-    *total = sh[T / 32 - 1];
-    __syncthreads();
-    return before + x - v;
+    *total = all;
+    return before;
 }
 
 template <int T>
 __global__ void __launch_bounds__(T)
-k_deflate_big(int64_t nprob, const int64_t *__restrict__ off, const double *__restrict__ d,
-              const double *__restrict__ z, double sqrt_rho, double tau, double *__restrict__ wd,
-              double *__restrict__ wz, int8_t *__restrict__ kept, int32_t *__restrict__ surv, R1Out o)
+k_deflate(int64_t nprob, const int64_t *__restrict__ off, const double *__restrict__ d,
+          const double *__restrict__ z, double sqrt_rho, double tau, double *__restrict__ wd,
+          double *__restrict__ wz, int8_t *__restrict__ kept, int32_t *__restrict__ surv, R1Out o)
 {
-    __shared__ int sh[32];
-    __shared__ int s_bad, s_ng;
-    __shared__ double s_w[T / 32];
+    constexpr int NWARP = T / 32;
+    __shared__ int sh[NWARP];
+    __shared__ int s_ng;
+    __shared__ double s_w[NWARP];
+    const unsigned FULL = 0xffffffffu;
     const int64_t p = blockIdx.x;
     if (p >= nprob) return;
     const int64_t b0 = off[p];
     const int m = (int)(off[p + 1] - b0);
-    if (m <= DEFL_BIG) return;
-    const int tid = threadIdx.x;
-    if (tid == 0) s_bad = 0;
-    __syncthreads();
+    if ((m <= DEFL_BIG) != (T == 32)) return;       // the other launch's problem
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const unsigned below = (1u << lane) - 1u;
+    const int seg = ((m + T - 1) / T) * 32;          // entries per warp, a multiple of 32
+    const int beg = min(m, warp * seg), end = min(m, beg + seg);
     // A: copy, mask, survivor list
-    int S = 0;
-    for (int c = 0; c < m; c += T) {
-        const int i = c + tid;
-        int keep = 0;
-        if (i < m) {
-            double di = d[b0 + i], zi = z[b0 + i] * sqrt_rho;
-            if (!isfinite(di) || !isfinite(zi)) s_bad = 1;
-            keep = !(fabs(zi) < tau);
+    const long long tbits = __double_as_longlong(tau);        // tau >= 0: doubles compare as their bits
+    bool bad = false;
+    int cnt = 0;
+#pragma unroll 4
+    for (int c = beg; c < end; c += 32) {
+        const int i = c + lane;
+        bool keep = false;
+        if (i < end) {
+            // (comparisons on the bits: FP64 ones are what bounds a large problem's CTA)
+            const double di = d[b0 + i], z0 = z[b0 + i], zi = sqrt_rho == 1.0 ? z0 : z0 * sqrt_rho;
+            bad = bad || ff_exp(di) == 0x7FF || ff_exp(zi) == 0x7FF;
+            keep = !((__double_as_longlong(zi) & 0x7FFFFFFFFFFFFFFFll) < tbits);
             wd[b0 + i] = di;
             wz[b0 + i] = keep ? zi : 0.0;
-            kept[b0 + i] = (int8_t)keep;
+            kept[b0 + i] = keep ? 1 : 0;
         }
-        int tot;
-        int pre = block_exscan<T>(keep, sh, &tot);
-        if (keep) surv[b0 + S + pre] = i;
-        S += tot;
+        cnt += __popc(__ballot_sync(FULL, keep));
+    }
+    if (__any_sync(FULL, bad) && lane == 0) sdc_latch(o.status, SUPERDC_DEV_NONFINITE);
+    int S;
+    int pos = seg_base<T>(cnt, sh, &S);
+#pragma unroll 4
+    for (int c = beg; c < end; c += 32) {
+        const int i = c + lane;
+        const bool keep = i < end && kept[b0 + i] != 0;
+        const unsigned mask = __ballot_sync(FULL, keep);
+        if (keep) surv[b0 + pos + __popc(mask & below)] = i;
+        pos += __popc(mask);
     }
     __syncthreads();
-    if (tid == 0 && s_bad) sdc_latch(o.status, SUPERDC_DEV_NONFINITE);
     // B: Givens scan over the survivors.  The candidate of every test is the
     // previous survivor, so a test can differ from its value on the original
-    // data only right after a rotation.  B1 evaluates every adjacent test on
-    // the original values in parallel and marks the survivors whose test
-    // passes (kept = 2, "chain heads").  B2 takes the positions in rounds of
-    // T: every head of the round walks its chain in its own thread on the
-    // original values (rotate, re-test the next pair with the rotated values,
-    // until a test fails; at most WALK_CAP steps); one thread then decides in
-    // order which heads start a chain of the sequential scan (a head inside or
-    // at the end of the previous chain does not) and gives each chain its
-    // offset in the rotation list; finally the chains write their rotations in
-    // parallel (chains are disjoint; a chain longer than WALK_CAP is finished
-    // and written by that one thread).  Each chain evaluates the same
-    // explicitly rounded operations in the same order as the plain sequential
-    // scan (k_deflate), so decisions and rotated values agree bit for bit.
-    for (int t = 1 + tid; t < S; t += T) {
-        const int ia = surv[b0 + t - 1], ib = surv[b0 + t];
-        const double da = wd[b0 + ia], za = wz[b0 + ia], db = wd[b0 + ib], zb = wz[b0 + ib];
-        const double lhs = fabs(__dmul_rn(__dmul_rn(__dsub_rn(da, db), za), zb));
-        const double rhs = __dmul_rn(__dadd_rn(__dmul_rn(za, za), __dmul_rn(zb, zb)), tau);
-        if (lhs < rhs) kept[b0 + ib] = 2;
+    // data only right after a rotation.  First every adjacent test on the
+    // original values; the positions whose test passes are the "chain heads",
+    // listed in order (o.src holds the flags and o.perm the list: both are
+    // written only later).  The heads are then taken T at a time: each walks its
+    // chain in its own thread on the original values (rotate, re-test the next
+    // pair with the rotated values, until a test fails; at most WALK_CAP
+    // steps); one thread then decides in order which heads start a chain of the
+    // sequential scan (a head inside or at the end of the previous chain does
+    // not) and gives each chain its offset in the rotation list; finally the
+    // chains write their rotations in parallel (chains are disjoint; a chain
+    // longer than WALK_CAP is finished and written by that one thread).
+    const int sseg = ((S + T - 1) / T) * 32, sbeg = min(S, warp * sseg), send = min(S, sbeg + sseg);
+    cnt = 0;
+#pragma unroll 2
+    for (int c = sbeg; c < send; c += 32) {
+        const int t = c + lane;
+        bool hf = false;
+        if (t < send && t > 0) {
+            const int ia = surv[b0 + t - 1], ib = surv[b0 + t];
+            const double da = wd[b0 + ia], za = wz[b0 + ia], db = wd[b0 + ib], zb = wz[b0 + ib];
+            // |da - db| |za| |zb| is at least 2^el and the right-hand side less than
+            // 2^(er + 4): most pairs are told apart by the exponents
+            const double dd = __dsub_rn(da, db);
+            const int ea = ff_exp(za) - 1023, eb = ff_exp(zb) - 1023, ed = ff_exp(dd) - 1023;
+            const int el = ed + ea + eb, er = 2 * max(ea, eb) + ff_exp(tau) - 1023;
+            const bool plain = min(min(ea, eb), ed) > -300 && max(max(ea, eb), ed) < 300;
+            if (!(plain && el > er + 4)) {
+                const double lhs = fabs(__dmul_rn(__dmul_rn(dd, za), zb));
+                const double rhs = __dmul_rn(__dadd_rn(__dmul_rn(za, za), __dmul_rn(zb, zb)), tau);
+                hf = lhs < rhs;
+            }
+        }
+        if (t < send) o.src[b0 + t] = hf;
+        cnt += __popc(__ballot_sync(FULL, hf));
     }
-    __syncthreads();
-    {
+    int nheads;
+    pos = seg_base<T>(cnt, sh, &nheads);
+    if (tid == 0) s_ng = 0;
+    if (nheads > 0) {
         __shared__ int h_pos[T], h_end[T], h_off[T];
-        __shared__ int s_nh, s_eprev;
+        __shared__ int s_eprev;
+        for (int c = sbeg; c < send; c += 32) {
+            const int t = c + lane;
+            const bool hf = t < send && o.src[b0 + t] != 0;
+            const unsigned mask = __ballot_sync(FULL, hf);
+            if (hf) o.perm[b0 + pos + __popc(mask & below)] = t;
+            pos += __popc(mask);
+        }
         // one chain from position h (candidate s_{h-1}); write = false: count
         // only.  Returns the first position whose test fails (or S), or -1 when
         // max_steps rotations were taken without reaching it.  nrot >= 0: take
@@ -277,20 +212,16 @@ k_deflate_big(int64_t nprob, const int64_t *__restrict__ off, const double *__re
             }
             return t2;
         };
-        if (tid == 0) { s_eprev = 0; s_ng = 0; }
-        for (int c = 1; c < S; c += T) {
-            const int t = c + tid;
-            const int hf = (t < S && kept[b0 + surv[b0 + t]] == 2) ? 1 : 0;
-            int nh;
-            const int pre = block_exscan<T>(hf, sh, &nh);
-            if (hf) h_pos[pre] = t;
-            __syncthreads();
-            if (nh == 0) continue;
+        if (tid == 0) s_eprev = 0;
+        __syncthreads();
+        for (int h0 = 0; h0 < nheads; h0 += T) {
+            const int nh = min(T, nheads - h0);
             // speculative walks; a head at or before the previous chain's end is
             // not a chain start, and such a head may read rotated values, so its
             // result is only used once that has been ruled out
             if (tid < nh) {
-                const int h = h_pos[tid];
+                const int h = o.perm[b0 + h0 + tid];
+                h_pos[tid] = h;
                 h_end[tid] = (h <= s_eprev) ? 0 : walk(h, WALK_CAP, false, 0, -1);
             }
             __syncthreads();
@@ -319,57 +250,62 @@ k_deflate_big(int64_t nprob, const int64_t *__restrict__ off, const double *__re
     }
     __syncthreads();
     // C: compaction, kept slots in index order, then deflated slots in index order
-    int mk = 0;
-    double wpart = 0.0;
-    for (int c = 0; c < m; c += T) {
-        const int i = c + tid;
-        const int k = (i < m) ? (int)(kept[b0 + i] != 0) : 0;
-        int tot;
-        int pre = block_exscan<T>(k, sh, &tot);
-        if (k) {
-            double zi = wz[b0 + i];
-            o.dk[b0 + mk + pre] = wd[b0 + i];
-            o.zk[b0 + mk + pre] = zi;
-            o.src[b0 + mk + pre] = i;
-            wpart = __dadd_rn(wpart, __dmul_rn(zi, zi));
-        }
-        mk += tot;
+    cnt = 0;
+#pragma unroll 4
+    for (int c = beg; c < end; c += 32) {
+        const int i = c + lane;
+        cnt += __popc(__ballot_sync(FULL, i < end && kept[b0 + i] != 0));
     }
-    int nd = 0;
-    for (int c = 0; c < m; c += T) {
-        const int i = c + tid;
-        const int dflt = (i < m) ? (int)(kept[b0 + i] == 0) : 0;
-        int tot;
-        int pre = block_exscan<T>(dflt, sh, &tot);
-        if (dflt) {
-            o.dk[b0 + mk + nd + pre] = wd[b0 + i];
-            o.src[b0 + mk + nd + pre] = i;
+    int mk;
+    pos = seg_base<T>(cnt, sh, &mk);
+    double wpart = 0.0;
+#pragma unroll 4
+    for (int c = beg; c < end; c += 32) {
+        const int i = c + lane;
+        const bool k = i < end && kept[b0 + i] != 0;
+        const unsigned mask = __ballot_sync(FULL, k);
+        const int before = pos + __popc(mask & below);            // kept entries before i
+        if (i < end) {
+            const int64_t q = b0 + (k ? before : mk + i - before);
+            o.dk[q] = wd[b0 + i];
+            o.src[q] = i;
+            if (k) {
+                const double zi = wz[b0 + i];
+                o.zk[q] = zi;
+                wpart = fma(zi, zi, wpart);
+            }
         }
-        nd += tot;
+        pos += __popc(mask);
     }
     // deterministic sum of kept z^2
-    for (int of = 16; of > 0; of >>= 1) wpart += __shfl_xor_sync(0xffffffffu, wpart, of);
-    if ((tid & 31) == 0) s_w[tid >> 5] = wpart;
+    for (int of = 16; of > 0; of >>= 1) wpart += __shfl_xor_sync(FULL, wpart, of);
+    if (lane == 0) s_w[warp] = wpart;
     __syncthreads();
-    // D: deflated values sorted by (value, index): they are in index order and
-    // out of order only inside tau-sized intervals, so insertion is short
     if (tid == 0) {
         double W = 0.0;
-        for (int w = 0; w < T / 32; w++) W += s_w[w];
+        for (int w = 0; w < NWARP; w++) W += s_w[w];
         o.wsum[p] = W;
         o.mk[p] = mk;
         o.ngiv[p] = s_ng;
-        for (int q = mk + 1; q < m; q++) {
-            double v = o.dk[b0 + q];
-            int sv = o.src[b0 + q];
-            int s2 = q;
-            while (s2 > mk && o.dk[b0 + s2 - 1] > v) {
-                o.dk[b0 + s2] = o.dk[b0 + s2 - 1];
-                o.src[b0 + s2] = o.src[b0 + s2 - 1];
-                s2--;
+    }
+    // D: deflated values sorted by (value, index): they are in index order and
+    // out of order only inside tau-sized intervals, so a few odd-even
+    // exchanges (of values strictly out of order: ties keep their order) do
+    if (m - mk >= 2) {
+        for (int idle = 0, ph = 0; idle < 2; ph ^= 1) {
+            bool sw = false;
+            for (int q = mk + ph + 2 * tid; q + 1 < m; q += 2 * T) {
+                const double v0 = o.dk[b0 + q], v1 = o.dk[b0 + q + 1];
+                if (v0 > v1) {
+                    const int s0 = o.src[b0 + q], s1 = o.src[b0 + q + 1];
+                    o.dk[b0 + q] = v1;
+                    o.dk[b0 + q + 1] = v0;
+                    o.src[b0 + q] = s1;
+                    o.src[b0 + q + 1] = s0;
+                    sw = true;
+                }
             }
-            o.dk[b0 + s2] = v;
-            o.src[b0 + s2] = sv;
+            idle = __syncthreads_or(sw) ? 0 : idle + 1;
         }
     }
     __syncthreads();
@@ -381,6 +317,17 @@ k_deflate_big(int64_t nprob, const int64_t *__restrict__ off, const double *__re
         o.vhat[b0 + s2] = 0.0;
         o.bnorm[b0 + s2] = 1.0;
         if (o.sweeps) o.sweeps[b0 + s2] = 0;
+    }
+}
+
+// the two launches of a batch: problems up to DEFL_BIG entries, and larger ones
+void launch_deflate(const R1Args &a, const R1Out &o, int big_t, double *wd, double *wz, int8_t *kept, int32_t *surv,
+                    cudaStream_t st)
+{
+    k_deflate<32><<<(unsigned)a.nprob, 32, 0, st>>>(a.nprob, a.off, a.d, a.z, a.sqrt_rho, a.tau, wd, wz, kept, surv, o);
+    if (a.total > DEFL_BIG) {
+        auto fn = big_t == 1024 ? k_deflate<1024> : k_deflate<DB_T>;
+        fn<<<(unsigned)a.nprob, big_t, 0, st>>>(a.nprob, a.off, a.d, a.z, a.sqrt_rho, a.tau, wd, wz, kept, surv, o);
     }
 }
 
@@ -934,13 +881,7 @@ superdc_status r1_run(const R1Args &a_in, cudaStream_t st)
     SDC_CHECK(sc.get(&ucount, 2));
     SDC_CHECK(units_attr());
 
-    const int tpb = 128;
-    PROF_LAUNCH("deflate", st, k_deflate<<<(unsigned)((a.nprob + tpb - 1) / tpb), tpb, 0, st>>>(
-        a.nprob, a.off, a.d, a.z, a.sqrt_rho, a.tau, wd, wz, kept, a.o));
-    if (a.total > DEFL_BIG)
-        PROF_LAUNCH("deflate", st, (nsm > a.nprob ? k_deflate_big<1024> : k_deflate_big<DB_T>)<<<
-                                       (unsigned)a.nprob, nsm > a.nprob ? 1024 : DB_T, 0, st>>>(
-            a.nprob, a.off, a.d, a.z, a.sqrt_rho, a.tau, wd, wz, kept, surv, a.o));
+    PROF_LAUNCH("deflate", st, launch_deflate(a, a.o, nsm > a.nprob ? 1024 : DB_T, wd, wz, kept, surv, st));
     // problems whose kept size reaches the threshold take the triangular FMM
     // path; the direct kernels below skip them
     FmmPlan fp;
@@ -1088,12 +1029,7 @@ extern "C" superdc_status superdc_secular_batched_noalloc(int64_t nprob, const i
     int *ucount = (int *)(base + NA_UCNT);
     SDC_CHECK(units_attr());
     const int nsm = sdc_num_sms();
-    const int tpb = 128;
-    k_deflate<<<(unsigned)((a.nprob + tpb - 1) / tpb), tpb, 0, st>>>(a.nprob, a.off, a.d, a.z, a.sqrt_rho, a.tau,
-                                                                      wd, wz, kept, a.o);
-    if (a.total > DEFL_BIG)
-        k_deflate_big<DB_T><<<(unsigned)a.nprob, DB_T, 0, st>>>(a.nprob, a.off, a.d, a.z, a.sqrt_rho, a.tau, wd, wz,
-                                                           kept, surv, a.o);
+    launch_deflate(a, a.o, DB_T, wd, wz, kept, surv, st);
     const int TR = 128;
     k_tiles<<<1, 1024, 0, st>>>(a.nprob, a.o.mk, TR, tile_off);
     const unsigned grid = (unsigned)(nsm * 8);
