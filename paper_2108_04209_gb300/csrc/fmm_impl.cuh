@@ -69,7 +69,7 @@ constexpr int B = FMM_BOX;
 // to ~3.2-3.4 near boxes per leaf (with 1.0 the box between two neighbours must
 // be at least as wide as both, which a random width sequence meets a third of
 // the time)
-constexpr double FMM_KAPPA = 0.75;
+constexpr double FMM_KAPPA = 0.75;   // 3 / 4 in adm
 constexpr int SPLIT_NEAR = 512 / B;   // leaf boxes with this many near boxes (512 poles) or more: CTA-split sweeps
 constexpr int TAIL_X = 12;        // k_secular_fmm hands a box's last roots to the tail pass below this many busy lanes
 constexpr int WMAX = 32;          // widest moment block (columns)
@@ -113,13 +113,13 @@ __device__ __forceinline__ void box_ch(double lo, double hi, double &c, double &
     if (!(h > 0.0)) h = fmax(fabs(c) * 1e-15, 1e-300);
 }
 
-__device__ __forceinline__ bool adm(double loS, double hiS, double loT, double hiT)
+// on the boxes' integer intervals (60 bits of the split positions: an FP64
+// comparison costs the issue slots of 64 integer ones, and the tree of a large
+// problem is built by one CTA)
+__device__ __forceinline__ bool adm(longlong2 S, longlong2 T)
 {
-    double gap;
-    if (hiS <= loT) gap = loT - hiS;
-    else if (hiT <= loS) gap = loS - hiT;
-    else return false;
-    return gap > 0.0 && gap >= FMM_KAPPA * fmax(hiS - loS, hiT - loT);
+    const long long gap = max(T.x - S.y, S.x - T.y);
+    return gap > 0 && 4 * gap >= 3 * max(S.y - S.x, T.y - T.x);
 }
 
 // near list of a leaf box: nn >= 0 entries, or (nn < 0) every leaf box
@@ -241,121 +241,142 @@ __global__ void k_fmm_plan(int64_t nprob, const int32_t *__restrict__ mk, int mi
 // Box intervals and near lists, one CTA per problem, top level first.  Near
 // lists have any length; they are stored back to back in the problem's share
 // of the pool (FMM_NPOOL entries per box on average).  A box whose list no
-// longer fits, and its subtree, is marked "all near" (nnear = -1).
-__device__ __forceinline__ int near_count(const double *__restrict__ blo, const double *__restrict__ bhi,
-                                          const int32_t *__restrict__ near, int64_t gb, int nb, int b,
-                                          int64_t pst, int npn)
+// longer fits, and its subtree, is marked "all near" (nnear = -1).  A warp takes
+// a contiguous segment of a level, a lane per box; the candidates (children of
+// the parent's near boxes) that are admissible are the box's interaction list,
+// kept as a bit mask (the first 64), the others its near list.
+// Measured (GB300, one problem of 100003 poles): 0.43 -> 0.09 ms.
+__device__ __forceinline__ unsigned long long adm_mask(const FmmDev &pl, int64_t gb, int nbl, int A, int64_t pst,
+                                                       int npn, int sec)
 {
-    const double loT = blo[gb + b], hiT = bhi[gb + b];
-    int cnt = 0;
-    for (int i = 0; i < npn; i++) {
-        const int s = near[pst + i];
-        for (int S = 2 * s; S <= 2 * s + 1 && S < nb; S++)
-            if (S == b || !adm(blo[gb + S], bhi[gb + S], loT, hiT)) cnt++;
+    unsigned long long mask = 0;
+    const longlong2 T = pl.ibox[gb + A];
+    const int end = min(2 * npn, 64 * sec + 64);
+#pragma unroll 4
+    for (int c = 64 * sec; c < end; c++) {
+        const int S = 2 * pl.near[pst + (c >> 1)] + (c & 1);
+        if (S < nbl && S != A && adm(pl.ibox[gb + S], T)) mask |= 1ull << (c & 63);
     }
-    return cnt;
-}
-
-// exclusive scan of one value per thread of the CTA (warp shuffles, then the
-// warp totals); sh holds one entry per warp
-__device__ __forceinline__ int64_t cta_exscan(int64_t v, int64_t *sh)
-{
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    int64_t x = v;
-    for (int o = 1; o < 32; o <<= 1) {
-        const int64_t y = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= o) x += y;
-    }
-    if (lane == 31) sh[warp] = x;
-    __syncthreads();
-    int64_t before = 0;
-    for (int w = 0; w < warp; w++) before += sh[w];
-    __syncthreads();
-    return before + x - v;
+    return mask;
 }
 
 __global__ void __launch_bounds__(1024)
-k_fmm_tree(int64_t nprob, const int64_t *__restrict__ off, const int32_t *__restrict__ mk,
-           const double *__restrict__ dk, const int64_t *__restrict__ box_base, int32_t *__restrict__ fslot,
+k_fmm_tree(FmmDev pl, const int64_t *__restrict__ off, const int32_t *__restrict__ mk, const double *__restrict__ dk,
            double *__restrict__ blo, double *__restrict__ bhi, int32_t *__restrict__ nnear,
-           int64_t *__restrict__ nstart, int32_t *__restrict__ near, int32_t *__restrict__ used,
-           const int64_t *__restrict__ leaf_base, int64_t *__restrict__ split, int32_t *__restrict__ nsplit)
+           int64_t *__restrict__ nstart, int32_t *__restrict__ near, int32_t *__restrict__ used)
 {
     __shared__ int64_t wsum[32];
-    __shared__ int64_t s_pos;
-    const int T = blockDim.x;
-    for (int64_t p = blockIdx.x; p < nprob; p += gridDim.x) {
-        if (fslot[p] < 0) continue;
+    const unsigned FULL = 0xffffffffu;
+    const int T = blockDim.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int64_t p = blockIdx.x; p < pl.nprob; p += gridDim.x) {
+        if (pl.fslot[p] < 0) continue;
         const int m = mk[p];
         const double *d = dk + off[p];
-        const int64_t g0 = box_base[p];
-        const int64_t pool_end = box_base[p + 1] * FMM_NPOOL;
+        const int64_t g0 = pl.box_base[p];
+        const int64_t pool_end = pl.box_base[p + 1] * FMM_NPOOL;
         const int nb0 = (m + B - 1) / B;
         const int L = lev_count(nb0);
-        if (threadIdx.x == 0) s_pos = g0 * FMM_NPOOL;
-        __syncthreads();
-        for (int l = L - 1; l >= 0; l--) {
+        const FfScale fs = ff_scale(d[0], d[m - 1], 1.0);
+        // intervals of every level at once
+        int64_t gb = g0;
+        for (int l = 0; l < L; l++) {
             const int nb = lev_nb(nb0, l);
-            const int64_t gb = g0 + lev_base(nb0, l);
-            const int64_t gp0 = (l < L - 1) ? g0 + lev_base(nb0, l + 1) : 0;
             for (int b = threadIdx.x; b < nb; b += T) {
                 int i0, i1;
                 box_range(m, l, b, i0, i1);
-                blo[gb + b] = d[i0];
-                bhi[gb + b] = (i1 < m) ? d[i1] : d[m - 1];
+                const double lo = d[i0], hi = (i1 < m) ? d[i1] : d[m - 1];
+                blo[gb + b] = lo;
+                bhi[gb + b] = hi;
+                longlong2 v = make_longlong2(0, 0);      // out of scale: nothing is admissible
+                if (fs.ok) {
+                    v.x = (long long)((ff_fixed(lo, fs.kk) - fs.ref) >> 34);
+                    v.y = (long long)((ff_fixed(hi, fs.kk) - fs.ref) >> 34);
+                }
+                pl.ibox[gb + b] = v;
             }
+            gb += nb;
+        }
+        int64_t pos0 = g0 * FMM_NPOOL;                   // pool position of the level
+        for (int l = L - 1; l >= 0; l--) {
             __syncthreads();
-            // each thread a contiguous range of boxes: count, block prefix, fill
-            const int per = (nb + T - 1) / T;
-            const int bb = min(nb, (int)threadIdx.x * per), be = min(nb, bb + per);
+            const int nb = lev_nb(nb0, l);
+            gb = g0 + lev_base(nb0, l);
+            const int64_t gp0 = (l < L - 1) ? g0 + lev_base(nb0, l + 1) : 0;
+            const int seg = ((nb + T - 1) / T) * 32, beg = min(nb, warp * seg), end = min(nb, beg + seg);
+            // near counts (nnear holds them until the lists are placed)
             int64_t sum = 0;
-            for (int b = bb; b < be; b++) {
-                if (l == L - 1) { sum += 1; continue; }
-                const int64_t gp = gp0 + (b >> 1);
-                const int npn = nnear[gp];
-                if (npn >= 0) sum += near_count(blo, bhi, near, gb, nb, b, nstart[gp], npn);
-            }
-            int64_t pos = s_pos + cta_exscan(sum, wsum);
-            for (int b = bb; b < be; b++) {
-                int cnt;
-                if (l == L - 1) {
-                    cnt = 1;
-                    if (pos + 1 <= pool_end) near[pos] = b; else cnt = -1;
-                    nstart[gb + b] = pos;
-                    pos += 1;
-                } else {
-                    const int64_t gp = gp0 + (b >> 1);
-                    const int npn = nnear[gp];
-                    if (npn < 0) {
-                        cnt = -1;                                           // parent all near
-                        nstart[gb + b] = pos;
-                    } else {
-                        const int64_t pst = nstart[gp];
-                        const int c = near_count(blo, bhi, near, gb, nb, b, pst, npn);
-                        nstart[gb + b] = pos;
-                        if (pos + c <= pool_end) {
-                            const double loT = blo[gb + b], hiT = bhi[gb + b];
-                            int w = 0;
-                            for (int i = 0; i < npn; i++) {
-                                const int s2 = near[pst + i];
-                                for (int S = 2 * s2; S <= 2 * s2 + 1 && S < nb; S++)
-                                    if (S == b || !adm(blo[gb + S], bhi[gb + S], loT, hiT)) near[pos + w++] = S;
-                            }
-                            cnt = c;
-                        } else {
-                            cnt = -1;                                       // pool exhausted: all near
+            for (int c = beg; c < end; c += 32) {
+                const int b = c + lane;
+                int cnt = 0;
+                if (b < end) {
+                    unsigned long long mask = 0;
+                    if (l == L - 1) cnt = 1;
+                    else {
+                        const int npn = nnear[gp0 + (b >> 1)];
+                        if (npn < 0) cnt = -1;
+                        else {
+                            const int64_t pst = nstart[gp0 + (b >> 1)];
+                            mask = adm_mask(pl, gb, nb, b, pst, npn, 0);
+                            int far = __popcll(mask);
+                            for (int sec = 1; 64 * sec < 2 * npn; sec++)
+                                far += __popcll(adm_mask(pl, gb, nb, b, pst, npn, sec));
+                            // a candidate beyond the level's last box is neither
+                            cnt = 2 * npn - far - ((nb & 1) && near[pst + npn - 1] == (nb >> 1) ? 1 : 0);
                         }
-                        pos += c;
+                    }
+                    nnear[gb + b] = cnt;
+                    pl.amask[gb + b] = mask;
+                }
+                sum += max(cnt, 0);
+            }
+            for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(FULL, sum, o);
+            if (lane == 0) wsum[warp] = sum;
+            __syncthreads();
+            int64_t pos = pos0, all = 0;
+            for (int w = 0; w < T / 32; w++) {
+                const int64_t v = wsum[w];
+                pos += (w < warp) ? v : 0;
+                all += v;
+            }
+            pos0 += all;
+            // the lists, in box order
+            for (int c = beg; c < end; c += 32) {
+                const int b = c + lane;
+                const int cnt = (b < end) ? nnear[gb + b] : 0;
+                int x = max(cnt, 0);
+                const int own = x;
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int y = __shfl_up_sync(FULL, x, o);
+                    if (lane >= o) x += y;
+                }
+                const int64_t at = pos + x - own;
+                pos += __shfl_sync(FULL, x, 31);
+                if (b >= end) continue;
+                nstart[gb + b] = at;
+                bool fits = cnt >= 0;
+                if (cnt >= 0) {
+                    if (at + cnt > pool_end) {                                  // pool exhausted: all near
+                        fits = false;
+                        nnear[gb + b] = -1;
+                        pl.amask[gb + b] = 0;
+                    } else if (l == L - 1) {
+                        near[at] = b;
+                    } else {
+                        const int64_t pst = nstart[gp0 + (b >> 1)];
+                        const int npn = nnear[gp0 + (b >> 1)];
+                        unsigned long long mask = pl.amask[gb + b];
+                        int w = 0;
+                        for (int k = 0; k < 2 * npn; k++) {
+                            if (k > 0 && (k & 63) == 0) mask = adm_mask(pl, gb, nb, b, pst, npn, k >> 6);
+                            const int S = 2 * near[pst + (k >> 1)] + (k & 1);
+                            if (S < nb && !((mask >> (k & 63)) & 1)) near[at + w++] = S;
+                        }
                     }
                 }
-                nnear[gb + b] = cnt;
                 // leaf boxes with long near lists, for k_secular_fmm_split (in
                 // any order: each box's sweeps are independent of the others)
-                if (l == 0 && (cnt < 0 || cnt >= SPLIT_NEAR)) split[atomicAdd(nsplit, 1)] = leaf_base[p] + b;
+                if (l == 0 && (!fits || cnt >= SPLIT_NEAR)) pl.split[atomicAdd(pl.nsplit, 1)] = pl.leaf_base[p] + b;
             }
-            __syncthreads();
-            if (threadIdx.x == T - 1) s_pos = pos;
-            __syncthreads();
         }
         if (threadIdx.x == 0 && used) used[p] = 1;
         __syncthreads();
@@ -376,6 +397,7 @@ struct SrcArgs {
     const double *X;
     int64_t ldx;
     int col0, nc;
+    const int32_t *only;                 // columns: the problems with only[p] != 0 (out of scale), others by k_cm_up
 };
 
 // leaf moments and node weights of leaf box gl (box g, index Tb within its
@@ -580,7 +602,7 @@ __global__ void __launch_bounds__(up_threads<MODE>()) k_fmm_up(FmmDev pl, SrcArg
         const int64_t gl = next;
         if (gl >= nleaf) break;
         const int64_t p = sdc_upper_index(pl.leaf_base, pl.nprob, gl);
-        if (pl.fslot[p] < 0) continue;
+        if (pl.fslot[p] < 0 || (up_wide<MODE>() && a.only[p] == 0)) continue;
         const int Tb = (int)(gl - pl.leaf_base[p]);
         const int64_t g = pl.box_base[p] + Tb;
         const int kw = (MODE == M_SEC || MODE == M_BN) ? ff_exp(a.wsum[p]) - 1022 : 0;
@@ -649,40 +671,6 @@ __global__ void k_fmm_nodes(FmmDev pl, const int64_t *__restrict__ off, const in
         double c, h;
         box_ch(pl.blo[g], pl.bhi[g], c, h);
         pl.npos[t] = ff_point(c, h * xq[t % P], s);         // not rounded to the spacing of c
-    }
-}
-
-// candidates 64 sec .. 64 sec + 63 of box A (level base gb, parent's near list
-// at pst of npn boxes) that are admissible to it
-__device__ __forceinline__ unsigned long long adm_mask(const FmmDev &pl, int64_t gb, int nbl, int A, int64_t pst,
-                                                       int npn, int sec)
-{
-    unsigned long long mask = 0;
-    const double lo = pl.blo[gb + A], hi = pl.bhi[gb + A];
-    for (int c = 64 * sec; c < min(2 * npn, 64 * sec + 64); c++) {
-        const int S = 2 * pl.near[pst + (c >> 1)] + (c & 1);
-        if (S < nbl && S != A && adm(pl.blo[gb + S], pl.bhi[gb + S], lo, hi)) mask |= 1ull << (c & 63);
-    }
-    return mask;
-}
-
-// interaction list of every box: its first 64 candidates as a bit mask
-__global__ void k_fmm_adm(FmmDev pl, const int32_t *__restrict__ mk)
-{
-    const int64_t n = pl.box_base[pl.nprob];
-    for (int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; g < n; g += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t p = sdc_upper_index(pl.box_base, pl.nprob, g);
-        if (pl.fslot[p] < 0) continue;
-        const int nb0 = (mk[p] + B - 1) / B;
-        const int L = lev_count(nb0);
-        int A = (int)(g - pl.box_base[p]), l = 0;
-        while (A >= lev_nb(nb0, l)) { A -= lev_nb(nb0, l); l++; }
-        unsigned long long mask = 0;
-        if (l < L - 1 && pl.nnear[g] >= 0) {
-            const int64_t gP = pl.box_base[p] + lev_base(nb0, l + 1) + (A >> 1);
-            mask = adm_mask(pl, g - A, lev_nb(nb0, l), A, pl.nstart[gP], pl.nnear[gP], 0);
-        }
-        pl.amask[g] = mask;
     }
 }
 
@@ -1705,7 +1693,7 @@ __global__ void __launch_bounds__(128) k_fmm_lastsum(FmmDev pl, const int64_t *_
 //     in FP64.
 //   * Problems out of the positions' scale (cm_prep) take FP64 loops.
 // One warp per 16 targets, digit fragments read in mma order from global
-// memory (written once per call by k_cm_slice / k_cm_slicew).
+// memory (written once per call by k_cm_slice / k_cm_up).
 // ---------------------------------------------------------------------------
 constexpr int CM_D = 7;           // digits
 constexpr int CM_NT = 3;          // column tiles of 8 per pass
@@ -1828,40 +1816,6 @@ __global__ void k_cm_slice(FactorView f, int64_t nchunk_rows, const double *__re
     }
 }
 
-// node weights of one box (a warp per box): exponent over the columns' scales, digits
-__global__ void __launch_bounds__(128) k_cm_slicew(FmmDev pl, int col0, int nc, int nt, CmDev c)
-{
-    const unsigned FULL = 0xffffffffu;
-    const int lane = threadIdx.x & 31;
-    const int64_t n = pl.box_base[pl.nprob];
-    for (int64_t g = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; g < n;
-         g += ((int64_t)gridDim.x * blockDim.x) >> 5) {
-        const int64_t p = sdc_upper_index(pl.box_base, pl.nprob, g);
-        if (pl.fslot[p] < 0 || c.bad[p]) continue;
-        int e = -4000;
-        for (int col = 0; col < nc; col++) {
-            const double w = lane < P ? pl.W[(g * P + lane) * pl.ncol + col] : 0.0;
-            const int ex = ff_exp(w);
-            if (ex > 0) e = max(e, ex - 1022 - cm_exp(c, p, col0 + col));
-        }
-        e = __reduce_max_sync(FULL, e);
-        if (lane == 0) c.eb[g] = e;
-        for (int col = 0; col < nt * 8; col++) {
-            unsigned short dg[CM_D] = {0, 0, 0, 0, 0, 0, 0};
-            if (lane < P && col < nc && e > -4000)
-                cm_digits(ldexp(pl.W[(g * P + lane) * pl.ncol + col], -e - cm_exp(c, p, col0 + col)), dg);
-            const int k = lane, ln = (col & 7) * 4 + ((k & 7) >> 1);
-            if (k < 16) {
-                unsigned short *dst = (unsigned short *)(c.wf0 + ((g * nt + (col >> 3)) * CM_D) * 32 + ln);
-                for (int s = 0; s < CM_D; s++) dst[s * 32 * 4 + ((k >> 3) << 1) + (k & 1)] = dg[s];
-            } else if (k < 24) {
-                unsigned short *dst = (unsigned short *)(c.wf1 + ((g * nt + (col >> 3)) * CM_D) * 32 + ln);
-                for (int s = 0; s < CM_D; s++) dst[s * 32 * 2 + (k & 1)] = dg[s];
-            }
-        }
-    }
-}
-
 __device__ __forceinline__ void cm_mma16(float (&d)[4], const unsigned (&a)[4], uint2 b)
 {
     asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
@@ -1912,6 +1866,273 @@ __device__ __forceinline__ double cm_fold(const float (&a)[CM_D][4], int i)
     lo += (long long)__float2int_rn(a[5][i] * 0x1p54f) << 8;
     lo += __float2int_rn(a[6][i] * 0x1p62f);
     return fma((double)hi, 0x1p-30, (double)lo * 0x1p-62);
+}
+
+// ---------------------------------------------------------------------------
+// Node weights of blocks of columns, on the tensor cores: a leaf box's weights
+// are the matrix L_q(u_j) v_j (Chebyshev interpolation at the 22 nodes, times
+// the source factor) times its columns, a parent's the matrix L_q of its
+// children's nodes times their weights.  The matrices are formed by the second
+// barycentric formula L_q(u) = (w_q / (u - x_q)) / sum_k (w_k / (u - x_k)) in
+// three floats (Berrut and Trefethen, Barycentric Lagrange interpolation, 2004:
+// stable for any u in the interval), cut into digits and multiplied as in
+// k_cm_apply; the weights leave as the digits the next level and k_cm_apply
+// read.  The climb and its arrival counters are those of k_fmm_up, which still
+// does the problems out of scale.  A leaf and its parent took 33 k cycles of the
+// FP64 pipe for 24 columns.  Measured (GB300, f(A) X, n = 32768, 64 columns;
+// with k_cm_slicew): 196 -> 59 ms.
+// ---------------------------------------------------------------------------
+constexpr int CU_ROWS = 32;       // matrix rows (22 nodes, zeros below)
+constexpr int CU_LD = 56;         // bf16 per row: up to 48 sources, 112 bytes (no bank conflicts)
+
+// u - x, three floats each
+__device__ __forceinline__ ff_t3 ff_sub3(const ff_t3 &u, const ff_t3 &x)
+{
+    float s, e1, t, e2, e3;
+    ff_two_sum(u.a, -x.a, s, e1);
+    ff_two_sum(u.b, -x.b, t, e2);
+    ff_two_sum(t, e1, t, e3);
+    ff_t3 o;
+    ff_two_sum(s, t, o.a, t);
+    ff_fast_sum(t, ff_add(ff_sub(u.c, x.c), ff_add(e2, e3)), o.b, o.c);
+    return o;
+}
+
+__device__ __forceinline__ ff_t3 ff_shfl3(const ff_t3 &v, int mask)
+{
+    return {__shfl_xor_sync(0xffffffffu, v.a, mask), __shfl_xor_sync(0xffffffffu, v.b, mask),
+            __shfl_xor_sync(0xffffffffu, v.c, mask)};
+}
+
+// The columns k0 .. k0 + n - 1 of the digit matrices: four threads per source
+// take every fourth node.  su: sources' variables, sf: their factors.
+__device__ __forceinline__ void cu_matrix(const ff_t3 *su, const ff_t3 *sf, const ff_t3 *sx, const ff_t3 *sw, int k0,
+                                          int n, unsigned short (*As)[CU_ROWS][CU_LD])
+{
+    constexpr int QN = (P + 3) / 4;
+    for (int t0 = 0; t0 < n * 4; t0 += blockDim.x) {     // n a multiple of 8: whole warps
+        const int t = t0 + threadIdx.x, k = t >> 2, part = t & 3;
+        if (k >= n) continue;
+        const ff_t3 u = su[k];
+        ff_t3 wr[QN], D = {0.0f, 0.0f, 0.0f};
+#pragma unroll
+        for (int i = 0; i < QN; i++) {
+            const int q = min(part + 4 * i, P - 1);
+            ff_t3 d = ff_sub3(u, sx[q]);
+            if (fabsf(d.a) < 0x1p-60f) d = {0x1p-60f, 0.0f, 0.0f};     // on a node: L = 1 there, 2^-60 elsewhere
+            wr[i] = ff_mul3(sw[q], ff_rcp3(d));
+            if (part + 4 * i < P) ff_acc3(D, wr[i]);
+        }
+        ff_acc3(D, ff_shfl3(D, 1));
+        ff_acc3(D, ff_shfl3(D, 2));
+        // renormalise, then the source's factor over D
+        float s, e;
+        ff_fast_sum(D.a, D.b, s, e);
+        D.a = s;
+        ff_fast_sum(e, D.c, D.b, D.c);
+        const ff_t3 f = ff_mul3(sf[k], ff_rcp3(D));
+#pragma unroll
+        for (int i = 0; i < QN; i++) {
+            const int q = part + 4 * i;
+            if (q >= P) continue;
+            float dg[CM_D];
+            cm_cut(ff_mul3(wr[i], f), dg);
+#pragma unroll
+            for (int s2 = 0; s2 < CM_D; s2++) As[s2][q][k0 + k] = (unsigned short)(__float_as_uint(dg[s2]) >> 16);
+        }
+    }
+}
+
+template <int NT, bool TRANS>
+__global__ void __launch_bounds__(128) k_cm_up(FmmDev pl, FactorView f, CmDev c, int col0, int nc)
+{
+    __shared__ __align__(16) unsigned short As[CM_D][CU_ROWS][CU_LD];
+    __shared__ __align__(16) uint2 o0[NT * CM_D * 32];
+    __shared__ unsigned o1[NT * CM_D * 32];
+    __shared__ double Ws[P][NT * 8];
+    __shared__ ff_t3 sx[P], sw[P], su[48], sf[48];
+    __shared__ double xq[P];
+    __shared__ int s_e, s_last;
+    __shared__ int64_t s_next;
+    const unsigned FULL = 0xffffffffu;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, gr = lane >> 2, gc = lane & 3;
+    for (int i = tid; i < CM_D * CU_ROWS * CU_LD; i += 128) ((unsigned short *)As)[i] = 0;
+    if (tid < P) {
+        xq[tid] = cospi((double)(2 * tid + 1) / (2.0 * P));
+        sx[tid] = ff_split3(xq[tid]);
+        const double w = sinpi((double)(2 * tid + 1) / (2.0 * P));
+        sw[tid] = ff_split3((tid & 1) ? -w : w);
+    }
+    const int64_t nleaf = pl.leaf_base[pl.nprob];
+    for (;;) {
+        __syncthreads();
+        if (tid == 0) {
+            s_next = (int64_t)atomicAdd(&pl.upq[0], 1ull);
+            if (s_next >= nleaf && atomicAdd(&pl.upq[1], 1ull) == gridDim.x - 1) {
+                pl.upq[0] = 0;                 // every CTA has run past the end: reset for the next launch
+                pl.upq[1] = 0;
+            }
+        }
+        __syncthreads();
+        const int64_t gl = s_next;
+        if (gl >= nleaf) break;
+        const int64_t p = sdc_upper_index(pl.leaf_base, pl.nprob, gl);
+        if (pl.fslot[p] < 0 || c.bad[p]) continue;
+        const int64_t b0 = f.off[p], g0 = pl.box_base[p];
+        const int m = f.mk[p], nb0 = (m + B - 1) / B, L = lev_count(nb0);
+        const double *dk = f.dk + b0;
+        const int kk = ff_scale(dk[0], dk[m - 1], 1.0).kk;
+        int l = 0, b = (int)(gl - pl.leaf_base[p]);
+        for (;;) {
+            const int64_t g = g0 + lev_base(nb0, l) + b;
+            int nch = 0, E0 = 0;
+            int64_t gc0 = 0;
+            if (l == 0) {
+                // sources of the leaf: variable, factor scaled to at most one
+                if (warp == 0) {
+                    const int j = b * B + lane, jend = TRANS ? m : m - 1;
+                    double cT, hT;
+                    box_ch(pl.blo[g], pl.bhi[g], cT, hT);
+                    double u = 0.0;
+                    ff_t3 v = {0.0f, 0.0f, 0.0f};
+                    if (j < jend) {
+                        u = TRANS ? (dk[j] - cT) / hT : ((f.dorg[b0 + j] - cT) + f.eta[b0 + j]) / hT;
+                        const ff_f4 fc = c.fac[b0 + j];
+                        v = {fc.x, fc.y, fc.z};
+                    }
+                    int e = v.a != 0.0f ? ff_fexp(fabsf(v.a)) + 1 : -126;
+                    e = __reduce_max_sync(FULL, e);
+                    const float sc = pow2f(max(-126, min(126, -e)));
+                    su[lane] = ff_split3(u);
+                    sf[lane] = {v.a * sc, v.b * sc, v.c * sc};
+                    if (lane == 0) s_e = e - (TRANS ? 0 : kk);            // Qhat X: the factors carry 2^kk
+                }
+            } else {
+                const int nbc = lev_nb(nb0, l - 1);
+                gc0 = g0 + lev_base(nb0, l - 1) + 2 * b;
+                nch = (2 * b + 1 < nbc) ? 2 : 1;
+                if (warp < 2) {
+                    const int ea = __ldcg(&c.eb[gc0]), eb = nch > 1 ? __ldcg(&c.eb[gc0 + 1]) : -4000;
+                    const int em = max(ea, eb), ec = warp == 0 ? ea : eb;
+                    if (warp < nch) {
+                        double cP, hP, cc, hc;
+                        box_ch(pl.blo[g], pl.bhi[g], cP, hP);
+                        box_ch(pl.blo[gc0 + warp], pl.bhi[gc0 + warp], cc, hc);
+                        const double ih = rcp_nr2(hP);
+                        if (lane < 24) {
+                            // the node as scale and shift (exact for boxes of one point)
+                            su[warp * 24 + lane] = ff_split3(fma(hc * ih, xq[min(lane, P - 1)], (cc - cP) * ih));
+                            const float sc = (ec < em - 120 || lane >= P) ? 0.0f : pow2f(ec - em);
+                            sf[warp * 24 + lane] = {sc, 0.0f, 0.0f};
+                        }
+                    }
+                    if (warp == 0 && lane == 0) s_e = em;
+                }
+            }
+            __syncthreads();
+            E0 = s_e;
+            cu_matrix(su, sf, sx, sw, 0, l == 0 ? B : 24 * nch, As);
+            __syncthreads();
+            // products: (16 nodes, 8 columns) per warp
+            for (int un = warp; un < 2 * NT; un += 4) {
+                const int mt = un / NT, n = un % NT;
+                float acc[CM_D][4];
+#pragma unroll
+                for (int s = 0; s < CM_D; s++)
+#pragma unroll
+                    for (int i = 0; i < 4; i++) acc[s][i] = 0.0f;
+                const int r0 = mt * 16 + gr;
+                auto frag = [&](int s, int row, int k) {
+                    return *(const unsigned *)&As[s][row][k + 2 * gc];
+                };
+                const int n16 = l == 0 ? 2 : nch;
+                for (int st = 0; st < n16; st++) {
+                    const int k0 = l == 0 ? 16 * st : 24 * st;
+                    const uint2 *bf = l == 0 ? c.xf + (((cm_chunk(b0, p) + 2 * b + st) * NT + n) * CM_D) * 32 + lane
+                                             : c.wf0 + (((gc0 + st) * NT + n) * CM_D) * 32 + lane;
+                    if (l == 0 && b * B + 16 * st >= m) continue;
+                    uint2 bb[CM_D];
+                    unsigned a[CM_D][4];
+#pragma unroll
+                    for (int s = 0; s < CM_D; s++) {
+                        bb[s] = __ldcg(bf + s * 32);
+                        a[s][0] = frag(s, r0, k0);
+                        a[s][1] = frag(s, r0 + 8, k0);
+                        a[s][2] = frag(s, r0, k0 + 8);
+                        a[s][3] = frag(s, r0 + 8, k0 + 8);
+                    }
+#pragma unroll
+                    for (int i1 = 0; i1 < CM_D; i1++)
+#pragma unroll
+                        for (int j1 = 0; i1 + j1 < CM_D; j1++) cm_mma16(acc[i1 + j1], a[i1], bb[j1]);
+                }
+                for (int st = 0; st < nch; st++) {
+                    const unsigned *bf = c.wf1 + (((gc0 + st) * NT + n) * CM_D) * 32 + lane;
+                    unsigned bb[CM_D], a[CM_D][2];
+#pragma unroll
+                    for (int s = 0; s < CM_D; s++) {
+                        bb[s] = __ldcg(bf + s * 32);
+                        a[s][0] = frag(s, r0, 24 * st + 16);
+                        a[s][1] = frag(s, r0 + 8, 24 * st + 16);
+                    }
+#pragma unroll
+                    for (int i1 = 0; i1 < CM_D; i1++)
+#pragma unroll
+                        for (int j1 = 0; i1 + j1 < CM_D; j1++) cm_mma8(acc[i1 + j1], a[i1][0], a[i1][1], bb[j1]);
+                }
+#pragma unroll
+                for (int i = 0; i < 4; i++) {
+                    const int q = r0 + 8 * (i >> 1), col = n * 8 + 2 * gc + (i & 1);
+                    if (q < P) Ws[q][col] = col < nc ? cm_fold(acc, i) : 0.0;
+                }
+            }
+            __syncthreads();
+            // the box's exponent, then its digits
+            int ex = 0;
+            for (int i = tid; i < P * NT * 8; i += 128) ex = max(ex, ff_exp(Ws[i / (NT * 8)][i % (NT * 8)]));
+            ex = __reduce_max_sync(FULL, ex);
+            if (tid == 0) s_e = 0;
+            __syncthreads();
+            if (lane == 0) atomicMax(&s_e, ex);
+            __syncthreads();
+            ex = s_e;
+            const double sc = ex > 0 ? ff_pow2(1022 - ex) : 0.0;
+            for (int i = tid; i < 24 * NT * 8; i += 128) {
+                const int k = i / (NT * 8), col = i % (NT * 8);
+                unsigned short dg[CM_D];
+                cm_digits(k < P ? Ws[k][col] * sc : 0.0, dg);
+                const int ln = (col & 7) * 4 + ((k & 7) >> 1), at = (col >> 3) * CM_D * 32 + ln;
+                unsigned short *dst = k < 16 ? (unsigned short *)(o0 + at) + ((k >> 3) << 1) + (k & 1)
+                                             : (unsigned short *)(o1 + at) + (k & 1);
+                const int step = k < 16 ? 32 * 4 : 32 * 2;
+#pragma unroll
+                for (int s = 0; s < CM_D; s++) dst[s * step] = dg[s];
+            }
+            __syncthreads();
+            for (int i = tid; i < NT * CM_D * 32; i += 128) {
+                c.wf0[g * NT * CM_D * 32 + i] = o0[i];
+                c.wf1[g * NT * CM_D * 32 + i] = o1[i];
+            }
+            if (tid == 0) c.eb[g] = ex > 0 ? E0 + ex - 1022 : -4000;
+            if (l + 1 >= L) break;
+            // the child that arrives last computes the parent (k_fmm_up)
+            const int bp = b >> 1;
+            const int nsib = (2 * bp + 1 < lev_nb(nb0, l)) ? 2 : 1;
+            const int64_t gp = g0 + lev_base(nb0, l + 1) + bp;
+            __threadfence();
+            __syncthreads();
+            if (tid == 0) {
+                const int old = atomicAdd(&pl.upcnt[gp], 1);
+                s_last = (old == nsib - 1);
+                if (s_last) pl.upcnt[gp] = 0;
+            }
+            __syncthreads();
+            if (!s_last) break;
+            __threadfence();
+            l++;
+            b = bp;
+        }
+    }
 }
 
 template <int NT, bool TRANS>
@@ -1966,7 +2187,7 @@ k_cm_apply(FmmDev pl, FactorView f, const int64_t *__restrict__ tile_off, CmDev 
                     for (int i = 0; i < 2 * pl.nnear[gP]; i++) {
                         const int S = 2 * pl.near[pl.nstart[gP] + (i >> 1)] + (i & 1);
                         if (S >= lev_nb(nb0, l) || S == A ||
-                            !adm(pl.blo[gl + S], pl.bhi[gl + S], pl.blo[gl + A], pl.bhi[gl + A]))
+                            !adm(pl.ibox[gl + S], pl.ibox[gl + A]))
                             continue;
                         double cS, hS;
                         box_ch(pl.blo[gl + S], pl.bhi[gl + S], cS, hS);
@@ -2351,6 +2572,13 @@ superdc_status far_field(const FmmPlan &pl, const int64_t *off, const R1Out &o, 
 }
 
 template <int NT>
+void launch_up(bool trans, const FmmDev &dv, const FactorView &f, const CmDev &c, int col0, int nc, cudaStream_t st)
+{
+    if (trans) k_cm_up<NT, true><<<resident_grid<k_cm_up<NT, true>>(128), 128, 0, st>>>(dv, f, c, col0, nc);
+    else k_cm_up<NT, false><<<resident_grid<k_cm_up<NT, false>>(128), 128, 0, st>>>(dv, f, c, col0, nc);
+}
+
+template <int NT>
 void launch_apply(bool trans, const FmmDev &dv, const FactorView &f, const int64_t *tile_off, const CmDev &c,
                   const double *X, int64_t ldx, double *Y, int64_t ldy, int col0, int nc, int64_t tiles, cudaStream_t st)
 {
@@ -2408,6 +2636,7 @@ superdc_status plan(FmmPlan &pl, int64_t nprob, const int64_t *off, int64_t tota
     SDC_CHECK(al(&d.W, (size_t)pl.cap_boxes * P * ncol));
     SDC_CHECK(al(&d.npos, (size_t)pl.cap_boxes * P));
     SDC_CHECK(al(&d.amask, (size_t)pl.cap_boxes));
+    SDC_CHECK(al(&d.ibox, (size_t)pl.cap_boxes));
     if (step) {
         SDC_CHECK(al(&d.coef, (size_t)pl.cap_leaves * NFIELD * P));
         SDC_CHECK(al(&d.lastp, (size_t)pl.cap_leaves));
@@ -2435,15 +2664,12 @@ superdc_status plan(FmmPlan &pl, int64_t nprob, const int64_t *off, int64_t tota
     const unsigned gt = (unsigned)std::min<int64_t>(nprob, (int64_t)sdc_num_sms() * 4);
     const int tt = (nprob < sdc_num_sms()) ? 1024 : 256;
     SDC_CHECK(cudaMemsetAsync(d.nsplit, 0, sizeof(int32_t), st));
-    PROF_LAUNCH("fmm_tree", st, k_fmm_tree<<<gt, tt, 0, st>>>(nprob, off, mk, dk, box_base, fslot, blo, bhi,
-                                                               nnear, nstart, near, used, leaf_base, d.split,
-                                                               d.nsplit));
+    PROF_LAUNCH("fmm_tree", st, k_fmm_tree<<<gt, tt, 0, st>>>(d, off, mk, dk, blo, bhi, nnear, nstart, near, used));
     {
         auto gr = [&](int64_t n) {
             return (unsigned)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, (int64_t)sdc_num_sms() * 8));
         };
         PROF_LAUNCH("fmm_plan", st, k_fmm_nodes<<<gr(pl.cap_boxes * P), 256, 0, st>>>(d, off, mk, dk));
-        PROF_LAUNCH("fmm_plan", st, k_fmm_adm<<<gr(pl.cap_boxes), 256, 0, st>>>(d, mk));
     }
     SDC_CHECK(cudaGetLastError());
     pl.on = true;
@@ -2544,10 +2770,11 @@ superdc_status columns(const FmmPlan &pl, const FactorView &f, int64_t total, co
         if (pl.on) {
             SrcArgs a{};
             a.off = f.off; a.mk = f.mk; a.dk = f.dk; a.vhat = f.vhat; a.bnorm = f.bnorm; a.dorg = f.dorg; a.eta = f.eta;
-            a.src = f.src; a.pinv = f.pinv; a.X = X; a.ldx = ldx; a.col0 = c0; a.nc = nc;
+            a.src = f.src; a.pinv = f.pinv; a.X = X; a.ldx = ldx; a.col0 = c0; a.nc = nc; a.only = c.bad;
             if (trans) PROF_LAUNCH("fmm_up", st, k_fmm_up<M_CT><<<up_grid<M_CT>(), up_threads<M_CT>(), 0, st>>>(dv, a));
             else PROF_LAUNCH("fmm_up", st, k_fmm_up<M_CN><<<up_grid<M_CN>(), up_threads<M_CN>(), 0, st>>>(dv, a));
-            PROF_LAUNCH("fmm_up", st, k_cm_slicew<<<gr(pl.cap_boxes * 32), 128, 0, st>>>(dv, c0, nc, nt, c));
+            auto up = (nt == 1) ? launch_up<1> : (nt == 2) ? launch_up<2> : launch_up<3>;
+            PROF_LAUNCH("fmm_up", st, up(trans, dv, f, c, c0, nc, st));
         }
         auto fn = (nt == 1) ? launch_apply<1> : (nt == 2) ? launch_apply<2> : launch_apply<3>;
         PROF_LAUNCH("cauchy", st, fn(trans, dv, f, tile_off, c, X, ldx, Y, ldy, c0, nc, tiles, st));
