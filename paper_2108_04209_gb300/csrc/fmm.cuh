@@ -51,7 +51,7 @@ struct FmmDev {
     unsigned long long *upq;               // upward pass: next unclaimed leaf box, CTAs past the end
     int64_t *split;                        // leaf boxes with long near lists (any order) and their
     int32_t *nsplit;                       // count, filled by the tree build
-    int32_t *ffbad;                        // per problem: 1 if the split FP32 forms (split.cuh) are not
+    int32_t *ffbad;                        // per problem (then for any): 1 if the split FP32 forms (split.cuh) are not
                                            // allowed; written with the secular roots, read by zhat and b
     int64_t cap_f;                         // capacity of the FMM problem list
     int ncol;                              // width of the node weights (columns)

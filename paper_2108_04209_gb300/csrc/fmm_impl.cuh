@@ -397,7 +397,8 @@ struct SrcArgs {
     const double *X;
     int64_t ldx;
     int col0, nc;
-    const int32_t *only;                 // columns: the problems with only[p] != 0 (out of scale), others by k_cm_up
+    const int32_t *only;                 // k_fmm_up: the problems with only[p] != 0 (out of scale); the others
+                                         // are k_fmm_up1's and k_cm_up's
 };
 
 // leaf moments and node weights of leaf box gl (box g, index Tb within its
@@ -409,7 +410,7 @@ constexpr int UP_ROWS = (B > 2 * P) ? B : 2 * P;   // rows of the staging arrays
 
 template <int MODE, int WW>
 __device__ __forceinline__ void leaf_moments(const FmmDev &pl, const SrcArgs &a, int64_t p, int64_t gl, int64_t g,
-                                             int Tb, int nw, int kw, double (*Tt)[P + 1], double (*Wt)[WW + 1],
+                                             int Tb, int nw, double (*Tt)[P + 1], double (*Wt)[WW + 1],
                                              double (*Ms)[WW + 1], const double *Tx)
 {
     const int tid = threadIdx.x;
@@ -486,7 +487,6 @@ __device__ __forceinline__ void leaf_moments(const FmmDev &pl, const SrcArgs &a,
         double s = Ms[0][q];
         for (int n = 1; n < P; n++) s = fma(Tx[qn * P + n], Ms[n][q], s);     // Tx holds 2 T_n
         pl.W[(g * P + qn) * pl.ncol + q] = s * (1.0 / P);
-        if (WW == 1) pl.nwt[g * P + qn] = ff_weight(s * (1.0 / P), kw);       // for k_fmm_far
     }
     // Chebyshev recurrence per source, moments, moments -> node weights
     const int64_t cnt = max(0, min(B, jend - Tb * B));
@@ -500,7 +500,7 @@ __device__ __forceinline__ void leaf_moments(const FmmDev &pl, const SrcArgs &a,
 // through L2 (ld.global.cg): the sibling's were written by another CTA of the
 // same launch, which published them before its arrival count.
 template <int WW>
-__device__ __forceinline__ void m2m_box(const FmmDev &pl, int64_t p, int nb0, int l, int b, int64_t g, int nw, int kw,
+__device__ __forceinline__ void m2m_box(const FmmDev &pl, int64_t p, int nb0, int l, int b, int64_t g, int nw,
                                         double (*Tv)[P + 1], double (*Wc)[WW + 1], double (*Ms)[WW + 1],
                                         const double *Tx, const double *xq)
 {
@@ -551,7 +551,6 @@ __device__ __forceinline__ void m2m_box(const FmmDev &pl, int64_t p, int nb0, in
         double s = Ms[0][q];
         for (int n = 1; n < P; n++) s = fma(Tx[qn * P + n], Ms[n][q], s);     // Tx holds 2 T_n
         pl.W[(g * P + qn) * pl.ncol + q] = s * (1.0 / P);
-        if (WW == 1) pl.nwt[g * P + qn] = ff_weight(s * (1.0 / P), kw);       // for k_fmm_far
     }
     // children's node positions, the children's weights into moments, moments -> weights
     fl_add(pl, (int64_t)nch * 2 * P * (P - 2) + (int64_t)nch * 2 * P * P * nw + 2 * P * P * nw);
@@ -583,6 +582,7 @@ __global__ void __launch_bounds__(up_threads<MODE>()) k_fmm_up(FmmDev pl, SrcArg
     __shared__ double Tx[P * P], xq[P];
     __shared__ int last;
     __shared__ int64_t next;
+    if (a.only[pl.nprob] == 0) return;             // no problem out of scale
     cheb_tables(xq, Tx, 2.0);          // 2 T_n(x_q), n >= 1: the moments -> weights sums
     const int nw = (MODE == M_CT || MODE == M_CN) ? a.nc : 1;
     const int tid = threadIdx.x;
@@ -602,11 +602,10 @@ __global__ void __launch_bounds__(up_threads<MODE>()) k_fmm_up(FmmDev pl, SrcArg
         const int64_t gl = next;
         if (gl >= nleaf) break;
         const int64_t p = sdc_upper_index(pl.leaf_base, pl.nprob, gl);
-        if (pl.fslot[p] < 0 || (up_wide<MODE>() && a.only[p] == 0)) continue;
+        if (pl.fslot[p] < 0 || a.only[p] == 0) continue;
         const int Tb = (int)(gl - pl.leaf_base[p]);
         const int64_t g = pl.box_base[p] + Tb;
-        const int kw = (MODE == M_SEC || MODE == M_BN) ? ff_exp(a.wsum[p]) - 1022 : 0;
-        leaf_moments<MODE, WW>(pl, a, p, gl, g, Tb, nw, kw, Tt, Wt, Ms, Tx);
+        leaf_moments<MODE, WW>(pl, a, p, gl, g, Tb, nw, Tt, Wt, Ms, Tx);
         const int nb0 = (a.mk[p] + B - 1) / B;
         const int L = lev_count(nb0);
         int l = 0, b = Tb;
@@ -624,7 +623,183 @@ __global__ void __launch_bounds__(up_threads<MODE>()) k_fmm_up(FmmDev pl, SrcArg
             __syncthreads();
             if (!last) break;
             __threadfence();
-            m2m_box<WW>(pl, p, nb0, l + 1, bp, gp, nw, kw, Tt, Wt, Ms, Tx, xq);
+            m2m_box<WW>(pl, p, nb0, l + 1, bp, gp, nw, Tt, Wt, Ms, Tx, xq);
+            l++;
+            b = bp;
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------
+// The upward pass of the one-column sums in split arithmetic, one warp per box:
+// the weight of node q is sum_j f_j w_q / (u_j - x_q), f_j = (weight of source
+// j) / sum_k w_k / (u_j - x_k) (second barycentric formula; the sources are a
+// leaf's poles, or the nodes of a box's children).  First a lane per source for
+// f, then a lane per node.  The dipoles of zhat (lambda_j minus d_j, nearly
+// cancelling) keep FP64 at the leaves: the moments' own difference recurrence.
+// Climb and counters as in k_fmm_up, which does the problems out of scale.
+// Measured (GB300, 4096 problems of 32..2048 poles): 1.9 + 1.9 + 2.3 -> 1.1 + 1.1 + 1.4 ms
+// (secular, b, zhat).
+// ---------------------------------------------------------------------------
+template <int MODE>
+__global__ void __launch_bounds__(128) k_fmm_up1(FmmDev pl, SrcArgs a)
+{
+    __shared__ double xq[P], wq[P], Tx[(MODE == M_LOW) ? P * P : 1];
+    __shared__ double Tt[(MODE == M_LOW) ? 4 : 1][(MODE == M_LOW) ? B : 1][P + 1];
+    __shared__ ff_f2 sx[P], sw[P], su[4][2 * P], sf[4][2 * P];
+    const unsigned FULL = 0xffffffffu;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (MODE == M_LOW) cheb_tables(xq, Tx, 2.0);
+    if (threadIdx.x < P) {
+        const int q = threadIdx.x;
+        const double w = sinpi((double)(2 * q + 1) / (2.0 * P));
+        if (MODE != M_LOW) xq[q] = cospi((double)(2 * q + 1) / (2.0 * P));
+        wq[q] = (q & 1) ? -w : w;
+        sx[q] = ff_weight(xq[q], 0);
+        sw[q] = ff_weight(wq[q], 0);
+    }
+    __syncthreads();
+    // d = u - x, away from zero (on a node: its weight is one, the others' 2^-60)
+    auto diff = [&](const ff_f2 &u, const ff_f2 &x, float &t, float &tl) {
+        float s, e;
+        ff_two_sum(u.x, -x.x, s, e);
+        ff_fast_sum(s, ff_add(e, ff_sub(u.y, x.y)), t, tl);
+        if (fabsf(t) < 0x1p-60f) { t = 0x1p-60f; tl = 0.0f; }
+    };
+    // f of the source in this lane
+    auto factor = [&](const ff_f2 &u, const ff_f2 &w) {
+        FfAcc D = {};
+#pragma unroll
+        for (int q = 0; q < P; q++) {
+            float t, tl, p, pr;
+            diff(u, sx[q], t, tl);
+            ff_div(sw[q], t, tl, p, pr);
+            ff_addto(D, p, pr);
+            if ((q & 7) == 7) ff_norm(D);
+        }
+        ff_norm(D);
+        ff_f2 f;
+        ff_div(w, D.b, D.bl, f.x, f.y);
+        return f;
+    };
+    // weight of node lane from n sources (in units of the split weights)
+    auto weight = [&](int n) {
+        FfAcc S = {};
+        const ff_f2 x = sx[min(lane, P - 1)];
+#pragma unroll 8
+        for (int j = 0; j < n; j++) {
+            float t, tl, p, pr;
+            diff(su[warp][j], x, t, tl);
+            ff_div(sf[warp][j], t, tl, p, pr);
+            ff_addto(S, p, pr);
+            if ((j & 7) == 7) ff_norm(S);
+        }
+        return ((double)S.b + (double)S.bl) * wq[min(lane, P - 1)];
+    };
+    const int64_t nleaf = pl.leaf_base[pl.nprob];
+    for (;;) {
+        int64_t gl = 0;
+        if (lane == 0) {
+            gl = (int64_t)atomicAdd(&pl.upq[0], 1ull);
+            if (gl >= nleaf && atomicAdd(&pl.upq[1], 1ull) == 4ull * gridDim.x - 1) {
+                pl.upq[0] = 0;                 // every warp has run past the end: reset for the next launch
+                pl.upq[1] = 0;
+            }
+        }
+        gl = __shfl_sync(FULL, gl, 0);
+        if (gl >= nleaf) break;
+        const int64_t p = sdc_upper_index(pl.leaf_base, pl.nprob, gl);
+        if (pl.fslot[p] < 0 || pl.ffbad[p]) continue;
+        const int64_t b0 = a.off[p], g0 = pl.box_base[p];
+        const int m = a.mk[p], nb0 = (m + B - 1) / B, L = lev_count(nb0);
+        const int kw = (MODE == M_LOW) ? 0 : ff_exp(a.wsum[p]) - 1022;
+        int l = 0, b = (int)(gl - pl.leaf_base[p]);
+        for (;;) {
+            const int64_t g = g0 + lev_base(nb0, l) + b;
+            double s;                          // weight of node lane, times 2^-kw
+            __syncwarp();
+            if (l == 0 && MODE == M_LOW) {
+                // D_n = T_n(b) - T_n(a) with b = a + delta, by the recurrence
+                // D_{n+1} = 2 delta T_n(b) + 2 a D_n - D_{n-1} (no cancellation)
+                double c, h, av = 0.0, dl = 0.0;
+                box_ch(pl.blo[g], pl.bhi[g], c, h);
+                const int j = b * B + lane;
+                if (j < m - 1) {
+                    const double ih = 1.0 / h;
+                    av = (a.dk[b0 + j] - c) * ih;
+                    dl = ((a.dorg[b0 + j] - a.dk[b0 + j]) + a.eta[b0 + j]) * ih;
+                }
+                const double bv = av + dl, a2 = 2.0 * av, d2 = 2.0 * dl, b2 = 2.0 * bv;
+                double tb0 = 1.0, tb1 = bv, D0 = 0.0, D1 = dl;
+                double *T = Tt[(MODE == M_LOW) ? warp : 0][(MODE == M_LOW) ? lane : 0];
+                T[1] = D1;
+                for (int n = 1; n < P - 1; n++) {
+                    const double D2 = fma(d2, tb1, fma(a2, D1, -D0)), tb2 = fma(b2, tb1, -tb0);
+                    T[n + 1] = D2;
+                    D0 = D1; D1 = D2; tb0 = tb1; tb1 = tb2;
+                }
+                __syncwarp();
+                double mom = 0.0;
+                const int n = min(lane, P - 1);
+                for (int k = 0; k < B && n > 0; k++) mom += Tt[(MODE == M_LOW) ? warp : 0][(MODE == M_LOW) ? k : 0][n];
+                __syncwarp();
+                Tt[(MODE == M_LOW) ? warp : 0][0][n] = mom;          // every lane has read its column
+                __syncwarp();
+                s = 0.0;
+                for (int k = 1; k < P; k++) s = fma(Tx[n * P + k], Tt[(MODE == M_LOW) ? warp : 0][0][k], s);
+                s *= 1.0 / P;
+            } else if (l == 0) {
+                double c, h;
+                box_ch(pl.blo[g], pl.bhi[g], c, h);
+                const int j = b * B + lane;
+                ff_f2 u = {0.0f, 0.0f}, w = {0.0f, 0.0f};
+                if (j < m) {
+                    const double z = (MODE == M_SEC) ? a.zk[b0 + j] : a.vhat[b0 + j];
+                    u = ff_weight((a.dk[b0 + j] - c) * rcp_nr2(h), 0);
+                    w = ff_weight(z * z, kw);
+                }
+                su[warp][lane] = u;
+                sf[warp][lane] = factor(u, w);
+                __syncwarp();
+                s = weight(min(B, m - b * B));
+            } else {
+                const int nbc = lev_nb(nb0, l - 1), nch = (2 * b + 1 < nbc) ? 2 : 1;
+                const int64_t gc = g0 + lev_base(nb0, l - 1) + 2 * b;
+                double cP, hP;
+                box_ch(pl.blo[g], pl.bhi[g], cP, hP);
+                const double ih = rcp_nr2(hP);
+                for (int ci = 0; ci < nch; ci++) {
+                    double cc, hc;
+                    box_ch(pl.blo[gc + ci], pl.bhi[gc + ci], cc, hc);
+                    const int q = min(lane, P - 1);
+                    // the node as scale and shift (exact for boxes of one point)
+                    const ff_f2 u = ff_weight(fma(hc * ih, xq[q], (cc - cP) * ih), 0);
+                    const float2 w = __ldcg((const float2 *)&pl.nwt[(gc + ci) * P + q]);
+                    const ff_f2 f = factor(u, {w.x, w.y});
+                    if (lane < P) {
+                        su[warp][ci * P + lane] = u;
+                        sf[warp][ci * P + lane] = f;
+                    }
+                }
+                __syncwarp();
+                s = weight(nch * P);
+            }
+            if (lane < P) {
+                pl.nwt[g * P + lane] = ff_weight(s, 0);
+                if (MODE == M_SEC) pl.W[(g * P + lane) * pl.ncol] = s * ff_pow2(kw);       // k_secular_last
+            }
+            if (l + 1 >= L) break;
+            const int bp = b >> 1, nsib = (2 * bp + 1 < lev_nb(nb0, l)) ? 2 : 1;
+            const int64_t gp = g0 + lev_base(nb0, l + 1) + bp;
+            __threadfence();
+            __syncwarp();
+            int last = 0;
+            if (lane == 0) {
+                last = atomicAdd(&pl.upcnt[gp], 1) == nsib - 1;
+                if (last) pl.upcnt[gp] = 0;
+            }
+            if (!__shfl_sync(FULL, last, 0)) break;
+            __threadfence();
             l++;
             b = bp;
         }
@@ -943,6 +1118,7 @@ __global__ void k_ff_prep(int64_t nprob, const int64_t *__restrict__ off, int64_
         const FfScale s = ff_scale(o.dk[b0], o.dk[b0 + m - 1], o.wsum[p]);
         if (!s.ok || o.unshifted || (j + 1 < m && !ff_gap_ok(o.dk[x], o.dk[x + 1], s.kk))) {
             bad[p] = 1;
+            bad[nprob] = 1;
             continue;
         }
         const double z = o.zk[x];
@@ -1719,7 +1895,7 @@ __device__ __forceinline__ void cm_digits(double y, unsigned short *out)
 // positions and factors of the sources, and the problems out of scale
 struct CmDev {
     ff_f4 *pos, *fac;            // per slot: source position, source factor (three floats)
-    int32_t *bad;                // per problem
+    int32_t *bad;                // per problem, then whether any is
     int32_t *cmax;               // per (problem, column of the call): biased exponent of max |x|
     int64_t ccols;               // columns of the call (stride of cmax)
     uint2 *xf;                   // column digits in mma order: [chunk][tile][digit][lane]
@@ -1749,6 +1925,7 @@ __global__ void k_cm_prep(FactorView f, int64_t total, CmDev c)
         ok = ok && ev > 923 && ev < 1113 && eb > 923 && eb < 1113;
         if (!ok) {
             c.bad[p] = 1;
+            c.bad[f.nprob] = 1;
             continue;
         }
         const ff_t3 t = ff_split3(v);
@@ -2564,7 +2741,11 @@ template <int MODE, int KER>
 superdc_status far_field(const FmmPlan &pl, const int64_t *off, const R1Out &o, cudaStream_t st)
 {
     const FmmDev &dv = pl.dv;
-    PROF_LAUNCH("fmm_up", st, k_fmm_up<MODE><<<up_grid<MODE>(), up_threads<MODE>(), 0, st>>>(dv, src_from_r1(off, o)));
+    SrcArgs a = src_from_r1(off, o);
+    a.only = dv.ffbad;
+    const unsigned gu = (unsigned)std::min<int64_t>((pl.cap_leaves + 3) / 4, resident_grid<k_fmm_up1<MODE>>(128));
+    PROF_LAUNCH("fmm_up", st, k_fmm_up1<MODE><<<gu, 128, 0, st>>>(dv, a));
+    PROF_LAUNCH("fmm_up", st, k_fmm_up<MODE><<<up_grid<MODE>(), up_threads<MODE>(), 0, st>>>(dv, a));
     const int64_t want = (pl.cap_leaves + FAR_NW - 1) / FAR_NW;
     const unsigned g = (unsigned)std::min<int64_t>(want, resident_grid<k_fmm_far<KER>>(FAR_NW * 32));
     PROF_LAUNCH("fmm_far", st, k_fmm_far<KER><<<g, FAR_NW * 32, 0, st>>>(dv, off, o));
@@ -2644,7 +2825,7 @@ superdc_status plan(FmmPlan &pl, int64_t nprob, const int64_t *off, int64_t tota
         SDC_CHECK(al(&d.ntail, 2));
         SDC_CHECK(cudaMemsetAsync(d.ntail, 0, 2 * sizeof(unsigned int), st));
         SDC_CHECK(al(&d.nwt, (size_t)pl.cap_boxes * P));
-        SDC_CHECK(al(&d.ffbad, nprob));
+        SDC_CHECK(al(&d.ffbad, nprob + 1));
     }
     SDC_CHECK(al(&d.upcnt, pl.cap_boxes));
     SDC_CHECK(cudaMemsetAsync(d.upcnt, 0, (size_t)pl.cap_boxes * sizeof(int32_t), st));
@@ -2693,7 +2874,7 @@ superdc_status secular(const FmmPlan &pl, const int64_t *off, const R1Out &o, do
     SdcScratch sc(st);
     SDC_CHECK(sc.get(&fd, (size_t)pl.total));
     SDC_CHECK(sc.get(&fw, (size_t)pl.total));
-    SDC_CHECK(cudaMemsetAsync(pl.dv.ffbad, 0, (size_t)pl.dv.nprob * sizeof(int32_t), st));
+    SDC_CHECK(cudaMemsetAsync(pl.dv.ffbad, 0, (size_t)(pl.dv.nprob + 1) * sizeof(int32_t), st));
     const unsigned gp = (unsigned)std::max<int64_t>(1, std::min<int64_t>((pl.total + 255) / 256,
                                                                          (int64_t)sdc_num_sms() * 8));
     PROF_LAUNCH("fmm_secular", st, k_ff_prep<<<gp, 256, 0, st>>>(pl.dv.nprob, off, pl.total, pl.dv.fslot, o, fd, fw,
@@ -2743,7 +2924,7 @@ superdc_status columns(const FmmPlan &pl, const FactorView &f, int64_t total, co
     c.ccols = ncols;
     SDC_CHECK(sc.get(&c.pos, (size_t)total));
     SDC_CHECK(sc.get(&c.fac, (size_t)total));
-    SDC_CHECK(sc.get(&c.bad, (size_t)f.nprob));
+    SDC_CHECK(sc.get(&c.bad, (size_t)f.nprob + 1));
     SDC_CHECK(sc.get(&c.cmax, (size_t)f.nprob * ncols));
     SDC_CHECK(sc.get(&c.xf, (size_t)chunks * ntmax * CM_D * 32));
     if (trans) SDC_CHECK(sc.get(&c.lastp, (size_t)tiles * CM_NT * 8));
@@ -2752,7 +2933,7 @@ superdc_status columns(const FmmPlan &pl, const FactorView &f, int64_t total, co
         SDC_CHECK(sc.get(&c.wf1, (size_t)pl.cap_boxes * ntmax * CM_D * 32));
         SDC_CHECK(sc.get(&c.eb, (size_t)pl.cap_boxes));
     }
-    SDC_CHECK(cudaMemsetAsync(c.bad, 0, (size_t)f.nprob * sizeof(int32_t), st));
+    SDC_CHECK(cudaMemsetAsync(c.bad, 0, ((size_t)f.nprob + 1) * sizeof(int32_t), st));
     SDC_CHECK(cudaMemsetAsync(c.cmax, 0, (size_t)f.nprob * ncols * sizeof(int32_t), st));
     auto gr = [&](int64_t n) {
         return (unsigned)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, (int64_t)sdc_num_sms() * 8));

@@ -160,6 +160,16 @@ FF_HD void ff_term(const ff_f4 &d, const ff_f2 &w, const ff_f4 &x, float &p, flo
     q = ff_mul(p, r);
 }
 
+// p + pl = w / (t + tl)
+FF_HD void ff_div(const ff_f2 &w, float t, float tl, float &p, float &pl)
+{
+    float r = ff_rcp(t);
+    r = ff_fma(r, ff_fma(-t, r, 1.0f), r);
+    const float rl = ff_mul(r, ff_fma(-tl, r, ff_fma(-t, r, 1.0f)));
+    p = ff_mul(w.x, r);
+    pl = ff_fma(w.y, r, ff_fma(w.x, rl, ff_fma(w.x, r, -p)));
+}
+
 // p + pl = w / (d - x)^2
 FF_HD void ff_term2(const ff_f4 &d, const ff_f2 &w, const ff_f4 &x, float &p, float &pl)
 {
