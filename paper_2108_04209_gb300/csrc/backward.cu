@@ -33,6 +33,7 @@
 #include "cauchy.cuh"
 #include "fmm.cuh"
 #include "prof.cuh"
+#include "tiles.cuh"
 #include "secular.cuh"
 
 namespace {
@@ -244,26 +245,6 @@ __global__ void k_bw_rotate(int64_t nprob, const int64_t *__restrict__ off, int6
     }
 }
 
-__global__ void k_tiles_b(int64_t nprob, const int32_t *__restrict__ mk, int tr, int64_t *__restrict__ tile_off)
-{
-    __shared__ int64_t part[1024];
-    const int T = blockDim.x;
-    int64_t per = (nprob + T - 1) / T;
-    int64_t beg = threadIdx.x * per, end = min(nprob, beg + per);
-    int64_t s = 0;
-    for (int64_t q = beg; q < end; q++) s += (mk[q] + tr - 1) / tr;
-    part[threadIdx.x] = s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int64_t acc = 0;
-        for (int i = 0; i < T; i++) { int64_t v = part[i]; part[i] = acc; acc += v; }
-        tile_off[nprob] = acc;
-    }
-    __syncthreads();
-    int64_t acc = part[threadIdx.x];
-    for (int64_t q = beg; q < end; q++) { tile_off[q] = acc; acc += (mk[q] + tr - 1) / tr; }
-}
-
 }  // namespace
 
 // Adjoint of one batched rank-one step given its factor view (pinv and d_K
@@ -284,7 +265,7 @@ superdc_status r1_backward_fv(const FactorView &f, int64_t total, const double *
     SDC_CHECK(sc.get(&tile_off, f.nprob + 1));
     SDC_CHECK(cudaMemsetAsync(u, 0, total * sizeof(double), st));
     SDC_CHECK(cudaMemsetAsync(g, 0, total * sizeof(double), st));
-    k_tiles_b<<<1, 1024, 0, st>>>(f.nprob, f.mk, BW_T, tile_off);
+    k_tiles<<<1, tiles_threads(f.nprob), 0, st>>>(f.nprob, f.mk, BW_T, tile_off);
     superdc_status s = SUPERDC_OK;
     const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(total / BW_T + f.nprob, (int64_t)nsm * 8));
     if (ncols > 0) {

@@ -11,30 +11,11 @@
 #include "cauchy.cuh"
 #include "fmm.cuh"
 #include "prof.cuh"
+#include "tiles.cuh"
 
 namespace {
 
 constexpr int TR = 64;    // kept rows per tile of the application kernels
-
-__global__ void k_tiles_c(int64_t nprob, const int32_t *__restrict__ mk, int tr, int64_t *__restrict__ tile_off)
-{
-    __shared__ int64_t part[1024];
-    const int T = blockDim.x;
-    int64_t per = (nprob + T - 1) / T;
-    int64_t beg = threadIdx.x * per, end = min(nprob, beg + per);
-    int64_t s = 0;
-    for (int64_t p = beg; p < end; p++) s += (mk[p] + tr - 1) / tr;
-    part[threadIdx.x] = s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int64_t acc = 0;
-        for (int i = 0; i < T; i++) { int64_t v = part[i]; part[i] = acc; acc += v; }
-        tile_off[nprob] = acc;
-    }
-    __syncthreads();
-    int64_t acc = part[threadIdx.x];
-    for (int64_t p = beg; p < end; p++) { tile_off[p] = acc; acc += (mk[p] + tr - 1) / tr; }
-}
 
 // rotations of the deflation, in scan order (forward) or reversed with the
 // transposed rotation (inverse).  The rotation list is a sequence of chains
@@ -108,7 +89,7 @@ superdc_status run(const FactorView &f, int64_t total, double *Xmut, const doubl
     int64_t *tile_off = nullptr;
     SdcScratch sc(st);
     SDC_CHECK(sc.get(&tile_off, f.nprob + 1));
-    k_tiles_c<<<1, 1024, 0, st>>>(f.nprob, f.mk, TR, tile_off);
+    k_tiles<<<1, tiles_threads(f.nprob), 0, st>>>(f.nprob, f.mk, TR, tile_off);
     const int gthreads = 128;
     if (trans)
         PROF_LAUNCH("givens", st, k_givens<<<(unsigned)(nsm * 8), gthreads, 0, st>>>(f, total, Xmut, ldx, ncols, 0));

@@ -51,6 +51,7 @@
 #include "fmm.cuh"
 #include "secular.cuh"
 #include "prof.cuh"
+#include "tiles.cuh"
 
 #if !defined(FMM_BOX) || !defined(FMM_NS)
 #error "define FMM_BOX (indices per leaf box) and FMM_NS (namespace) before including fmm_impl.cuh"
@@ -183,15 +184,12 @@ __global__ void k_fmm_plan(int64_t nprob, const int32_t *__restrict__ mk, int mi
                            int64_t *__restrict__ leaf_base, int32_t *__restrict__ fslot,
                            int32_t *__restrict__ fprob, int32_t *__restrict__ nfmm)
 {
-    __shared__ int64_t sb[1024], sl[1024];
-    __shared__ int sf[1024];
-    __shared__ int ok;
+    __shared__ int64_t sh[32];
     const int T = blockDim.x;
     const int64_t per = (nprob + T - 1) / T;
     const int64_t beg = std::min<int64_t>(nprob, (int64_t)threadIdx.x * per);
     const int64_t end = std::min<int64_t>(nprob, beg + per);
-    int64_t nbx = 0, nlf = 0;
-    int nf = 0;
+    int64_t nbx = 0, nlf = 0, nf = 0;
     for (int64_t p = beg; p < end; p++) {
         const int m = mk[p];
         if (!fmm_cand(m, min_m)) continue;
@@ -200,27 +198,16 @@ __global__ void k_fmm_plan(int64_t nprob, const int32_t *__restrict__ mk, int mi
         nlf += nb0;
         nf++;
     }
-    sb[threadIdx.x] = nbx;
-    sl[threadIdx.x] = nlf;
-    sf[threadIdx.x] = nf;
-    __syncthreads();
+    int64_t tb, tl, tf;
+    int64_t ab = cta_exscan(nbx, sh, &tb), al = cta_exscan(nlf, sh, &tl);
+    int af = (int)cta_exscan(nf, sh, &tf);
+    const bool ok = tb <= cap_boxes && tl <= cap_leaves && tf <= cap_f;
+    if (!ok) { ab = 0; al = 0; }
     if (threadIdx.x == 0) {
-        int64_t ab = 0, al = 0;
-        int af = 0;
-        for (int i = 0; i < T; i++) {
-            int64_t vb = sb[i], vl = sl[i];
-            int vf = sf[i];
-            sb[i] = ab; sl[i] = al; sf[i] = af;
-            ab += vb; al += vl; af += vf;
-        }
-        ok = (ab <= cap_boxes && al <= cap_leaves && af <= cap_f) ? 1 : 0;
-        box_base[nprob] = ok ? ab : 0;
-        leaf_base[nprob] = ok ? al : 0;
-        *nfmm = ok ? af : 0;
+        box_base[nprob] = ok ? tb : 0;
+        leaf_base[nprob] = ok ? tl : 0;
+        *nfmm = ok ? (int)tf : 0;
     }
-    __syncthreads();
-    int64_t ab = ok ? sb[threadIdx.x] : 0, al = ok ? sl[threadIdx.x] : 0;
-    int af = ok ? sf[threadIdx.x] : 0;
     for (int64_t p = beg; p < end; p++) {
         box_base[p] = ab;
         leaf_base[p] = al;
@@ -2838,7 +2825,7 @@ superdc_status plan(FmmPlan &pl, int64_t nprob, const int64_t *off, int64_t tota
     d.flops = prof_counter("fmm_flops");
     d.box_base = box_base; d.leaf_base = leaf_base; d.fslot = fslot; d.fprob = fprob; d.nfmm = nfmm;
     d.blo = blo; d.bhi = bhi; d.nnear = nnear; d.near = near; d.nstart = nstart;
-    PROF_LAUNCH("fmm_plan", st, k_fmm_plan<<<1, 1024, 0, st>>>(nprob, mk, min_m, pl.cap_boxes, pl.cap_leaves,
+    PROF_LAUNCH("fmm_plan", st, k_fmm_plan<<<1, tiles_threads(nprob), 0, st>>>(nprob, mk, min_m, pl.cap_boxes, pl.cap_leaves,
                                                                pl.cap_f, box_base, leaf_base, fslot, fprob, nfmm));
     // one CTA per problem; a batch of fewer problems than SMs (the top tree
     // levels) gives each tree 1024 threads instead of 256

@@ -26,6 +26,7 @@
 #include "prof.cuh"
 #include "secular.cuh"
 #include "fmm.cuh"
+#include "tiles.cuh"
 #include <algorithm>
 #include <mutex>
 
@@ -331,30 +332,6 @@ void launch_deflate(const R1Args &a, const R1Out &o, int big_t, double *wd, doub
     }
 }
 
-// ---------------------------------------------------------------------------
-// Prefix of root tiles per problem (single CTA).
-// ---------------------------------------------------------------------------
-__global__ void k_tiles(int64_t nprob, const int32_t *__restrict__ mk, int tr, int64_t *__restrict__ tile_off)
-{
-    __shared__ int64_t part[1024];
-    const int T = blockDim.x;
-    int64_t per = (nprob + T - 1) / T;
-    int64_t beg = threadIdx.x * per, end = min(nprob, beg + per);
-    int64_t s = 0;
-    for (int64_t p = beg; p < end; p++) s += (mk[p] + tr - 1) / tr;
-    part[threadIdx.x] = s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int64_t acc = 0;
-        for (int i = 0; i < T; i++) { int64_t v = part[i]; part[i] = acc; acc += v; }
-        tile_off[nprob] = acc;
-    }
-    __syncthreads();
-    int64_t acc = part[threadIdx.x];
-    for (int64_t p = beg; p < end; p++) { tile_off[p] = acc; acc += (mk[p] + tr - 1) / tr; }
-}
-
-
 // Work units of the secular kernel: (problem, first root, end root), at most
 // ubig roots each.  A unit stages its problem's poles in shared memory (all of
 // them when they fit in SEC_CHUNK, else in chunks per sweep).  Units are
@@ -369,7 +346,7 @@ __global__ void k_units(int64_t nprob, const int32_t *__restrict__ mk, const int
                         int *__restrict__ counter)
 {
     extern __shared__ unsigned long long keys[];   // SORT_MAX entries when sorting
-    __shared__ int part[1024];
+    __shared__ int sh[32];
     const int T = blockDim.x;
     const bool sorted = nprob <= SORT_MAX;
     int64_t n2 = 1;
@@ -399,23 +376,19 @@ __global__ void k_units(int64_t nprob, const int32_t *__restrict__ mk, const int
     }
     // units per problem (in the chosen order), block-wide prefix
     int64_t per = (nprob + T - 1) / T;
-    int64_t beg = threadIdx.x * per, end = min(nprob, beg + per);
+    int64_t beg = min(nprob, threadIdx.x * per), end = min(nprob, beg + per);
     int cnt = 0;
     for (int64_t q = beg; q < end; q++) {
         int64_t pp = sorted ? (int64_t)(0xFFFFFFFFu - (unsigned)(keys[q] & 0xFFFFFFFFull)) : q;
         int m = (fslot && fslot[pp] >= 0) ? 0 : mk[pp];   // FMM problems: not here
         cnt += (m + ubig - 1) / ubig;
     }
-    part[threadIdx.x] = cnt;
-    __syncthreads();
+    int all;
+    int u = cta_exscan(cnt, sh, &all);
     if (threadIdx.x == 0) {
-        int acc = 0;
-        for (int i = 0; i < T; i++) { int v = part[i]; part[i] = acc; acc += v; }
-        *nunits = acc;
+        *nunits = all;
         *counter = 0;
     }
-    __syncthreads();
-    int u = part[threadIdx.x];
     for (int64_t q = beg; q < end; q++) {
         int64_t pp = sorted ? (int64_t)(0xFFFFFFFFu - (unsigned)(keys[q] & 0xFFFFFFFFull)) : q;
         int m = (fslot && fslot[pp] >= 0) ? 0 : mk[pp];
@@ -597,19 +570,35 @@ k_secular(const int64_t *__restrict__ off, const int4 *__restrict__ units,
     }
 }
 
+// Tiles of the direct zhat and b kernels: TR targets per CTA, SW groups of TR
+// threads that split the sources.  Many rows: 128 targets, one group (the staged
+// sources serve four warps).  Fewer rows than two such tiles per SM: 32 targets
+// and eight warps, as a thread's chain over every source, not the throughput,
+// sets the time (GB300, 16 problems of 8..300: zhat 0.123 -> 0.025, b 0.127 -> 0.024 ms).
+bool direct_split(int64_t rows) { return rows < (int64_t)sdc_num_sms() * 256; }
+
+template <int SW>
+__device__ __forceinline__ void grp_sync()
+{
+    if (SW > 1) __syncwarp();
+    else __syncthreads();
+}
+
 // ---------------------------------------------------------------------------
 // Loewner zhat, eq. (4.23):
 //   vhat_i^2 = (lambda_{m-1} - d_i) prod_{j<i} (lambda_j - d_i)/(d_j - d_i)
 //                                   prod_{i<=j<m-1} (lambda_j - d_i)/(d_{j+1} - d_i)
 // with lambda_j - d_i = (d_{K_j} - d_i) + eta_j.
 // ---------------------------------------------------------------------------
-template <int TR>
-__global__ void __launch_bounds__(TR)
+template <int TR, int SW>
+__global__ void __launch_bounds__(TR * SW)
 k_lowner(int64_t nprob, const int64_t *__restrict__ off, const int64_t *__restrict__ tile_off, R1Out o,
          const int32_t *__restrict__ fslot, unsigned long long *__restrict__ queue)
 {
     __shared__ int64_t s_tile;
-    __shared__ ff_w4 sd[TR], sl[TR];
+    __shared__ ff_w4 sd[SW][TR], sl[SW][TR];
+    __shared__ FfProd part[SW > 1 ? SW : 1][2][SW > 1 ? TR : 1];
+    const int tl = threadIdx.x % TR, grp = threadIdx.x / TR;
     const int64_t ntiles = tile_off[nprob];
     for (int64_t it = blockIdx.x;; it += gridDim.x) {
         int64_t tile = it;
@@ -624,11 +613,11 @@ k_lowner(int64_t nprob, const int64_t *__restrict__ off, const int64_t *__restri
         if (fslot && fslot[p] >= 0) continue;   // FMM problem
         const int64_t b0 = off[p];
         const int m = o.mk[p];
-        const int i = (int)(tile - tile_off[p]) * TR + threadIdx.x;
+        const int i = (int)(tile - tile_off[p]) * TR + tl;
         const double *dk = o.dk + b0, *dorg = o.dorg + b0, *eta = o.eta + b0;
         const FfScale fs = ff_scale(dk[0], dk[m - 1], o.wsum[p]);
         bool okt = fs.ok && !o.unshifted && m >= 2;
-        for (int j = threadIdx.x; okt && j + 1 < m; j += TR) okt = ff_gap_ok(dk[j], dk[j + 1], fs.kk);
+        for (int j = threadIdx.x; okt && j + 1 < m; j += TR * SW) okt = ff_gap_ok(dk[j], dk[j + 1], fs.kk);
         const bool ok = __syncthreads_and(okt);
         const double di = i < m ? dk[i] : 0.0;
         double pn = 1.0, pd = 1.0;
@@ -639,15 +628,30 @@ k_lowner(int64_t nprob, const int64_t *__restrict__ off, const int64_t *__restri
             FfProd num = {1ull << 63, 0}, den = {1ull << 63, 0};
             const ff_w4 d4 = ff_words4(ff_fixed(di, fs.kk) - fs.ref);
             const ff_u96 dw = {d4.lo, d4.mid, d4.hi};
-            for (int c0 = 0; c0 < m - 1; c0 += TR) {
-                const int cn = min(TR, m - 1 - c0), j = c0 + threadIdx.x;
-                __syncthreads();
-                if (threadIdx.x < cn) {
-                    sd[threadIdx.x] = ff_words4(ff_fixed(dk[j], fs.kk) - fs.ref);
-                    sl[threadIdx.x] = ff_words4(ff_fixed(dorg[j], fs.kk) + ff_fixed(eta[j], fs.kk) - fs.ref);
+            for (int c0 = grp * TR; c0 < m - 1; c0 += SW * TR) {
+                const int cn = min(TR, m - 1 - c0), j = c0 + tl;
+                grp_sync<SW>();
+                if (tl < cn) {
+                    sd[grp][tl] = ff_words4(ff_fixed(dk[j], fs.kk) - fs.ref);
+                    sl[grp][tl] = ff_words4(ff_fixed(dorg[j], fs.kk) + ff_fixed(eta[j], fs.kk) - fs.ref);
                 }
+                grp_sync<SW>();
+                ff_prod_sweep(sd[grp], sl[grp], cn, c0, i, dw, num, den);
+            }
+            if (SW > 1) {
+                part[SW > 1 ? grp : 0][0][SW > 1 ? tl : 0] = num;
+                part[SW > 1 ? grp : 0][1][SW > 1 ? tl : 0] = den;
                 __syncthreads();
-                ff_prod_sweep(sd, sl, cn, c0, i, dw, num, den);
+                if (grp > 0) continue;
+                for (int w = 1; w < SW; w++) {
+                    const FfProd a = part[SW > 1 ? w : 0][0][SW > 1 ? tl : 0], c = part[SW > 1 ? w : 0][1][SW > 1 ? tl : 0];
+                    num.m = ff_mulhi(num.m, a.m);
+                    den.m = ff_mulhi(den.m, c.m);
+                    num.e += a.e + 64;
+                    den.e += c.e + 64;
+                    ff_prod_norm(num);
+                    ff_prod_norm(den);
+                }
             }
             if (i >= m) continue;
             lowner_edges(dk, dorg, eta, di, i, m, pn, pd, ex);
@@ -655,7 +659,7 @@ k_lowner(int64_t nprob, const int64_t *__restrict__ off, const int64_t *__restri
             pd *= (double)den.m;
             ex += num.e - den.e;
         } else {
-            if (i >= m) continue;
+            if (i >= m || grp > 0) continue;
             // numerator and denominator products kept apart (one division per
             // entry instead of one per factor); every 8 factors both are brought
             // back to [1/2, 1) by exponent arithmetic, the exponents summed in ex
@@ -689,14 +693,16 @@ k_lowner(int64_t nprob, const int64_t *__restrict__ off, const int64_t *__restri
 // ---------------------------------------------------------------------------
 // b_j = (sum_i vhat_i^2 / ((d_i - d_{K_j}) - eta_j)^2)^(-1/2), eq. (4.27)
 // ---------------------------------------------------------------------------
-template <int TR>
-__global__ void __launch_bounds__(TR)
+template <int TR, int SW>
+__global__ void __launch_bounds__(TR * SW)
 k_bnorm(int64_t nprob, const int64_t *__restrict__ off, const int64_t *__restrict__ tile_off, R1Out o,
          const int32_t *__restrict__ fslot, unsigned long long *__restrict__ queue)
 {
     __shared__ int64_t s_tile;
-    __shared__ ff_f4 sd[TR], sv[TR];
-    __shared__ double red[TR / 32];
+    __shared__ ff_f4 sd[SW][TR], sv[SW][TR];
+    __shared__ ff_t3 part[SW > 1 ? SW : 1][SW > 1 ? TR : 1];
+    __shared__ double red[TR * SW / 32];
+    const int tl = threadIdx.x % TR, grp = threadIdx.x / TR;
     const int64_t ntiles = tile_off[nprob];
     for (int64_t it = blockIdx.x;; it += gridDim.x) {
         int64_t tile = it;
@@ -711,11 +717,11 @@ k_bnorm(int64_t nprob, const int64_t *__restrict__ off, const int64_t *__restric
         if (fslot && fslot[p] >= 0) continue;   // FMM problem
         const int64_t b0 = off[p];
         const int m = o.mk[p];
-        const int j = (int)(tile - tile_off[p]) * TR + threadIdx.x;
+        const int j = (int)(tile - tile_off[p]) * TR + tl;
         const double *dk = o.dk + b0, *v = o.vhat + b0;
         const FfScale fs = ff_scale(dk[0], dk[m - 1], o.wsum[p]);
         bool okt = fs.ok && !o.unshifted && m >= 2;
-        for (int i = threadIdx.x; okt && i + 1 < m; i += TR) okt = ff_gap_ok(dk[i], dk[i + 1], fs.kk);
+        for (int i = threadIdx.x; okt && i + 1 < m; i += TR * SW) okt = ff_gap_ok(dk[i], dk[i + 1], fs.kk);
         const bool ok = __syncthreads_and(okt);
         const double dK = j < m ? o.dorg[b0 + j] : 0.0, e = j < m ? o.eta[b0 + j] : 1.0;
         if (ok) {
@@ -726,25 +732,31 @@ k_bnorm(int64_t nprob, const int64_t *__restrict__ off, const int64_t *__restric
             const ff_f4 x = ff_point(dK, e, fs);
             const int kv = fs.kw >> 1;
             const double sc = ff_pow2(-kv);
-            for (int c0 = 0; c0 < m; c0 += TR) {
+            for (int c0 = grp * TR; c0 < m; c0 += SW * TR) {
                 const int cn = min(TR, m - c0);
-                __syncthreads();
-                if (threadIdx.x < cn) {
-                    const ff_t3 t = ff_split3(v[c0 + threadIdx.x] * sc);
-                    sd[threadIdx.x] = ff_pole(dk[c0 + threadIdx.x], fs);
-                    sv[threadIdx.x] = {t.a, t.b, t.c, 0.0f};
+                grp_sync<SW>();
+                if (tl < cn) {
+                    const ff_t3 t = ff_split3(v[c0 + tl] * sc);
+                    sd[grp][tl] = ff_pole(dk[c0 + tl], fs);
+                    sv[grp][tl] = {t.a, t.b, t.c, 0.0f};
                 }
-                __syncthreads();
-                ff_sqr_sweep(sd, sv, cn, c0, K, x, S);
+                grp_sync<SW>();
+                ff_sqr_sweep(sd[grp], sv[grp], cn, c0, K, x, S);
             }
-            if (j < m - 1) {
+            if (SW > 1) {
+                part[SW > 1 ? grp : 0][SW > 1 ? tl : 0] = S;
+                __syncthreads();
+                if (grp == 0)
+                    for (int w = 1; w < SW; w++) ff_acc3(S, part[SW > 1 ? w : 0][SW > 1 ? tl : 0]);
+            }
+            if (grp == 0 && j < m - 1) {
                 const double r = v[K] * rcp_nr2(-e);
                 o.bnorm[b0 + j] = 1.0 / sqrt(fma(r, r, ff_join3(S) * ff_pow2(2 * (kv + fs.kk))));
             }
             if (m - 1 - (int)(tile - tile_off[p]) * TR < TR) {
                 const double dl = o.dorg[b0 + m - 1], el = o.eta[b0 + m - 1];
                 double s = 0.0;
-                for (int i = threadIdx.x; i < m; i += TR) {
+                for (int i = threadIdx.x; i < m; i += TR * SW) {
                     const double vr = v[i] * rcp_nr2((dk[i] - dl) - el);
                     s = fma(vr, vr, s);
                 }
@@ -753,13 +765,13 @@ k_bnorm(int64_t nprob, const int64_t *__restrict__ off, const int64_t *__restric
                 __syncthreads();
                 if (threadIdx.x == 0) {
                     s = 0.0;
-                    for (int w = 0; w < TR / 32; w++) s += red[w];
+                    for (int w = 0; w < TR * SW / 32; w++) s += red[w];
                     o.bnorm[b0 + m - 1] = 1.0 / sqrt(s);
                 }
             }
             continue;
         }
-        if (j >= m) continue;
+        if (j >= m || grp > 0) continue;
         double s = 0.0;
         for (int i = 0; i < m; i++) {
             double t = (dk[i] - dK) - e;
@@ -892,8 +904,8 @@ superdc_status r1_run(const R1Args &a_in, cudaStream_t st)
         if (fs != SUPERDC_OK) { fmm_free(fp, st); return fs; }
     }
     const int32_t *fslot = fp.on ? fp.dv.fslot : nullptr;
-    const int TR = 128;
-    PROF_LAUNCH("tiles", st, k_tiles<<<1, 1024, 0, st>>>(a.nprob, a.o.mk, TR, tile_off));
+    const bool dsplit = direct_split(a.rows >= 0 ? a.rows : a.total);
+    PROF_LAUNCH("tiles", st, k_tiles<<<1, tiles_threads(a.nprob), 0, st>>>(a.nprob, a.o.mk, dsplit ? 32 : 128, tile_off));
     const unsigned grid = (unsigned)(nsm * 8);
     const size_t ksm = (a.nprob <= SORT_MAX) ? (size_t)SORT_MAX * sizeof(unsigned long long) : 0;
     const int slots = nsm * 6;
@@ -912,9 +924,12 @@ superdc_status r1_run(const R1Args &a_in, cudaStream_t st)
     unsigned long long *tq = nullptr;          // tile queues of the direct Loewner and b kernels
     SDC_CHECK(sc.get(&tq, 2));
     SDC_CHECK(cudaMemsetAsync(tq, 0, 2 * sizeof(unsigned long long), st));
-    PROF_LAUNCH("lowner", st, k_lowner<128><<<grid, 128, 0, st>>>(a.nprob, a.off, tile_off, a.o, fslot, tq));
+    const auto k_low = dsplit ? k_lowner<32, 8> : k_lowner<128, 1>;
+    const auto k_b = dsplit ? k_bnorm<32, 8> : k_bnorm<128, 1>;
+    const int dthreads = dsplit ? 256 : 128;
+    PROF_LAUNCH("lowner", st, k_low<<<grid, dthreads, 0, st>>>(a.nprob, a.off, tile_off, a.o, fslot, tq));
     if (fs == SUPERDC_OK) fs = fmm_lowner(fp, a.off, a.o, st);
-    PROF_LAUNCH("bnorm", st, k_bnorm<128><<<grid, 128, 0, st>>>(a.nprob, a.off, tile_off, a.o, fslot, tq + 1));
+    PROF_LAUNCH("bnorm", st, k_b<<<grid, dthreads, 0, st>>>(a.nprob, a.off, tile_off, a.o, fslot, tq + 1));
     if (fs == SUPERDC_OK) fs = fmm_bnorm(fp, a.off, a.o, st);
     PROF_LAUNCH("merge", st, k_merge<<<(unsigned)(nsm * 8), 256, 0, st>>>(a.nprob, a.off, a.total, a.o));
     const cudaError_t le = cudaGetLastError();
@@ -1030,8 +1045,8 @@ extern "C" superdc_status superdc_secular_batched_noalloc(int64_t nprob, const i
     SDC_CHECK(units_attr());
     const int nsm = sdc_num_sms();
     launch_deflate(a, a.o, DB_T, wd, wz, kept, surv, st);
-    const int TR = 128;
-    k_tiles<<<1, 1024, 0, st>>>(a.nprob, a.o.mk, TR, tile_off);
+    const bool dsplit = direct_split(a.total);
+    k_tiles<<<1, tiles_threads(a.nprob), 0, st>>>(a.nprob, a.o.mk, dsplit ? 32 : 128, tile_off);
     const unsigned grid = (unsigned)(nsm * 8);
     const size_t ksm = (a.nprob <= SORT_MAX) ? (size_t)SORT_MAX * sizeof(unsigned long long) : 0;
     const int slots = nsm * 6;
@@ -1045,8 +1060,11 @@ extern "C" superdc_status superdc_secular_batched_noalloc(int64_t nprob, const i
     else
         k_secular<4, false><<<(unsigned)slots, 128, 0, st>>>(a.off, units, ucount, ucount + 1, a.o, a.stop_c,
                                                               a.max_iter);
-    k_lowner<128><<<grid, 128, 0, st>>>(a.nprob, a.off, tile_off, a.o, nullptr, nullptr);
-    k_bnorm<128><<<grid, 128, 0, st>>>(a.nprob, a.off, tile_off, a.o, nullptr, nullptr);
+    const auto k_low = dsplit ? k_lowner<32, 8> : k_lowner<128, 1>;
+    const auto k_b = dsplit ? k_bnorm<32, 8> : k_bnorm<128, 1>;
+    const int dthreads = dsplit ? 256 : 128;
+    k_low<<<grid, dthreads, 0, st>>>(a.nprob, a.off, tile_off, a.o, nullptr, nullptr);
+    k_b<<<grid, dthreads, 0, st>>>(a.nprob, a.off, tile_off, a.o, nullptr, nullptr);
     k_merge<<<(unsigned)(nsm * 8), 256, 0, st>>>(a.nprob, a.off, a.total, a.o);
     SDC_CHECK(cudaGetLastError());
     return SUPERDC_OK;
