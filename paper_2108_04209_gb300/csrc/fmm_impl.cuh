@@ -839,10 +839,96 @@ __global__ void k_fmm_nodes(FmmDev pl, const int64_t *__restrict__ off, const in
 constexpr int FAR_NW = 4;         // warps (leaf boxes) per CTA
 constexpr int FAR_TAKE = 4;       // list entries taken per level and round
 
+// Series of a leaf box in mixed precision: sum_{n < LOWN} a_n u^n (monomials, FP64)
+// plus sum_{n >= LOWN} c_n T_n(u) (Chebyshev, single precision).  A box of the
+// lists is at least its own width away, so c_n falls as 5.8^-n: the single
+// precision part is below 2^-30 of the sum and its rounding below 2^-52; the
+// monomials' amplification, at most 2.4^n, is below that decay.  11 FP64
+// instructions per evaluation instead of 43 (Clenshaw over all of them): 180
+// instead of 690 cycles of the SM for a warp.
+constexpr int LOWN = 12;
+
+__device__ __forceinline__ double low_eval(const double *__restrict__ a, double u)
+{
+    double s = a[LOWN - 1];
+#pragma unroll
+    for (int n = LOWN - 2; n >= 0; n--) s = fma(s, u, a[n]);
+    return s;
+}
+
+// single precision series; LO: its first LO coefficients are zero and not stored
+template <int LO>
+__device__ __forceinline__ float clenshawf(const float *__restrict__ a, float u)
+{
+    const float u2 = u + u;
+    float b1 = 0.0f, b2 = 0.0f;
+#pragma unroll
+    for (int n = P - 1; n >= 1; n--) {
+        const float b0 = fmaf(u2, b1, (n >= LO) ? a[n - LO] - b2 : -b2);
+        b2 = b1;
+        b1 = b0;
+    }
+    return fmaf(u, b1, (LO == 0) ? a[0] - b2 : -b2);
+}
+
+// M[n * LOWN + k]: coefficient of u^k in T_n
+__device__ __forceinline__ void mono_table(double *M)
+{
+    if (threadIdx.x < LOWN) {
+        const int k = threadIdx.x;
+        int c0 = 0, c1 = 0;                       // coefficients of u^k in T_{n-1}, T_{n-2}
+        for (int n = 0; n < LOWN; n++) {
+            const int up = __shfl_up_sync((1u << LOWN) - 1u, c0, 1);
+            const int c = (n == 0) ? (k == 0) : (n == 1) ? (k == 1) : 2 * (k ? up : 0) - c1;
+            c1 = c0;
+            c0 = c;
+            M[n * LOWN + k] = (double)c;
+        }
+    }
+}
+
+// a leaf's series (coefficient lane in a) into the mixed form at cf, the single
+// precision part times sc; one warp, t: LOWN entries of shared memory
+__device__ __forceinline__ void store_series(double a, double sc, const double *M, double *t, double *__restrict__ cf)
+{
+    const int lane = threadIdx.x & 31;
+    __syncwarp();
+    if (lane < LOWN) t[lane] = a;
+    __syncwarp();
+    if (lane < LOWN) {
+        double s = 0.0;
+        for (int n = 0; n < LOWN; n++) s = fma(M[n * LOWN + lane], t[n], s);
+        cf[lane] = s;
+    } else if (lane < P) {
+        ((float *)(cf + LOWN))[lane - LOWN] = (float)(a * sc);
+    }
+}
+
+// far field of a root in its leaf box gl (K_SEC's layouts): FP64 sums of a problem out of scale
+__device__ __forceinline__ void far_eval(const FmmDev &pl, int64_t gl, double u, Acc &A)
+{
+    const double *cf = pl.coef + gl * NFIELD * P;
+    A.psi += clenshaw(cf, u);
+    A.phi += clenshaw(cf + P, u);
+    A.dpsi += clenshaw(cf + 2 * P, u);
+    A.dphi += clenshaw(cf + 3 * P, u);
+}
+
+// the same of a split sweep: single precision parts into S, the FP64 part returned
+__device__ __forceinline__ double far_split(const FmmDev &pl, int64_t gl, double u, FfAcc &S)
+{
+    const double *cf = pl.coef + gl * NFIELD * P;
+    const float *ff = (const float *)(cf + LOWN), *fd = (const float *)(cf + P);
+    const float uf = ff_top(u, 0);
+    ff_merge(S, clenshawf<LOWN>(ff, uf), 0.0f, clenshawf<0>(fd, uf), clenshawf<0>(fd + P, uf),
+             clenshawf<0>(fd + 2 * P, uf));
+    return low_eval(cf, u);
+}
+
 template <int KER>
 __global__ void __launch_bounds__(FAR_NW * 32) k_fmm_far(FmmDev pl, const int64_t *__restrict__ off, R1Out o)
 {
-    __shared__ double Tx[P * P], xq[P];
+    __shared__ double Tx[P * P], xq[P], Mt[LOWN * LOWN];
     __shared__ float Tf[(KER == K_SEC) ? P * P : 1];
     __shared__ ff_logtab lt[(KER == K_LOG) ? 128 : 1];
     __shared__ ff_f4 sp[FAR_NW][P];
@@ -853,6 +939,7 @@ __global__ void __launch_bounds__(FAR_NW * 32) k_fmm_far(FmmDev pl, const int64_
     const unsigned FULL = 0xffffffffu;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, q = min(lane, P - 1);
     cheb_tables(xq, Tx);
+    mono_table(Mt);
     if (KER == K_LOG)
         for (int i = threadIdx.x; i < 128; i += blockDim.x) {
             const float c = ff_logc(i);
@@ -1012,11 +1099,11 @@ __global__ void __launch_bounds__(FAR_NW * 32) k_fmm_far(FmmDev pl, const int64_
             if (q == 0) { dl *= 0.5f; dr *= 0.5f; }
             if (lane < P) {
                 float *ff = (float *)(cf + P);
-                cf[lane] = a;
                 ff[lane] = l;
                 ff[P + lane] = dl * ih;
                 ff[2 * P + lane] = dr * ih;
             }
+            store_series(a, ff_pow2(-(fs.kk + fs.kw)), Mt, sF[warp], cf);
         } else if (KER == K_SEC) {
             const double F[4] = {L1, R1, L2, R2};
             for (int k = 0; k < 4; k++) {
@@ -1024,8 +1111,12 @@ __global__ void __launch_bounds__(FAR_NW * 32) k_fmm_far(FmmDev pl, const int64_
                 if (lane < P) cf[k * P + lane] = a;
             }
         } else if (KER == K_2) {
-            const double a = series(ok ? ((double)AL.s + (double)AL.sl) * (c1 * ff_pow2(fs.kk)) : L2 + R2);
-            if (lane < P) cf[lane] = a;
+            if (ok) {
+                store_series(series((double)AL.s + (double)AL.sl), 1.0, Mt, sF[warp], cf);
+            } else {
+                const double a = series(L2 + R2);
+                if (lane < P) cf[lane] = a;
+            }
         } else {
             // F' -> antiderivative G = sum B_k T_k (k = 1..P; T_P vanishes at the
             // nodes but not at 0), F(u) = F(centre) + h (G(u) - G(0))
@@ -1041,45 +1132,13 @@ __global__ void __launch_bounds__(FAR_NW * 32) k_fmm_far(FmmDev pl, const int64_
             else if (lane >= 2 && lane <= P) bk = (sF[warp][lane - 1] - sF[warp][lane + 1]) * (0.5 / lane);
             double g0s = (lane >= 2 && lane <= P && !(lane & 1)) ? ((lane & 2) ? -bk : bk) : 0.0;   // T_k(0)
             for (int s = 16; s > 0; s >>= 1) g0s += __shfl_xor_sync(FULL, g0s, s);
-            if (lane < P) cf[lane] = (lane == 0) ? c - hT * g0s : hT * bk;
+            const double a2 = (lane == 0) ? c - hT * g0s : hT * bk;
+            if (ok) store_series(a2, 1.0, Mt, sF[warp], cf);
+            else if (lane < P) cf[lane] = a2;
         }
         if (pl.flops && lane == 0 && npair)
             atomicAdd(pl.flops, (unsigned long long)npair * P * (P * (KER == K_SEC ? 7 : 5) + (KER == K_LOG ? 3 : 0)) +
                                     2 * P * P);
-    }
-}
-
-// far field of a root at u in its leaf box gl (K_SEC's layouts)
-__device__ __forceinline__ float clenshawf(const float *__restrict__ a, float u)
-{
-    const float u2 = u + u;
-    float b1 = 0.0f, b2 = 0.0f;
-#pragma unroll
-    for (int n = P - 1; n >= 1; n--) {
-        const float b0 = fmaf(u2, b1, a[n] - b2);
-        b2 = b1;
-        b1 = b0;
-    }
-    return fmaf(u, b1, a[0] - b2);
-}
-
-__device__ __forceinline__ void far_eval(const FmmDev &pl, int64_t gl, bool ok, double u, int kk, int kw, Acc &A)
-{
-    const double *cf = pl.coef + gl * NFIELD * P;
-    if (ok) {
-        const double S = clenshaw(cf, u);
-        const float *ff = (const float *)(cf + P);
-        const float uf = (float)u;
-        const double ps = (double)clenshawf(ff, uf) * ff_pow2(kk + kw), c2 = ff_pow2(2 * kk + kw);
-        A.psi += ps;
-        A.phi += S - ps;
-        A.dpsi = fma((double)clenshawf(ff + P, uf), c2, A.dpsi);
-        A.dphi = fma((double)clenshawf(ff + 2 * P, uf), c2, A.dphi);
-    } else {
-        A.psi += clenshaw(cf, u);
-        A.phi += clenshaw(cf + P, u);
-        A.dpsi += clenshaw(cf + 2 * P, u);
-        A.dphi += clenshaw(cf + 3 * P, u);
     }
 }
 
@@ -1180,6 +1239,7 @@ k_secular_fmm(FmmDev pl, FfDev ff, const int64_t *__restrict__ off, R1Out o, dou
         Root R;
         R.dK = 0.0; R.y = 1.0; R.phase = 1;
         if (act) R.init(dk, zk, k, m, W, o.unshifted != 0);
+        double uK = (R.dK - cT) * ihT;                  // the root's origin in the leaf's coordinate
         while (__any_sync(FULL, act)) {
             const int kwlo = __reduce_min_sync(FULL, act ? k : 0x7fffffff);
             const int kwhi = __reduce_max_sync(FULL, act ? k : -1);
@@ -1197,17 +1257,24 @@ k_secular_fmm(FmmDev pl, FfDev ff, const int64_t *__restrict__ off, R1Out o, dou
                 else if (p0) sweep<false>(sd + i * B, sw + i * B, 0, cnt, j0, kk, kwlo, kwhi, R.dK, R.y, A);
                 else         sweep<true>(sd + i * B, sw + i * B, 0, cnt, j0, kk, kwlo, kwhi, R.dK, R.y, A);
             }
-            if (ok) A = ff_collect(S, R, fs.kk, fs.kw);
-            // far field at the plain position x = d_K + y (local shifting)
-            if (act) far_eval(pl, gl, ok, ((R.dK + R.y) - cT) * ihT, fs.kk, fs.kw, A);
+            // far field at x = d_K + y, then the step
             bool fin = false;
-            if (act && R.update(A, tol, max_iter, o.status)) {
+            const bool moved = R.phase == 0;
+            if (act) {
+                if (ok) {
+                    const double low = far_split(pl, gl, fma(R.y, ihT, uK), S);
+                    fin = R.update_split(S, low, fs.kk, fs.kw, tol, max_iter, o.status);
+                } else {
+                    far_eval(pl, gl, ((R.dK + R.y) - cT) * ihT, A);
+                    fin = R.update(A, tol, max_iter, o.status);
+                }
+            }
+            if (fin) {
                 o.org[b0 + k] = R.K;
                 o.eta[b0 + k] = R.y;
                 o.dorg[b0 + k] = R.dK;
                 o.lamk[b0 + k] = R.dK + R.y;
                 if (o.sweeps) o.sweeps[b0 + k] = R.nsw;
-                fin = true;
             }
             const unsigned mask = __ballot_sync(FULL, fin);
             if (fin) {
@@ -1215,6 +1282,7 @@ k_secular_fmm(FmmDev pl, FfDev ff, const int64_t *__restrict__ off, R1Out o, dou
                 act = k < kend;
                 if (act) R.init(dk, zk, k, m, W, o.unshifted != 0);
             }
+            if (__any_sync(FULL, moved || fin)) uK = (R.dK - cT) * ihT;
             next += __popc(mask);
             // no root left to refill and fewer than TAIL_X lanes busy: the
             // stragglers go to k_secular_tail, which runs 32 of them per warp
@@ -1304,8 +1372,8 @@ k_secular_tail(FmmDev pl, FfDev ff, const int64_t *__restrict__ off, R1Out o, do
             if (lane == 0) atomicAdd(terms, (unsigned long long)nt);
         }
         Acc A = {0.0, 0.0, 0.0, 0.0};
+        FfAcc S = {};
         if (act && ok) {
-            FfAcc S = {};
             const ff_f4 x = ff_point(R.dK, R.y, fs);
             for (int i = 0; i < nn; i++) {
                 const int j0 = near_box_chk(pl, g, nnr, i, (m + B - 1) / B, o.status) * B;
@@ -1320,7 +1388,6 @@ k_secular_tail(FmmDev pl, FfDev ff, const int64_t *__restrict__ off, R1Out o, do
                 }
                 ff_close(S);
             }
-            A = ff_collect(S, R, fs.kk, fs.kw, part == 0);
         } else if (act) {
             for (int i = 0; i < nn; i++) {
                 const int j0 = near_box_chk(pl, g, nnr, i, (m + B - 1) / B, o.status) * B;
@@ -1337,14 +1404,27 @@ k_secular_tail(FmmDev pl, FfDev ff, const int64_t *__restrict__ off, R1Out o, do
         }
         // the four lanes of a root are consecutive: butterfly over lane bits 0, 1
         for (int sh = 1; sh < TAIL_LANES; sh <<= 1) {
-            A.psi += __shfl_xor_sync(FULL, A.psi, sh);
-            A.phi += __shfl_xor_sync(FULL, A.phi, sh);
-            A.dpsi += __shfl_xor_sync(FULL, A.dpsi, sh);
-            A.dphi += __shfl_xor_sync(FULL, A.dphi, sh);
+            const float v0 = __shfl_xor_sync(FULL, S.s, sh), v1 = __shfl_xor_sync(FULL, S.sl, sh);
+            const float v2 = __shfl_xor_sync(FULL, S.psi, sh), v3 = __shfl_xor_sync(FULL, S.dpsi, sh);
+            ff_merge(S, v0, v1, v2, v3, __shfl_xor_sync(FULL, S.dphi, sh));
         }
+        if (__any_sync(FULL, act && !ok))
+            for (int sh = 1; sh < TAIL_LANES; sh <<= 1) {
+                A.psi += __shfl_xor_sync(FULL, A.psi, sh);
+                A.phi += __shfl_xor_sync(FULL, A.phi, sh);
+                A.dpsi += __shfl_xor_sync(FULL, A.dpsi, sh);
+                A.dphi += __shfl_xor_sync(FULL, A.dphi, sh);
+            }
         if (act) {
-            far_eval(pl, gl, ok, ((R.dK + R.y) - cT) * ihT, fs.kk, fs.kw, A);
-            if (R.update(A, tol, max_iter, o.status)) {
+            bool fin;
+            if (ok) {
+                const double low = far_split(pl, gl, ((R.dK + R.y) - cT) * ihT, S);
+                fin = R.update_split(S, low, fs.kk, fs.kw, tol, max_iter, o.status);
+            } else {
+                far_eval(pl, gl, ((R.dK + R.y) - cT) * ihT, A);
+                fin = R.update(A, tol, max_iter, o.status);
+            }
+            if (fin) {
                 if (part == 0) {
                     const int k = R.k;
                     o.org[b0 + k] = R.K;
@@ -1371,6 +1451,7 @@ k_secular_fmm_split(FmmDev pl, FfDev ff, const int64_t *__restrict__ off, R1Out 
 {
     __shared__ __align__(16) unsigned char stage[SPW][B * (sizeof(ff_f4) + sizeof(ff_f2))];
     __shared__ double red[SPW][4][32];
+    __shared__ float fred[SPW][5][32];
     const unsigned FULL = 0xffffffffu;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     ff_f4 *const fd = (ff_f4 *)stage[warp];
@@ -1437,23 +1518,46 @@ k_secular_fmm_split(FmmDev pl, FfDev ff, const int64_t *__restrict__ off, R1Out 
                     else if (p0) sweep<false>(sd, sw, 0, cnt, j0, kk, kwlo, kwhi, R.dK, R.y, A);
                     else         sweep<true>(sd, sw, 0, cnt, j0, kk, kwlo, kwhi, R.dK, R.y, A);
                 }
-                if (ok) A = ff_collect(fa, R, fs.kk, fs.kw, warp == 0);
-                if (warp == 0 && act) far_eval(pl, gl, ok, ((R.dK + R.y) - cT) * ihT, fs.kk, fs.kw, A);
-                red[warp][0][lane] = A.psi;
-                red[warp][1][lane] = A.phi;
-                red[warp][2][lane] = A.dpsi;
-                red[warp][3][lane] = A.dphi;
-                __syncthreads();
-                Acc T = {0.0, 0.0, 0.0, 0.0};
-#pragma unroll
-                for (int w = 0; w < SPW; w++) {      // same order in every warp
-                    T.psi += red[w][0][lane];
-                    T.phi += red[w][1][lane];
-                    T.dpsi += red[w][2][lane];
-                    T.dphi += red[w][3][lane];
+                const double u = ((R.dK + R.y) - cT) * ihT;
+                if (!ok && warp == 0 && act) far_eval(pl, gl, u, A);
+                if (ok) {
+                    fred[warp][0][lane] = fa.s;
+                    fred[warp][1][lane] = fa.sl;
+                    fred[warp][2][lane] = fa.psi;
+                    fred[warp][3][lane] = fa.dpsi;
+                    fred[warp][4][lane] = fa.dphi;
+                } else {
+                    red[warp][0][lane] = A.psi;
+                    red[warp][1][lane] = A.phi;
+                    red[warp][2][lane] = A.dpsi;
+                    red[warp][3][lane] = A.dphi;
                 }
                 __syncthreads();
-                if (act && R.update(T, tol, max_iter, warp == 0 ? o.status : nullptr)) {
+                // same order in every warp
+                Acc T = {0.0, 0.0, 0.0, 0.0};
+                FfAcc S = {};
+#pragma unroll
+                for (int w = 0; w < SPW; w++) {
+                    if (ok) {
+                        ff_merge(S, fred[w][0][lane], fred[w][1][lane], fred[w][2][lane], fred[w][3][lane],
+                                 fred[w][4][lane]);
+                    } else {
+                        T.psi += red[w][0][lane];
+                        T.phi += red[w][1][lane];
+                        T.dpsi += red[w][2][lane];
+                        T.dphi += red[w][3][lane];
+                    }
+                }
+                __syncthreads();
+                int32_t *const sts = warp == 0 ? o.status : nullptr;
+                bool fin = false;
+                if (act && ok) {
+                    const double low = far_split(pl, gl, u, S);
+                    fin = R.update_split(S, low, fs.kk, fs.kw, tol, max_iter, sts);
+                } else if (act) {
+                    fin = R.update(T, tol, max_iter, sts);
+                }
+                if (fin) {
                     if (warp == 0) {
                         o.org[b0 + k] = R.K;
                         o.eta[b0 + k] = R.y;
@@ -1707,11 +1811,22 @@ __global__ void __launch_bounds__(B) k_lowner_fmm(FmmDev pl, const int64_t *__re
         if (act) {
             double cT, hT;
             box_ch(pl.blo[g], pl.bhi[g], cT, hT);
-            const double Lf = clenshaw(pl.coef + gl * NFIELD * P, (di - cT) / hT);
-            double prod = pr.pn / pr.pd;
+            const double *cf = pl.coef + gl * NFIELD * P;
+            const double u = (di - cT) * rcp_any(hT);
+            double Lf, v;
             int ex = pr.ex;
-            if (ex & 1) { prod *= 2.0; ex -= 1; }
-            double v = ldexp(sqrt(prod), ex / 2) * exp(0.5 * Lf);
+            if (ok) {
+                // pn and pd are normal and positive: exponents apart, then the
+                // quotient's root without divide and square root
+                Lf = low_eval(cf, u) + (double)clenshawf<LOWN>((const float *)(cf + LOWN), ff_top(u, 0));
+                v = root_quot(pr.pn, pr.pd, ex);
+            } else {
+                Lf = clenshaw(cf, u);
+                double prod = pr.pn / pr.pd;
+                if (ex & 1) { prod *= 2.0; ex -= 1; }
+                v = sqrt(prod);
+            }
+            v = ldexp(v, ex / 2) * exp(0.5 * Lf);
             if (!isfinite(v)) sdc_latch(o.status, SUPERDC_DEV_NONFINITE);
             o.vhat[b0 + i] = (o.zk[b0 + i] < 0.0) ? -v : v;
         }
@@ -1731,7 +1846,7 @@ __global__ void __launch_bounds__(B) k_bnorm_fmm(FmmDev pl, const int64_t *__res
     __shared__ __align__(16) double stage[4 * B];
     double *const sd = stage, *const sv = stage + B;                // FP64 sums
     ff_f4 *const fd = (ff_f4 *)stage, *const fv = fd + B;           // three-float sums
-    __shared__ double red[B];
+    static_assert(B == 32, "one warp per leaf box");
     const int tid = threadIdx.x;
     const int64_t nleaf = pl.leaf_base[pl.nprob];
     for (int64_t gl = blockIdx.x; gl < nleaf; gl += gridDim.x) {
@@ -1744,19 +1859,27 @@ __global__ void __launch_bounds__(B) k_bnorm_fmm(FmmDev pl, const int64_t *__res
         const int j = Tb * B + tid;
         const bool act = j < m - 1;
         const double dK = act ? o.dorg[b0 + j] : 0.0, e = act ? o.eta[b0 + j] : 0.0;
+        const bool ok = pl.ffbad[p] == 0;
+        const FfScale fs = ff_scale(o.dk[b0], o.dk[b0 + m - 1], o.wsum[p]);
         double s = 0.0;
+        float tail = 0.0f;                        // the far field's single precision part
         if (act) {
             double cT, hT;
             box_ch(pl.blo[g], pl.bhi[g], cT, hT);
-            s = clenshaw(pl.coef + gl * NFIELD * P, ((dK + e) - cT) / hT);
+            const double *cf = pl.coef + gl * NFIELD * P;
+            const double u = ((dK + e) - cT) * rcp_any(hT);
+            if (ok) {
+                s = low_eval(cf, u) * ff_pow2(2 * fs.kk + fs.kw);
+                tail = clenshawf<LOWN>((const float *)(cf + LOWN), ff_top(u, 0));
+            } else {
+                s = clenshaw(cf, u);
+            }
         }
-        const bool ok = pl.ffbad[p] == 0;
-        const FfScale fs = ff_scale(o.dk[b0], o.dk[b0 + m - 1], o.wsum[p]);
         const int kv = fs.kw >> 1;
         const int K = act ? o.org[b0 + j] : -1;
         const ff_f4 x = ff_point(dK, e, fs);
         const double sc = ok ? ff_pow2(-kv) : 1.0;
-        ff_t3 s3 = {0.0f, 0.0f, 0.0f};
+        ff_t3 s3 = {(fs.kw & 1) ? tail + tail : tail, 0.0f, 0.0f};      // in units of 2^(2 (kv + kk))
         const int nnr = pl.nnear[g];
         const int nn = near_len(nnr, (m + B - 1) / B);
         int64_t nsrc = 0;
@@ -1791,7 +1914,7 @@ __global__ void __launch_bounds__(B) k_bnorm_fmm(FmmDev pl, const int64_t *__res
             const double vr = o.vhat[b0 + K] * rcp_nr2(-e);         // the origin's term
             s = fma(vr, vr, fma(ff_join3(s3), ff_pow2(2 * (kv + fs.kk)), s));
         }
-        if (act) o.bnorm[b0 + j] = 1.0 / sqrt(s);
+        if (act) o.bnorm[b0 + j] = rsqrt_any(s);
         // this box's sources in the sum for the last target
         double t = 0.0;
         if (j < m) {
@@ -1799,14 +1922,8 @@ __global__ void __launch_bounds__(B) k_bnorm_fmm(FmmDev pl, const int64_t *__res
             const double vr = o.vhat[b0 + j] * r;
             t = vr * vr;
         }
-        __syncthreads();
-        red[tid] = t;
-        __syncthreads();
-        if (tid == 0) {
-            double a = 0.0;
-            for (int q = 0; q < B; q++) a += red[q];
-            pl.lastp[gl] = a;
-        }
+        for (int sh = 16; sh > 0; sh >>= 1) t += __shfl_xor_sync(0xffffffffu, t, sh);
+        if (tid == 0) pl.lastp[gl] = t;
         // near terms (6 each, as the direct kernel), Clenshaw, the last target's share
         const int64_t nt = max(0, min(B, (m - 1) - Tb * B)), ns = max(0, min(B, m - Tb * B));
         fl_add(pl, nt * (6 * nsrc + 2 * P + 2) + ns * 7);

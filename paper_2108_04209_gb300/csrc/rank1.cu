@@ -337,12 +337,13 @@ void launch_deflate(const R1Args &a, const R1Out &o, int big_t, double *wd, doub
 // them when they fit in SEC_CHUNK, else in chunks per sweep).  Units are
 // ordered by decreasing problem size (largest first) so the long units start
 // early, and capping the roots per unit spreads a large problem over several
-// SMs, which keeps the tail of the launch short.
+// SMs, which keeps the tail of the launch short.  With last != 0 a problem's last
+// root, a chain of its own, gets a unit (fourth entry 1) ahead of the others.
 constexpr int SEC_UNIT_BIG = 2048;
 constexpr int SORT_MAX = 8192;
 
 __global__ void k_units(int64_t nprob, const int32_t *__restrict__ mk, const int32_t *__restrict__ fslot, int ubig,
-                        int whole_small, int4 *__restrict__ units, int *__restrict__ nunits,
+                        int last, int4 *__restrict__ units, int *__restrict__ nunits,
                         int *__restrict__ counter)
 {
     extern __shared__ unsigned long long keys[];   // SORT_MAX entries when sorting
@@ -381,7 +382,7 @@ __global__ void k_units(int64_t nprob, const int32_t *__restrict__ mk, const int
     for (int64_t q = beg; q < end; q++) {
         int64_t pp = sorted ? (int64_t)(0xFFFFFFFFu - (unsigned)(keys[q] & 0xFFFFFFFFull)) : q;
         int m = (fslot && fslot[pp] >= 0) ? 0 : mk[pp];   // FMM problems: not here
-        cnt += (m + ubig - 1) / ubig;
+        cnt += (m + ubig - 1) / ubig + (last && m >= 2 ? 1 : 0);
     }
     int all;
     int u = cta_exscan(cnt, sh, &all);
@@ -393,6 +394,7 @@ __global__ void k_units(int64_t nprob, const int32_t *__restrict__ mk, const int
         int64_t pp = sorted ? (int64_t)(0xFFFFFFFFu - (unsigned)(keys[q] & 0xFFFFFFFFull)) : q;
         int m = (fslot && fslot[pp] >= 0) ? 0 : mk[pp];
         if (m <= 0) continue;
+        if (last && m >= 2) units[u++] = make_int4((int)pp, m - 1, m, 1);
         for (int r = 0; r < m; r += ubig) units[u++] = make_int4((int)pp, r, min(m, r + ubig), 0);
     }
 }
@@ -422,6 +424,7 @@ k_secular(const int64_t *__restrict__ off, const int4 *__restrict__ units,
     ff_f2 *const fw = (ff_f2 *)(fd + SEC_CHUNK);
     double *const sd = (double *)stage, *const sw = sd + SEC_CHUNK;
     __shared__ double red[SPLIT ? NW : 1][4][32];
+    __shared__ float fred[SPLIT ? NW : 1][5][32];
     __shared__ double s_dK[SPLIT ? 32 : 1], s_y[SPLIT ? 32 : 1];
     __shared__ int s_ph[SPLIT ? 32 : 1], s_fin[SPLIT ? 32 : 1];
     __shared__ int s_unit;
@@ -447,6 +450,21 @@ k_secular(const int64_t *__restrict__ off, const int4 *__restrict__ units,
         bool okt = fs.ok && !o.unshifted && m >= 2;
         for (int j = threadIdx.x; okt && j + 1 < m; j += NW * 32) okt = ff_gap_ok(dk[j], dk[j + 1], fs.kk);
         const bool ok = __syncthreads_and(okt);
+        auto last_root = [&]() {
+            Root R;
+            last_root_warp(dk, zk, m, W, tol, max_iter, o.status, R);
+            if (lane == 0) {
+                o.org[b0 + m - 1] = R.K;
+                o.eta[b0 + m - 1] = R.y;
+                o.dorg[b0 + m - 1] = R.dK;
+                o.lamk[b0 + m - 1] = R.dK + R.y;
+                if (o.sweeps) o.sweeps[b0 + m - 1] = R.nsw;
+            }
+        };
+        if (SPLIT && U.w) {                       // the last root's unit
+            if (ok && warp == 0) last_root();
+            continue;
+        }
         const int uend = ok ? min(U.z, m - 1) : U.z;
         const int len = uend - U.y;
         const int wbeg = SPLIT ? U.y : U.y + (int)(((int64_t)len * warp) / NW);
@@ -497,28 +515,40 @@ k_secular(const int64_t *__restrict__ off, const int4 *__restrict__ units,
                     else         sweep<true>(sd, sw, j0, j1, c0, kk, kwlo, kwhi, R.dK, R.y, A);
                 }
             }
-            if (ok) A = ff_collect(S, R, fs.kk, fs.kw, !SPLIT || warp == 0);
             bool fin = false;
             if (SPLIT) {
                 // the warps hold the same roots: warp 0 alone reduces the partial
                 // sums (fixed order) and updates, the others take the new iterate
                 // (an FP64 instruction costs its pipe slot in every warp that runs it)
-                red[SPLIT ? warp : 0][0][lane] = A.psi;
-                red[SPLIT ? warp : 0][1][lane] = A.phi;
-                red[SPLIT ? warp : 0][2][lane] = A.dpsi;
-                red[SPLIT ? warp : 0][3][lane] = A.dphi;
+                if (ok) {
+                    float (*const fr)[32] = fred[SPLIT ? warp : 0];
+                    fr[0][lane] = S.s; fr[1][lane] = S.sl; fr[2][lane] = S.psi; fr[3][lane] = S.dpsi; fr[4][lane] = S.dphi;
+                } else {
+                    red[SPLIT ? warp : 0][0][lane] = A.psi;
+                    red[SPLIT ? warp : 0][1][lane] = A.phi;
+                    red[SPLIT ? warp : 0][2][lane] = A.dpsi;
+                    red[SPLIT ? warp : 0][3][lane] = A.dphi;
+                }
                 __syncthreads();
                 if (warp == 0) {
                     Acc T = {0.0, 0.0, 0.0, 0.0};
+                    if (ok) {
 #pragma unroll
-                    for (int w = 0; w < (SPLIT ? NW : 1); w++) {
-                        T.psi += red[w][0][lane];
-                        T.phi += red[w][1][lane];
-                        T.dpsi += red[w][2][lane];
-                        T.dphi += red[w][3][lane];
+                        for (int w = 1; w < (SPLIT ? NW : 1); w++)
+                            ff_merge(S, fred[w][0][lane], fred[w][1][lane], fred[w][2][lane], fred[w][3][lane],
+                                     fred[w][4][lane]);
+                    } else {
+#pragma unroll
+                        for (int w = 0; w < (SPLIT ? NW : 1); w++) {
+                            T.psi += red[w][0][lane];
+                            T.phi += red[w][1][lane];
+                            T.dpsi += red[w][2][lane];
+                            T.dphi += red[w][3][lane];
+                        }
                     }
                     if (act) {
-                        fin = R.update(T, tol, max_iter, o.status);
+                        fin = ok ? R.update_split(S, 0.0, fs.kk, fs.kw, tol, max_iter, o.status)
+                                 : R.update(T, tol, max_iter, o.status);
                         if (fin) {
                             o.org[b0 + k] = R.K;
                             o.eta[b0 + k] = R.y;
@@ -540,7 +570,8 @@ k_secular(const int64_t *__restrict__ off, const int4 *__restrict__ units,
                     fin = s_fin[SPLIT ? lane : 0] != 0;
                 }
             } else if (act) {
-                fin = R.update(A, tol, max_iter, o.status);
+                fin = ok ? R.update_split(S, 0.0, fs.kk, fs.kw, tol, max_iter, o.status)
+                         : R.update(A, tol, max_iter, o.status);
                 if (fin) {
                     o.org[b0 + k] = R.K;
                     o.eta[b0 + k] = R.y;
@@ -557,16 +588,7 @@ k_secular(const int64_t *__restrict__ off, const int4 *__restrict__ units,
             }
             next += __popc(mask);
         }
-        if (ok && U.z == m && warp == NW - 1) {
-            last_root_warp(dk, zk, m, W, tol, max_iter, o.status, R);
-            if (lane == 0) {
-                o.org[b0 + m - 1] = R.K;
-                o.eta[b0 + m - 1] = R.y;
-                o.dorg[b0 + m - 1] = R.dK;
-                o.lamk[b0 + m - 1] = R.dK + R.y;
-                if (o.sweeps) o.sweeps[b0 + m - 1] = R.nsw;
-            }
-        }
+        if (!SPLIT && ok && U.z == m && warp == NW - 1) last_root();
     }
 }
 
@@ -680,11 +702,8 @@ k_lowner(int64_t nprob, const int64_t *__restrict__ off, const int64_t *__restri
                 }
             }
         }
-        double prod = pn / pd;
-        if (ex & 1) { prod *= 2.0; ex -= 1; }
-        double vs = sqrt(prod);
-        vs = ldexp(vs, ex / 2);
-        double v = vs;
+        double v = root_quot(pn, pd, ex);
+        v = ldexp(v, ex / 2);
         if (!isfinite(v)) sdc_latch(o.status, SUPERDC_DEV_NONFINITE);
         o.vhat[b0 + i] = (o.zk[b0 + i] < 0.0) ? -v : v;
     }
@@ -751,7 +770,7 @@ k_bnorm(int64_t nprob, const int64_t *__restrict__ off, const int64_t *__restric
             }
             if (grp == 0 && j < m - 1) {
                 const double r = v[K] * rcp_nr2(-e);
-                o.bnorm[b0 + j] = 1.0 / sqrt(fma(r, r, ff_join3(S) * ff_pow2(2 * (kv + fs.kk))));
+                o.bnorm[b0 + j] = rsqrt_any(fma(r, r, ff_join3(S) * ff_pow2(2 * (kv + fs.kk))));
             }
             if (m - 1 - (int)(tile - tile_off[p]) * TR < TR) {
                 const double dl = o.dorg[b0 + m - 1], el = o.eta[b0 + m - 1];
@@ -766,7 +785,7 @@ k_bnorm(int64_t nprob, const int64_t *__restrict__ off, const int64_t *__restric
                 if (threadIdx.x == 0) {
                     s = 0.0;
                     for (int w = 0; w < TR * SW / 32; w++) s += red[w];
-                    o.bnorm[b0 + m - 1] = 1.0 / sqrt(s);
+                    o.bnorm[b0 + m - 1] = rsqrt_any(s);
                 }
             }
             continue;
@@ -889,7 +908,7 @@ superdc_status r1_run(const R1Args &a_in, cudaStream_t st)
     SDC_CHECK(sc.get(&a.o.lamk, a.total));
     int4 *units = nullptr;
     int *ucount = nullptr;
-    SDC_CHECK(sc.get(&units, a.nprob + a.total / 32 + 2));
+    SDC_CHECK(sc.get(&units, 2 * a.nprob + a.total / 32 + 2));
     SDC_CHECK(sc.get(&ucount, 2));
     SDC_CHECK(units_attr());
 
@@ -912,7 +931,7 @@ superdc_status r1_run(const R1Args &a_in, cudaStream_t st)
     bool split;
     int ubig;
     secular_schedule(a.rows >= 0 ? a.rows : a.total, a.sched, a.tile_roots, slots, &split, &ubig);
-    PROF_LAUNCH("units", st, k_units<<<1, 1024, ksm, st>>>(a.nprob, a.o.mk, fslot, ubig, split ? 0 : 1, units,
+    PROF_LAUNCH("units", st, k_units<<<1, 1024, ksm, st>>>(a.nprob, a.o.mk, fslot, ubig, split ? 1 : 0, units,
                                                            ucount, ucount + 1));
     if (split)
         PROF_LAUNCH("secular", st, (k_secular<4, true><<<(unsigned)slots, 128, 0, st>>>(
@@ -969,7 +988,7 @@ constexpr size_t NA_DORG = NA_WZ + na_round(NA_T * sizeof(double));
 constexpr size_t NA_WSUM = NA_DORG + na_round(NA_T * sizeof(double));
 constexpr size_t NA_TILE = NA_WSUM + na_round(NA_P * sizeof(double));
 constexpr size_t NA_UNITS = NA_TILE + na_round((NA_P + 1) * sizeof(int64_t));
-constexpr size_t NA_SURV = NA_UNITS + na_round((NA_P + NA_T / 32 + 2) * sizeof(int4));
+constexpr size_t NA_SURV = NA_UNITS + na_round((2 * NA_P + NA_T / 32 + 2) * sizeof(int4));
 constexpr size_t NA_PINV = NA_SURV + na_round(NA_T * sizeof(int32_t));
 constexpr size_t NA_KEPT = NA_PINV + na_round(NA_T * sizeof(int32_t));
 constexpr size_t NA_UCNT = NA_KEPT + na_round(NA_T * sizeof(int8_t));
@@ -1053,7 +1072,7 @@ extern "C" superdc_status superdc_secular_batched_noalloc(int64_t nprob, const i
     bool split;
     int ubig;
     secular_schedule(a.total, a.sched, a.tile_roots, slots, &split, &ubig);
-    k_units<<<1, 1024, ksm, st>>>(a.nprob, a.o.mk, nullptr, ubig, split ? 0 : 1, units, ucount, ucount + 1);
+    k_units<<<1, 1024, ksm, st>>>(a.nprob, a.o.mk, nullptr, ubig, split ? 1 : 0, units, ucount, ucount + 1);
     if (split)
         k_secular<4, true><<<(unsigned)slots, 128, 0, st>>>(a.off, units, ucount, ucount + 1, a.o, a.stop_c,
                                                              a.max_iter);

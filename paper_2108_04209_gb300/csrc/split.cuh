@@ -219,6 +219,19 @@ FF_HD void ff_close(FfAcc &A)
     A.b = A.bl = 0.0f;
 }
 
+// another part's sums of the same root into A (the same result either way round)
+FF_HD void ff_merge(FfAcc &A, float s, float sl, float psi, float dpsi, float dphi)
+{
+    const float t = ff_add(A.s, s);
+    const float v = ff_sub(t, A.s);
+    const float l = ff_add(ff_add(ff_sub(A.s, ff_sub(t, v)), ff_sub(s, v)), ff_add(A.sl, sl));
+    A.s = ff_add(t, l);
+    A.sl = ff_sub(l, ff_sub(A.s, t));
+    A.psi += psi;
+    A.dpsi += dpsi;
+    A.dphi += dphi;
+}
+
 // the term of pole j when it may lie on either side of root k; the two next to
 // the root are left out
 FF_HD void ff_select(FfAcc &A, float p, float pl, float q, int j, int k)
