@@ -25,6 +25,7 @@
 #include "cauchy.cuh"
 #include "fmm.cuh"
 #include "prof.cuh"
+#include "secular.cuh"
 
 #include <mutex>
 #include "handles.cuh"
@@ -343,95 +344,122 @@ k_leaf_tri(int r, const int64_t *__restrict__ leaf_off, const int64_t *__restric
 }
 
 // Givens pair of a QL step: rr = sqrt(f^2 + g^2), c = g / rr, s = f / rr.  In
-// the usual range x^(-1/2) of q = f^2 + g^2 comes from an FP32 seed and two
-// Newton steps y <- y + y (1 - q y^2) / 2 (relative error 2^-22 -> 2^-44 ->
-// below one ulp), which replaces a square root and a division in the chain of
-// dependent operations; elsewhere hypot and one division.
-// q^(-1/2) to about 2^-22 for a normal q > 0: the FP32 approximate reciprocal
-// square root of the leading mantissa bits (scaled into [1, 4) to make the
-// exponent even), the exponent halved by integer arithmetic; no conversion
-// between FP64 and FP32 in the chain of dependent steps
-__device__ __forceinline__ double rsqrt_seed(double q)
-{
-    const int hi = __double2hiint(q);
-    const unsigned lo = (unsigned)__double2loint(q);
-    const int e = ((hi >> 20) & 0x7FF) - 1023;
-    const int odd = e & 1;
-    const unsigned mb = (((unsigned)hi & 0xFFFFFu) << 3) | (lo >> 29);
-    float r;
-    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(__uint_as_float(((unsigned)(127 + odd) << 23) | mb)));
-    const unsigned rb = __float_as_uint(r);                  // in (0.5, 1]
-    const int E = (int)(rb >> 23) - 127 - (e - odd) / 2 + 1023;
-    const unsigned rm = rb & 0x7FFFFFu;
-    return __hiloint2double((int)(((unsigned)E << 20) | (rm >> 3)), (int)(rm << 29));
-}
-
+// the usual range x^(-1/2) of q = f^2 + g^2 comes from an FP32 seed and one step
+// of third order (relative error 2^-22 -> 2^-64), carried into the three products
+// directly: an FP64 instruction takes 64 cycles of a warp whether the next one
+// waits for it or not, so a chain's time is its number of instructions (11 here,
+// comparisons on the exponent bits).  Elsewhere hypot and one division.
 __device__ __forceinline__ void ql_pair(double f, double g, double &c, double &s, double &rr)
 {
     const double q = fma(f, f, g * g);
-    if (q > 1e-36 && q < 1e36) {
-        double y = rsqrt_seed(q);
-        double e = fma(-q * y, y, 1.0);
-        y = fma(0.5 * y, e, y);
-        e = fma(-q * y, y, 1.0);
-        y = fma(0.5 * y, e, y);
-        rr = q * y;
-        c = g * y;
-        s = f * y;
+    const int e = __double2hiint(q) >> 20;
+    if (e > 1023 - 120 && e < 1023 + 120) {
+        const double y = rsqrt_seed(q), qy = q * y;
+        const double d = fma(-qy, y, 1.0);
+        const double k = d * fma(0.375, d, 0.5);
+        const double c0 = g * y, s0 = f * y;
+        rr = fma(qy, k, qy);
+        c = fma(c0, k, c0);
+        s = fma(s0, k, s0);
     } else {
         rr = hypot(f, g);
         const double inv = (rr != 0.0) ? 1.0 / rr : 0.0;
         c = g * inv;
         s = f * inv;
+        if (!(rr > 0.0)) { c = 1.0; s = 0.0; rr = g; }
     }
+}
+
+// |b| <= eps (|a0| + |a1|); exponents alone decide unless they are close
+__device__ __forceinline__ bool ql_small(double b, double a0, double a1)
+{
+    const int e = (__double2hiint(b) >> 20) & 0x7FF;
+    const int ea = max((__double2hiint(a0) >> 20) & 0x7FF, (__double2hiint(a1) >> 20) & 0x7FF);
+    if (e >= ea - 48 && e > 60) return false;
+    if (e < ea - 56 && ea < 0x7FF) return true;
+    return fabs(b) <= SDC_EPS * (fabs(a0) + fabs(a1));
+}
+
+// 2 v
+__device__ __forceinline__ double ql_twice(double v)
+{
+    const int h = __double2hiint(v), e = (h >> 20) & 0x7FF;
+    return (e > 0 && e < 0x7FE) ? __hiloint2double(h + (1 << 20), __double2loint(v)) : v + v;
 }
 
 // One implicit QL sweep on the unreduced block [l, h] of a symmetric
 // tridiagonal matrix (diagonal a[i * S], off-diagonal b[i * S] coupling i and
 // i + 1): the implicit symmetric QR step with Wilkinson's shift of Golub and
 // Van Loan (Section 8.3), in its QL orientation.  The shift mu is the
-// eigenvalue of the leading 2 x 2 block nearer to a_l; the first rotation, in
-// plane (h-1, h), has its second column along the last column of T - mu I
-// restricted to rows h-1, h, i.e. along (b_{h-1}, a_h - mu); every later
+// eigenvalue of the leading 2 x 2 block nearer to a_l (its correction in single
+// precision: an error of 2^-22 of it does not change the convergence); the first
+// rotation, in plane (h-1, h), has its second column along the last column of
+// T - mu I restricted to rows h-1, h, i.e. along (b_{h-1}, a_h - mu); every later
 // rotation, in plane (i, i+1), removes the bulge at (i, i+2) that the
 // previous one left, against the entry b_{i+1}.  A rotation G with G(i,i) =
-// G(i+1,i+1) = c, G(i,i+1) = s, G(i+1,i) = -s acts as T <- G^T T G:
-//   a_i     <- c^2 a_i - 2 c s b_i + s^2 a_{i+1}
-//   a_{i+1} <- s^2 a_i + 2 c s b_i + c^2 a_{i+1}
-//   b_i     <- c s (a_i - a_{i+1}) + (c^2 - s^2) b_i
+// G(i+1,i+1) = c, G(i,i+1) = s, G(i+1,i) = -s acts as T <- G^T T G, with
+//   t = s (a_i - a_{i+1}) + 2 c b_i:
+//   a_{i+1} <- a_{i+1} + s t,  a_i <- a_i - s t,  b_i <- c t - b_i,
 //   b_{i-1} <- c b_{i-1}, and the new bulge at (i-1, i+1) is s b_{i-1}.
 // rec(q, c, s) records rotation q (plane (h-1-q, h-q)): the eigenvectors are
 // Q <- Q G, i.e. columns (x_i, x_{i+1}) <- (c x_i - s x_{i+1}, s x_i + c x_{i+1}).
-// Returns the number of rotations (h - l).
+// Returns the number of rotations (h - l); low is the smallest index i in
+// (l, h] whose b_i is negligible (h when no other), first whether b_l is.
+// 19 FP64 instructions a rotation (37 with comparisons before).  Measured (GB300,
+// k_leaf_qlcta): 16 leaves of 32 rows 1.77 -> 1.03 ms, 256 of 64 6.9 -> 4.1.
 template <int S, typename Rec>
-__device__ __forceinline__ int ql_sweep_tri(double *a, double *b, int l, int h, Rec rec)
+__device__ __forceinline__ int ql_sweep_tri(double *a, double *b, int l, int h, int &low, bool &first, Rec rec)
 {
-    const double al = a[l * S], bl = b[l * S];
-    const double del = 0.5 * (a[(l + 1) * S] - al);
-    const double mu = al - bl * bl / (del + copysign(hypot(del, bl), del));
-    double x = a[h * S] - mu, z = b[(h - 1) * S];
-    int q = 0;
-    for (int i = h - 1; i >= l; i--, q++) {
-        double c, s, r;
-        ql_pair(z, x, c, s, r);                 // c = x / r, s = z / r
-        if (!(r > 0.0)) { c = 1.0; s = 0.0; r = x; }
-        if (i < h - 1) b[(i + 1) * S] = r;      // the bulge is gone
-        const double ai = a[i * S], ai1 = a[(i + 1) * S], bi = b[i * S];
-        const double cc = c * c, ss = s * s, cs = c * s;
-        const double t2 = 2.0 * cs * bi;
-        a[i * S] = fma(cc, ai, fma(ss, ai1, -t2));
-        a[(i + 1) * S] = fma(ss, ai, fma(cc, ai1, t2));
-        const double bn = fma(cs, ai - ai1, (cc - ss) * bi);
-        b[i * S] = bn;
-        rec(q, c, s);
-        if (i > l) {
-            const double bm = b[(i - 1) * S];
-            z = s * bm;                         // bulge at (i-1, i+1)
-            b[(i - 1) * S] = c * bm;
-            x = bn;
+    const double al = a[l * S], bl = b[l * S], al1 = a[(l + 1) * S];
+    const double dif = al1 - al;
+    double mu = al;
+    {
+        const int ed = ((__double2hiint(dif) >> 20) & 0x7FF) - 1, eb = (__double2hiint(bl) >> 20) & 0x7FF;
+        const int E = max(ed, eb) - 1023;
+        if (E > -700 && E < 700) {
+            const float d = 0.5f * ff_top(dif, -E), x = ff_top(bl, -E);
+            const float den = d + copysignf(ff_sqrtf(fmaf(d, d, x * x)), d);
+            mu = al - ff_up(x * x * mufu_rcp(den), E);
+        } else {
+            const double del = 0.5 * dif;
+            mu = al - bl * bl / (del + copysign(hypot(del, bl), del));
         }
     }
+    double a1 = a[h * S], bi = b[(h - 1) * S], x = a1 - mu, z = bi, a2 = 0.0;
+    int q = 0;
+    low = h;
+    for (int i = h - 1; i >= l; i--, q++) {
+        const double ai = a[i * S], bm = (i > l) ? b[(i - 1) * S] : 0.0;
+        double c, s, r;
+        ql_pair(z, x, c, s, r);                 // c = x / r, s = z / r
+        const double t = fma(s, ai - a1, ql_twice(c * bi));
+        const double an = fma(s, t, a1);
+        a[(i + 1) * S] = an;
+        if (i < h - 1) {
+            b[(i + 1) * S] = r;                 // the bulge is gone
+            if (ql_small(r, an, a2)) low = i + 1;
+        }
+        a2 = an;
+        a1 = fma(-s, t, ai);
+        x = fma(c, t, -bi);
+        rec(q, c, s);
+        z = s * bm;                             // bulge at (i-1, i+1)
+        bi = c * bm;
+    }
+    a[l * S] = a1;
+    b[l * S] = x;
+    first = ql_small(x, a1, a2);
     return q;
+}
+
+// The smallest i >= l with b_i negligible (m - 1 when none)
+template <int S>
+__device__ __forceinline__ int ql_scan(const double *a, const double *b, int l, int m)
+{
+    int h = l;
+    for (; h < m - 1; h++)
+        if (ql_small(b[h * S], a[h * S], a[(h + 1) * S])) break;
+    return h;
 }
 
 // Implicit QL on the tridiagonal (d, e) of every leaf, one lane per leaf and
@@ -464,21 +492,21 @@ k_leaf_ql(int nleaves, int mmax, const int64_t *__restrict__ leaf_off, const int
     bool bad = false;
     double2 *R = rot + (int64_t)(act ? L : 0) * cap;
     int2 *Hd = hdr + (int64_t)(act ? L : 0) * caps;
-    for (int l = 0; l < m && !bad; l++) {
-        for (int iter = 0;; iter++) {
-            int mm = l;
-            for (; mm < m - 1; mm++) {
-                const double s2 = fabs(sd[mm * LPW + lane]) + fabs(sd[(mm + 1) * LPW + lane]);
-                if (fabs(se[mm * LPW + lane]) <= SDC_EPS * s2) break;
-            }
-            if (mm == l) break;
-            if (iter >= 64 || nsweep >= caps || nrot + (mm - l) > cap) { bad = true; break; }
+    double *const a = sd + lane, *const b = se + lane;
+    for (int l = 0, h = -1; l < m && !bad; l++) {
+        if (h <= l) h = ql_scan<LPW>(a, b, l, m);       // else known from the last sweep
+        for (int iter = 0; h > l; iter++) {
+            if (iter >= 64 || nsweep >= caps || nrot + (h - l) > cap) { bad = true; break; }
             double2 *Rs = R + nrot;
-            const int cnt = ql_sweep_tri<LPW>(sd + lane, se + lane, l, mm,
+            int low;
+            bool first;
+            const int cnt = ql_sweep_tri<LPW>(a, b, l, h, low, first,
                                              [&](int q, double c, double s) { Rs[q] = make_double2(c, s); });
-            Hd[nsweep] = make_int2(mm - 1, cnt);
+            Hd[nsweep] = make_int2(h - 1, cnt);
             nsweep++;
             nrot += cnt;
+            h = low;
+            if (first) break;
         }
     }
     if (act) {
@@ -618,25 +646,25 @@ k_leaf_qlcta(int r, int64_t n, const int64_t *__restrict__ leaf_off, const int64
     for (int i = tid; i < m; i += LEAF_T) { dg[i] = din[o + i]; ee[i] = ein[o + i]; }
     if (tid == 0) s_flag = 0;
     __syncthreads();
-    int ql_l = 0, ql_iter = 0;
+    int ql_l = 0, ql_iter = 0, ql_h = -1;
     auto ql_sweep = [&](int b) -> int {
         double *bc = rc + b * m, *bs = rs + b * m;
         while (ql_l < m) {
             const int l = ql_l;
-            int mm = l;
-            for (; mm < m - 1; mm++) {
-                const double dd2 = fabs(dg[mm]) + fabs(dg[mm + 1]);
-                if (fabs(ee[mm]) <= SDC_EPS * dd2) break;
-            }
-            if (mm == l || ql_iter >= 64) {
-                if (mm != l) s_flag = 1;
+            if (ql_iter == 0 && ql_h <= l) ql_h = ql_scan<1>(dg, ee, l, m);      // else known from the last sweep
+            if (ql_h <= l || ql_iter >= 64) {
+                if (ql_h > l) s_flag = 1;
                 ql_l++;
                 ql_iter = 0;
                 continue;
             }
             ql_iter++;
-            const int cnt = ql_sweep_tri<1>(dg, ee, l, mm, [&](int q, double c, double s) { bc[q] = c; bs[q] = s; });
-            s_first_b[b] = mm - 1;
+            int low;
+            bool first;
+            s_first_b[b] = ql_h - 1;
+            const int cnt = ql_sweep_tri<1>(dg, ee, l, ql_h, low, first, [&](int q, double c, double s) { bc[q] = c; bs[q] = s; });
+            ql_h = low;
+            if (first) { ql_l++; ql_iter = 0; }
             return cnt;
         }
         return -1;
