@@ -352,7 +352,7 @@ extern "C" superdc_status superdc_rank1_apply(int64_t nprob, const int64_t *offs
 #ifdef SUPERDC_CHECK
     f.status = fwd->status;
 #endif
-    f.fmm_min_m = fmm_resolve(opts->fmm_min_m);
+    f.fmm_min_m = fmm_resolve_rows(opts->fmm_min_m, total);
     superdc_status s;
     if (trans) {
         SDC_CHECK(sc.get(&Xw, (size_t)total * ncols));

@@ -1351,7 +1351,7 @@ superdc_status superdc_eig_plan(const superdc_hss *h, const superdc_opts *opts, 
     superdc_eigfact *f = new superdc_eigfact();
     f->h = h; f->n = n; f->r = r; f->lmax = lmax;
     f->opts = *opts;
-    f->fmm_min_m = fmm_resolve(opts->fmm_min_m);
+    f->fmm_min_m = fmm_resolve_rows(opts->fmm_min_m, n);
     auto fail = [&](cudaError_t e) {
         superdc_eigfact_free(f);
         return e == cudaErrorMemoryAllocation ? SUPERDC_ERR_OOM : SUPERDC_ERR_CUDA;
@@ -1795,7 +1795,7 @@ superdc_status superdc_apply_function(const superdc_eigfact *f, const double *fv
 superdc_status superdc_eigfact_set_fmm_min_m(superdc_eigfact *f, int32_t fmm_min_m)
 {
     if (!f) return SUPERDC_ERR_ARG;
-    f->fmm_min_m = fmm_resolve(fmm_min_m);
+    f->fmm_min_m = fmm_resolve_rows(fmm_min_m, f->n);
     return SUPERDC_OK;
 }
 

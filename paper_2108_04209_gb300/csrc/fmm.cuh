@@ -97,3 +97,12 @@ superdc_status fmm_columns(const FmmPlan &pl, const FactorView &f, int64_t total
 // threshold an option value selects (> 0 itself, 0 the default, < 0 off).
 int fmm_default_min_m();
 inline int fmm_resolve(int32_t opt) { return opt > 0 ? opt : (opt == 0 ? fmm_default_min_m() : 0); }
+
+// The same for eigendecompositions and applications of their factors, whose
+// levels have rows rows each: with few rows the launches and chains of the tree
+// and its passes cost more than they save (fmm.cu).
+int fmm_few_rows_min_m();
+inline int fmm_resolve_rows(int32_t opt, int64_t rows)
+{
+    return (opt == 0 && rows < (int64_t)sdc_num_sms() * 128) ? fmm_few_rows_min_m() : fmm_resolve(opt);
+}
