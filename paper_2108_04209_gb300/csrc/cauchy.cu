@@ -61,26 +61,6 @@ __global__ void k_givens(FactorView f, int64_t total, double *X, int64_t ldx, in
     }
 }
 
-// deflated slots: identity part of the factor
-__global__ void k_defl_copy(FactorView f, int64_t total, const double *__restrict__ X, int64_t ldx,
-                            double *__restrict__ Y, int64_t ldy, int ncols, int trans)
-{
-    for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < total * ncols;
-         x += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t slotg = x % total;
-        const int col = (int)(x / total);
-        if (slotg < f.off[0] || slotg >= f.off[f.nprob]) continue;
-        const int64_t p = sdc_upper_index(f.off, f.nprob, slotg);
-        const int64_t b0 = f.off[p];
-        const int s = (int)(slotg - b0);
-        if (s < f.mk[p]) continue;
-        const int64_t ps = SDC_IDX(f.pinv[slotg], f.off[p + 1] - b0, f.status);
-        const int64_t sr = SDC_IDX(f.src[slotg], f.off[p + 1] - b0, f.status);
-        if (trans) Y[b0 + ps + (int64_t)col * ldy] = X[b0 + sr + (int64_t)col * ldx];
-        else       Y[b0 + sr + (int64_t)col * ldy] = X[b0 + ps + (int64_t)col * ldx];
-    }
-}
-
 superdc_status run(const FactorView &f, int64_t total, double *Xmut, const double *X, int64_t ldx, double *Y,
                    int64_t ldy, int ncols, bool trans, cudaStream_t st, const FmmPlan *shared)
 {
@@ -104,8 +84,6 @@ superdc_status run(const FactorView &f, int64_t total, double *Xmut, const doubl
         if (fs != SUPERDC_OK) { fmm_free(fp, st); return fs; }
     }
     const superdc_status fs = fmm_columns(use_shared ? *shared : fp, f, total, tile_off, X, ldx, Y, ldy, ncols, trans, st);
-    PROF_LAUNCH("deflcopy", st, k_defl_copy<<<(unsigned)(nsm * 8), 256, 0, st>>>(f, total, X, ldx, Y, ldy, ncols,
-                                                                                  trans ? 1 : 0));
     if (!trans)
         PROF_LAUNCH("givens", st, k_givens<<<(unsigned)(nsm * 8), gthreads, 0, st>>>(f, total, Y, ldy, ncols, 1));
     const cudaError_t le = cudaGetLastError();

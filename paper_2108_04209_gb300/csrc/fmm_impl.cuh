@@ -1972,12 +1972,14 @@ __global__ void __launch_bounds__(128) k_fmm_lastsum(FmmDev pl, const int64_t *_
 //     eta_j) and the last eigenvalue (outside the positions' range) are added
 //     in FP64.
 //   * Problems out of the positions' scale (cm_prep) take FP64 loops.
-// One warp per 16 targets, digit fragments read in mma order from global
-// memory (written once per call by k_cm_slice / k_cm_up).
+// Digit fragments of the columns are read in mma order from global memory
+// (written once per pass of 64 columns by k_cm_slice / k_cm_up).
 // ---------------------------------------------------------------------------
 constexpr int CM_D = 7;           // digits
-constexpr int CM_NT = 3;          // column tiles of 8 per pass
-constexpr int CM_TR = 64;         // targets per CTA (4 warps)
+constexpr int CM_NT = 8;          // column tiles of 8 per pass
+constexpr int CM_TR = 64;         // targets per entry of tile_off, four CTAs of 16
+constexpr int CM_TAKE = 8;        // far boxes taken per level and round
+constexpr int CM_BC = 24;         // columns per pass of the FP64 loops
 
 __device__ __forceinline__ float pow2f(int e) { return __int_as_float((e + 127) << 23); }      // -126 <= e <= 127
 
@@ -2006,7 +2008,7 @@ struct CmDev {
     uint2 *wf0;                  // node weights' digits: nodes 0..15 [box][tile][digit][lane]
     unsigned *wf1;               //                       nodes 16..21
     int32_t *eb;                 // per box: exponent of its node weights over the columns' scales
-    double *lastp;               // per (tile of 64, column): partial sums for the last eigenvalue
+    double *lastp;               // per (tile of 64, column of the pass): partial sums for the last eigenvalue
 };
 
 template <bool TRANS>
@@ -2097,12 +2099,12 @@ __global__ void k_cm_slice(FactorView f, int64_t nchunk_rows, const double *__re
     }
 }
 
-__device__ __forceinline__ void cm_mma16(float (&d)[4], const unsigned (&a)[4], uint2 b)
+__device__ __forceinline__ void cm_mma16(float (&d)[4], const uint4 &a, uint2 b)
 {
     asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
                  "{%0,%1,%2,%3};"
                  : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b.x), "r"(b.y));
+                 : "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b.x), "r"(b.y));
 }
 
 __device__ __forceinline__ void cm_mma8(float (&d)[4], unsigned a0, unsigned a1, unsigned b)
@@ -2136,17 +2138,24 @@ __device__ __forceinline__ unsigned cm_pack(float lo, float hi)
     return __byte_perm(__float_as_uint(lo), __float_as_uint(hi), 0x7632);
 }
 
-// exact sums of the orders i + j = 2..8 -> double (unit entries)
+// exact sums of the orders i + j = 2..8 (unit entries) in two integers: hi 2^-30 + lo 2^-62
+struct CmSum { long long hi, lo; };
+
+__device__ __forceinline__ void cm_add(CmSum &v, const float (&a)[CM_D][4], int i)
+{
+    v.hi += ((long long)__float2int_rn(a[0][i] * 0x1p14f) << 16) + ((long long)__float2int_rn(a[1][i] * 0x1p22f) << 8) +
+            __float2int_rn(a[2][i] * 0x1p30f);
+    v.lo += ((long long)__float2int_rn(a[3][i] * 0x1p38f) << 24) + ((long long)__float2int_rn(a[4][i] * 0x1p46f) << 16) +
+            ((long long)__float2int_rn(a[5][i] * 0x1p54f) << 8) + __float2int_rn(a[6][i] * 0x1p62f);
+}
+
+__device__ __forceinline__ double cm_value(const CmSum &v) { return fma((double)v.hi, 0x1p-30, (double)v.lo * 0x1p-62); }
+
 __device__ __forceinline__ double cm_fold(const float (&a)[CM_D][4], int i)
 {
-    long long hi = (long long)__float2int_rn(a[0][i] * 0x1p14f) << 16;
-    hi += (long long)__float2int_rn(a[1][i] * 0x1p22f) << 8;
-    hi += __float2int_rn(a[2][i] * 0x1p30f);
-    long long lo = (long long)__float2int_rn(a[3][i] * 0x1p38f) << 24;
-    lo += (long long)__float2int_rn(a[4][i] * 0x1p46f) << 16;
-    lo += (long long)__float2int_rn(a[5][i] * 0x1p54f) << 8;
-    lo += __float2int_rn(a[6][i] * 0x1p62f);
-    return fma((double)hi, 0x1p-30, (double)lo * 0x1p-62);
+    CmSum v = {0, 0};
+    cm_add(v, a, i);
+    return cm_value(v);
 }
 
 // ---------------------------------------------------------------------------
@@ -2161,7 +2170,7 @@ __device__ __forceinline__ double cm_fold(const float (&a)[CM_D][4], int i)
 // read.  The climb and its arrival counters are those of k_fmm_up, which still
 // does the problems out of scale.  A leaf and its parent took 33 k cycles of the
 // FP64 pipe for 24 columns.  Measured (GB300, f(A) X, n = 32768, 64 columns;
-// with k_cm_slicew): 196 -> 59 ms.
+// 24 columns a pass): 196 -> 59 ms, with 64 columns a pass 36.
 // ---------------------------------------------------------------------------
 constexpr int CU_ROWS = 32;       // matrix rows (22 nodes, zeros below)
 constexpr int CU_LD = 56;         // bf16 per row: up to 48 sources, 112 bytes (no bank conflicts)
@@ -2224,13 +2233,13 @@ __device__ __forceinline__ void cu_matrix(const ff_t3 *su, const ff_t3 *sf, cons
     }
 }
 
-template <int NT, bool TRANS>
-__global__ void __launch_bounds__(128) k_cm_up(FmmDev pl, FactorView f, CmDev c, int col0, int nc)
+template <int NTM, bool TRANS>          // NTM: most column tiles of a pass (shared memory)
+__global__ void __launch_bounds__(128) k_cm_up(FmmDev pl, FactorView f, CmDev c, int col0, int nc, int nt)
 {
     __shared__ __align__(16) unsigned short As[CM_D][CU_ROWS][CU_LD];
-    __shared__ __align__(16) uint2 o0[NT * CM_D * 32];
-    __shared__ unsigned o1[NT * CM_D * 32];
-    __shared__ double Ws[P][NT * 8];
+    __shared__ __align__(16) uint2 o0[2 * CM_D * 32];        // digits of two column tiles
+    __shared__ unsigned o1[2 * CM_D * 32];
+    __shared__ double Ws[P][NTM * 8];
     __shared__ ff_t3 sx[P], sw[P], su[48], sf[48];
     __shared__ double xq[P];
     __shared__ int s_e, s_last;
@@ -2315,8 +2324,8 @@ __global__ void __launch_bounds__(128) k_cm_up(FmmDev pl, FactorView f, CmDev c,
             cu_matrix(su, sf, sx, sw, 0, l == 0 ? B : 24 * nch, As);
             __syncthreads();
             // products: (16 nodes, 8 columns) per warp
-            for (int un = warp; un < 2 * NT; un += 4) {
-                const int mt = un / NT, n = un % NT;
+            for (int un = warp; un < 2 * nt; un += 4) {
+                const int mt = un & 1, n = un >> 1;
                 float acc[CM_D][4];
 #pragma unroll
                 for (int s = 0; s < CM_D; s++)
@@ -2329,18 +2338,16 @@ __global__ void __launch_bounds__(128) k_cm_up(FmmDev pl, FactorView f, CmDev c,
                 const int n16 = l == 0 ? 2 : nch;
                 for (int st = 0; st < n16; st++) {
                     const int k0 = l == 0 ? 16 * st : 24 * st;
-                    const uint2 *bf = l == 0 ? c.xf + (((cm_chunk(b0, p) + 2 * b + st) * NT + n) * CM_D) * 32 + lane
-                                             : c.wf0 + (((gc0 + st) * NT + n) * CM_D) * 32 + lane;
+                    const uint2 *bf = l == 0 ? c.xf + (((cm_chunk(b0, p) + 2 * b + st) * nt + n) * CM_D) * 32 + lane
+                                             : c.wf0 + (((gc0 + st) * nt + n) * CM_D) * 32 + lane;
                     if (l == 0 && b * B + 16 * st >= m) continue;
                     uint2 bb[CM_D];
-                    unsigned a[CM_D][4];
+                    uint4 a[CM_D];
 #pragma unroll
                     for (int s = 0; s < CM_D; s++) {
                         bb[s] = __ldcg(bf + s * 32);
-                        a[s][0] = frag(s, r0, k0);
-                        a[s][1] = frag(s, r0 + 8, k0);
-                        a[s][2] = frag(s, r0, k0 + 8);
-                        a[s][3] = frag(s, r0 + 8, k0 + 8);
+                        a[s] = make_uint4(frag(s, r0, k0), frag(s, r0 + 8, k0), frag(s, r0, k0 + 8),
+                                          frag(s, r0 + 8, k0 + 8));
                     }
 #pragma unroll
                     for (int i1 = 0; i1 < CM_D; i1++)
@@ -2348,7 +2355,7 @@ __global__ void __launch_bounds__(128) k_cm_up(FmmDev pl, FactorView f, CmDev c,
                         for (int j1 = 0; i1 + j1 < CM_D; j1++) cm_mma16(acc[i1 + j1], a[i1], bb[j1]);
                 }
                 for (int st = 0; st < nch; st++) {
-                    const unsigned *bf = c.wf1 + (((gc0 + st) * NT + n) * CM_D) * 32 + lane;
+                    const unsigned *bf = c.wf1 + (((gc0 + st) * nt + n) * CM_D) * 32 + lane;
                     unsigned bb[CM_D], a[CM_D][2];
 #pragma unroll
                     for (int s = 0; s < CM_D; s++) {
@@ -2370,7 +2377,7 @@ __global__ void __launch_bounds__(128) k_cm_up(FmmDev pl, FactorView f, CmDev c,
             __syncthreads();
             // the box's exponent, then its digits
             int ex = 0;
-            for (int i = tid; i < P * NT * 8; i += 128) ex = max(ex, ff_exp(Ws[i / (NT * 8)][i % (NT * 8)]));
+            for (int i = tid; i < P * nt * 8; i += 128) ex = max(ex, ff_exp(Ws[i / (nt * 8)][i % (nt * 8)]));
             ex = __reduce_max_sync(FULL, ex);
             if (tid == 0) s_e = 0;
             __syncthreads();
@@ -2378,21 +2385,25 @@ __global__ void __launch_bounds__(128) k_cm_up(FmmDev pl, FactorView f, CmDev c,
             __syncthreads();
             ex = s_e;
             const double sc = ex > 0 ? ff_pow2(1022 - ex) : 0.0;
-            for (int i = tid; i < 24 * NT * 8; i += 128) {
-                const int k = i / (NT * 8), col = i % (NT * 8);
-                unsigned short dg[CM_D];
-                cm_digits(k < P ? Ws[k][col] * sc : 0.0, dg);
-                const int ln = (col & 7) * 4 + ((k & 7) >> 1), at = (col >> 3) * CM_D * 32 + ln;
-                unsigned short *dst = k < 16 ? (unsigned short *)(o0 + at) + ((k >> 3) << 1) + (k & 1)
-                                             : (unsigned short *)(o1 + at) + (k & 1);
-                const int step = k < 16 ? 32 * 4 : 32 * 2;
+            for (int n0 = 0; n0 < nt; n0 += 2) {
+                const int nb = min(2, nt - n0);
+                for (int i = tid; i < 24 * nb * 8; i += 128) {
+                    const int k = i / (nb * 8), col = i % (nb * 8);
+                    unsigned short dg[CM_D];
+                    cm_digits(k < P ? Ws[k][n0 * 8 + col] * sc : 0.0, dg);
+                    const int ln = (col & 7) * 4 + ((k & 7) >> 1), at = (col >> 3) * CM_D * 32 + ln;
+                    unsigned short *dst = k < 16 ? (unsigned short *)(o0 + at) + ((k >> 3) << 1) + (k & 1)
+                                                 : (unsigned short *)(o1 + at) + (k & 1);
+                    const int step = k < 16 ? 32 * 4 : 32 * 2;
 #pragma unroll
-                for (int s = 0; s < CM_D; s++) dst[s * step] = dg[s];
-            }
-            __syncthreads();
-            for (int i = tid; i < NT * CM_D * 32; i += 128) {
-                c.wf0[g * NT * CM_D * 32 + i] = o0[i];
-                c.wf1[g * NT * CM_D * 32 + i] = o1[i];
+                    for (int s = 0; s < CM_D; s++) dst[s * step] = dg[s];
+                }
+                __syncthreads();
+                for (int i = tid; i < nb * CM_D * 32; i += 128) {
+                    c.wf0[(g * nt + n0) * CM_D * 32 + i] = o0[i];
+                    c.wf1[(g * nt + n0) * CM_D * 32 + i] = o1[i];
+                }
+                __syncthreads();
             }
             if (tid == 0) c.eb[g] = ex > 0 ? E0 + ex - 1022 : -4000;
             if (l + 1 >= L) break;
@@ -2416,22 +2427,45 @@ __global__ void __launch_bounds__(128) k_cm_up(FmmDev pl, FactorView f, CmDev c,
     }
 }
 
-template <int NT, bool TRANS>
-__global__ void __launch_bounds__(128)
+// digits of the kernel entries of up to 32 sources (22 nodes) and 16 targets, in mma order
+struct __align__(16) CmFrag { uint4 k[2][CM_D][32]; };
+
+// The CTA's four warps form the digits of four boxes at a time (near boxes of 32
+// sources, or the 22 nodes of far boxes), then multiply: warp w has the column
+// tiles w % NTP + NTP i (i < TPW) of every (4 / NTP)-th box.
+// What bounds it: forming a 16 x 16 block takes 800 warp instructions (three-float
+// quotient and 7 digits an entry), its products 28 mma per column tile.  One warp
+// per 16 targets with three tiles of its own held 255 registers: 8 warps per SM at
+// 26 % of the issue slots, and every 24 columns formed the entries again.  Here a
+// warp holds one or two tiles and an entry is formed once for 64 columns.
+// Measured (GB300, f(A) X, n = 32768, 64 columns): 86 -> 57 ms; the
+// eigendecomposition of n = 131072 (1 to 19 columns): 61 -> 58 ms.
+template <int NTP, int TPW, bool TRANS>
+__global__ void __launch_bounds__(128, TPW == 1 ? 4 : 3)
 k_cm_apply(FmmDev pl, FactorView f, const int64_t *__restrict__ tile_off, CmDev c, const double *__restrict__ X,
-           int64_t ldx, double *__restrict__ Y, int64_t ldy, int col0, int nc)
+           int64_t ldx, double *__restrict__ Y, int64_t ldy, int col0, int nc, int nt)
 {
-    __shared__ int list[4][32 * FAR_TAKE];
+    constexpr int NS = 4 / NTP;                          // warps that share a column tile
+    __shared__ CmFrag sA[4];
+    __shared__ int2 list[32 * CM_TAKE];                  // far boxes: index, exponent of its weights
+    __shared__ int64_t s_pst[32];                        // per level: the list's start, the target's ancestor
+    __shared__ int s_lb[32];
+    __shared__ double s_lo[32], s_hi[32];
+    __shared__ int s_total, s_ET;
+    // a warp that multiplies what it formed itself needs no barrier
+    auto boxes_sync = [&]() { if (NS == 4) __syncwarp(); else __syncthreads(); };
     const unsigned FULL = 0xffffffffu;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, gr = lane >> 2, gc = lane & 3;
-    const int64_t ntiles = tile_off[f.nprob];
-    for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    const int tl = warp % NTP, grp = warp / NTP;
+    const int64_t ntiles = tile_off[f.nprob] * 4;
+    for (int64_t it = blockIdx.x; it < ntiles; it += gridDim.x) {
+        const int64_t tile = it >> 2;
         const int64_t p = sdc_upper_index(tile_off, f.nprob, tile);
         const int64_t b0 = f.off[p];
         const int m = f.mk[p];
-        const int t0 = (int)(tile - tile_off[p]) * CM_TR + warp * 16;
+        const int t0 = (int)(tile - tile_off[p]) * CM_TR + (int)(it & 3) * 16;
         const int tend = TRANS ? m - 1 : m;              // T: the last target is summed by k_cm_last
-        if (t0 >= tend) continue;
+        if (t0 >= tend || c.bad[p]) continue;            // out of scale: k_cm_rest
         const bool tree = pl.fslot && pl.fslot[p] >= 0;
         const double *dk = f.dk + b0, *dorg = f.dorg + b0, *eta = f.eta + b0;
         const int nb0 = (m + B - 1) / B, Tb = t0 / B;
@@ -2439,270 +2473,274 @@ k_cm_apply(FmmDev pl, FactorView f, const int64_t *__restrict__ tile_off, CmDev 
         const int nnr = tree ? pl.nnear[gbx + Tb] : -1;
         const int nn = near_len(nnr, nb0);               // without a tree: every box
         const int nsrc = TRANS ? m : m - 1;
-        if (c.bad[p]) {
-            // FP64: a row per lane pair, half of the columns each
-            const int r = min(t0 + (lane & 15), tend - 1), h = lane >> 4;
-            const double a0 = TRANS ? dorg[r] : dk[r], a1 = TRANS ? eta[r] : 0.0;
-            double acc[NT * 4] = {};
-            auto add = [&](double t, double s, const double *col, int64_t st) {
-                const double w = s * rcp_nr2(t);
-#pragma unroll
-                for (int q = 0; q < NT * 4; q++)
-                    if (h * NT * 4 + q < nc) acc[q] = fma(w, col[(int64_t)(h * NT * 4 + q) * st], acc[q]);
-            };
-            for (int i = 0; i < nn; i++) {
-                const int j0 = SDC_IDX(near_box(pl, gbx + Tb, nnr, i), nb0, f.status) * B;
-                for (int j = j0; j < min(j0 + B, nsrc); j++) {
-                    if (TRANS) add((dk[j] - a0) - a1, f.vhat[b0 + j], X + b0 + f.src[b0 + j] + (int64_t)col0 * ldx, ldx);
-                    else add((a0 - dorg[j]) - eta[j], f.bnorm[b0 + j], X + b0 + f.pinv[b0 + j] + (int64_t)col0 * ldx, ldx);
-                }
-            }
-            if (!TRANS) add((a0 - dorg[m - 1]) - eta[m - 1], f.bnorm[b0 + m - 1],
-                            X + b0 + f.pinv[b0 + m - 1] + (int64_t)col0 * ldx, ldx);
-            if (tree && nnr >= 0) {
-                const int L = lev_count(nb0);
-                const double x = TRANS ? a0 + a1 : a0;
-                for (int l = 0; l < L - 1; l++) {
-                    const int A = Tb >> l;
-                    const int64_t gl = gbx + lev_base(nb0, l), gP = gbx + lev_base(nb0, l + 1) + (A >> 1);
-                    for (int i = 0; i < 2 * pl.nnear[gP]; i++) {
-                        const int S = 2 * pl.near[pl.nstart[gP] + (i >> 1)] + (i & 1);
-                        if (S >= lev_nb(nb0, l) || S == A ||
-                            !adm(pl.ibox[gl + S], pl.ibox[gl + A]))
-                            continue;
-                        double cS, hS;
-                        box_ch(pl.blo[gl + S], pl.bhi[gl + S], cS, hS);
-                        for (int q = 0; q < P; q++) {
-                            const double s = cS + hS * cospi((double)(2 * q + 1) / (2.0 * P));
-                            add(TRANS ? s - x : x - s, 1.0, pl.W + ((gl + S) * P + q) * pl.ncol, 1);
-                        }
-                    }
-                }
-            }
-            const int64_t row = b0 + (TRANS ? f.pinv[b0 + r] : f.src[b0 + r]);
-            const double sc = TRANS ? f.bnorm[b0 + r] : f.vhat[b0 + r];
-            if (t0 + (lane & 15) < tend)
-#pragma unroll
-                for (int q = 0; q < NT * 4; q++)
-                    if (h * NT * 4 + q < nc) Y[row + (int64_t)(col0 + h * NT * 4 + q) * ldy] = sc * acc[q];
-            continue;
-        }
         const FfScale fs = ff_scale(dk[0], dk[m - 1], 1.0);
         // the two rows of this lane: positions and the powers of two of their near entries
         ff_f4 x[2];
         float rs[2];
+        double ns[2];                                    // near sums times this (2^kk by the factors of Qhat X)
         int skip[2];                                     // T: the origin's index; N: the target (skip, skip - 1)
 #pragma unroll
         for (int h = 0; h < 2; h++) {
             const int r = min(t0 + gr + 8 * h, tend - 1);
             const double sc = TRANS ? f.bnorm[b0 + r] : f.vhat[b0 + r];
             x[h] = TRANS ? ff_point(dorg[r], eta[r], fs) : ff_pole(dk[r], fs);
-            const int e = ff_exp(sc) - 1023 + (TRANS ? fs.kk : 0);
-            rs[h] = pow2f(max(-126, min(126, e)));
+            const int e = max(-126, min(126, ff_exp(sc) - 1023 + (TRANS ? fs.kk : 0)));
+            rs[h] = pow2f(e);
+            ns[h] = ff_pow2((TRANS ? fs.kk : 0) - e);
             skip[h] = TRANS ? (dorg[r] == dk[r] ? r : r + 1) : r;
         }
-        float acc[NT][CM_D][4];
-        double y[NT][4];
+        float acc[TPW][CM_D][4];
+        CmSum sum[TPW][4];                               // of the folds: FP64 only once per field
+        double y[TPW][4];
         auto clear = [&]() {
 #pragma unroll
-            for (int n = 0; n < NT; n++)
+            for (int t = 0; t < TPW; t++)
 #pragma unroll
                 for (int s = 0; s < CM_D; s++)
 #pragma unroll
-                    for (int i = 0; i < 4; i++) acc[n][s][i] = 0.0f;
+                    for (int i = 0; i < 4; i++) acc[t][s][i] = 0.0f;
+        };
+        auto fold = [&]() {
+#pragma unroll
+            for (int t = 0; t < TPW; t++)
+#pragma unroll
+                for (int i = 0; i < 4; i++) cm_add(sum[t][i], acc[t], i);
+            clear();
+        };
+        // y += the sums of all warps times sc (rows gr, gr + 8), in the first group's warps
+        auto collect = [&](double sc0, double sc1) {
+            fold();
+            if (NS > 1) {
+                CmSum *red = (CmSum *)sA;
+                __syncthreads();                         // every warp is done with the digits
+                if (grp > 0)
+#pragma unroll
+                    for (int q = 0; q < 4 * TPW; q++)
+                        red[(((grp - 1) * NTP + tl) * 4 * TPW + q) * 32 + lane] = sum[q >> 2][q & 3];
+                __syncthreads();
+                if (grp == 0)
+                    for (int w = 0; w < NS - 1; w++)
+#pragma unroll
+                        for (int q = 0; q < 4 * TPW; q++) {
+                            const CmSum v = red[((w * NTP + tl) * 4 * TPW + q) * 32 + lane];
+                            sum[q >> 2][q & 3].hi += v.hi;
+                            sum[q >> 2][q & 3].lo += v.lo;
+                        }
+            }
+#pragma unroll
+            for (int t = 0; t < TPW; t++)
+#pragma unroll
+                for (int i = 0; i < 4; i++) {
+                    if (grp == 0) y[t][i] = fma(cm_value(sum[t][i]), i < 2 ? sc0 : sc1, y[t][i]);
+                    sum[t][i] = {0, 0};
+                }
+            __syncthreads();
+        };
+        // the products of the staged digits k[half] of box v with this warp's column tiles
+        auto mult16 = [&](int v, int half, const uint2 *__restrict__ bf) {
+            uint4 a[CM_D];
+#pragma unroll
+            for (int s = 0; s < CM_D; s++) a[s] = sA[v].k[half][s][lane];
+#pragma unroll
+            for (int t = 0; t < TPW; t++) {
+                const int n = tl + NTP * t;
+                if (n >= nt) break;
+                uint2 b[CM_D];
+#pragma unroll
+                for (int s = 0; s < CM_D; s++) b[s] = bf[(n * CM_D + s) * 32 + lane];
+#pragma unroll
+                for (int i1 = 0; i1 < CM_D; i1++)
+#pragma unroll
+                    for (int j1 = 0; i1 + j1 < CM_D; j1++) cm_mma16(acc[t][i1 + j1], a[i1], b[j1]);
+            }
+        };
+        auto mult8 = [&](int v, const unsigned *__restrict__ bf) {
+            uint2 a[CM_D];
+#pragma unroll
+            for (int s = 0; s < CM_D; s++) a[s] = ((const uint2 *)sA[v].k[1][s])[lane];
+#pragma unroll
+            for (int t = 0; t < TPW; t++) {
+                const int n = tl + NTP * t;
+                if (n >= nt) break;
+                unsigned b[CM_D];
+#pragma unroll
+                for (int s = 0; s < CM_D; s++) b[s] = bf[(n * CM_D + s) * 32 + lane];
+#pragma unroll
+                for (int i1 = 0; i1 < CM_D; i1++)
+#pragma unroll
+                    for (int j1 = 0; i1 + j1 < CM_D; j1++) cm_mma8(acc[t][i1 + j1], a[i1].x, a[i1].y, b[j1]);
+            }
         };
         clear();
 #pragma unroll
-        for (int n = 0; n < NT; n++)
+        for (int t = 0; t < TPW; t++)
 #pragma unroll
-            for (int i = 0; i < 4; i++) y[n][i] = 0.0;
+            for (int i = 0; i < 4; i++) { y[t][i] = 0.0; sum[t][i] = {0, 0}; }
+        __syncthreads();                                 // the previous tile's list and digits
         // ---- far field: the nodes of the interaction lists
-        int ET = -4000, far_src = 0;
+        int far_src = 0;
         if (tree && nnr >= 0) {
+            // warp 0, lane l: the list of the tile's ancestor on level l
             const int L = lev_count(nb0);
-            int A = 0, npn = 0, lb = 0, nbl = 0;
+            int A = 0, npn = 0, nbl = 0, lb = 0, sec = 0;
             int64_t pst = 0;
             unsigned long long mask = 0;
-            double lo = 0.0, hi = 0.0;
-            if (lane < L - 1) {
+            if (warp == 0 && lane < L - 1) {
                 A = Tb >> lane;
                 lb = lev_base(nb0, lane);
                 nbl = lev_nb(nb0, lane);
                 const int64_t gP = gbx + lev_base(nb0, lane + 1) + (A >> 1);
                 npn = pl.nnear[gP];
                 pst = pl.nstart[gP];
-                lo = pl.blo[gbx + lb + A];
-                hi = pl.bhi[gbx + lb + A];
-                // largest weight over distance of the list
-                for (int sec = 0; sec == 0 || 64 * sec < 2 * npn; sec++) {
-                    unsigned long long mk = sec == 0 ? pl.amask[gbx + lb + A] : adm_mask(pl, gbx + lb, nbl, A, pst, npn, sec);
-                    if (sec == 0) mask = mk;
-                    while (mk) {
-                        const int i = __ffsll((long long)mk) - 1;
-                        mk &= mk - 1;
-                        const int64_t gS = gbx + lb + 2 * pl.near[pst + ((64 * sec + i) >> 1)] + (i & 1);
-                        const double gap = fmax(lo - pl.bhi[gS], pl.blo[gS] - hi);
-                        if (c.eb[gS] > -4000) ET = max(ET, c.eb[gS] - (ff_exp(gap) - 1023 + fs.kk));
-                    }
-                }
+                mask = pl.amask[gbx + lb + A];
+                s_pst[lane] = pst;
+                s_lb[lane] = lb;
+                s_lo[lane] = pl.blo[gbx + lb + A];
+                s_hi[lane] = pl.bhi[gbx + lb + A];
             }
-            ET = __reduce_max_sync(FULL, ET);
-            int sec = 0, nsum = 0;
-            while (ET > -4000 && __any_sync(FULL, mask != 0 || 64 * (sec + 1) < 2 * npn)) {
-                if (mask == 0 && 64 * (sec + 1) < 2 * npn) {
-                    sec++;
-                    mask = adm_mask(pl, gbx + lb, nbl, A, pst, npn, sec);
+            for (;;) {
+                // a round: warp 0 numbers the boxes, every thread looks one up; the
+                // round's digits share the largest weight over distance, 2^ET
+                if (warp == 0) {
+                    int total = -1;
+                    if (__any_sync(FULL, mask != 0 || 64 * (sec + 1) < 2 * npn)) {
+                        if (mask == 0 && 64 * (sec + 1) < 2 * npn) {
+                            sec++;
+                            mask = adm_mask(pl, gbx + lb, nbl, A, pst, npn, sec);
+                        }
+                        const int cnt = min(CM_TAKE, __popcll(mask));
+                        int pos = cnt;
+                        for (int s = 1; s < 32; s <<= 1) {
+                            const int v = __shfl_up_sync(FULL, pos, s);
+                            if (lane >= s) pos += v;
+                        }
+                        total = __shfl_sync(FULL, pos, 31);
+                        pos -= cnt;
+                        for (int i = 0; i < cnt; i++) {
+                            const int bt = __ffsll((long long)mask) - 1;
+                            mask &= mask - 1;
+                            list[pos + i] = make_int2(64 * sec + bt, lane);
+                        }
+                    }
+                    if (lane == 0) { s_total = total; s_ET = -4000; }
                 }
-                const int cnt = min(FAR_TAKE, __popcll(mask));
-                int pos = cnt;
-                for (int s = 1; s < 32; s <<= 1) {
-                    const int v = __shfl_up_sync(FULL, pos, s);
-                    if (lane >= s) pos += v;
+                __syncthreads();
+                const int total = s_total;
+                if (total < 0) break;
+                for (int t = threadIdx.x; t < total; t += 128) {
+                    const int2 q = list[t];
+                    const int S = s_lb[q.y] + 2 * pl.near[s_pst[q.y] + (q.x >> 1)] + (q.x & 1);
+                    const int e = c.eb[gbx + S];
+                    const double gap = fmax(s_lo[q.y] - pl.bhi[gbx + S], pl.blo[gbx + S] - s_hi[q.y]);
+                    list[t] = make_int2(S, e);
+                    if (e > -4000) atomicMax(&s_ET, e - (ff_exp(gap) - 1023 + fs.kk));
                 }
-                const int total = __shfl_sync(FULL, pos, 31);
-                pos -= cnt;
-                __syncwarp();
-                for (int i = 0; i < cnt; i++) {
-                    const int b = __ffsll((long long)mask) - 1;
-                    mask &= mask - 1;
-                    list[warp][pos + i] = lb + 2 * pl.near[pst + ((64 * sec + b) >> 1)] + (b & 1);
-                }
-                __syncwarp();
+                __syncthreads();
+                const int ET = s_ET;
+                int nsum = 0;
                 far_src += total * P;
-                for (int i = 0; i < total; i++) {
-                    const int64_t gS = gbx + list[warp][i];
-                    const int e = c.eb[gS] - ET;
-                    if (e < -62) continue;               // below the last digit
-                    const float sc = TRANS ? pow2f(e) : -pow2f(e);
-                    const ff_f4 *np = pl.npos + gS * P;
-                    unsigned a[CM_D][4];
-                    // nodes 0..15
+                for (int i = 0; i < total; i += 4) {
+                    const int u = i + warp;
+                    if (u < total && list[u].y - ET >= -62) {    // else below the last digit
+                        const float sc = TRANS ? pow2f(list[u].y - ET) : -pow2f(list[u].y - ET);
+                        const ff_f4 *np = pl.npos + (gbx + list[u].x) * P;
+                        // nodes 0..15, then 16..21
 #pragma unroll
-                    for (int kp = 0; kp < 2; kp++) {
-                        const ff_f4 s0 = np[2 * gc + 8 * kp], s1 = np[2 * gc + 8 * kp + 1];
+                        for (int kp = 0; kp < 3; kp++) {
+                            const bool in = kp < 2 || gc < 3;
+                            const int q0 = in ? 2 * gc + 8 * kp : 0;
+                            const ff_f4 s0 = np[q0], s1 = np[q0 + 1];
+                            unsigned a[2][CM_D];
 #pragma unroll
-                        for (int h = 0; h < 2; h++) {
-                            ff_t3 u = ff_rcp3(ff_diff3(s0, x[h])), v = ff_rcp3(ff_diff3(s1, x[h]));
-                            u = {u.a * sc, u.b * sc, u.c * sc};
-                            v = {v.a * sc, v.b * sc, v.c * sc};
-                            float d0[CM_D], d1[CM_D];
-                            cm_cut(u, d0);
-                            cm_cut(v, d1);
+                            for (int h = 0; h < 2; h++) {
+                                ff_t3 w = ff_rcp3(ff_diff3(s0, x[h])), v = ff_rcp3(ff_diff3(s1, x[h]));
+                                w = {w.a * sc, w.b * sc, w.c * sc};
+                                v = {v.a * sc, v.b * sc, v.c * sc};
+                                float d0[CM_D], d1[CM_D];
+                                cm_cut(w, d0);
+                                cm_cut(v, d1);
 #pragma unroll
-                            for (int s = 0; s < CM_D; s++) a[s][2 * kp + h] = cm_pack(d0[s], d1[s]);
+                                for (int s = 0; s < CM_D; s++) a[h][s] = in ? cm_pack(d0[s], d1[s]) : 0u;
+                            }
+#pragma unroll
+                            for (int s = 0; s < CM_D; s++)
+                                if (kp < 2) ((uint2 *)&sA[warp].k[0][s][lane])[kp] = make_uint2(a[0][s], a[1][s]);
+                                else ((uint2 *)sA[warp].k[1][s])[lane] = make_uint2(a[0][s], a[1][s]);
                         }
                     }
-#pragma unroll
-                    for (int n = 0; n < NT; n++) {
-                        const uint2 *bf = c.wf0 + ((gS * NT + n) * CM_D) * 32 + lane;
-                        uint2 b[CM_D];
-#pragma unroll
-                        for (int s = 0; s < CM_D; s++) b[s] = bf[s * 32];
-#pragma unroll
-                        for (int i1 = 0; i1 < CM_D; i1++)
-#pragma unroll
-                            for (int j1 = 0; i1 + j1 < CM_D; j1++) cm_mma16(acc[n][i1 + j1], a[i1], b[j1]);
-                    }
-                    // nodes 16..21
-                    {
-                        const bool in = gc < 3;
-                        const ff_f4 s0 = np[in ? 16 + 2 * gc : 0], s1 = np[in ? 17 + 2 * gc : 1];
-#pragma unroll
-                        for (int h = 0; h < 2; h++) {
-                            ff_t3 u = ff_rcp3(ff_diff3(s0, x[h])), v = ff_rcp3(ff_diff3(s1, x[h]));
-                            u = {u.a * sc, u.b * sc, u.c * sc};
-                            v = {v.a * sc, v.b * sc, v.c * sc};
-                            float d0[CM_D], d1[CM_D];
-                            cm_cut(u, d0);
-                            cm_cut(v, d1);
-#pragma unroll
-                            for (int s = 0; s < CM_D; s++) a[s][h] = in ? cm_pack(d0[s], d1[s]) : 0u;
+                    boxes_sync();
+                    for (int v = grp; v < 4 && i + v < total; v += NS)
+                        if (list[i + v].y - ET >= -62) {
+                            const int64_t at = (gbx + list[i + v].x) * nt * CM_D * 32;
+                            mult16(v, 0, c.wf0 + at);
+                            mult8(v, c.wf1 + at);
                         }
-                    }
-#pragma unroll
-                    for (int n = 0; n < NT; n++) {
-                        const unsigned *bf = c.wf1 + ((gS * NT + n) * CM_D) * 32 + lane;
-                        unsigned b[CM_D];
-#pragma unroll
-                        for (int s = 0; s < CM_D; s++) b[s] = bf[s * 32];
-#pragma unroll
-                        for (int i1 = 0; i1 < CM_D; i1++)
-#pragma unroll
-                            for (int j1 = 0; i1 + j1 < CM_D; j1++) cm_mma8(acc[n][i1 + j1], a[i1][0], a[i1][1], b[j1]);
-                    }
-                    if (++nsum == 5) {                   // 110 sources: fold before the sums leave 24 bits
+                    nsum += NTP;
+                    if (nsum + NTP > 5) {                // 110 sources: fold before the sums leave 24 bits
                         nsum = 0;
-#pragma unroll
-                        for (int n = 0; n < NT; n++)
-#pragma unroll
-                            for (int q = 0; q < 4; q++) y[n][q] += cm_fold(acc[n], q);
-                        clear();
+                        fold();
                     }
+                    boxes_sync();
                 }
-                __syncwarp();
+                const double sc = ET > -4000 ? ff_pow2(ET + fs.kk) : 0.0;
+                collect(sc, sc);
             }
-            const double sc = ET > -4000 ? ff_pow2(ET + fs.kk) : 0.0;
-#pragma unroll
-            for (int n = 0; n < NT; n++)
-#pragma unroll
-                for (int q = 0; q < 4; q++) y[n][q] = (y[n][q] + cm_fold(acc[n], q)) * sc;
-            clear();
         }
         // ---- near field
-        // near sums carry the row's power of two (and 2^kk by the factors of Qhat X)
-        double ns[2];
-#pragma unroll
-        for (int h = 0; h < 2; h++) ns[h] = TRANS ? ff_pow2(fs.kk) / (double)rs[h] : 1.0 / (double)rs[h];
         const int64_t ch0 = cm_chunk(b0, p);
-        if (pl.flops && lane == 0)
+        if (pl.flops && threadIdx.x == 0)
             atomicAdd(pl.flops, (unsigned long long)min(16, tend - t0) * (far_src + (int64_t)nn * B) * (3 + 2 * nc));
-        int steps = 0;
-        for (int i = 0; i < 2 * nn; i++) {
-            const int k0 = SDC_IDX(near_box(pl, gbx + Tb, nnr, i >> 1), nb0, f.status) * B + (i & 1) * 16;
-            if (k0 >= nsrc) continue;
-            unsigned a[CM_D][4];
+        int nsum = 0;
+        for (int i = 0; i < nn; i += 4) {
+            const int u = i + warp;
+            const int kb = u < nn ? SDC_IDX(near_box(pl, gbx + Tb, nnr, u), nb0, f.status) * B : nsrc;
+#pragma unroll 1
+            for (int half = 0; half < 2; half++) {
+                const int k0 = kb + 16 * half;
+                if (k0 >= nsrc) break;
 #pragma unroll
-            for (int kp = 0; kp < 2; kp++) {
-                const int ka = k0 + 2 * gc + 8 * kp, kb = ka + 1;
-                const int64_t ia = b0 + min(ka, nsrc - 1), ib = b0 + min(kb, nsrc - 1);
-                const ff_f4 sa = c.pos[ia], sb = c.pos[ib], fa = c.fac[ia], fb = c.fac[ib];
-                const ff_t3 va = {fa.x, fa.y, fa.z}, vb = {fb.x, fb.y, fb.z};
+                for (int kp = 0; kp < 2; kp++) {
+                    const int ka = k0 + 2 * gc + 8 * kp, kc = ka + 1;
+                    const int64_t ia = b0 + min(ka, nsrc - 1), ib = b0 + min(kc, nsrc - 1);
+                    const ff_f4 sa = c.pos[ia], sb = c.pos[ib], fa = c.fac[ia], fb = c.fac[ib];
+                    const ff_t3 va = {fa.x, fa.y, fa.z}, vb = {fb.x, fb.y, fb.z};
+                    unsigned a[2][CM_D];
 #pragma unroll
-                for (int h = 0; h < 2; h++) {
-                    const ff_t3 ta = TRANS ? ff_diff3(sa, x[h]) : ff_diff3(x[h], sa);
-                    const ff_t3 tb = TRANS ? ff_diff3(sb, x[h]) : ff_diff3(x[h], sb);
-                    ff_t3 u = ff_mul3(va, ff_rcp3(ta)), v = ff_mul3(vb, ff_rcp3(tb));
-                    const bool ua = ka < nsrc && (TRANS ? ka != skip[h] : (unsigned)(skip[h] - ka) > 1u);
-                    const bool ub = kb < nsrc && (TRANS ? kb != skip[h] : (unsigned)(skip[h] - kb) > 1u);
-                    u = {ua ? u.a * rs[h] : 0.0f, ua ? u.b * rs[h] : 0.0f, ua ? u.c * rs[h] : 0.0f};
-                    v = {ub ? v.a * rs[h] : 0.0f, ub ? v.b * rs[h] : 0.0f, ub ? v.c * rs[h] : 0.0f};
-                    float d0[CM_D], d1[CM_D];
-                    cm_cut(u, d0);
-                    cm_cut(v, d1);
+                    for (int h = 0; h < 2; h++) {
+                        const ff_t3 ta = TRANS ? ff_diff3(sa, x[h]) : ff_diff3(x[h], sa);
+                        const ff_t3 tb = TRANS ? ff_diff3(sb, x[h]) : ff_diff3(x[h], sb);
+                        ff_t3 w = ff_mul3(va, ff_rcp3(ta)), v = ff_mul3(vb, ff_rcp3(tb));
+                        const bool ua = ka < nsrc && (TRANS ? ka != skip[h] : (unsigned)(skip[h] - ka) > 1u);
+                        const bool ub = kc < nsrc && (TRANS ? kc != skip[h] : (unsigned)(skip[h] - kc) > 1u);
+                        w = {ua ? w.a * rs[h] : 0.0f, ua ? w.b * rs[h] : 0.0f, ua ? w.c * rs[h] : 0.0f};
+                        v = {ub ? v.a * rs[h] : 0.0f, ub ? v.b * rs[h] : 0.0f, ub ? v.c * rs[h] : 0.0f};
+                        float d0[CM_D], d1[CM_D];
+                        cm_cut(w, d0);
+                        cm_cut(v, d1);
 #pragma unroll
-                    for (int s = 0; s < CM_D; s++) a[s][2 * kp + h] = cm_pack(d0[s], d1[s]);
+                        for (int s = 0; s < CM_D; s++) a[h][s] = cm_pack(d0[s], d1[s]);
+                    }
+#pragma unroll
+                    for (int s = 0; s < CM_D; s++)
+                        ((uint2 *)&sA[warp].k[half][s][lane])[kp] = make_uint2(a[0][s], a[1][s]);
                 }
             }
-#pragma unroll
-            for (int n = 0; n < NT; n++) {
-                const uint2 *bf = c.xf + (((ch0 + (k0 >> 4)) * NT + n) * CM_D) * 32 + lane;
-                uint2 b[CM_D];
-#pragma unroll
-                for (int s = 0; s < CM_D; s++) b[s] = bf[s * 32];
-#pragma unroll
-                for (int i1 = 0; i1 < CM_D; i1++)
-#pragma unroll
-                    for (int j1 = 0; i1 + j1 < CM_D; j1++) cm_mma16(acc[n][i1 + j1], a[i1], b[j1]);
+            boxes_sync();
+            for (int v = grp; v < 4 && i + v < nn; v += NS) {
+                const int kv = SDC_IDX(near_box(pl, gbx + Tb, nnr, i + v), nb0, f.status) * B;
+                for (int half = 0; half < 2; half++)
+                    if (kv + 16 * half < nsrc)
+                        mult16(v, half, c.xf + (ch0 + (kv >> 4) + half) * nt * CM_D * 32);
             }
-            if (++steps == 8) {                          // 128 sources
-                steps = 0;
-#pragma unroll
-                for (int n = 0; n < NT; n++)
-#pragma unroll
-                    for (int q = 0; q < 4; q++) y[n][q] = fma(cm_fold(acc[n], q), ns[q >> 1], y[n][q]);
-                clear();
+            nsum += NTP;
+            if (nsum + NTP > 4) {                        // 128 sources
+                nsum = 0;
+                fold();
             }
+            boxes_sync();
         }
+        collect(ns[0], ns[1]);
+        if (grp > 0 || tl >= nt) continue;
         // ---- FP64 terms: lane r < 16 has row r's coefficients
         double g0 = 0.0, g1 = 0.0, g2 = 0.0;
         int64_t r0 = 0, r1 = 0, r2 = 0;
@@ -2734,21 +2772,108 @@ k_cm_apply(FmmDev pl, FactorView f, const int64_t *__restrict__ tile_off, CmDev 
             const double sc = TRANS ? f.bnorm[b0 + r] : f.vhat[b0 + r];
             const int64_t row = b0 + (TRANS ? f.pinv[b0 + r] : f.src[b0 + r]);
 #pragma unroll
-            for (int n = 0; n < NT; n++)
+            for (int t = 0; t < TPW; t++)
 #pragma unroll
                 for (int q = 0; q < 2; q++) {
-                    const int col = n * 8 + 2 * gc + q;
+                    const int col = (tl + NTP * t) * 8 + 2 * gc + q;
                     if (col >= nc) continue;
-                    const int i = 2 * h + q;
                     const int cm = c.cmax[p * c.ccols + col0 + col];
-                    double v = fma(cm_fold(acc[n], i), ns[h], y[n][i]);
-                    v = cm >= 0x7FF ? nan("") : ldexp(v, cm - 1022);
+                    double v = y[t][2 * h + q];
+                    v = cm >= 0x7FF ? nan("") : cm > 30 ? v * ff_pow2(min(cm - 1022, 1023)) * (cm > 2045 ? 2.0 : 1.0)
+                                                        : ldexp(v, cm - 1022);
                     const double *xc = X + (int64_t)(col0 + col) * ldx;
                     v = fma(u0, xc[q0], v);
                     if (!TRANS) v = fma(u1, xc[q1], fma(u2, xc[q2], v));
                     Y[row + (int64_t)(col0 + col) * ldy] = sc * v;
                 }
         }
+    }
+}
+
+// What the tiles leave out, CM_BC columns per launch: the deflated slots (identity
+// part of the factor) and, in FP64, the problems out of the positions' scale (a
+// warp per 16 targets, a row per lane pair, half of the columns each).
+template <bool TRANS>
+__global__ void __launch_bounds__(128)
+k_cm_rest(FmmDev pl, FactorView f, int64_t total, const int64_t *__restrict__ tile_off, CmDev c,
+          const double *__restrict__ X, int64_t ldx, double *__restrict__ Y, int64_t ldy, int col0, int nc)
+{
+    for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < total * nc;
+         x += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t slotg = x % total;
+        const int64_t col = col0 + x / total;
+        if (slotg < f.off[0] || slotg >= f.off[f.nprob]) continue;
+        const int64_t p = sdc_upper_index(f.off, f.nprob, slotg);
+        const int64_t b0 = f.off[p];
+        if ((int)(slotg - b0) < f.mk[p]) continue;
+        const int64_t ps = SDC_IDX(f.pinv[slotg], f.off[p + 1] - b0, f.status);
+        const int64_t sr = SDC_IDX(f.src[slotg], f.off[p + 1] - b0, f.status);
+        if (TRANS) Y[b0 + ps + col * ldy] = X[b0 + sr + col * ldx];
+        else       Y[b0 + sr + col * ldy] = X[b0 + ps + col * ldx];
+    }
+    if (c.bad[f.nprob] == 0) return;
+    constexpr int NT = CM_BC / 8;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t ntiles = tile_off[f.nprob];
+    for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+        const int64_t p = sdc_upper_index(tile_off, f.nprob, tile);
+        if (!c.bad[p]) continue;
+        const int64_t b0 = f.off[p];
+        const int m = f.mk[p];
+        const int t0 = (int)(tile - tile_off[p]) * CM_TR + warp * 16;
+        const int tend = TRANS ? m - 1 : m;              // T: the last target is summed by k_cm_last
+        if (t0 >= tend) continue;
+        const bool tree = pl.fslot && pl.fslot[p] >= 0;
+        const double *dk = f.dk + b0, *dorg = f.dorg + b0, *eta = f.eta + b0;
+        const int nb0 = (m + B - 1) / B, Tb = t0 / B;
+        const int64_t gbx = tree ? pl.box_base[p] : 0;
+        const int nnr = tree ? pl.nnear[gbx + Tb] : -1;
+        const int nn = near_len(nnr, nb0);               // without a tree: every box
+        const int nsrc = TRANS ? m : m - 1;
+                                const int r = min(t0 + (lane & 15), tend - 1), h = lane >> 4;
+                    const double a0 = TRANS ? dorg[r] : dk[r], a1 = TRANS ? eta[r] : 0.0;
+                    double acc[NT * 4] = {};
+                    auto add = [&](double t, double s, const double *col, int64_t st) {
+                        const double w = s * rcp_nr2(t);
+        #pragma unroll
+                        for (int q = 0; q < NT * 4; q++)
+                            if (h * NT * 4 + q < nc) acc[q] = fma(w, col[(int64_t)(h * NT * 4 + q) * st], acc[q]);
+                    };
+                    for (int i = 0; i < nn; i++) {
+                        const int j0 = SDC_IDX(near_box(pl, gbx + Tb, nnr, i), nb0, f.status) * B;
+                        for (int j = j0; j < min(j0 + B, nsrc); j++) {
+                            if (TRANS) add((dk[j] - a0) - a1, f.vhat[b0 + j], X + b0 + f.src[b0 + j] + (int64_t)col0 * ldx, ldx);
+                            else add((a0 - dorg[j]) - eta[j], f.bnorm[b0 + j], X + b0 + f.pinv[b0 + j] + (int64_t)col0 * ldx, ldx);
+                        }
+                    }
+                    if (!TRANS) add((a0 - dorg[m - 1]) - eta[m - 1], f.bnorm[b0 + m - 1],
+                                    X + b0 + f.pinv[b0 + m - 1] + (int64_t)col0 * ldx, ldx);
+                    if (tree && nnr >= 0) {
+                        const int L = lev_count(nb0);
+                        const double x = TRANS ? a0 + a1 : a0;
+                        for (int l = 0; l < L - 1; l++) {
+                            const int A = Tb >> l;
+                            const int64_t gl = gbx + lev_base(nb0, l), gP = gbx + lev_base(nb0, l + 1) + (A >> 1);
+                            for (int i = 0; i < 2 * pl.nnear[gP]; i++) {
+                                const int S = 2 * pl.near[pl.nstart[gP] + (i >> 1)] + (i & 1);
+                                if (S >= lev_nb(nb0, l) || S == A ||
+                                    !adm(pl.ibox[gl + S], pl.ibox[gl + A]))
+                                    continue;
+                                double cS, hS;
+                                box_ch(pl.blo[gl + S], pl.bhi[gl + S], cS, hS);
+                                for (int q = 0; q < P; q++) {
+                                    const double s = cS + hS * cospi((double)(2 * q + 1) / (2.0 * P));
+                                    add(TRANS ? s - x : x - s, 1.0, pl.W + ((gl + S) * P + q) * pl.ncol, 1);
+                                }
+                            }
+                        }
+                    }
+                    const int64_t row = b0 + (TRANS ? f.pinv[b0 + r] : f.src[b0 + r]);
+                    const double sc = TRANS ? f.bnorm[b0 + r] : f.vhat[b0 + r];
+                    if (t0 + (lane & 15) < tend)
+        #pragma unroll
+                        for (int q = 0; q < NT * 4; q++)
+                            if (h * NT * 4 + q < nc) Y[row + (int64_t)(col0 + h * NT * 4 + q) * ldy] = sc * acc[q];
     }
 }
 
@@ -2856,21 +2981,28 @@ superdc_status far_field(const FmmPlan &pl, const int64_t *off, const R1Out &o, 
     return SUPERDC_OK;
 }
 
-template <int NT>
-void launch_up(bool trans, const FmmDev &dv, const FactorView &f, const CmDev &c, int col0, int nc, cudaStream_t st)
+void launch_up(bool trans, const FmmDev &dv, const FactorView &f, const CmDev &c, int col0, int nc, int nt,
+               cudaStream_t st)
 {
-    if (trans) k_cm_up<NT, true><<<resident_grid<k_cm_up<NT, true>>(128), 128, 0, st>>>(dv, f, c, col0, nc);
-    else k_cm_up<NT, false><<<resident_grid<k_cm_up<NT, false>>(128), 128, 0, st>>>(dv, f, c, col0, nc);
+    auto run = [&](auto K, unsigned g) { K<<<g, 128, 0, st>>>(dv, f, c, col0, nc, nt); };
+    if (nt <= 3) {
+        if (trans) run(k_cm_up<3, true>, resident_grid<k_cm_up<3, true>>(128));
+        else run(k_cm_up<3, false>, resident_grid<k_cm_up<3, false>>(128));
+    } else {
+        if (trans) run(k_cm_up<CM_NT, true>, resident_grid<k_cm_up<CM_NT, true>>(128));
+        else run(k_cm_up<CM_NT, false>, resident_grid<k_cm_up<CM_NT, false>>(128));
+    }
 }
 
-template <int NT>
+template <int NTP, int TPW>
 void launch_apply(bool trans, const FmmDev &dv, const FactorView &f, const int64_t *tile_off, const CmDev &c,
-                  const double *X, int64_t ldx, double *Y, int64_t ldy, int col0, int nc, int64_t tiles, cudaStream_t st)
+                  const double *X, int64_t ldx, double *Y, int64_t ldy, int col0, int nc, int nt, int64_t tiles,
+                  cudaStream_t st)
 {
-    const int64_t res = trans ? resident_grid<k_cm_apply<NT, true>>(128) : resident_grid<k_cm_apply<NT, false>>(128);
-    const unsigned g = (unsigned)std::max<int64_t>(1, std::min(tiles, res));
-    if (trans) k_cm_apply<NT, true><<<g, 128, 0, st>>>(dv, f, tile_off, c, X, ldx, Y, ldy, col0, nc);
-    else k_cm_apply<NT, false><<<g, 128, 0, st>>>(dv, f, tile_off, c, X, ldx, Y, ldy, col0, nc);
+    // four CTAs per tile of 64 rows; problems differ in size, so the CTAs are scheduled and not persistent
+    const unsigned g = (unsigned)std::max<int64_t>(1, std::min<int64_t>(4 * tiles, 1 << 20));
+    if (trans) k_cm_apply<NTP, TPW, true><<<g, 128, 0, st>>>(dv, f, tile_off, c, X, ldx, Y, ldy, col0, nc, nt);
+    else k_cm_apply<NTP, TPW, false><<<g, 128, 0, st>>>(dv, f, tile_off, c, X, ldx, Y, ldy, col0, nc, nt);
 }
 
 }  // namespace
@@ -3028,8 +3160,9 @@ superdc_status columns(const FmmPlan &pl, const FactorView &f, int64_t total, co
     c.ccols = ncols;
     SDC_CHECK(sc.get(&c.pos, (size_t)total));
     SDC_CHECK(sc.get(&c.fac, (size_t)total));
-    SDC_CHECK(sc.get(&c.bad, (size_t)f.nprob + 1));
-    SDC_CHECK(sc.get(&c.cmax, (size_t)f.nprob * ncols));
+    const size_t nflag = (size_t)f.nprob + 1 + (size_t)f.nprob * ncols;
+    SDC_CHECK(sc.get(&c.bad, nflag));
+    c.cmax = c.bad + f.nprob + 1;
     SDC_CHECK(sc.get(&c.xf, (size_t)chunks * ntmax * CM_D * 32));
     if (trans) SDC_CHECK(sc.get(&c.lastp, (size_t)tiles * CM_NT * 8));
     if (pl.on) {
@@ -3037,8 +3170,7 @@ superdc_status columns(const FmmPlan &pl, const FactorView &f, int64_t total, co
         SDC_CHECK(sc.get(&c.wf1, (size_t)pl.cap_boxes * ntmax * CM_D * 32));
         SDC_CHECK(sc.get(&c.eb, (size_t)pl.cap_boxes));
     }
-    SDC_CHECK(cudaMemsetAsync(c.bad, 0, ((size_t)f.nprob + 1) * sizeof(int32_t), st));
-    SDC_CHECK(cudaMemsetAsync(c.cmax, 0, (size_t)f.nprob * ncols * sizeof(int32_t), st));
+    SDC_CHECK(cudaMemsetAsync(c.bad, 0, nflag * sizeof(int32_t), st));
     auto gr = [&](int64_t n) {
         return (unsigned)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, (int64_t)sdc_num_sms() * 8));
     };
@@ -3052,22 +3184,28 @@ superdc_status columns(const FmmPlan &pl, const FactorView &f, int64_t total, co
         const int nc = std::min(CM_NT * 8, ncols - c0), nt = (nc + 7) / 8;
         if (trans) PROF_LAUNCH("cauchy", st, k_cm_slice<true><<<gr(rows * nt * 8), 256, 0, st>>>(f, rows, X, ldx, c0, nc, nt, c));
         else PROF_LAUNCH("cauchy", st, k_cm_slice<false><<<gr(rows * nt * 8), 256, 0, st>>>(f, rows, X, ldx, c0, nc, nt, c));
-        if (pl.on) {
-            SrcArgs a{};
-            a.off = f.off; a.mk = f.mk; a.dk = f.dk; a.vhat = f.vhat; a.bnorm = f.bnorm; a.dorg = f.dorg; a.eta = f.eta;
-            a.src = f.src; a.pinv = f.pinv; a.X = X; a.ldx = ldx; a.col0 = c0; a.nc = nc; a.only = c.bad;
-            if (trans) PROF_LAUNCH("fmm_up", st, k_fmm_up<M_CT><<<up_grid<M_CT>(), up_threads<M_CT>(), 0, st>>>(dv, a));
-            else PROF_LAUNCH("fmm_up", st, k_fmm_up<M_CN><<<up_grid<M_CN>(), up_threads<M_CN>(), 0, st>>>(dv, a));
-            auto up = (nt == 1) ? launch_up<1> : (nt == 2) ? launch_up<2> : launch_up<3>;
-            PROF_LAUNCH("fmm_up", st, up(trans, dv, f, c, c0, nc, st));
-        }
-        auto fn = (nt == 1) ? launch_apply<1> : (nt == 2) ? launch_apply<2> : launch_apply<3>;
-        PROF_LAUNCH("cauchy", st, fn(trans, dv, f, tile_off, c, X, ldx, Y, ldy, c0, nc, tiles, st));
+        if (pl.on) PROF_LAUNCH("fmm_up", st, launch_up(trans, dv, f, c, c0, nc, nt, st));
+        auto fn = (nt == 1) ? launch_apply<1, 1> : (nt == 2) ? launch_apply<2, 1> : (nt <= 4) ? launch_apply<4, 1>
+                                                                                              : launch_apply<4, 2>;
+        PROF_LAUNCH("cauchy", st, fn(trans, dv, f, tile_off, c, X, ldx, Y, ldy, c0, nc, nt, tiles, st));
         if (trans) {
             PROF_LAUNCH("cauchy", st, k_cm_last<<<(unsigned)std::min<int64_t>(tiles, (int64_t)sdc_num_sms() * 16), 64, 0,
                                                  st>>>(f, tile_off, c, X, ldx, c0, nc));
             PROF_LAUNCH("cauchy", st, k_cm_lastsum<<<gr(f.nprob * nc * 32), 128, 0, st>>>(f, tile_off, c, Y, ldy, c0, nc));
         }
+    }
+    for (int c0 = 0; c0 < ncols; c0 += CM_BC) {
+        const int nc = std::min(CM_BC, ncols - c0);
+        if (pl.on) {
+            // node weights in FP64 of the problems out of scale (nothing to do as a rule)
+            SrcArgs a{};
+            a.off = f.off; a.mk = f.mk; a.dk = f.dk; a.vhat = f.vhat; a.bnorm = f.bnorm; a.dorg = f.dorg; a.eta = f.eta;
+            a.src = f.src; a.pinv = f.pinv; a.X = X; a.ldx = ldx; a.col0 = c0; a.nc = nc; a.only = c.bad;
+            if (trans) PROF_LAUNCH("fmm_up", st, k_fmm_up<M_CT><<<up_grid<M_CT>(), up_threads<M_CT>(), 0, st>>>(dv, a));
+            else PROF_LAUNCH("fmm_up", st, k_fmm_up<M_CN><<<up_grid<M_CN>(), up_threads<M_CN>(), 0, st>>>(dv, a));
+        }
+        if (trans) PROF_LAUNCH("deflcopy", st, k_cm_rest<true><<<gr(total * nc), 128, 0, st>>>(dv, f, total, tile_off, c, X, ldx, Y, ldy, c0, nc));
+        else PROF_LAUNCH("deflcopy", st, k_cm_rest<false><<<gr(total * nc), 128, 0, st>>>(dv, f, total, tile_off, c, X, ldx, Y, ldy, c0, nc));
     }
     SDC_CHECK(cudaGetLastError());
     return SUPERDC_OK;
