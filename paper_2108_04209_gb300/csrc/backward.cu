@@ -58,16 +58,29 @@ __global__ void k_prep(int64_t nprob, const int64_t *__restrict__ off, int64_t t
     }
 }
 
-// Per kept root k, columns [c0, c0 + nc): u_k and g_k.  Both sums run over the
-// pairs with one factor per pair, s_kl = sum_c (ybar_kc alpha_lc - y_kc beta_lc):
-//   u_k -= 1/2 sum_l s_kl / (lambda_k - lambda_l),
-//   g_k += b_k sum_l s_kl / (lambda_k - lambda_l)^2,
-// so a pair costs 2 nc + 10 FP64 operations instead of 4 nc plus a division, and
-// every column count pays for its own columns only.  A CTA takes 32 targets and
-// its eight warps split the sources (a tile of 128 targets left most SMs idle
-// below 20000 rows).  Measured (GB300, n = 4096 tree adjoint, 7 columns on
-// average, 36 steps): 104.7 -> 11.4 ms; k_bw_dz 19.3 -> 3.9 ms.
-template <int NC>
+// 1 / t rounded to nearest (Markstein, 1990: a reciprocal within an ulp, corrected
+// by its residual)
+__device__ __forceinline__ double rcp_rn(double t)
+{
+    const int e = (__double2hiint(t) >> 20) & 0x7FF;
+    if (e < 31 || e > 2015) return 1.0 / t;
+    const double r = rcp_nr2(t);
+    return fma(r, fma(-t, r, 1.0), r);
+}
+
+// Per kept root k, columns [c0, c0 + nc): u_k and g_k from the four sums P, R,
+// Gamma, Delta of every column, each added up in the order of the sources.  (One
+// factor per pair, s_kl = sum_c (ybar_kc alpha_lc - y_kc beta_lc), takes half of
+// the operations and cancels before it divides, but its g differs from these sums
+// by their own rounding, up to 1e-9 of the result at close pairs.)
+// A CTA takes 32 targets: its eight warps form the reciprocals of 32 sources at a
+// time, then every warp carries one or two sums pairs (P, Gamma or R, Delta of a
+// column) through them, so a pair costs 10 + 4 nc FP64 operations, a chain 2 or 4
+// per source, and every column count pays for its own columns only (a thread
+// with all sums of 8 columns, 128 targets per CTA, left most SMs idle below 20000
+// rows).  Measured (GB300, n = 4096 tree adjoint, 7 columns on average, 36 steps):
+// 104.7 -> 17.8 ms; k_bw_dz 19.3 -> 3.5 ms.
+template <int NU>                       // sum pairs per warp
 __global__ void __launch_bounds__(BW_W * 32)
 k_bw_lamlam(int64_t nprob, const int64_t *__restrict__ off, const int64_t *__restrict__ tile_off,
             const int32_t *__restrict__ mk, const double *__restrict__ dorg, const double *__restrict__ eta,
@@ -75,8 +88,8 @@ k_bw_lamlam(int64_t nprob, const int64_t *__restrict__ off, const int64_t *__res
             const double *__restrict__ Y, int64_t ld, const double *__restrict__ Ybar, int64_t ldb, int c0, int nc,
             double *__restrict__ u, double *__restrict__ g)
 {
-    __shared__ double sK[BW_W][BW_S], sE[BW_W][BW_S], sA[BW_W][NC][BW_S], sB[BW_W][NC][BW_S];
-    __shared__ double red[2][BW_W][BW_T];
+    __shared__ double sK[BW_S], sE[BW_S], sV[2 * BW_C][BW_S], sR[2][BW_S][BW_T];
+    __shared__ double red[2][2 * BW_C][BW_T];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t ntiles = tile_off[nprob];
     for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
@@ -86,59 +99,74 @@ k_bw_lamlam(int64_t nprob, const int64_t *__restrict__ off, const int64_t *__res
         const int k = (int)(tile - tile_off[p]) * BW_T + lane;
         const bool act = k < m;
         const double dKk = act ? dorg[b0 + k] : 0.0, ek = act ? eta[b0 + k] : 0.0;
-        const int64_t rowk = act ? b0 + pinv[b0 + k] : b0;
-        double y[NC], yb[NC];
-#pragma unroll
-        for (int c = 0; c < NC; c++) {
-            y[c] = (act && c < nc) ? -Y[rowk + ld * (c0 + c)] : 0.0;
-            yb[c] = (act && c < nc) ? Ybar[rowk + ldb * (c0 + c)] : 0.0;
-        }
         // exponent of the largest |lambda|: differences above 2^-32 of it are not degenerate
         const double lmax = fmax(fabs(dorg[b0] + eta[b0]), fabs(dorg[b0 + m - 1] + eta[b0 + m - 1]));
         const int emin = ((__double2hiint(lmax) >> 20) & 0x7FF) + 1 - 32;
-        double su = 0.0, sg = 0.0;
-        for (int l0 = warp * BW_S; l0 < m; l0 += BW_W * BW_S) {
+        double s1[NU], s2[NU];
+#pragma unroll
+        for (int i = 0; i < NU; i++) s1[i] = s2[i] = 0.0;
+        for (int l0 = 0; l0 < m; l0 += BW_S) {
             const int cn = min(BW_S, m - l0);
-            __syncwarp();
+            __syncthreads();
             if (lane < cn) {
                 const int64_t s = b0 + l0 + lane;
                 const double bl = bnorm[s];
                 const int64_t row = b0 + pinv[s];
-                sK[warp][lane] = dorg[s];
-                sE[warp][lane] = eta[s];
-#pragma unroll
-                for (int c = 0; c < NC; c++) {
-                    sA[warp][c][lane] = (c < nc) ? bl * Y[row + ld * (c0 + c)] : 0.0;
-                    sB[warp][c][lane] = (c < nc) ? bl * Ybar[row + ldb * (c0 + c)] : 0.0;
+                if (warp == 0) { sK[lane] = dorg[s]; sE[lane] = eta[s]; }
+                for (int c = warp; c < nc; c += BW_W) {
+                    sV[2 * c][lane] = bl * Ybar[row + ldb * (c0 + c)];
+                    sV[2 * c + 1][lane] = bl * Y[row + ld * (c0 + c)];
                 }
             }
-            __syncwarp();
-#pragma unroll 2
-            for (int ll = 0; ll < cn; ll++) {
-                const double dl = (dKk - sK[warp][ll]) + (ek - sE[warp][ll]);     // lambda_k - lambda_l
+            __syncthreads();
+#pragma unroll
+            for (int i = 0; i < BW_S / BW_W; i++) {
+                const int ll = warp * (BW_S / BW_W) + i;
+                if (ll >= cn) break;
+                const double dl = (dKk - sK[ll]) + (ek - sE[ll]);     // lambda_k - lambda_l
                 bool use = l0 + ll != k;
                 // numerically degenerate pairs form one eigenspace: no coupling
                 if (((__double2hiint(dl) >> 20) & 0x7FF) < emin)
-                    use = use && fabs(dl) > 1e-10 * fmax(fabs(dKk + ek), fabs(sK[warp][ll] + sE[warp][ll]));
-                double s = 0.0;
+                    use = use && fabs(dl) > 1e-10 * fmax(fabs(dKk + ek), fabs(sK[ll] + sE[ll]));
+                const double r = use ? rcp_rn(dl) : 0.0;
+                sR[0][ll][lane] = r;
+                sR[1][ll][lane] = r * r;
+            }
+            __syncthreads();
 #pragma unroll
-                for (int c = 0; c < NC; c++) s = fma(yb[c], sA[warp][c][ll], fma(y[c], sB[warp][c][ll], s));
-                const double r = use ? rcp_nr2(dl) : 0.0;
-                const double t = s * r;
-                su += t;
-                sg = fma(t, r, sg);
+            for (int i = 0; i < NU; i++) {
+                const int q = warp + BW_W * i;
+                if (q >= 2 * nc) break;
+                double a = s1[i], b = s2[i];
+#pragma unroll 4
+                for (int ll = 0; ll < cn; ll++) {
+                    const double v = sV[q][ll];
+                    a = fma(-v, sR[0][ll][lane], a);     // sum beta_l/(lambda_l - lambda_k), or of alpha_l
+                    b = fma(v, sR[1][ll][lane], b);
+                }
+                s1[i] = a;
+                s2[i] = b;
             }
         }
-        red[0][warp][lane] = su;
-        red[1][warp][lane] = sg;
+#pragma unroll
+        for (int i = 0; i < NU; i++)
+            if (warp + BW_W * i < 2 * nc) {
+                red[0][warp + BW_W * i][lane] = s1[i];
+                red[1][warp + BW_W * i][lane] = s2[i];
+            }
         __syncthreads();
         if (warp == 0 && act) {
-            double a = 0.0, b = 0.0;
-            for (int w = 0; w < BW_W; w++) { a += red[0][w][lane]; b += red[1][w][lane]; }
-            u[b0 + k] += -0.5 * a;
-            g[b0 + k] += bnorm[b0 + k] * b;
+            const double bk = bnorm[b0 + k];
+            const int64_t row = b0 + pinv[b0 + k];
+            double uu = 0.0, gg = 0.0;
+            for (int c = 0; c < nc; c++) {
+                const double y = Y[row + ld * (c0 + c)], yb = Ybar[row + ldb * (c0 + c)];
+                uu += -0.5 * (y * red[0][2 * c][lane] - yb * red[0][2 * c + 1][lane]);
+                gg += (bk * yb) * red[1][2 * c + 1][lane] - (bk * y) * red[1][2 * c][lane];
+            }
+            u[b0 + k] += uu;
+            g[b0 + k] += gg;
         }
-        __syncthreads();
     }
 }
 
@@ -278,8 +306,7 @@ superdc_status r1_backward_fv(const FactorView &f, int64_t total, const double *
         if (s == SUPERDC_OK) s = cauchy_apply_N(f, total, Ybar, ldy, X_bar, ldxb, ncols, st);
         for (int c0 = 0; c0 < ncols && s == SUPERDC_OK; c0 += BW_C) {
             const int nc = std::min(BW_C, ncols - c0);
-            auto fn = nc <= 1 ? k_bw_lamlam<1> : nc <= 2 ? k_bw_lamlam<2> : nc <= 4 ? k_bw_lamlam<4>
-                    : nc <= 6 ? k_bw_lamlam<6> : k_bw_lamlam<BW_C>;
+            auto fn = 2 * nc <= BW_W ? k_bw_lamlam<1> : k_bw_lamlam<2 * BW_C / BW_W>;
             PROF_LAUNCH("bw_lamlam", st, fn<<<grid, BW_W * 32, 0, st>>>(
                 f.nprob, f.off, tile_off, f.mk, f.dorg, f.eta, f.bnorm, f.pinv, Y, total, Ybar, ldy, c0, nc, u, g));
         }
