@@ -213,11 +213,12 @@ constexpr int LEAF_T = 256;
 // Then implicit QL iterations with the usual shift from the leading 2x2 block
 // on (d, e).  A QL sweep is one chain of dependent scalar steps, and on this
 // GPU a scalar FP64 chain is slow, so the chains run in parallel:
-//   large leaves (one CTA per SM): k_leaf_ql runs one leaf per lane and
+//   large leaves (one CTA per SM), and small ones in great number (six per
+//                 SM): k_leaf_ql runs one leaf per lane and
 //                 records every sweep's rotations; k_leaf_rot applies them to
 //                 the rows of Q (each row independently, a leaf's rows split
 //                 over several CTAs), k_leaf_out sorts and emits;
-//   small leaves: k_leaf_qlcta, in each leaf's CTA, thread 0 computes one
+//   other leaves: k_leaf_qlcta, in each leaf's CTA, thread 0 computes one
 //                 sweep while the other warps apply the previous one, and
 //                 several CTAs share an SM.
 // Outputs: eigenvalues ascending (ties by index), Q columns in that order,
@@ -1423,7 +1424,12 @@ superdc_status superdc_eig_plan(const superdc_hss *h, const superdc_opts *opts, 
     EIG_CHECK(dalloc(&w.eq, n, &f->slabs));
     // leaf eigensolver layout and kernel attributes (set here, not in the run)
     const size_t mm = (size_t)h->mmax;
-    w.leaf_batched = mm >= 96;
+    // small leaves chase in their own CTAs until a sub-core has two chains to issue
+    // (an FP64 instruction holds it for 64 cycles, whatever the lanes): then a warp
+    // carries several leaves, one per lane.  GB300, own CTA / lane: 512 leaves of 32
+    // rows 1.60 / 1.74 ms, of 80 11.3 / 11.9; 1024 of 48 7.2 / 5.6, of 64 12.3 / 10.0;
+    // 2048 of 32 5.8 / 3.4
+    w.leaf_batched = mm >= 96 || h->nleaves >= 6 * sdc_num_sms();
     w.smem1 = (mm * (mm | 1) + std::max(mm * (size_t)r, mm)) * sizeof(double);
     w.smem2 = 2 * mm * 32 * sizeof(double);
     // leaves per warp of the QL chase: about one warp per scheduler (4 per SM)
@@ -1672,7 +1678,7 @@ superdc_status superdc_eig_run(superdc_eigfact *f, cudaStream_t st, double *lamb
                 a.o.fmm_used = S.fmm + q;
                 a.o.unshifted = opts->shifted ? 0 : 1;
                 const int c = ctot - (j + 1);
-                // the step's FMM plan (tree, near lists, M2L kernel matrices)
+                // the step's FMM plan (tree, near lists, interaction masks)
                 // also serves the Cauchy-like update of the remaining columns
                 FmmPlan keep;
                 if (opts->batching && c > 0 && c <= 24) { a.keep = &keep; a.keep_width = c; }
