@@ -63,7 +63,9 @@ typedef struct {
                              FMM with local shifting (Sections 4.1.2, 4.2.2, 4.3) for the secular
                              sweeps, zhat, b and the Cauchy-like applications; smaller ones the
                              direct tiled evaluator.  0 = the library default (the crossover
-                             measured on GB300), < 0 = direct evaluator only */
+                             measured on GB300: 512; in eigendecompositions and applications
+                             whose levels have fewer than 128 rows per SM 1536), < 0 = direct
+                             evaluator only */
     int32_t shifted;      /* 1 (default): every secular root is solved and stored relative to its
                              nearest pole (the local shifting of Section 4.2, eqs. (4.13)-(4.21));
                              0: ablation, the roots are solved and stored as plain positions, so

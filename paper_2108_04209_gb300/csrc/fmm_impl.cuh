@@ -3,9 +3,8 @@
 // Geometry.  The kept poles d_0 < ... < d_{m-1} of a problem and the targets
 // (roots x_k in (d_k, d_{k+1}), eigenvalues lambda_j, or the poles themselves)
 // interlace (eq. (4.4)), so one index-based binary tree serves both: a leaf
-// box holds B consecutive indices (32 or 64; this file is compiled once per
-// box size, fmm32.cu and fmm64.cu), so d_k and x_k of the same k always share
-// a box (the paper's first design point), and every box carries the interval
+// box holds B = 32 consecutive indices (fmm32.cu), so d_k and x_k of the same k
+// always share a box (the paper's first design point), and every box carries the interval
 // [d_{i0}, d_{i1}] of its points (the last box ends at d_{m-1}).  The index
 // split adapts the boxes to clustered spectra (second design point); whether
 // two boxes interact through expansions is decided geometrically: boxes S, T
@@ -20,16 +19,18 @@
 // far from it, direct sums over the leaf boxes next to it) or are spread over
 // the leaf boxes; as a source it is added directly to every target.
 //
-// Expansions.  Chebyshev interpolation with FMM_P first-kind nodes per box:
-// source moments M_n = sum_j w_j T_n(u_j) of the leaf boxes, node weights
-// W_q = sum_j w_j L_q(u_j) from the moments, parents' moments exactly from
-// the children's weights (T_n(alpha u + beta) has degree n < P; upward
-// pass); every box
-// receives the kernel sums of its interaction list (children of its parent's
-// near list that are admissible to it) at its own Chebyshev nodes (M2L), the
-// parents' fields are interpolated down the tree (L2L), and on the leaves the
-// field becomes Chebyshev coefficients evaluated at the targets by Clenshaw.
-// Work is O(m P^2 / B) for the far field plus O(m B) for the near field.
+// Expansions.  Chebyshev interpolation with FMM_P first-kind nodes per box: node
+// weights W_q = sum_j w_j L_q(u_j) of the leaf boxes, parents' weights from the
+// children's nodes (upward pass: k_fmm_up1 for one column, k_cm_up for blocks of
+// columns, k_fmm_up for problems out of the split arithmetic's scale).  Every leaf
+// box then sums the node weights of the boxes in the interaction lists (children of
+// the parent's near list that are admissible) of itself and of its ancestors: at its
+// own Chebyshev nodes for the one-column fields (k_fmm_far), whose coefficients are
+// evaluated at the targets; at the targets themselves for blocks of columns
+// (k_cm_apply).  There is no translation between boxes and no downward pass: in split
+// FP32 arithmetic and on the tensor cores a node sum costs less than reading or
+// forming a translation matrix.  Work is O(m P log m) for the far field plus O(m B)
+// for the near field.
 //
 // Triangularity.  A far box lies entirely to the left or right of the target
 // box in index order, so its sums go to the lower (psi, C_L w, S_L w) or the
@@ -44,7 +45,7 @@
 // Because the poles and weights of a secular equation do not change during
 // the iteration and every root stays inside its bracket, the far-field
 // expansions on the leaf boxes' (fixed) intervals are computed once per
-// problem; each sweep costs a near-field pass plus one Clenshaw evaluation.
+// problem; each sweep costs a near-field pass plus one series evaluation.
 #include <algorithm>
 #include <mutex>
 #include "common.cuh"
@@ -813,7 +814,8 @@ enum { K_SEC = 0, K_1 = 1, K_2 = 2, K_1N = 3, K_LOG = 4 };
 // Measured (GB300, 4096 problems of 32..2048 poles; translations, then down):
 // secular 6.2 + 2.1 -> 1.4 ms, b 3.4 + 2.1 -> 1.5, Loewner 5.1 + 2.1 -> 1.5; the
 // sweeps read one FP64 and three FP32 series instead of four FP64 ones, 10.1 ->
-// 6.8 ms (tail pass 2.3 -> 1.4).  zhat's error falls from 5.4e-13 to 1.6e-13 (4000 poles).
+// 6.8 ms (tail pass 2.3 -> 1.4; with the mixed series below 5.2 and 0.9).  zhat's error
+// falls from 5.4e-13 to 1.6e-13 (4000 poles).
 // ---------------------------------------------------------------------------
 
 // positions of every box's Chebyshev nodes as split parts
@@ -841,9 +843,9 @@ constexpr int FAR_TAKE = 4;       // list entries taken per level and round
 
 // Series of a leaf box in mixed precision: sum_{n < LOWN} a_n u^n (monomials, FP64)
 // plus sum_{n >= LOWN} c_n T_n(u) (Chebyshev, single precision).  A box of the
-// lists is at least its own width away, so c_n falls as 5.8^-n: the single
-// precision part is below 2^-30 of the sum and its rounding below 2^-52; the
-// monomials' amplification, at most 2.4^n, is below that decay.  11 FP64
+// lists is at least 3/4 of the larger width away, so c_n falls as 4.8^-n
+// (FMM_KAPPA): the single precision part is below 2^-27 of the sum and its rounding
+// below 2^-51; the monomials' amplification, at most 2.4^n, is below that decay.  11 FP64
 // instructions per evaluation instead of 43 (Clenshaw over all of them): 180
 // instead of 690 cycles of the SM for a warp.
 constexpr int LOWN = 12;
