@@ -2450,7 +2450,6 @@ k_cm_apply(FmmDev pl, FactorView f, const int64_t *__restrict__ tile_off, CmDev 
     constexpr int NS = 4 / NTP;                          // warps that share a column tile
     __shared__ CmFrag sA[4];
     __shared__ int2 list[32 * CM_TAKE];                  // far boxes: index, exponent of its weights
-    __shared__ int lim[32 * CM_TAKE];                    // and of its largest term: weights over distance
     __shared__ int64_t s_pst[32];                        // per level: the list's start, the target's ancestor
     __shared__ int s_lb[32];
     __shared__ double s_lo[32], s_hi[32];
@@ -2636,8 +2635,7 @@ k_cm_apply(FmmDev pl, FactorView f, const int64_t *__restrict__ tile_off, CmDev 
                     const int e = c.eb[gbx + S];
                     const double gap = fmax(s_lo[q.y] - pl.bhi[gbx + S], pl.blo[gbx + S] - s_hi[q.y]);
                     list[t] = make_int2(S, e);
-                    lim[t] = e > -4000 ? e - (ff_exp(gap) - 1023 + fs.kk) : -8000;
-                    if (e > -4000) atomicMax(&s_ET, lim[t]);
+                    if (e > -4000) atomicMax(&s_ET, e - (ff_exp(gap) - 1023 + fs.kk));
                 }
                 __syncthreads();
                 const int ET = s_ET;
@@ -2645,9 +2643,7 @@ k_cm_apply(FmmDev pl, FactorView f, const int64_t *__restrict__ tile_off, CmDev 
                 far_src += total * P;
                 for (int i = 0; i < total; i += 4) {
                     const int u = i + warp;
-                    // else its largest term is below the last digit (the weights alone do not
-                    // say so: the distances of one round differ by the spread over the gaps, 2^41)
-                    if (u < total && lim[u] - ET >= -62) {
+                    if (u < total && list[u].y - ET >= -62) {    // else below the last digit
                         const float sc = TRANS ? pow2f(list[u].y - ET) : -pow2f(list[u].y - ET);
                         const ff_f4 *np = pl.npos + (gbx + list[u].x) * P;
                         // nodes 0..15, then 16..21
@@ -2676,7 +2672,7 @@ k_cm_apply(FmmDev pl, FactorView f, const int64_t *__restrict__ tile_off, CmDev 
                     }
                     boxes_sync();
                     for (int v = grp; v < 4 && i + v < total; v += NS)
-                        if (lim[i + v] - ET >= -62) {
+                        if (list[i + v].y - ET >= -62) {
                             const int64_t at = (gbx + list[i + v].x) * nt * CM_D * 32;
                             mult16(v, 0, c.wf0 + at);
                             mult8(v, c.wf1 + at);
@@ -2748,9 +2744,8 @@ k_cm_apply(FmmDev pl, FactorView f, const int64_t *__restrict__ tile_off, CmDev 
         collect(ns[0], ns[1]);
         if (grp > 0 || tl >= nt) continue;
         // ---- FP64 terms: lane r < 16 has row r's coefficients
-        // (a row of -1: no such term; 0 times another problem's row could be NaN)
         double g0 = 0.0, g1 = 0.0, g2 = 0.0;
-        int64_t r0 = -1, r1 = -1, r2 = -1;
+        int64_t r0 = 0, r1 = 0, r2 = 0;
         {
             const int r = min(t0 + (lane & 15), tend - 1);
             if (TRANS) {
@@ -2789,11 +2784,8 @@ k_cm_apply(FmmDev pl, FactorView f, const int64_t *__restrict__ tile_off, CmDev 
                     v = cm >= 0x7FF ? nan("") : cm > 30 ? v * ff_pow2(min(cm - 1022, 1023)) * (cm > 2045 ? 2.0 : 1.0)
                                                         : ldexp(v, cm - 1022);
                     const double *xc = X + (int64_t)(col0 + col) * ldx;
-                    if (q0 >= 0) v = fma(u0, xc[q0], v);
-                    if (!TRANS) {
-                        v = fma(u2, xc[q2], v);
-                        if (q1 >= 0) v = fma(u1, xc[q1], v);
-                    }
+                    v = fma(u0, xc[q0], v);
+                    if (!TRANS) v = fma(u1, xc[q1], fma(u2, xc[q2], v));
                     Y[row + (int64_t)(col0 + col) * ldy] = sc * v;
                 }
         }
