@@ -2450,6 +2450,7 @@ k_cm_apply(FmmDev pl, FactorView f, const int64_t *__restrict__ tile_off, CmDev 
     constexpr int NS = 4 / NTP;                          // warps that share a column tile
     __shared__ CmFrag sA[4];
     __shared__ int2 list[32 * CM_TAKE];                  // far boxes: index, exponent of its weights
+    __shared__ int lim[32 * CM_TAKE];                    // and of its largest term: weights over distance
     __shared__ int64_t s_pst[32];                        // per level: the list's start, the target's ancestor
     __shared__ int s_lb[32];
     __shared__ double s_lo[32], s_hi[32];
@@ -2635,7 +2636,8 @@ k_cm_apply(FmmDev pl, FactorView f, const int64_t *__restrict__ tile_off, CmDev 
                     const int e = c.eb[gbx + S];
                     const double gap = fmax(s_lo[q.y] - pl.bhi[gbx + S], pl.blo[gbx + S] - s_hi[q.y]);
                     list[t] = make_int2(S, e);
-                    if (e > -4000) atomicMax(&s_ET, e - (ff_exp(gap) - 1023 + fs.kk));
+                    lim[t] = e > -4000 ? e - (ff_exp(gap) - 1023 + fs.kk) : -8000;
+                    if (e > -4000) atomicMax(&s_ET, lim[t]);
                 }
                 __syncthreads();
                 const int ET = s_ET;
@@ -2643,7 +2645,9 @@ k_cm_apply(FmmDev pl, FactorView f, const int64_t *__restrict__ tile_off, CmDev 
                 far_src += total * P;
                 for (int i = 0; i < total; i += 4) {
                     const int u = i + warp;
-                    if (u < total && list[u].y - ET >= -62) {    // else below the last digit
+                    // else its largest term is below the last digit (the weights alone do not
+                    // say so: the distances of one round differ by the spread over the gaps, 2^41)
+                    if (u < total && lim[u] - ET >= -62) {
                         const float sc = TRANS ? pow2f(list[u].y - ET) : -pow2f(list[u].y - ET);
                         const ff_f4 *np = pl.npos + (gbx + list[u].x) * P;
                         // nodes 0..15, then 16..21
@@ -2672,7 +2676,7 @@ k_cm_apply(FmmDev pl, FactorView f, const int64_t *__restrict__ tile_off, CmDev 
                     }
                     boxes_sync();
                     for (int v = grp; v < 4 && i + v < total; v += NS)
-                        if (list[i + v].y - ET >= -62) {
+                        if (lim[i + v] - ET >= -62) {
                             const int64_t at = (gbx + list[i + v].x) * nt * CM_D * 32;
                             mult16(v, 0, c.wf0 + at);
                             mult8(v, c.wf1 + at);

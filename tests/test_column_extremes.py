@@ -1,0 +1,59 @@
+"""Blocks of columns through the factors of rank-one steps where a column's
+entries or the poles differ by many orders of magnitude: graded columns over a
+tight cluster.
+
+Reference and bound: the dense Qhat of the step's own outputs, (8 eps m + 1e-13
+sqrt(m)) max|x| per entry (test_column_blocks)."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+import paper_2108_04209_gb300 as sdc  # noqa: E402
+from tests import parity as P  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+
+
+def _factor(d, z, tau):
+    """Factor of a batch (lists of poles and weights) and its dense Qhat per problem."""
+    offs = np.concatenate([[0], np.cumsum([len(x) for x in d])]).astype(np.int64)
+    o, dd, zz = (torch.from_numpy(a).cuda() for a in (offs, np.concatenate(d), np.concatenate(z)))
+    fact = sdc.secular_batched(o, dd, zz, 1.0, sdc.default_opts(tau=tau))
+    host = {k: (v.cpu().numpy() if v is not None else None) for k, v in fact.items()}
+    g = [P.gpu_problem(host, offs, p) for p in range(len(d))]
+    return offs, o, fact, g, [P.dense_qhat(x) for x in g]
+
+
+def _apply(o, fact, X, trans, fmm):
+    return sdc.apply_rank1(o, fact, torch.from_numpy(X).cuda(), trans=trans,
+                           opts=sdc.default_opts(fmm_min_m=fmm)).cpu().numpy()
+
+
+def _tol(m, x):
+    return (8 * 2.0 ** -52 * m + 1e-13 * np.sqrt(m)) * np.abs(x).max(axis=0)
+
+
+@pytest.mark.parametrize("fmm", [-1, 256], ids=["direct", "tree"])
+@pytest.mark.parametrize("gap", [-40, -36, -30])
+def test_graded_columns_over_a_tight_cluster(gap, fmm):
+    """512 of 1024 poles a gap of 2^-30 to 2^-40 of the spread apart, boxes of the
+    cluster with entries 2^-20 to 2^-45 of the column's largest: their far boxes
+    are near in position, so small weights still count."""
+    rng = np.random.default_rng(5)
+    m = 1024
+    d = np.sort(np.concatenate([0.25 + np.arange(512) * 2.0 ** gap, rng.uniform(0.3, 1.0, 511), [1.25]]))
+    z = rng.standard_normal(m) / np.sqrt(m)
+    offs, o, fact, g, Q = _factor([d], [z], 1e-30)
+    assert g[0]["mk"] == m
+    X = np.zeros((m, 12))
+    for c in range(12):
+        X[256:288, c] = 1.0                       # one box of the cluster, another far from it below
+        X[384:416, c] = 2.0 ** -(20 + 2.25 * c)
+        if c >= 6:
+            X[:, c] = np.where(np.arange(m) < 300, X[:, c], 2.0 ** -(10 + 3 * c) * rng.standard_normal(m))
+    for trans in (True, False):
+        Y = _apply(o, fact, X, trans, fmm)
+        ref = (Q[0].T if trans else Q[0]) @ X
+        err = np.abs(Y - ref)
+        assert np.all(err <= _tol(m, X)), (trans, err.max())
