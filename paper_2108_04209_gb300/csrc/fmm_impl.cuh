@@ -2748,8 +2748,9 @@ k_cm_apply(FmmDev pl, FactorView f, const int64_t *__restrict__ tile_off, CmDev 
         collect(ns[0], ns[1]);
         if (grp > 0 || tl >= nt) continue;
         // ---- FP64 terms: lane r < 16 has row r's coefficients
+        // (a row of -1: no such term; 0 times another problem's row could be NaN)
         double g0 = 0.0, g1 = 0.0, g2 = 0.0;
-        int64_t r0 = 0, r1 = 0, r2 = 0;
+        int64_t r0 = -1, r1 = -1, r2 = -1;
         {
             const int r = min(t0 + (lane & 15), tend - 1);
             if (TRANS) {
@@ -2788,8 +2789,11 @@ k_cm_apply(FmmDev pl, FactorView f, const int64_t *__restrict__ tile_off, CmDev 
                     v = cm >= 0x7FF ? nan("") : cm > 30 ? v * ff_pow2(min(cm - 1022, 1023)) * (cm > 2045 ? 2.0 : 1.0)
                                                         : ldexp(v, cm - 1022);
                     const double *xc = X + (int64_t)(col0 + col) * ldx;
-                    v = fma(u0, xc[q0], v);
-                    if (!TRANS) v = fma(u1, xc[q1], fma(u2, xc[q2], v));
+                    if (q0 >= 0) v = fma(u0, xc[q0], v);
+                    if (!TRANS) {
+                        v = fma(u2, xc[q2], v);
+                        if (q1 >= 0) v = fma(u1, xc[q1], v);
+                    }
                     Y[row + (int64_t)(col0 + col) * ldy] = sc * v;
                 }
         }

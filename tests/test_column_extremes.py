@@ -1,6 +1,6 @@
 """Blocks of columns through the factors of rank-one steps where a column's
 entries or the poles differ by many orders of magnitude: graded columns over a
-tight cluster.
+tight cluster, non-finite entries.
 
 Reference and bound: the dense Qhat of the step's own outputs, (8 eps m + 1e-13
 sqrt(m)) max|x| per entry (test_column_blocks)."""
@@ -57,3 +57,25 @@ def test_graded_columns_over_a_tight_cluster(gap, fmm):
         ref = (Q[0].T if trans else Q[0]) @ X
         err = np.abs(Y - ref)
         assert np.all(err <= _tol(m, X)), (trans, err.max())
+
+
+@pytest.mark.parametrize("bad", [np.nan, np.inf])
+@pytest.mark.parametrize("ncols", [3, 40])
+def test_first_row_stays_in_its_problem(bad, ncols):
+    """A NaN or infinity in the block's row 0 reaches the first problem's rows of
+    its column only, every row of the others is as without it."""
+    rng = np.random.default_rng(6)
+    sizes = (33, 1, 2, 40, 700)
+    d = [np.sort(rng.uniform(-1, 1, m)) for m in sizes]
+    z = [rng.standard_normal(m) / np.sqrt(m) for m in sizes]
+    offs, o, fact, g, Q = _factor(d, z, 1e-30)
+    X = rng.standard_normal((int(offs[-1]), ncols))
+    X[0, 1] = bad
+    for fmm in (-1, 256):
+        for trans in (True, False):
+            Y = _apply(o, fact, X, trans, fmm)
+            assert not np.any(np.isfinite(Y[:33, 1]))
+            for p in range(1, len(sizes)):
+                x, y = X[offs[p]:offs[p + 1]], Y[offs[p]:offs[p + 1]]
+                ref = (Q[p].T if trans else Q[p]) @ x
+                assert np.all(np.abs(y - ref) <= _tol(sizes[p], x)), (trans, p)
