@@ -2004,7 +2004,7 @@ __device__ __forceinline__ void cm_digits(double y, unsigned short *out)
 struct CmDev {
     ff_f4 *pos, *fac;            // per slot: source position, source factor (three floats)
     int32_t *bad;                // per problem, then whether any is
-    int32_t *cmax;               // per (problem, column of the call): biased exponent of max |x|
+    int32_t *cmax;               // per (problem, column of the call): biased exponent of max |x| of the kept rows
     int64_t ccols;               // columns of the call (stride of cmax)
     uint2 *xf;                   // column digits in mma order: [chunk][tile][digit][lane]
     uint2 *wf0;                  // node weights' digits: nodes 0..15 [box][tile][digit][lane]
@@ -2042,6 +2042,10 @@ __global__ void k_cm_prep(FactorView f, int64_t total, CmDev c)
     }
 }
 
+// Scale of every column over its problem's kept rows (a deflated row passes through
+// unchanged, whatever its size).  A problem with a non-finite entry takes the FP64
+// loops: the digits of one column share the boxes' scales with the others.
+template <bool TRANS>
 __global__ void k_cm_colmax(FactorView f, int64_t total, const double *__restrict__ X, int64_t ldx, int ncols,
                             CmDev c)
 {
@@ -2053,16 +2057,23 @@ __global__ void k_cm_colmax(FactorView f, int64_t total, const double *__restric
         int e = 0;
         if (x >= f.off[0] && x < f.off[f.nprob]) {
             p = sdc_upper_index(f.off, f.nprob, x);
-            e = ff_exp(X[x + (int64_t)col * ldx]);
+            const int64_t b0 = f.off[p];
+            if (x - b0 < f.mk[p]) e = ff_exp(X[b0 + (TRANS ? f.src[x] : f.pinv[x]) + (int64_t)col * ldx]);
         }
         // one atomic per run of lanes with the same problem and column
         const unsigned grp = __match_any_sync(__activemask(), p * ncols + col);
         const int mx = __reduce_max_sync(grp, e);
-        if (p >= 0 && (int)(threadIdx.x & 31) == __ffs(grp) - 1 && mx > 0) atomicMax(&c.cmax[p * c.ccols + col], mx);
+        if (p >= 0 && (int)(threadIdx.x & 31) == __ffs(grp) - 1 && mx > 0) {
+            atomicMax(&c.cmax[p * c.ccols + col], mx);
+            if (mx == 0x7FF) {
+                c.bad[p] = 1;
+                c.bad[f.nprob] = 1;
+            }
+        }
     }
 }
 
-// 2^-e x with |x| < 2^e for every row of the problem (e from the biased exponent)
+// 2^-e x with |x| < 2^e for every kept row of the problem (e from the biased exponent)
 __device__ __forceinline__ int cm_exp(const CmDev &c, int64_t p, int col) { return c.cmax[p * c.ccols + col] - 1022; }
 
 // digits of the columns [col0, col0 + nc) of the kept slots; row: src (TRANS) or pinv
@@ -2786,8 +2797,7 @@ k_cm_apply(FmmDev pl, FactorView f, const int64_t *__restrict__ tile_off, CmDev 
                     if (col >= nc) continue;
                     const int cm = c.cmax[p * c.ccols + col0 + col];
                     double v = y[t][2 * h + q];
-                    v = cm >= 0x7FF ? nan("") : cm > 30 ? v * ff_pow2(min(cm - 1022, 1023)) * (cm > 2045 ? 2.0 : 1.0)
-                                                        : ldexp(v, cm - 1022);
+                    v = cm > 30 ? v * ff_pow2(min(cm - 1022, 1023)) * (cm > 2045 ? 2.0 : 1.0) : ldexp(v, cm - 1022);
                     const double *xc = X + (int64_t)(col0 + col) * ldx;
                     if (q0 >= 0) v = fma(u0, xc[q0], v);
                     if (!TRANS) {
@@ -3187,7 +3197,8 @@ superdc_status columns(const FmmPlan &pl, const FactorView &f, int64_t total, co
     const int64_t rows = chunks * 16;
     if (trans) PROF_LAUNCH("cauchy", st, k_cm_prep<true><<<gr(total), 256, 0, st>>>(f, total, c));
     else PROF_LAUNCH("cauchy", st, k_cm_prep<false><<<gr(total), 256, 0, st>>>(f, total, c));
-    PROF_LAUNCH("cauchy", st, k_cm_colmax<<<gr(total * ncols), 256, 0, st>>>(f, total, X, ldx, ncols, c));
+    if (trans) PROF_LAUNCH("cauchy", st, k_cm_colmax<true><<<gr(total * ncols), 256, 0, st>>>(f, total, X, ldx, ncols, c));
+    else PROF_LAUNCH("cauchy", st, k_cm_colmax<false><<<gr(total * ncols), 256, 0, st>>>(f, total, X, ldx, ncols, c));
     FmmDev dv = pl.dv;
     if (!pl.on) dv = FmmDev{};
     for (int c0 = 0; c0 < ncols; c0 += CM_NT * 8) {

@@ -1,6 +1,7 @@
 """Blocks of columns through the factors of rank-one steps where a column's
 entries or the poles differ by many orders of magnitude: graded columns over a
-tight cluster, non-finite entries.
+tight cluster, non-finite entries,
+and deflated rows of any value.
 
 Reference and bound: the dense Qhat of the step's own outputs, (8 eps m + 1e-13
 sqrt(m)) max|x| per entry (test_column_blocks)."""
@@ -79,3 +80,64 @@ def test_first_row_stays_in_its_problem(bad, ncols):
                 x, y = X[offs[p]:offs[p + 1]], Y[offs[p]:offs[p + 1]]
                 ref = (Q[p].T if trans else Q[p]) @ x
                 assert np.all(np.abs(y - ref) <= _tol(sizes[p], x)), (trans, p)
+
+
+@pytest.mark.parametrize("fmm", [-1, 256], ids=["direct", "tree"])
+@pytest.mark.parametrize("value", [np.nan, np.inf, 1e12, 1e300])
+def test_deflated_rows_keep_to_themselves(value, fmm):
+    """The identity part of the factor: a deflated row passes its entry on unchanged
+    and has no part in the kept rows, whose error stays relative to the kept
+    entries."""
+    rng = np.random.default_rng(7)
+    sizes = (40, 900)
+    d = [np.sort(rng.uniform(-1, 1, m)) for m in sizes]
+    z = [rng.standard_normal(m) / np.sqrt(m) for m in sizes]
+    for v in z:
+        v[5::11] = 0.0                            # deflated without a rotation: rows 5, 16, ...
+    offs, o, fact, g, Q = _factor(d, z, 1e-30)
+    n = int(offs[-1])
+    X0 = rng.standard_normal((n, 9))
+    for trans in (True, False):
+        X = X0.copy()
+        gone = np.zeros(n, bool)                  # output rows of the deflated slots
+        for p, q in enumerate(g):
+            assert q["mk"] == sizes[p] - len(range(5, sizes[p], 11))
+            slots = np.arange(q["mk"], q["m"])
+            merged = np.argsort(q["perm"])[slots]
+            X[offs[p] + (q["src"][slots] if trans else merged), 3] = value
+            gone[offs[p] + (merged if trans else q["src"][slots])] = True
+        Y = _apply(o, fact, X, trans, fmm)
+        assert np.array_equal(Y[gone, 3], np.full(gone.sum(), value), equal_nan=True)
+        for p, q in enumerate(Q):
+            s = slice(int(offs[p]), int(offs[p + 1]))
+            ref = (q.T if trans else q) @ X0[s]
+            keep = ~gone[s]
+            err = np.abs(Y[s] - ref)[keep]
+            assert np.all(err <= _tol(sizes[p], X0[s])), (trans, p, err.max())
+
+
+@pytest.mark.parametrize("fmm", [-1, 256], ids=["direct", "tree"])
+def test_non_finite_column_leaves_the_others(fmm):
+    """Columns beside one with a NaN or an infinity are those of the block without
+    it to rounding: both sides sum the same terms (near, or the same nodes), each
+    with 4 eps |C_ij| |x_i|, rows of Qhat have norm one, so 16 eps sqrt(m) max|x|
+    covers both; an infinite entry gives signed infinities."""
+    rng = np.random.default_rng(8)
+    m = 1537
+    d, z = np.sort(rng.uniform(-1, 1, m)), rng.standard_normal(m) / np.sqrt(m)
+    offs, o, fact, g, Q = _factor([d], [z], 1e-30)
+    X = rng.standard_normal((m, 9))
+    ok = [c for c in range(9) if c != 4]
+    for trans in (True, False):
+        ref = _apply(o, fact, X, trans, fmm)
+        Qt = Q[0].T if trans else Q[0]
+        for bad in (np.nan, np.inf):
+            Z = X.copy()
+            Z[70, 4] = bad
+            Y = _apply(o, fact, Z, trans, fmm)
+            err = np.abs(Y - ref)[:, ok].max()
+            assert err <= 16 * 2.0 ** -52 * np.sqrt(m) * np.abs(X).max(), (trans, bad, err)
+            if fmm < 0 and bad == np.inf:
+                assert np.array_equal(Y[:, 4], np.sign(Qt[:, 70]) * np.inf)
+            else:
+                assert not np.any(np.isfinite(Y[:, 4]))
