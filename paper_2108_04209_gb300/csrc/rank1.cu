@@ -50,6 +50,15 @@ constexpr int DEFL_BIG = 128;     // problems larger than this deflate with more
 // ---------------------------------------------------------------------------
 constexpr int DB_T = 512;         // threads per problem; 1024 when a batch has fewer problems than SMs
 constexpr int WALK_CAP = 64;      // speculative steps of one chain before one thread finishes it
+constexpr int ORDER_PHASES = 32;  // exchange phases on the deflated values before they are merge-sorted
+
+// doubles ordered as integers: as <, with both zeros equal and every NaN at an end
+// (a total order, so that equal keys and indexes keep a permutation)
+__device__ __forceinline__ long long order_key(double v)
+{
+    const long long b = __double_as_longlong(v);
+    return (b << 1) == 0 ? 0 : ff_ord(v);
+}
 
 // sum of cnt over the warps before this one; *total over all (every thread calls)
 template <int T>
@@ -289,13 +298,21 @@ k_deflate(int64_t nprob, const int64_t *__restrict__ off, const double *__restri
         o.mk[p] = mk;
         o.ngiv[p] = s_ng;
     }
-    // D: deflated values sorted by (value, index): they are in index order and
-    // out of order only inside tau-sized intervals, so a few odd-even
-    // exchanges (of values strictly out of order: ties keep their order) do
-    if (m - mk >= 2) {
-        for (int idle = 0, ph = 0; idle < 2; ph ^= 1) {
+    // D: deflated values sorted by (value, index).  They are in index order; only
+    // a rotated value can be out of order, in a cluster by a few places, which
+    // odd-even exchanges (of values strictly out of order: ties keep their order)
+    // settle in as many phases.  But a rotation next to a much larger weight moves
+    // its value across all entries up to the next survivor: what is not in order
+    // after ORDER_PHASES is merge-sorted, a thread per entry placing it by binary
+    // search in the neighbouring run, with the copies wd and surv, read for the last
+    // time above, as the other buffer.  (GB300, 30000 entries, one value moved
+    // across all of them: 137 ms by exchanges alone, @@ ms now.)
+    const int nd = m - mk;
+    if (nd >= 2) {
+        int idle = 0;
+        for (int ph = 0; idle < 2 && ph < ORDER_PHASES; ph++) {
             bool sw = false;
-            for (int q = mk + ph + 2 * tid; q + 1 < m; q += 2 * T) {
+            for (int q = mk + (ph & 1) + 2 * tid; q + 1 < m; q += 2 * T) {
                 const double v0 = o.dk[b0 + q], v1 = o.dk[b0 + q + 1];
                 if (v0 > v1) {
                     const int s0 = o.src[b0 + q], s1 = o.src[b0 + q + 1];
@@ -307,6 +324,41 @@ k_deflate(int64_t nprob, const int64_t *__restrict__ off, const double *__restri
                 }
             }
             idle = __syncthreads_or(sw) ? 0 : idle + 1;
+        }
+        if (idle < 2) {
+            double *va = o.dk + b0 + mk, *vb = wd + b0;
+            int32_t *ia = o.src + b0 + mk, *ib = surv + b0;
+            for (int lw = 0; lw < 31 && (1 << lw) < nd; lw++) {
+                const int w = 1 << lw;
+                for (int i = tid; i < nd; i += T) {
+                    const int r0 = i & ~(w - 1);                       // this entry's run, and its neighbour's
+                    const int q0 = min(nd, r0 ^ w), q1 = q0 + min(w, nd - q0);
+                    const double v = va[i];
+                    const int s = ia[i];
+                    const long long k = order_key(v);
+                    int lo = q0, hi = q1;
+                    while (lo < hi) {
+                        const int mid = (lo + hi) >> 1;
+                        const long long km = order_key(va[mid]);
+                        if (km < k || (km == k && ia[mid] < s)) lo = mid + 1; else hi = mid;
+                    }
+                    const int to = min(r0, r0 ^ w) + (i - r0) + (lo - q0);
+                    vb[to] = v;
+                    ib[to] = s;
+                }
+                __syncthreads();
+                double *const tv = va;
+                va = vb;
+                vb = tv;
+                int32_t *const ti = ia;
+                ia = ib;
+                ib = ti;
+            }
+            if (va == wd + b0)
+                for (int i = tid; i < nd; i += T) {
+                    o.dk[b0 + mk + i] = va[i];
+                    o.src[b0 + mk + i] = ia[i];
+                }
         }
     }
     __syncthreads();
