@@ -46,6 +46,7 @@ struct FmmDev {
     ff_f2 *nwt;
     unsigned long long *amask;
     longlong2 *ibox;                       // per box: its interval in integers (admissibility)
+    int32_t *coarse;                       // per FMM problem: 1 if the integers do not resolve its boxes
     int32_t *upcnt;                        // per box: children whose moments are done in the current
                                            // upward pass (the last one computes the box; reset by it)
     unsigned long long *upq;               // upward pass: next unclaimed leaf box, CTAs past the end

@@ -117,11 +117,26 @@ __device__ __forceinline__ void box_ch(double lo, double hi, double &c, double &
 
 // on the boxes' integer intervals (60 bits of the split positions: an FP64
 // comparison costs the issue slots of 64 integer ones, and the tree of a large
-// problem is built by one CTA)
+// problem is built by one CTA).  Good to a part in COARSE of the boxes' widths; a
+// problem with narrower leaf boxes (poles graded over many orders of magnitude) or
+// out of the positions' scale takes the FP64 form, for lack of which half of 40000
+// poles graded over 25 decades saw each other directly: step 186 ms against 6.8
+constexpr long long COARSE = 1ll << 20;
 __device__ __forceinline__ bool adm(longlong2 S, longlong2 T)
 {
     const long long gap = max(T.x - S.y, S.x - T.y);
     return gap > 0 && 4 * gap >= 3 * max(S.y - S.x, T.y - T.x);
+}
+
+__device__ __forceinline__ bool adm64(double loS, double hiS, double loT, double hiT)
+{
+    const double gap = fmax(loT - hiS, loS - hiT);
+    return gap > 0.0 && gap >= FMM_KAPPA * fmax(hiS - loS, hiT - loT);
+}
+
+__device__ __forceinline__ bool adm_box(const FmmDev &pl, int64_t S, int64_t T, bool coarse)
+{
+    return coarse ? adm64(pl.blo[S], pl.bhi[S], pl.blo[T], pl.bhi[T]) : adm(pl.ibox[S], pl.ibox[T]);
 }
 
 // near list of a leaf box: nn >= 0 entries, or (nn < 0) every leaf box
@@ -235,11 +250,18 @@ __global__ void k_fmm_plan(int64_t nprob, const int32_t *__restrict__ mk, int mi
 // kept as a bit mask (the first 64), the others its near list.
 // Measured (GB300, one problem of 100003 poles): 0.43 -> 0.09 ms.
 __device__ __forceinline__ unsigned long long adm_mask(const FmmDev &pl, int64_t gb, int nbl, int A, int64_t pst,
-                                                       int npn, int sec)
+                                                       int npn, int sec, bool coarse)
 {
     unsigned long long mask = 0;
-    const longlong2 T = pl.ibox[gb + A];
     const int end = min(2 * npn, 64 * sec + 64);
+    if (coarse) {
+        for (int c = 64 * sec; c < end; c++) {
+            const int S = 2 * pl.near[pst + (c >> 1)] + (c & 1);
+            if (S < nbl && S != A && adm_box(pl, gb + S, gb + A, true)) mask |= 1ull << (c & 63);
+        }
+        return mask;
+    }
+    const longlong2 T = pl.ibox[gb + A];
 #pragma unroll 4
     for (int c = 64 * sec; c < end; c++) {
         const int S = 2 * pl.near[pst + (c >> 1)] + (c & 1);
@@ -267,6 +289,7 @@ k_fmm_tree(FmmDev pl, const int64_t *__restrict__ off, const int32_t *__restrict
         const FfScale fs = ff_scale(d[0], d[m - 1], 1.0);
         // intervals of every level at once
         int64_t gb = g0;
+        bool narrow = !fs.ok;
         for (int l = 0; l < L; l++) {
             const int nb = lev_nb(nb0, l);
             for (int b = threadIdx.x; b < nb; b += T) {
@@ -275,15 +298,18 @@ k_fmm_tree(FmmDev pl, const int64_t *__restrict__ off, const int32_t *__restrict
                 const double lo = d[i0], hi = (i1 < m) ? d[i1] : d[m - 1];
                 blo[gb + b] = lo;
                 bhi[gb + b] = hi;
-                longlong2 v = make_longlong2(0, 0);      // out of scale: nothing is admissible
+                longlong2 v = make_longlong2(0, 0);
                 if (fs.ok) {
                     v.x = (long long)((ff_fixed(lo, fs.kk) - fs.ref) >> 34);
                     v.y = (long long)((ff_fixed(hi, fs.kk) - fs.ref) >> 34);
+                    narrow = narrow || (l == 0 && b + 1 < nb && v.y - v.x < COARSE);
                 }
                 pl.ibox[gb + b] = v;
             }
             gb += nb;
         }
+        const bool coarse = __syncthreads_or(narrow);
+        if (threadIdx.x == 0) pl.coarse[p] = coarse ? 1 : 0;
         int64_t pos0 = g0 * FMM_NPOOL;                   // pool position of the level
         for (int l = L - 1; l >= 0; l--) {
             __syncthreads();
@@ -304,10 +330,10 @@ k_fmm_tree(FmmDev pl, const int64_t *__restrict__ off, const int32_t *__restrict
                         if (npn < 0) cnt = -1;
                         else {
                             const int64_t pst = nstart[gp0 + (b >> 1)];
-                            mask = adm_mask(pl, gb, nb, b, pst, npn, 0);
+                            mask = adm_mask(pl, gb, nb, b, pst, npn, 0, coarse);
                             int far = __popcll(mask);
                             for (int sec = 1; 64 * sec < 2 * npn; sec++)
-                                far += __popcll(adm_mask(pl, gb, nb, b, pst, npn, sec));
+                                far += __popcll(adm_mask(pl, gb, nb, b, pst, npn, sec, coarse));
                             // a candidate beyond the level's last box is neither
                             cnt = 2 * npn - far - ((nb & 1) && near[pst + npn - 1] == (nb >> 1) ? 1 : 0);
                         }
@@ -355,7 +381,7 @@ k_fmm_tree(FmmDev pl, const int64_t *__restrict__ off, const int32_t *__restrict
                         unsigned long long mask = pl.amask[gb + b];
                         int w = 0;
                         for (int k = 0; k < 2 * npn; k++) {
-                            if (k > 0 && (k & 63) == 0) mask = adm_mask(pl, gb, nb, b, pst, npn, k >> 6);
+                            if (k > 0 && (k & 63) == 0) mask = adm_mask(pl, gb, nb, b, pst, npn, k >> 6, coarse);
                             const int S = 2 * near[pst + (k >> 1)] + (k & 1);
                             if (S < nb && !((mask >> (k & 63)) & 1)) near[at + w++] = S;
                         }
@@ -983,7 +1009,7 @@ __global__ void __launch_bounds__(FAR_NW * 32) k_fmm_far(FmmDev pl, const int64_
         while (__any_sync(FULL, mask != 0 || 64 * (sec + 1) < 2 * npn)) {
             if (mask == 0 && 64 * (sec + 1) < 2 * npn) {
                 sec++;
-                mask = adm_mask(pl, g0 + lb, lev_nb(nb0, lane), A, pst, npn, sec);
+                mask = adm_mask(pl, g0 + lb, lev_nb(nb0, lane), A, pst, npn, sec, !ok && pl.coarse[p] != 0);
             }
             const int cnt = min(FAR_TAKE, __popcll(mask));
             int pos = cnt;
@@ -2620,7 +2646,7 @@ k_cm_apply(FmmDev pl, FactorView f, const int64_t *__restrict__ tile_off, CmDev 
                     if (__any_sync(FULL, mask != 0 || 64 * (sec + 1) < 2 * npn)) {
                         if (mask == 0 && 64 * (sec + 1) < 2 * npn) {
                             sec++;
-                            mask = adm_mask(pl, gbx + lb, nbl, A, pst, npn, sec);
+                            mask = adm_mask(pl, gbx + lb, nbl, A, pst, npn, sec, false);   // coarse problems are out of scale
                         }
                         const int cnt = min(CM_TAKE, __popcll(mask));
                         int pos = cnt;
@@ -2877,7 +2903,7 @@ k_cm_rest(FmmDev pl, FactorView f, int64_t total, const int64_t *__restrict__ ti
                             for (int i = 0; i < 2 * pl.nnear[gP]; i++) {
                                 const int S = 2 * pl.near[pl.nstart[gP] + (i >> 1)] + (i & 1);
                                 if (S >= lev_nb(nb0, l) || S == A ||
-                                    !adm(pl.ibox[gl + S], pl.ibox[gl + A]))
+                                    !adm_box(pl, gl + S, gl + A, pl.coarse[p] != 0))
                                     continue;
                                 double cS, hS;
                                 box_ch(pl.blo[gl + S], pl.bhi[gl + S], cS, hS);
@@ -3074,6 +3100,7 @@ superdc_status plan(FmmPlan &pl, int64_t nprob, const int64_t *off, int64_t tota
     SDC_CHECK(al(&d.npos, (size_t)pl.cap_boxes * P));
     SDC_CHECK(al(&d.amask, (size_t)pl.cap_boxes));
     SDC_CHECK(al(&d.ibox, (size_t)pl.cap_boxes));
+    SDC_CHECK(al(&d.coarse, (size_t)nprob));
     if (step) {
         SDC_CHECK(al(&d.coef, (size_t)pl.cap_leaves * NFIELD * P));
         SDC_CHECK(al(&d.lastp, (size_t)pl.cap_leaves));
