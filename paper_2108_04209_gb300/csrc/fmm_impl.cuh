@@ -120,7 +120,7 @@ __device__ __forceinline__ void box_ch(double lo, double hi, double &c, double &
 // problem is built by one CTA).  Good to a part in COARSE of the boxes' widths; a
 // problem with narrower leaf boxes (poles graded over many orders of magnitude) or
 // out of the positions' scale takes the FP64 form, for lack of which half of 40000
-// poles graded over 25 decades saw each other directly: step 186 ms against 6.8
+// poles graded over 25 decades saw each other directly: step 186 ms against 3.1
 constexpr long long COARSE = 1ll << 20;
 __device__ __forceinline__ bool adm(longlong2 S, longlong2 T)
 {
@@ -477,16 +477,18 @@ __device__ __forceinline__ void leaf_moments(const FmmDev &pl, const SrcArgs &a,
             } else if (MODE == M_BN) {
                 const double v = act ? a.vhat[b0 + j] : 0.0;
                 Wt[tid][0] = v * v;
-            } else if (MODE == M_CT) {
-                const double v = act ? a.vhat[b0 + j] : 0.0;
-                const int64_t row = act ? b0 + a.src[b0 + j] : 0;
-                for (int q = 0; q < nw; q++) Wt[tid][q] = act ? v * a.X[row + (int64_t)(a.col0 + q) * a.ldx] : 0.0;
-            } else {
-                const double bj = act ? a.bnorm[b0 + j] : 0.0;
-                const int64_t row = act ? b0 + a.pinv[b0 + j] : 0;
-                for (int q = 0; q < nw; q++) Wt[tid][q] = act ? bj * a.X[row + (int64_t)(a.col0 + q) * a.ldx] : 0.0;
             }
         }
+    }
+    if (MODE == M_CT || MODE == M_CN) {
+        // the columns by all warps, a lane per source
+        const int js = Tb * B + (tid & 31);
+        const bool in = js < jend;
+        const double v = in ? (MODE == M_CT ? a.vhat[b0 + js] : a.bnorm[b0 + js]) : 0.0;
+        const int64_t row = in ? b0 + (MODE == M_CT ? a.src[b0 + js] : a.pinv[b0 + js]) : 0;
+#pragma unroll 4
+        for (int q = tid >> 5; q < nw; q += (int)blockDim.x >> 5)
+            Wt[tid & 31][q] = in ? v * a.X[row + (int64_t)(a.col0 + q) * a.ldx] : 0.0;
     }
     __syncthreads();
     for (int t = tid; t < P * nw; t += blockDim.x) {
@@ -583,7 +585,7 @@ __device__ __forceinline__ void m2m_box(const FmmDev &pl, int64_t p, int nb0, in
 // (secular, b, Loewner) take 64 threads (one per source of a box of 64, and
 // the 2P children's nodes of a box), the Cauchy-like ones 128 and WMAX columns.
 template <int MODE> constexpr bool up_wide() { return MODE == M_CT || MODE == M_CN; }
-template <int MODE> constexpr int up_threads() { return up_wide<MODE>() ? 128 : 64; }
+template <int MODE> constexpr int up_threads() { return up_wide<MODE>() ? 256 : 64; }
 template <int MODE> constexpr int up_cols() { return up_wide<MODE>() ? WMAX : 1; }
 
 template <int MODE>
@@ -622,8 +624,11 @@ __global__ void __launch_bounds__(up_threads<MODE>()) k_fmm_up(FmmDev pl, SrcArg
         leaf_moments<MODE, WW>(pl, a, p, gl, g, Tb, nw, Tt, Wt, Ms, Tx);
         const int nb0 = (a.mk[p] + B - 1) / B;
         const int L = lev_count(nb0);
+        // the two top levels' boxes are in no interaction list (the last root's sums
+        // take them, one column)
+        const int lend = up_wide<MODE>() ? L - 2 : L;
         int l = 0, b = Tb;
-        while (l + 1 < L) {
+        while (l + 1 < lend) {
             const int bp = b >> 1;
             const int nch = (2 * bp + 1 < lev_nb(nb0, l)) ? 2 : 1;
             const int64_t gp = pl.box_base[p] + lev_base(nb0, l + 1) + bp;
@@ -981,18 +986,15 @@ __global__ void __launch_bounds__(FAR_NW * 32) k_fmm_far(FmmDev pl, const int64_
     const int64_t nleaf = pl.leaf_base[pl.nprob];
     for (int64_t gl = (int64_t)blockIdx.x * FAR_NW + warp; gl < nleaf; gl += (int64_t)gridDim.x * FAR_NW) {
         const int64_t p = sdc_upper_index(pl.leaf_base, pl.nprob, gl);
-        if (pl.fslot[p] < 0) continue;
+        if (pl.fslot[p] < 0 || pl.ffbad[p]) continue;        // out of scale: k_fmm_far64
         const int64_t b0 = off[p], g0 = pl.box_base[p];
         const int m = o.mk[p], nb0 = (m + B - 1) / B, L = lev_count(nb0);
         const int Tb = (int)(gl - pl.leaf_base[p]);
-        const bool ok = pl.ffbad[p] == 0;
         const FfScale fs = ff_scale(o.dk[b0], o.dk[b0 + m - 1], o.wsum[p]);
         double cT, hT;
         box_ch(pl.blo[g0 + Tb], pl.bhi[g0 + Tb], cT, hT);
-        const double tq = cT + hT * xq[q];
         const ff_f4 x = ff_point(cT, hT * xq[q], fs), xc = ff_pole(cT, fs);
         FfAcc AL = {}, AR = {}, AC = {};          // AC: K_LOG, the sum at the centre
-        double L1 = 0.0, R1 = 0.0, L2 = 0.0, R2 = 0.0, C1 = 0.0;      // the same in FP64 (!ok)
         // lane l: the interaction list of the leaf's ancestor on level l
         int A = 0, npn = 0, sec = 0, lb = 0;
         int64_t pst = 0;
@@ -1009,7 +1011,7 @@ __global__ void __launch_bounds__(FAR_NW * 32) k_fmm_far(FmmDev pl, const int64_
         while (__any_sync(FULL, mask != 0 || 64 * (sec + 1) < 2 * npn)) {
             if (mask == 0 && 64 * (sec + 1) < 2 * npn) {
                 sec++;
-                mask = adm_mask(pl, g0 + lb, lev_nb(nb0, lane), A, pst, npn, sec, !ok && pl.coarse[p] != 0);
+                mask = adm_mask(pl, g0 + lb, lev_nb(nb0, lane), A, pst, npn, sec, false);     // coarse problems are out of scale
             }
             const int cnt = min(FAR_TAKE, __popcll(mask));
             int pos = cnt;
@@ -1030,7 +1032,7 @@ __global__ void __launch_bounds__(FAR_NW * 32) k_fmm_far(FmmDev pl, const int64_
             npair += total;
             ff_f4 v = {};
             ff_f2 w = {};
-            if (ok && total > 0) {
+            if (total > 0) {
                 const int64_t t = (g0 + (list[warp][0] >> 1)) * P + q;
                 v = pl.npos[t];
                 w = pl.nwt[t];
@@ -1038,61 +1040,46 @@ __global__ void __launch_bounds__(FAR_NW * 32) k_fmm_far(FmmDev pl, const int64_
             for (int i = 0; i < total; i++) {
                 const int e = list[warp][i];
                 const bool left = e & 1;
-                if (ok) {
-                    __syncwarp();
-                    if (lane < P) { sp[warp][lane] = v; sw[warp][lane] = w; }
-                    __syncwarp();
-                    const ff_f4 vq = v;
-                    const ff_f2 wq = w;
-                    if (i + 1 < total) {                         // the next pair's nodes, ahead of their use
-                        const int64_t t = (g0 + (list[warp][i + 1] >> 1)) * P + q;
-                        v = pl.npos[t];
-                        w = pl.nwt[t];
-                    }
-                    FfAcc S = (KER == K_SEC && !left) ? AR : AL;
+                __syncwarp();
+                if (lane < P) { sp[warp][lane] = v; sw[warp][lane] = w; }
+                __syncwarp();
+                const ff_f4 vq = v;
+                const ff_f2 wq = w;
+                if (i + 1 < total) {                         // the next pair's nodes, ahead of their use
+                    const int64_t t = (g0 + (list[warp][i + 1] >> 1)) * P + q;
+                    v = pl.npos[t];
+                    w = pl.nwt[t];
+                }
+                FfAcc S = (KER == K_SEC && !left) ? AR : AL;
 #pragma unroll 2
-                    for (int j = 0; j < P; j++) {
-                        float t, tp, tq2;
-                        if (KER == K_2) ff_term2(sp[warp][j], sw[warp][j], x, t, tp);
-                        else ff_term(sp[warp][j], sw[warp][j], x, t, tp, tq2);
-                        ff_addto(S, t, tp);
-                        if ((j & 7) == 7) ff_norm(S);
-                    }
-                    ff_close(S);
-                    if (KER == K_SEC && !left) AR = S; else AL = S;
-                    if (KER == K_LOG) {
-                        // node q of the source against the centre; the box's weights sum
-                        // to zero, so one exponent per box drops out
-                        float t, tl2, y, yl;
-                        ff_diff(vq, xc, t, tl2);
-                        if (t < 0.0f) { t = -t; tl2 = -tl2; }
-                        const int e0 = __shfl_sync(FULL, ff_fexp(t), 0);
-                        ff_log(t, tl2, e0, lt, y, yl);
-                        float pr, pe;
-                        ff_two_mul(wq.x, y, pr, pe);
-                        pe = ff_fma(wq.y, y, ff_fma(wq.x, yl, pe));
-                        if (lane < P) ff_addto(AC, pr, pe);
-                        ff_close(AC);
-                    }
-                } else {
-                    const int64_t gS = g0 + (e >> 1);
-                    double cS, hS;
-                    box_ch(pl.blo[gS], pl.bhi[gS], cS, hS);
-                    double a1 = 0.0, a2 = 0.0;
-                    for (int j = 0; j < P; j++) {
-                        const double r = rcp_nr2((cS + hS * xq[j]) - tq), a = pl.W[(gS * P + j) * pl.ncol] * r;
-                        a1 += a;
-                        a2 = fma(a, r, a2);
-                    }
-                    if (left) { L1 += a1; L2 += a2; } else { R1 += a1; R2 += a2; }
-                    if (KER == K_LOG && lane < P)
-                        C1 = fma(pl.W[(gS * P + lane) * pl.ncol], log(fabs((cS + hS * xq[lane]) - cT)), C1);
+                for (int j = 0; j < P; j++) {
+                    float t, tp, tq2;
+                    if (KER == K_2) ff_term2(sp[warp][j], sw[warp][j], x, t, tp);
+                    else ff_term(sp[warp][j], sw[warp][j], x, t, tp, tq2);
+                    ff_addto(S, t, tp);
+                    if ((j & 7) == 7) ff_norm(S);
+                }
+                ff_close(S);
+                if (KER == K_SEC && !left) AR = S; else AL = S;
+                if (KER == K_LOG) {
+                    // node q of the source against the centre; the box's weights sum
+                    // to zero, so one exponent per box drops out
+                    float t, tl2, y, yl;
+                    ff_diff(vq, xc, t, tl2);
+                    if (t < 0.0f) { t = -t; tl2 = -tl2; }
+                    const int e0 = __shfl_sync(FULL, ff_fexp(t), 0);
+                    ff_log(t, tl2, e0, lt, y, yl);
+                    float pr, pe;
+                    ff_two_mul(wq.x, y, pr, pe);
+                    pe = ff_fma(wq.y, y, ff_fma(wq.x, yl, pe));
+                    if (lane < P) ff_addto(AC, pr, pe);
+                    ff_close(AC);
                 }
             }
         }
         // the leaf's coefficients
         double *cf = pl.coef + gl * NFIELD * P;
-        const double c1 = ok ? ff_pow2(fs.kk + fs.kw) : 1.0;
+        const double c1 = ff_pow2(fs.kk + fs.kw);
         const double fn = (lane == 0) ? 1.0 / P : 2.0 / P;
         auto series = [&](double F) {              // coefficient lane of the series with node values F
             __syncwarp();
@@ -1102,7 +1089,7 @@ __global__ void __launch_bounds__(FAR_NW * 32) k_fmm_far(FmmDev pl, const int64_
             for (int j = 0; j < P; j++) a = fma(sF[warp][j], Tx[j * P + q], a);
             return a * fn;
         };
-        if (KER == K_SEC && ok) {
+        if (KER == K_SEC) {
             // psi + phi in FP64; psi and the two derivatives in single precision,
             // scaled like the near sums (ff_collect)
             const double a = series(((double)AL.s + (double)AL.sl + ((double)AR.s + (double)AR.sl)) * c1);
@@ -1132,24 +1119,13 @@ __global__ void __launch_bounds__(FAR_NW * 32) k_fmm_far(FmmDev pl, const int64_
                 ff[2 * P + lane] = dr * ih;
             }
             store_series(a, ff_pow2(-(fs.kk + fs.kw)), Mt, sF[warp], cf);
-        } else if (KER == K_SEC) {
-            const double F[4] = {L1, R1, L2, R2};
-            for (int k = 0; k < 4; k++) {
-                const double a = series(F[k]);
-                if (lane < P) cf[k * P + lane] = a;
-            }
         } else if (KER == K_2) {
-            if (ok) {
-                store_series(series((double)AL.s + (double)AL.sl), 1.0, Mt, sF[warp], cf);
-            } else {
-                const double a = series(L2 + R2);
-                if (lane < P) cf[lane] = a;
-            }
+            store_series(series((double)AL.s + (double)AL.sl), 1.0, Mt, sF[warp], cf);
         } else {
             // F' -> antiderivative G = sum B_k T_k (k = 1..P; T_P vanishes at the
             // nodes but not at 0), F(u) = F(centre) + h (G(u) - G(0))
-            const double a = series(ok ? -((double)AL.s + (double)AL.sl) * ff_pow2(fs.kk) : -(L1 + R1));
-            double c = ok ? (double)AC.s + (double)AC.sl : C1;
+            const double a = series(-((double)AL.s + (double)AL.sl) * ff_pow2(fs.kk));
+            double c = (double)AC.s + (double)AC.sl;
             if (lane >= P) c = 0.0;
             for (int s = 16; s > 0; s >>= 1) c += __shfl_xor_sync(FULL, c, s);
             __syncwarp();
@@ -1161,12 +1137,225 @@ __global__ void __launch_bounds__(FAR_NW * 32) k_fmm_far(FmmDev pl, const int64_
             double g0s = (lane >= 2 && lane <= P && !(lane & 1)) ? ((lane & 2) ? -bk : bk) : 0.0;   // T_k(0)
             for (int s = 16; s > 0; s >>= 1) g0s += __shfl_xor_sync(FULL, g0s, s);
             const double a2 = (lane == 0) ? c - hT * g0s : hT * bk;
-            if (ok) store_series(a2, 1.0, Mt, sF[warp], cf);
-            else if (lane < P) cf[lane] = a2;
+            store_series(a2, 1.0, Mt, sF[warp], cf);
         }
         if (pl.flops && lane == 0 && npair)
             atomicAdd(pl.flops, (unsigned long long)npair * P * (P * (KER == K_SEC ? 7 : 5) + (KER == K_LOG ? 3 : 0)) +
                                     2 * P * P);
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Far fields of the problems out of the split arithmetic's scale, in FP64 (poles
+// closer than its positions resolve): series of P coefficients per field and leaf
+// box.  A CTA takes a subtree of 2^sub leaf boxes: its top box sums the interaction
+// lists of itself and of every ancestor at its own nodes, the boxes below it their
+// own lists, plus the parent's series at their nodes; the series of the current
+// path stay in shared memory.  About 7 + 3.5 levels / 2^sub box pairs per leaf, as by
+// translation level by level but in one launch (summing every ancestor's list at
+// the leaf: 3.5 per level).  Fields: K_SEC the sums w/(s-t) to the left and right,
+// then w/(s-t)^2; K_2 w/(s-t)^2; K_LOG w log|s-t| as its derivative at the nodes,
+// integrated in coefficient space, plus the sum itself at the box's centre; K_1 and
+// K_1N nw columns w/(s-t), w/(t-s).
+// Measured (GB300): step of 40000 poles, one pair of them close, 2.22 ms (2.96 with
+// every list summed at the leaves, 2.57 by translations level by level, a launch per
+// level); 64 columns through 20000 such poles, both directions, with k_cm_rest 6.2
+// (17.0, 6.0); 124000 rows in 60 problems, 19 columns 6.6 (15.7, 7.0).
+// ---------------------------------------------------------------------------
+constexpr int SUB_MAX = 3;        // levels of a subtree below its top box
+constexpr int F64_COLS = 32;      // widest block of columns
+
+template <int KER> constexpr bool far_cols() { return KER == K_1 || KER == K_1N; }
+template <int KER> constexpr int far_fields() { return KER == K_SEC ? 4 : far_cols<KER>() ? F64_COLS : 1; }
+
+template <int KER> constexpr int far_threads() { return far_cols<KER>() ? 256 : 128; }
+
+template <int KER>
+__global__ void __launch_bounds__(far_threads<KER>())
+k_fmm_far64(FmmDev pl, const int32_t *__restrict__ mk, const int32_t *__restrict__ only, int nw, int sub,
+            double *__restrict__ coef, int nfield)
+{
+    constexpr bool COLS = far_cols<KER>();
+    constexpr int NF = far_fields<KER>(), NT = far_threads<KER>(), PARTS = NT / P, PAIRS = COLS ? 1 : 32;
+    constexpr int RMAX = (P * NF + NT - 1) / NT;
+    __shared__ double xq[P], tq[P], Tx[P * P];
+    __shared__ double stack[SUB_MAX + 1][NF][P];         // series of the path's boxes by level
+    __shared__ double Fs[NF][P], An[P + 2], Bk[P + 1];
+    __shared__ double sq[PAIRS][P], Ws[PAIRS * P][COLS ? NF : 1];
+    __shared__ double K1[COLS ? P : 1][P + 1];
+    __shared__ double red[COLS ? 1 : NF][COLS ? 1 : PARTS][P];
+    __shared__ int s_list[32], s_nlist;
+    __shared__ double s_ctr[4];
+    if (only[pl.nprob] == 0) return;                     // no problem out of scale
+    cheb_tables(xq, Tx);
+    // columns f0 .. f0 + nf - 1 of the nw (blockIdx.y: halves)
+    const int f0 = COLS ? (int)((int64_t)nw * blockIdx.y / gridDim.y) : 0;
+    const int tid = threadIdx.x, nf = COLS ? (int)((int64_t)nw * (blockIdx.y + 1) / gridDim.y) - f0 : NF;
+    const int64_t nleaf = pl.leaf_base[pl.nprob];
+    for (int64_t t = blockIdx.x;; t += gridDim.x) {
+        const int64_t w0 = t << sub;
+        if (w0 >= nleaf) break;
+        // the subtrees that start in this window of leaf boxes
+        for (int64_t gl = w0; gl < min(nleaf, w0 + ((int64_t)1 << sub)); gl++) {
+            const int64_t p = sdc_upper_index(pl.leaf_base, pl.nprob, gl);
+            if (pl.fslot[p] < 0 || only[p] == 0) continue;
+            const int Tb0 = (int)(gl - pl.leaf_base[p]);
+            const int nb0 = (mk[p] + B - 1) / B, L = lev_count(nb0), top = min(sub, L - 1);
+            if (Tb0 & ((1 << top) - 1)) continue;
+            const int64_t g0 = pl.box_base[p];
+            const bool coarse = pl.coarse[p] != 0;
+            int npair = 0;
+            for (int b = Tb0; b < min(nb0, Tb0 + (1 << top)); b++)
+                for (int l = b == Tb0 ? top : __ffs(b) - 1; l >= 0; l--) {
+                    const int64_t g = g0 + lev_base(nb0, l) + (b >> l);
+                    const bool near_all = pl.nnear[g] < 0;               // every source directly: no far field
+                    double cT, hT;
+                    box_ch(pl.blo[g], pl.bhi[g], cT, hT);
+                    __syncthreads();
+                    if (tid < P) tq[tid] = cT + hT * xq[tid];
+                    double acc[RMAX] = {};                               // COLS: entry (q, f)
+                    double a1[2] = {}, a2[2] = {}, c1 = 0.0;             // else node q, by side; the centre's sum
+                    const int q = tid % P, part = tid / P;
+                    // the interaction lists: of this box, and of its ancestors for the subtree's top
+                    for (int lv = l; lv < (near_all ? 0 : l == top ? L - 1 : l + 1); lv++) {
+                        const int A = b >> lv, nbl = lev_nb(nb0, lv);
+                        const int64_t gb = g0 + lev_base(nb0, lv), gP = g0 + lev_base(nb0, lv + 1) + (A >> 1);
+                        const int npn = pl.nnear[gP];
+                        const int64_t pst = pl.nstart[gP];
+                        for (int c0 = 0; c0 < 2 * npn; c0 += 32) {
+                            __syncthreads();
+                            if (tid < 32) {
+                                const int cd = c0 + tid;
+                                int S = -1;
+                                bool in = false;
+                                if (cd < 2 * npn) {
+                                    S = 2 * pl.near[pst + (cd >> 1)] + (cd & 1);
+                                    in = S < nbl && S != A && adm_box(pl, gb + S, gb + A, coarse);
+                                }
+                                const unsigned bal = __ballot_sync(0xffffffffu, in);
+                                if (in) s_list[__popc(bal & ((1u << tid) - 1u))] = S;
+                                if (tid == 0) s_nlist = __popc(bal);
+                            }
+                            __syncthreads();
+                            const int nlist = s_nlist;
+                            npair += nlist;
+                            for (int i0 = 0; i0 < nlist; i0 += PAIRS) {
+                                const int cnt = min(PAIRS, nlist - i0);
+                                if (i0 > 0) __syncthreads();
+                                for (int e = tid; e < cnt * P; e += NT) {
+                                    const int64_t gS = gb + s_list[i0 + e / P];
+                                    double cS, hS;
+                                    box_ch(pl.blo[gS], pl.bhi[gS], cS, hS);
+                                    sq[e / P][e % P] = cS + hS * xq[e % P];
+                                    if (!COLS) Ws[e][0] = pl.W[(gS * P + e % P) * pl.ncol];
+                                }
+                                if (COLS) {
+                                    const double *Wg = pl.W + (gb + s_list[i0]) * P * pl.ncol + f0;
+                                    for (int e = tid; e < P * nf; e += NT) Ws[e / nf][e % nf] = Wg[(e / nf) * pl.ncol + e % nf];
+                                }
+                                __syncthreads();
+                                if (COLS) {
+                                    for (int e = tid; e < P * P; e += NT) {
+                                        const double d = sq[0][e % P] - tq[e / P];
+                                        K1[e / P][e % P] = rcp_nr2(KER == K_1N ? -d : d);
+                                    }
+                                    __syncthreads();
+#pragma unroll
+                                    for (int r = 0; r < RMAX; r++) {
+                                        const int e = tid + r * NT;
+                                        if (e >= P * nf) break;
+                                        const int eq = e / nf, ef = e % nf;
+                                        double v = 0.0;
+                                        for (int j = 0; j < P; j++) v = fma(K1[COLS ? eq : 0][j], Ws[j][COLS ? ef : 0], v);
+                                        acc[r] += v;
+                                    }
+                                } else if (part < PARTS) {
+                                    for (int i = 0; i < cnt; i++) {
+                                        const bool left = KER != K_SEC || s_list[i0 + i] < A;
+                                        double v1 = 0.0, v2 = 0.0;
+                                        for (int j = part; j < P; j += PARTS) {
+                                            const double r = rcp_nr2(sq[COLS ? 0 : i][j] - tq[q]);
+                                            const double wr = Ws[i * P + j][0] * r;
+                                            if (KER != K_2) v1 += wr;
+                                            if (KER == K_SEC || KER == K_2) v2 = fma(wr, r, v2);
+                                        }
+                                        if (left) { a1[0] += v1; a2[0] += v2; } else { a1[1] += v1; a2[1] += v2; }
+                                    }
+                                }
+                                if (KER == K_LOG)
+                                    for (int e = tid; e < cnt * P; e += NT)
+                                        c1 = fma(Ws[e][0], log(fabs(sq[COLS ? 0 : e / P][e % P] - cT)), c1);
+                            }
+                        }
+                    }
+                    // node values
+                    if (COLS) {
+#pragma unroll
+                        for (int r = 0; r < RMAX; r++) {
+                            const int e = tid + r * NT;
+                            if (e < P * nf) Fs[e % nf][e / nf] = acc[r];
+                        }
+                    } else {
+                        if (part < PARTS) {
+                            const double v[4] = {KER == K_2 ? a2[0] : a1[0], a1[1], a2[0], a2[1]};
+#pragma unroll
+                            for (int k = 0; k < NF; k++) red[COLS ? 0 : k][COLS ? 0 : part][q] = v[k];
+                        }
+                        __syncthreads();
+                        for (int e = tid; e < P * NF; e += NT) {
+                            double v = 0.0;
+                            for (int i = 0; i < PARTS; i++) v += red[COLS ? 0 : e / P][COLS ? 0 : i][e % P];
+                            Fs[e / P][e % P] = v;
+                        }
+                    }
+                    if (KER == K_LOG) {
+                        // F' = -sum w/(s-t) -> antiderivative G = sum B_k T_k (k = 1..P; T_P vanishes at
+                        // the nodes but not at 0), F(u) = F(centre) + h (G(u) - G(0))
+                        for (int sh = 16; sh > 0; sh >>= 1) c1 += __shfl_xor_sync(0xffffffffu, c1, sh);
+                        __syncthreads();
+                        if (tid < P) {
+                            double v = 0.0;
+                            for (int j = 0; j < P; j++) v = fma(Fs[0][j], Tx[j * P + tid], v);
+                            An[tid] = -v * (tid == 0 ? 1.0 / P : 2.0 / P);
+                        }
+                        if (tid == 0) An[P] = An[P + 1] = 0.0;
+                        if ((tid & 31) == 0) s_ctr[tid >> 5] = c1;
+                        __syncthreads();
+                        if (tid >= 1 && tid <= P)
+                            Bk[tid] = tid == 1 ? An[0] - 0.5 * An[2] : (An[tid - 1] - An[tid + 1]) * (0.5 / tid);
+                        __syncthreads();
+                        if (tid < P) {
+                            double gq = 0.0, gz = 0.0;
+                            for (int k = 1; k < P; k++) gq = fma(Bk[k], Tx[tid * P + k], gq);
+                            for (int k = 2; k <= P; k += 2) gz += (k & 2) ? -Bk[k] : Bk[k];     // T_k(0)
+                            Fs[0][tid] = near_all ? 0.0 : (s_ctr[0] + s_ctr[1]) + (s_ctr[2] + s_ctr[3]) + hT * (gq - gz);
+                        }
+                    }
+                    __syncthreads();
+                    // the parent's series at this box's nodes (the node as scale and shift: forming
+                    // c + h x_q first would round it to the spacing of c, several percent of h on a
+                    // box of one point)
+                    if (l < top && !near_all) {
+                        const int64_t gP = g0 + lev_base(nb0, l + 1) + (b >> (l + 1));
+                        double cP, hP;
+                        box_ch(pl.blo[gP], pl.bhi[gP], cP, hP);
+                        const double ihP = rcp_any(hP);
+                        for (int e = tid; e < P * nf; e += NT)
+                            Fs[e / P][e % P] += clenshaw(stack[l + 1][e / P], fma(hT * ihP, xq[e % P], (cT - cP) * ihP));
+                        __syncthreads();
+                    }
+                    for (int e = tid; e < P * nf; e += NT) {
+                        double v = 0.0;
+                        for (int j = 0; j < P; j++) v = fma(Fs[e / P][j], Tx[j * P + e % P], v);
+                        v *= (e % P == 0) ? 1.0 / P : 2.0 / P;
+                        stack[l][e / P][e % P] = v;
+                        if (l == 0) coef[((pl.leaf_base[p] + b) * nfield + f0 + e / P) * P + e % P] = v;
+                    }
+                }
+            // kernel entry and its products; the series per box of the subtree
+            fl_add(pl, (int64_t)npair * P * P * (KER == K_SEC ? 7 : COLS ? 2 + 2 * nf : 5) +
+                           (int64_t)(2 << top) * 4 * P * P * nf);
+        }
     }
 }
 
@@ -2007,7 +2196,7 @@ constexpr int CM_D = 7;           // digits
 constexpr int CM_NT = 8;          // column tiles of 8 per pass
 constexpr int CM_TR = 64;         // targets per entry of tile_off, four CTAs of 16
 constexpr int CM_TAKE = 8;        // far boxes taken per level and round
-constexpr int CM_BC = 24;         // columns per pass of the FP64 loops
+constexpr int CM_BC = F64_COLS;   // columns per pass of the FP64 loops
 
 __device__ __forceinline__ float pow2f(int e) { return __int_as_float((e + 127) << 23); }      // -126 <= e <= 127
 
@@ -2037,6 +2226,7 @@ struct CmDev {
     unsigned *wf1;               //                       nodes 16..21
     int32_t *eb;                 // per box: exponent of its node weights over the columns' scales
     double *lastp;               // per (tile of 64, column of the pass): partial sums for the last eigenvalue
+    double *coef;                // per leaf box and column: far field's series of the problems out of scale
 };
 
 template <bool TRANS>
@@ -2836,10 +3026,12 @@ k_cm_apply(FmmDev pl, FactorView f, const int64_t *__restrict__ tile_off, CmDev 
     }
 }
 
-// What the tiles leave out, CM_BC columns per launch: the deflated slots (identity
-// part of the factor) and, in FP64, the problems out of the positions' scale (a
-// warp per 16 targets, a row per lane pair, half of the columns each).
-template <bool TRANS>
+// What the tiles leave out, at most NC columns per launch: the deflated slots
+// (identity part of the factor) and, in FP64, the problems out of the positions'
+// scale: a warp per leaf box (32 targets; without a tree every box is near), near
+// sources staged, far field from the box's series (k_fmm_far64, figures
+// there).  The inner loop runs all NC columns.
+template <bool TRANS, int NC>
 __global__ void __launch_bounds__(128)
 k_cm_rest(FmmDev pl, FactorView f, int64_t total, const int64_t *__restrict__ tile_off, CmDev c,
           const double *__restrict__ X, int64_t ldx, double *__restrict__ Y, int64_t ldy, int col0, int nc)
@@ -2858,69 +3050,84 @@ k_cm_rest(FmmDev pl, FactorView f, int64_t total, const int64_t *__restrict__ ti
         else       Y[b0 + sr + col * ldy] = X[b0 + ps + col * ldx];
     }
     if (c.bad[f.nprob] == 0) return;
-    constexpr int NT = CM_BC / 8;
+    __shared__ double sd[4][B], se[4][B], sf[4][B], sx[4][NC][B + 1];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t ntiles = tile_off[f.nprob];
-    for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    const int64_t nunit = tile_off[f.nprob] * (CM_TR / B);
+    for (int64_t u = (int64_t)blockIdx.x * 4 + warp; u < nunit; u += (int64_t)gridDim.x * 4) {
+        const int64_t tile = u / (CM_TR / B);
         const int64_t p = sdc_upper_index(tile_off, f.nprob, tile);
         if (!c.bad[p]) continue;
         const int64_t b0 = f.off[p];
         const int m = f.mk[p];
-        const int t0 = (int)(tile - tile_off[p]) * CM_TR + warp * 16;
+        const int Tb = (int)(tile - tile_off[p]) * (CM_TR / B) + (int)(u % (CM_TR / B));
         const int tend = TRANS ? m - 1 : m;              // T: the last target is summed by k_cm_last
-        if (t0 >= tend) continue;
+        if (Tb * B >= tend) continue;
         const bool tree = pl.fslot && pl.fslot[p] >= 0;
         const double *dk = f.dk + b0, *dorg = f.dorg + b0, *eta = f.eta + b0;
-        const int nb0 = (m + B - 1) / B, Tb = t0 / B;
-        const int64_t gbx = tree ? pl.box_base[p] : 0;
-        const int nnr = tree ? pl.nnear[gbx + Tb] : -1;
-        const int nn = near_len(nnr, nb0);               // without a tree: every box
-        const int nsrc = TRANS ? m : m - 1;
-                                const int r = min(t0 + (lane & 15), tend - 1), h = lane >> 4;
-                    const double a0 = TRANS ? dorg[r] : dk[r], a1 = TRANS ? eta[r] : 0.0;
-                    double acc[NT * 4] = {};
-                    auto add = [&](double t, double s, const double *col, int64_t st) {
-                        const double w = s * rcp_nr2(t);
-        #pragma unroll
-                        for (int q = 0; q < NT * 4; q++)
-                            if (h * NT * 4 + q < nc) acc[q] = fma(w, col[(int64_t)(h * NT * 4 + q) * st], acc[q]);
-                    };
-                    for (int i = 0; i < nn; i++) {
-                        const int j0 = SDC_IDX(near_box(pl, gbx + Tb, nnr, i), nb0, f.status) * B;
-                        for (int j = j0; j < min(j0 + B, nsrc); j++) {
-                            if (TRANS) add((dk[j] - a0) - a1, f.vhat[b0 + j], X + b0 + f.src[b0 + j] + (int64_t)col0 * ldx, ldx);
-                            else add((a0 - dorg[j]) - eta[j], f.bnorm[b0 + j], X + b0 + f.pinv[b0 + j] + (int64_t)col0 * ldx, ldx);
-                        }
-                    }
-                    if (!TRANS) add((a0 - dorg[m - 1]) - eta[m - 1], f.bnorm[b0 + m - 1],
-                                    X + b0 + f.pinv[b0 + m - 1] + (int64_t)col0 * ldx, ldx);
-                    if (tree && nnr >= 0) {
-                        const int L = lev_count(nb0);
-                        const double x = TRANS ? a0 + a1 : a0;
-                        for (int l = 0; l < L - 1; l++) {
-                            const int A = Tb >> l;
-                            const int64_t gl = gbx + lev_base(nb0, l), gP = gbx + lev_base(nb0, l + 1) + (A >> 1);
-                            for (int i = 0; i < 2 * pl.nnear[gP]; i++) {
-                                const int S = 2 * pl.near[pl.nstart[gP] + (i >> 1)] + (i & 1);
-                                if (S >= lev_nb(nb0, l) || S == A ||
-                                    !adm_box(pl, gl + S, gl + A, pl.coarse[p] != 0))
-                                    continue;
-                                double cS, hS;
-                                box_ch(pl.blo[gl + S], pl.bhi[gl + S], cS, hS);
-                                for (int q = 0; q < P; q++) {
-                                    const double s = cS + hS * cospi((double)(2 * q + 1) / (2.0 * P));
-                                    add(TRANS ? s - x : x - s, 1.0, pl.W + ((gl + S) * P + q) * pl.ncol, 1);
-                                }
-                            }
-                        }
-                    }
-                    const int64_t row = b0 + (TRANS ? f.pinv[b0 + r] : f.src[b0 + r]);
-                    const double sc = TRANS ? f.bnorm[b0 + r] : f.vhat[b0 + r];
-                    if (t0 + (lane & 15) < tend)
-        #pragma unroll
-                        for (int q = 0; q < NT * 4; q++)
-                            if (h * NT * 4 + q < nc) Y[row + (int64_t)(col0 + h * NT * 4 + q) * ldy] = sc * acc[q];
+        const int nb0 = (m + B - 1) / B, nsrc = TRANS ? m : m - 1;
+        const int64_t gx = tree ? pl.box_base[p] + Tb : 0;
+        const int nnr = tree ? pl.nnear[gx] : -1;
+        const int nn = near_len(nnr, nb0);
+        const int64_t nrow = f.off[p + 1] - b0;
+        const int r = min(Tb * B + lane, tend - 1);
+        const double a0 = TRANS ? dorg[r] : dk[r], a1 = TRANS ? eta[r] : 0.0;
+        double acc[NC];
+#pragma unroll
+        for (int q = 0; q < NC; q++) acc[q] = 0.0;
+        if (tree) {
+            double cT, hT;
+            box_ch(pl.blo[gx], pl.bhi[gx], cT, hT);
+            const double v = ((a0 + a1) - cT) * rcp_any(hT);
+            const double *cf = c.coef + (pl.leaf_base[p] + Tb) * CM_BC * P;
+#pragma unroll
+            for (int q = 0; q < NC; q++)
+                if (q < nc) acc[q] = clenshaw(cf + q * P, v);
+        }
+        for (int i = 0; i < nn; i++) {
+            const int j0 = SDC_IDX(near_box(pl, gx, nnr, i), nb0, f.status) * B, cnt = min(B, nsrc - j0);
+            __syncwarp();
+            if (lane < cnt) {
+                const int j = j0 + lane;
+                const int64_t row = b0 + SDC_IDX(TRANS ? f.src[b0 + j] : f.pinv[b0 + j], nrow, f.status);
+                sd[warp][lane] = TRANS ? dk[j] : dorg[j];
+                se[warp][lane] = TRANS ? 0.0 : eta[j];
+                sf[warp][lane] = TRANS ? f.vhat[b0 + j] : f.bnorm[b0 + j];
+#pragma unroll
+                for (int q = 0; q < NC; q++) sx[warp][q][lane] = (q < nc) ? X[row + (int64_t)(col0 + q) * ldx] : 0.0;
+            }
+            __syncwarp();
+#pragma unroll 2
+            for (int jj = 0; jj < cnt; jj++) {
+                const double t = TRANS ? (sd[warp][jj] - a0) - a1 : (a0 - sd[warp][jj]) - se[warp][jj];
+                const double w = sf[warp][jj] * rcp_nr2(t);      // before x: b_j x_j could underflow
+#pragma unroll
+                for (int q = 0; q < NC; q++) acc[q] = fma(sx[warp][q][jj], w, acc[q]);
+            }
+        }
+        if (!TRANS) {                                    // the last eigenvalue, outside the tree
+            const double w = f.bnorm[b0 + m - 1] * rcp_nr2((a0 - dorg[m - 1]) - eta[m - 1]);
+            const int64_t row = b0 + SDC_IDX(f.pinv[b0 + m - 1], nrow, f.status);
+#pragma unroll
+            for (int q = 0; q < NC; q++)
+                if (q < nc) acc[q] = fma(w, X[row + (int64_t)(col0 + q) * ldx], acc[q]);
+        }
+        if (Tb * B + lane < tend) {
+            const int64_t row = b0 + SDC_IDX(TRANS ? f.pinv[b0 + r] : f.src[b0 + r], nrow, f.status);
+            const double sc = TRANS ? f.bnorm[b0 + r] : f.vhat[b0 + r];
+#pragma unroll
+            for (int q = 0; q < NC; q++)
+                if (q < nc) Y[row + (int64_t)(col0 + q) * ldy] = sc * acc[q];
+        }
     }
+}
+
+template <int NC>
+void launch_rest(bool trans, const FmmDev &dv, const FactorView &f, int64_t total, const int64_t *tile_off,
+                 const CmDev &c, const double *X, int64_t ldx, double *Y, int64_t ldy, int col0, int nc, unsigned g,
+                 cudaStream_t st)
+{
+    if (trans) k_cm_rest<true, NC><<<g, 128, 0, st>>>(dv, f, total, tile_off, c, X, ldx, Y, ldy, col0, nc);
+    else k_cm_rest<false, NC><<<g, 128, 0, st>>>(dv, f, total, tile_off, c, X, ldx, Y, ldy, col0, nc);
 }
 
 // Row of the last eigenvalue of Qhat^T X: the sources of one tile of 64, FP64
@@ -3011,6 +3218,23 @@ SrcArgs src_from_r1(const int64_t *off, const R1Out &o)
     return a;
 }
 
+// Far fields of the problems with only[p] != 0.  Subtrees of 8 leaf boxes where that
+// leaves four to an SM (their lists differ in length), of 4 where it leaves one, the
+// columns in two halves where there are few.  GB300, applications of 19 columns to
+// 124000 rows, of 64 to 20000, poles graded: 8 boxes 36.3 and 13.8 ms, 4 boxes 29.9 and
+// 9.0, 2 boxes 30 and 10.7
+template <int KER>
+void launch_far64(const FmmPlan &pl, const int32_t *mk, const int32_t *only, int nw, double *coef, int nfield,
+                  cudaStream_t st)
+{
+    const int64_t nsm = sdc_num_sms();
+    const int sub = (pl.cap_leaves >> 3) >= 4 * nsm ? 3 : (pl.cap_leaves >> 2) >= nsm ? 2 : 1;
+    const int64_t units = (pl.cap_leaves >> sub) + 1;
+    const unsigned g = (unsigned)std::min<int64_t>(units, resident_grid<k_fmm_far64<KER>>(far_threads<KER>()));
+    const dim3 grid(g, far_cols<KER>() && nw > 8 && units < 2 * nsm ? 2 : 1);
+    PROF_LAUNCH("fmm_far", st, k_fmm_far64<KER><<<grid, far_threads<KER>(), 0, st>>>(pl.dv, mk, only, nw, sub, coef, nfield));
+}
+
 // far field of a one-column sum: node weights, then every leaf's series
 template <int MODE, int KER>
 superdc_status far_field(const FmmPlan &pl, const int64_t *off, const R1Out &o, cudaStream_t st)
@@ -3024,6 +3248,7 @@ superdc_status far_field(const FmmPlan &pl, const int64_t *off, const R1Out &o, 
     const int64_t want = (pl.cap_leaves + FAR_NW - 1) / FAR_NW;
     const unsigned g = (unsigned)std::min<int64_t>(want, resident_grid<k_fmm_far<KER>>(FAR_NW * 32));
     PROF_LAUNCH("fmm_far", st, k_fmm_far<KER><<<g, FAR_NW * 32, 0, st>>>(dv, off, o));
+    launch_far64<KER>(pl, o.mk, dv.ffbad, 1, dv.coef, NFIELD, st);
     return SUPERDC_OK;
 }
 
@@ -3216,6 +3441,7 @@ superdc_status columns(const FmmPlan &pl, const FactorView &f, int64_t total, co
         SDC_CHECK(sc.get(&c.wf0, (size_t)pl.cap_boxes * ntmax * CM_D * 32));
         SDC_CHECK(sc.get(&c.wf1, (size_t)pl.cap_boxes * ntmax * CM_D * 32));
         SDC_CHECK(sc.get(&c.eb, (size_t)pl.cap_boxes));
+        SDC_CHECK(sc.get(&c.coef, (size_t)pl.cap_leaves * CM_BC * P));
     }
     SDC_CHECK(cudaMemsetAsync(c.bad, 0, nflag * sizeof(int32_t), st));
     auto gr = [&](int64_t n) {
@@ -3251,9 +3477,12 @@ superdc_status columns(const FmmPlan &pl, const FactorView &f, int64_t total, co
             a.src = f.src; a.pinv = f.pinv; a.X = X; a.ldx = ldx; a.col0 = c0; a.nc = nc; a.only = c.bad;
             if (trans) PROF_LAUNCH("fmm_up", st, k_fmm_up<M_CT><<<up_grid<M_CT>(), up_threads<M_CT>(), 0, st>>>(dv, a));
             else PROF_LAUNCH("fmm_up", st, k_fmm_up<M_CN><<<up_grid<M_CN>(), up_threads<M_CN>(), 0, st>>>(dv, a));
+            if (trans) launch_far64<K_1>(pl, f.mk, c.bad, nc, c.coef, CM_BC, st);
+            else launch_far64<K_1N>(pl, f.mk, c.bad, nc, c.coef, CM_BC, st);
         }
-        if (trans) PROF_LAUNCH("deflcopy", st, k_cm_rest<true><<<gr(total * nc), 128, 0, st>>>(dv, f, total, tile_off, c, X, ldx, Y, ldy, c0, nc));
-        else PROF_LAUNCH("deflcopy", st, k_cm_rest<false><<<gr(total * nc), 128, 0, st>>>(dv, f, total, tile_off, c, X, ldx, Y, ldy, c0, nc));
+        auto fn = nc <= 2 ? launch_rest<2> : nc <= 4 ? launch_rest<4> : nc <= 8 ? launch_rest<8> : nc <= 12 ? launch_rest<12>
+                : nc <= 16 ? launch_rest<16> : nc <= 20 ? launch_rest<20> : nc <= 24 ? launch_rest<24> : launch_rest<CM_BC>;
+        PROF_LAUNCH("deflcopy", st, fn(trans, dv, f, total, tile_off, c, X, ldx, Y, ldy, c0, nc, gr(total * nc), st));
     }
     SDC_CHECK(cudaGetLastError());
     return SUPERDC_OK;
