@@ -1059,7 +1059,7 @@ __global__ void __launch_bounds__(FAR_NW * 32) k_fmm_far(FmmDev pl, const int64_
                     ff_addto(S, t, tp);
                     if ((j & 7) == 7) ff_norm(S);
                 }
-                ff_close(S);
+                if (KER == K_SEC) ff_close3(S); else ff_close(S);
                 if (KER == K_SEC && !left) AR = S; else AL = S;
                 if (KER == K_LOG) {
                     // node q of the source against the centre; the box's weights sum
@@ -1092,7 +1092,7 @@ __global__ void __launch_bounds__(FAR_NW * 32) k_fmm_far(FmmDev pl, const int64_
         if (KER == K_SEC) {
             // psi + phi in FP64; psi and the two derivatives in single precision,
             // scaled like the near sums (ff_collect)
-            const double a = series(((double)AL.s + (double)AL.sl + ((double)AR.s + (double)AR.sl)) * c1);
+            const double a = series(((double)AL.s + ((double)AL.sl + (double)AL.c) + ((double)AR.s + ((double)AR.sl + (double)AR.c))) * c1);
             if (lane < P) { fL[warp][lane] = AL.s; fR[warp][lane] = AR.s; }
             __syncwarp();
             float l = 0.0f, r = 0.0f;
@@ -1470,7 +1470,7 @@ k_secular_fmm(FmmDev pl, FfDev ff, const int64_t *__restrict__ off, R1Out o, dou
             for (int i = 0; i < nn; i++) {
                 const int j0 = near_box_chk(pl, g, nnr, i, (m + B - 1) / B, o.status) * B;
                 const int cnt = min(B, m - j0);
-                if (ok)      ff_sweep(fd + i * B, fw + i * B, 0, cnt, j0, kk, kwlo, kwhi, x, S);
+                if (ok)      ff_sweep<false>(fd + i * B, fw + i * B, 0, cnt, j0, kk, kwlo, kwhi, x, S);
                 else if (p0) sweep<false>(sd + i * B, sw + i * B, 0, cnt, j0, kk, kwlo, kwhi, R.dK, R.y, A);
                 else         sweep<true>(sd + i * B, sw + i * B, 0, cnt, j0, kk, kwlo, kwhi, R.dK, R.y, A);
             }
