@@ -654,7 +654,11 @@ __global__ void __launch_bounds__(up_threads<MODE>()) k_fmm_up(FmmDev pl, SrcArg
 // the weight of node q is sum_j f_j w_q / (u_j - x_q), f_j = (weight of source
 // j) / sum_k w_k / (u_j - x_k) (second barycentric formula; the sources are a
 // leaf's poles, or the nodes of a box's children).  First a lane per source for
-// f, then a lane per node.  The dipoles of zhat (lambda_j minus d_j, nearly
+// f, then a lane per node.  The secular sums (M_SEC) take blocks of 8
+// with three-float totals and f by a three-float quotient: with two floats all
+// through the weights' error grows with every level (against quadruple precision,
+// random leaves: 3.5e-15 there, 5.6e-15 three levels up, 2e-14 in the last root of
+// 60000 poles; so 1.6e-15 to 1.9e-15 on every level and 3e-15).  The dipoles of zhat (lambda_j minus d_j, nearly
 // cancelling) keep FP64 at the leaves: the moments' own difference recurrence.
 // Climb and counters as in k_fmm_up, which does the problems out of scale.
 // Measured (GB300, 4096 problems of 32..2048 poles): 1.9 + 1.9 + 2.3 -> 1.1 + 1.1 + 1.4 ms
@@ -694,12 +698,20 @@ __global__ void __launch_bounds__(128) k_fmm_up1(FmmDev pl, SrcArgs a)
             diff(u, sx[q], t, tl);
             ff_div(sw[q], t, tl, p, pr);
             ff_addto(D, p, pr);
-            if ((q & 7) == 7) ff_norm(D);
+            if ((q & 7) == 7) { if (MODE == M_SEC) ff_close3(D); else ff_norm(D); }
         }
-        ff_norm(D);
-        ff_f2 f;
-        ff_div(w, D.b, D.bl, f.x, f.y);
-        return f;
+        if (MODE != M_SEC) {
+            ff_norm(D);
+            ff_f2 f;
+            ff_div(w, D.b, D.bl, f.x, f.y);
+            return f;
+        }
+        ff_close3(D);
+        const ff_t3 f = ff_mul3({w.x, w.y, 0.0f}, ff_rcp3({D.s, D.sl, D.c}));
+        ff_f2 r;
+        r.x = f.a;
+        r.y = ff_add(f.b, f.c);
+        return r;
     };
     // weight of node lane from n sources (in units of the split weights)
     auto weight = [&](int n) {
@@ -711,9 +723,12 @@ __global__ void __launch_bounds__(128) k_fmm_up1(FmmDev pl, SrcArgs a)
             diff(su[warp][j], x, t, tl);
             ff_div(sf[warp][j], t, tl, p, pr);
             ff_addto(S, p, pr);
-            if ((j & 7) == 7) ff_norm(S);
+            if ((j & 7) == 7) { if (MODE == M_SEC) ff_close3(S); else ff_norm(S); }
         }
-        return ((double)S.b + (double)S.bl) * wq[min(lane, P - 1)];
+        if (MODE != M_SEC) return ((double)S.b + (double)S.bl) * wq[min(lane, P - 1)];
+        ff_close3(S);
+        ff_fold(S);
+        return ((double)S.s + (double)S.sl) * wq[min(lane, P - 1)];
     };
     const int64_t nleaf = pl.leaf_base[pl.nprob];
     for (;;) {
