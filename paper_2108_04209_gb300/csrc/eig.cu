@@ -205,6 +205,7 @@ __global__ void k_divide(const int32_t *__restrict__ nodes, int root, int r, con
 
 // ---------------------------------------------------------------------------
 constexpr int LEAF_T = 256;
+constexpr size_t LEAF_REC_MAX = (size_t)1 << 30;      // rotation records of small leaves (superdc_eig_plan)
 
 // Leaf eigendecompositions Dhat = D - U H U^T = Q diag(lambda) Q^T (Lemma 2.1).
 //   k_leaf_tri    one CTA per leaf: Dhat, Householder reduction to tridiagonal
@@ -1428,8 +1429,13 @@ superdc_status superdc_eig_plan(const superdc_hss *h, const superdc_opts *opts, 
     // (an FP64 instruction holds it for 64 cycles, whatever the lanes): then a warp
     // carries several leaves, one per lane.  GB300, own CTA / lane: 512 leaves of 32
     // rows 1.60 / 1.74 ms, of 80 11.3 / 11.9; 1024 of 48 7.2 / 5.6, of 64 12.3 / 10.0;
-    // 2048 of 32 5.8 / 3.4
-    w.leaf_batched = mm >= 96 || h->nleaves >= 6 * sdc_num_sms();
+    // 2048 of 32 5.8 / 3.4.  The lanes' rotation records (48 mm + 128 bytes a row, for
+    // the life of the plan) are what the own CTAs do without: beyond LEAF_REC_MAX,
+    // or where they do not fit, small leaves keep those
+    w.cap = 3 * (int64_t)mm * mm;
+    w.caps = 16 * (int64_t)mm;
+    const size_t rec = (size_t)h->nleaves * (w.cap * sizeof(*w.rot) + w.caps * sizeof(*w.hdr));
+    w.leaf_batched = mm >= 96 || (h->nleaves >= 6 * sdc_num_sms() && rec <= LEAF_REC_MAX);
     w.smem1 = (mm * (mm | 1) + std::max(mm * (size_t)r, mm)) * sizeof(double);
     w.smem2 = 2 * mm * 32 * sizeof(double);
     // leaves per warp of the QL chase: about one warp per scheduler (4 per SM)
@@ -1438,17 +1444,24 @@ superdc_status superdc_eig_plan(const superdc_hss *h, const superdc_opts *opts, 
     w.smem3 = mm * (mm | 1) * sizeof(double);
     w.smem4 = (mm * (mm | 1) + 4 * mm) * sizeof(double);
     w.smem5 = (size_t)LEAF_R * (mm | 1) * sizeof(double);
-    w.cap = 3 * (int64_t)mm * mm;
-    w.caps = 16 * (int64_t)mm;
     // leaves all of 128 rows: divide and conquer inside the leaves (blocks of
     // 32, two merge levels); its QL records fit the leaves' record buffers
     w.leaf_dc = (mm == DC_M);
     for (int L : h->leaves) w.leaf_dc = w.leaf_dc && h->size[L] == DC_M;
     const int64_t nblk = n / DC_B;
     if (w.leaf_batched) {
-        EIG_CHECK(dalloc(&w.rot, (size_t)h->nleaves * w.cap, &f->slabs));
-        EIG_CHECK(dalloc(&w.hdr, (size_t)h->nleaves * w.caps, &f->slabs));
-        EIG_CHECK(dalloc(&w.nsw, std::max<int64_t>(h->nleaves, w.leaf_dc ? nblk : 0), &f->slabs));
+        const size_t taken = f->slabs.size();
+        cudaError_t e = dalloc(&w.rot, (size_t)h->nleaves * w.cap, &f->slabs);
+        if (e == cudaSuccess) e = dalloc(&w.hdr, (size_t)h->nleaves * w.caps, &f->slabs);
+        if (e == cudaSuccess)
+            e = dalloc(&w.nsw, std::max<int64_t>(h->nleaves, w.leaf_dc ? nblk : 0), &f->slabs);
+        if (e == cudaErrorMemoryAllocation && mm < 96) {
+            cudaGetLastError();
+            for (; f->slabs.size() > taken; f->slabs.pop_back()) cudaFree(f->slabs.back());
+            w.leaf_batched = false;
+        } else {
+            EIG_CHECK(e);
+        }
     }
     if (w.leaf_dc) {
         std::vector<int64_t> bo(nblk), bm(nblk, DC_B), bq(nblk);
