@@ -411,7 +411,10 @@ struct SrcArgs {
     const double *X;
     int64_t ldx;
     int col0, nc;
-    const int32_t *only;                 // k_fmm_up: the problems with only[p] != 0 (out of scale); the others
+#ifdef SUPERDC_CHECK
+    int32_t *status;                     // index guards
+#endif
+    const int32_t *only;                 // the problems with only[p] != 0 (out of scale); the others
                                          // are k_fmm_up1's and k_cm_up's
 };
 
@@ -485,7 +488,7 @@ __device__ __forceinline__ void leaf_moments(const FmmDev &pl, const SrcArgs &a,
         const int js = Tb * B + (tid & 31);
         const bool in = js < jend;
         const double v = in ? (MODE == M_CT ? a.vhat[b0 + js] : a.bnorm[b0 + js]) : 0.0;
-        const int64_t row = in ? b0 + (MODE == M_CT ? a.src[b0 + js] : a.pinv[b0 + js]) : 0;
+        const int64_t row = in ? b0 + SDC_IDX(MODE == M_CT ? a.src[b0 + js] : a.pinv[b0 + js], a.off[p + 1] - b0, a.status) : 0;
 #pragma unroll 4
         for (int q = tid >> 5; q < nw; q += (int)blockDim.x >> 5)
             Wt[tid & 31][q] = in ? v * a.X[row + (int64_t)(a.col0 + q) * a.ldx] : 0.0;
@@ -1040,7 +1043,7 @@ __global__ void __launch_bounds__(FAR_NW * 32) k_fmm_far(FmmDev pl, const int64_
             for (int i = 0; i < cnt; i++) {
                 const int c = __ffsll((long long)mask) - 1;
                 mask &= mask - 1;
-                const int S = 2 * pl.near[pst + ((64 * sec + c) >> 1)] + (c & 1);
+                const int S = SDC_IDX(2 * pl.near[pst + ((64 * sec + c) >> 1)] + (c & 1), lev_nb(nb0, lane), o.status);
                 list[warp][pos + i] = ((lb + S) << 1) | (S < A ? 1 : 0);
             }
             __syncwarp();
@@ -1190,7 +1193,7 @@ template <int KER> constexpr int far_threads() { return far_cols<KER>() ? 256 : 
 template <int KER>
 __global__ void __launch_bounds__(far_threads<KER>())
 k_fmm_far64(FmmDev pl, const int32_t *__restrict__ mk, const int32_t *__restrict__ only, int nw, int sub,
-            double *__restrict__ coef, int nfield)
+            double *__restrict__ coef, int nfield, int32_t *word)
 {
     constexpr bool COLS = far_cols<KER>();
     constexpr int NF = far_fields<KER>(), NT = far_threads<KER>(), PARTS = NT / P, PAIRS = COLS ? 1 : 32;
@@ -1246,7 +1249,7 @@ k_fmm_far64(FmmDev pl, const int32_t *__restrict__ mk, const int32_t *__restrict
                                 int S = -1;
                                 bool in = false;
                                 if (cd < 2 * npn) {
-                                    S = 2 * pl.near[pst + (cd >> 1)] + (cd & 1);
+                                    S = SDC_IDX(2 * pl.near[pst + (cd >> 1)] + (cd & 1), nbl + 1, word);
                                     in = S < nbl && S != A && adm_box(pl, gb + S, gb + A, coarse);
                                 }
                                 const unsigned bal = __ballot_sync(0xffffffffu, in);
@@ -2291,7 +2294,8 @@ __global__ void k_cm_colmax(FactorView f, int64_t total, const double *__restric
         if (x >= f.off[0] && x < f.off[f.nprob]) {
             p = sdc_upper_index(f.off, f.nprob, x);
             const int64_t b0 = f.off[p];
-            if (x - b0 < f.mk[p]) e = ff_exp(X[b0 + (TRANS ? f.src[x] : f.pinv[x]) + (int64_t)col * ldx]);
+            if (x - b0 < f.mk[p])
+                e = ff_exp(X[b0 + SDC_IDX(TRANS ? f.src[x] : f.pinv[x], f.off[p + 1] - b0, f.status) + (int64_t)col * ldx]);
         }
         // one atomic per run of lanes with the same problem and column
         const unsigned grp = __match_any_sync(__activemask(), p * ncols + col);
@@ -2334,7 +2338,7 @@ __global__ void k_cm_slice(FactorView f, int64_t nchunk_rows, const double *__re
         if ((ch - first) * 16 >= m) continue;
         unsigned short dg[CM_D] = {0, 0, 0, 0, 0, 0, 0};
         if (col < nc && j < m && c.bad[lo] == 0) {
-            const int64_t r = b0 + (TRANS ? f.src[b0 + j] : f.pinv[b0 + j]);
+            const int64_t r = b0 + SDC_IDX(TRANS ? f.src[b0 + j] : f.pinv[b0 + j], f.off[lo + 1] - b0, f.status);
             const int e = cm_exp(c, lo, col0 + col);
             cm_digits(ldexp(X[r + (int64_t)(col0 + col) * ldx], -e), dg);
         }
@@ -2876,7 +2880,7 @@ k_cm_apply(FmmDev pl, FactorView f, const int64_t *__restrict__ tile_off, CmDev 
                 if (total < 0) break;
                 for (int t = threadIdx.x; t < total; t += 128) {
                     const int2 q = list[t];
-                    const int S = s_lb[q.y] + 2 * pl.near[s_pst[q.y] + (q.x >> 1)] + (q.x & 1);
+                    const int S = s_lb[q.y] + SDC_IDX(2 * pl.near[s_pst[q.y] + (q.x >> 1)] + (q.x & 1), lev_nb(nb0, q.y), f.status);
                     const int e = c.eb[gbx + S];
                     const double gap = fmax(s_lo[q.y] - pl.bhi[gbx + S], pl.blo[gbx + S] - s_hi[q.y]);
                     list[t] = make_int2(S, e);
@@ -3000,18 +3004,18 @@ k_cm_apply(FmmDev pl, FactorView f, const int64_t *__restrict__ tile_off, CmDev 
             if (TRANS) {
                 const int K = dorg[r] == dk[r] ? r : r + 1;
                 g0 = f.vhat[b0 + K] * rcp_nr2((dk[K] - dorg[r]) - eta[r]);
-                r0 = b0 + f.src[b0 + K];
+                r0 = b0 + SDC_IDX(f.src[b0 + K], f.off[p + 1] - b0, f.status);
             } else {
                 if (r < m - 1) {
                     g0 = f.bnorm[b0 + r] * rcp_nr2((dk[r] - dorg[r]) - eta[r]);
-                    r0 = b0 + f.pinv[b0 + r];
+                    r0 = b0 + SDC_IDX(f.pinv[b0 + r], f.off[p + 1] - b0, f.status);
                 }
                 if (r > 0) {
                     g1 = f.bnorm[b0 + r - 1] * rcp_nr2((dk[r] - dorg[r - 1]) - eta[r - 1]);
-                    r1 = b0 + f.pinv[b0 + r - 1];
+                    r1 = b0 + SDC_IDX(f.pinv[b0 + r - 1], f.off[p + 1] - b0, f.status);
                 }
                 g2 = f.bnorm[b0 + m - 1] * rcp_nr2((dk[r] - dorg[m - 1]) - eta[m - 1]);
-                r2 = b0 + f.pinv[b0 + m - 1];
+                r2 = b0 + SDC_IDX(f.pinv[b0 + m - 1], f.off[p + 1] - b0, f.status);
             }
         }
 #pragma unroll
@@ -3021,7 +3025,7 @@ k_cm_apply(FmmDev pl, FactorView f, const int64_t *__restrict__ tile_off, CmDev 
             const int64_t q0 = __shfl_sync(FULL, r0, src), q1 = __shfl_sync(FULL, r1, src), q2 = __shfl_sync(FULL, r2, src);
             if (r >= tend) continue;
             const double sc = TRANS ? f.bnorm[b0 + r] : f.vhat[b0 + r];
-            const int64_t row = b0 + (TRANS ? f.pinv[b0 + r] : f.src[b0 + r]);
+            const int64_t row = b0 + SDC_IDX(TRANS ? f.pinv[b0 + r] : f.src[b0 + r], f.off[p + 1] - b0, f.status);
 #pragma unroll
             for (int t = 0; t < TPW; t++)
 #pragma unroll
@@ -3164,7 +3168,7 @@ k_cm_last(FactorView f, const int64_t *__restrict__ tile_off, CmDev c, const dou
         row[threadIdx.x] = 0;
         if (i < m) {
             w[threadIdx.x] = f.vhat[b0 + i] * rcp_nr2((f.dk[b0 + i] - f.dorg[b0 + m - 1]) - f.eta[b0 + m - 1]);
-            row[threadIdx.x] = b0 + f.src[b0 + i];
+            row[threadIdx.x] = b0 + SDC_IDX(f.src[b0 + i], f.off[p + 1] - b0, f.status);
         }
         __syncthreads();
         for (int q = threadIdx.x; q < nc; q += CM_TR) {
@@ -3189,7 +3193,9 @@ k_cm_lastsum(FactorView f, const int64_t *__restrict__ tile_off, CmDev c, double
         double a = 0.0;
         for (int64_t t = tile_off[p] + lane; t < tile_off[p + 1]; t += 32) a += c.lastp[t * (CM_NT * 8) + q];
         for (int sh = 16; sh > 0; sh >>= 1) a += __shfl_xor_sync(0xffffffffu, a, sh);
-        if (lane == 0) Y[b0 + f.pinv[b0 + m - 1] + (int64_t)(col0 + q) * ldy] = f.bnorm[b0 + m - 1] * a;
+        if (lane == 0)
+            Y[b0 + SDC_IDX(f.pinv[b0 + m - 1], f.off[p + 1] - b0, f.status) + (int64_t)(col0 + q) * ldy] =
+                f.bnorm[b0 + m - 1] * a;
     }
 }
 
@@ -3232,6 +3238,9 @@ SrcArgs src_from_r1(const int64_t *off, const R1Out &o)
     SrcArgs a{};
     a.off = off; a.mk = o.mk; a.dk = o.dk; a.zk = o.zk; a.vhat = o.vhat; a.bnorm = o.bnorm;
     a.dorg = o.dorg; a.eta = o.eta; a.src = o.src; a.pinv = o.pinv; a.wsum = o.wsum;
+#ifdef SUPERDC_CHECK
+    a.status = o.status;
+#endif
     return a;
 }
 
@@ -3242,14 +3251,14 @@ SrcArgs src_from_r1(const int64_t *off, const R1Out &o)
 // 9.0, 2 boxes 30 and 10.7
 template <int KER>
 void launch_far64(const FmmPlan &pl, const int32_t *mk, const int32_t *only, int nw, double *coef, int nfield,
-                  cudaStream_t st)
+                  int32_t *word, cudaStream_t st)
 {
     const int64_t nsm = sdc_num_sms();
     const int sub = (pl.cap_leaves >> 3) >= 4 * nsm ? 3 : (pl.cap_leaves >> 2) >= nsm ? 2 : 1;
     const int64_t units = (pl.cap_leaves >> sub) + 1;
     const unsigned g = (unsigned)std::min<int64_t>(units, resident_grid<k_fmm_far64<KER>>(far_threads<KER>()));
     const dim3 grid(g, far_cols<KER>() && nw > 8 && units < 2 * nsm ? 2 : 1);
-    PROF_LAUNCH("fmm_far", st, k_fmm_far64<KER><<<grid, far_threads<KER>(), 0, st>>>(pl.dv, mk, only, nw, sub, coef, nfield));
+    PROF_LAUNCH("fmm_far", st, k_fmm_far64<KER><<<grid, far_threads<KER>(), 0, st>>>(pl.dv, mk, only, nw, sub, coef, nfield, word));
 }
 
 // far field of a one-column sum: node weights, then every leaf's series
@@ -3265,7 +3274,7 @@ superdc_status far_field(const FmmPlan &pl, const int64_t *off, const R1Out &o, 
     const int64_t want = (pl.cap_leaves + FAR_NW - 1) / FAR_NW;
     const unsigned g = (unsigned)std::min<int64_t>(want, resident_grid<k_fmm_far<KER>>(FAR_NW * 32));
     PROF_LAUNCH("fmm_far", st, k_fmm_far<KER><<<g, FAR_NW * 32, 0, st>>>(dv, off, o));
-    launch_far64<KER>(pl, o.mk, dv.ffbad, 1, dv.coef, NFIELD, st);
+    launch_far64<KER>(pl, o.mk, dv.ffbad, 1, dv.coef, NFIELD, o.status, st);
     return SUPERDC_OK;
 }
 
@@ -3471,6 +3480,10 @@ superdc_status columns(const FmmPlan &pl, const FactorView &f, int64_t total, co
     else PROF_LAUNCH("cauchy", st, k_cm_colmax<false><<<gr(total * ncols), 256, 0, st>>>(f, total, X, ldx, ncols, c));
     FmmDev dv = pl.dv;
     if (!pl.on) dv = FmmDev{};
+    int32_t *word = nullptr;                             // of the index guards (checked build)
+#ifdef SUPERDC_CHECK
+    word = f.status;
+#endif
     for (int c0 = 0; c0 < ncols; c0 += CM_NT * 8) {
         const int nc = std::min(CM_NT * 8, ncols - c0), nt = (nc + 7) / 8;
         if (trans) PROF_LAUNCH("cauchy", st, k_cm_slice<true><<<gr(rows * nt * 8), 256, 0, st>>>(f, rows, X, ldx, c0, nc, nt, c));
@@ -3492,10 +3505,13 @@ superdc_status columns(const FmmPlan &pl, const FactorView &f, int64_t total, co
             SrcArgs a{};
             a.off = f.off; a.mk = f.mk; a.dk = f.dk; a.vhat = f.vhat; a.bnorm = f.bnorm; a.dorg = f.dorg; a.eta = f.eta;
             a.src = f.src; a.pinv = f.pinv; a.X = X; a.ldx = ldx; a.col0 = c0; a.nc = nc; a.only = c.bad;
+#ifdef SUPERDC_CHECK
+            a.status = word;
+#endif
             if (trans) PROF_LAUNCH("fmm_up", st, k_fmm_up<M_CT><<<up_grid<M_CT>(), up_threads<M_CT>(), 0, st>>>(dv, a));
             else PROF_LAUNCH("fmm_up", st, k_fmm_up<M_CN><<<up_grid<M_CN>(), up_threads<M_CN>(), 0, st>>>(dv, a));
-            if (trans) launch_far64<K_1>(pl, f.mk, c.bad, nc, c.coef, CM_BC, st);
-            else launch_far64<K_1N>(pl, f.mk, c.bad, nc, c.coef, CM_BC, st);
+            if (trans) launch_far64<K_1>(pl, f.mk, c.bad, nc, c.coef, CM_BC, word, st);
+            else launch_far64<K_1N>(pl, f.mk, c.bad, nc, c.coef, CM_BC, word, st);
         }
         auto fn = nc <= 2 ? launch_rest<2> : nc <= 4 ? launch_rest<4> : nc <= 8 ? launch_rest<8> : nc <= 12 ? launch_rest<12>
                 : nc <= 16 ? launch_rest<16> : nc <= 20 ? launch_rest<20> : nc <= 24 ? launch_rest<24> : launch_rest<CM_BC>;
