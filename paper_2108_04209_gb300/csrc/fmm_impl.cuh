@@ -2050,19 +2050,10 @@ __global__ void __launch_bounds__(B) k_lowner_fmm(FmmDev pl, const int64_t *__re
             box_ch(pl.blo[g], pl.bhi[g], cT, hT);
             const double *cf = pl.coef + gl * NFIELD * P;
             const double u = (di - cT) * rcp_any(hT);
-            double Lf, v;
             int ex = pr.ex;
-            if (ok) {
-                // pn and pd are normal and positive: exponents apart, then the
-                // quotient's root without divide and square root
-                Lf = low_eval(cf, u) + (double)clenshawf<LOWN>((const float *)(cf + LOWN), ff_top(u, 0));
-                v = root_quot(pr.pn, pr.pd, ex);
-            } else {
-                Lf = clenshaw(cf, u);
-                double prod = pr.pn / pr.pd;
-                if (ex & 1) { prod *= 2.0; ex -= 1; }
-                v = sqrt(prod);
-            }
+            const double Lf = ok ? low_eval(cf, u) + (double)clenshawf<LOWN>((const float *)(cf + LOWN), ff_top(u, 0))
+                                 : clenshaw(cf, u);
+            double v = root_quot(pr.pn, pr.pd, ex);
             v = ldexp(v, ex / 2) * exp(0.5 * Lf);
             if (!isfinite(v)) sdc_latch(o.status, SUPERDC_DEV_NONFINITE);
             o.vhat[b0 + i] = (o.zk[b0 + i] < 0.0) ? -v : v;

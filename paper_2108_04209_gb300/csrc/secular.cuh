@@ -100,25 +100,12 @@ __device__ __forceinline__ double rsqrt_any(double q)
     return (e > 30 && e < 2016) ? rsqrt_nr(q) : 1.0 / sqrt(q);
 }
 
-// sqrt(n / d 2^ex) = result 2^(ex / 2), ex made even; n, d > 0
+// sqrt(n / d 2^ex) = result 2^(ex / 2), ex made even; n and d of one sign
 __device__ __forceinline__ double root_quot(double n, double d, int &ex)
 {
-    const int en = (__double2hiint(n) >> 20), ed = (__double2hiint(d) >> 20);     // sign included
-    if (!(en > 0 && en < 0x7FF && ed > 0 && ed < 0x7FF)) {
-        double q = n / d;
-        if (ex & 1) { q *= 2.0; ex -= 1; }
-        return sqrt(q);
-    }
-    ex += en - ed;
-    n = __hiloint2double((__double2hiint(n) & 0xFFFFF) | (1023 << 20), __double2loint(n));
-    d = __hiloint2double((__double2hiint(d) & 0xFFFFF) | (1023 << 20), __double2loint(d));
-    if (ex & 1) {
-        n = __hiloint2double(__double2hiint(n) + (1 << 20), __double2loint(n));
-        ex -= 1;
-    }
-    // q = n / d, then q q^(-1/2) and its residual
-    const double q = n * rcp_nr2(d), y = rsqrt_nr(q), s = q * y;
-    return fma(0.5 * y, fma(-s, s, q), s);
+    double q = n / d;
+    if (ex & 1) { q *= 2.0; ex -= 1; }
+    return sqrt(q);
 }
 
 // root of a*y^2 + b*y + c = 0 strictly inside (lo, hi), else the bracket middle
