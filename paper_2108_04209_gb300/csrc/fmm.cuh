@@ -64,8 +64,6 @@ struct FmmDev {
 struct FmmPlan {
     FmmDev dv{};
     int64_t cap_boxes = 0, cap_leaves = 0, cap_f = 0;
-    int lmax = 0;                          // upper bound on tree levels
-    int nb0max = 0;                        // upper bound on leaf boxes per problem
     int64_t total = 0;                     // extent of the row-indexed arrays
     bool on = false;                       // some problem may take the FMM path
     std::vector<void *> bufs;

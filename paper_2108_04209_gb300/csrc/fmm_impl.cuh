@@ -3,7 +3,7 @@
 // Geometry.  The kept poles d_0 < ... < d_{m-1} of a problem and the targets
 // (roots x_k in (d_k, d_{k+1}), eigenvalues lambda_j, or the poles themselves)
 // interlace (eq. (4.4)), so one index-based binary tree serves both: a leaf
-// box holds B = 32 consecutive indices (fmm32.cu), so d_k and x_k of the same k
+// box holds B = 32 consecutive indices, so d_k and x_k of the same k
 // always share a box (the paper's first design point), and every box carries the interval
 // [d_{i0}, d_{i1}] of its points (the last box ends at d_{m-1}).  The index
 // split adapts the boxes to clustered spectra (second design point); whether
@@ -54,15 +54,10 @@
 #include "prof.cuh"
 #include "tiles.cuh"
 
-#if !defined(FMM_BOX) || !defined(FMM_NS)
-#error "define FMM_BOX (indices per leaf box) and FMM_NS (namespace) before including fmm_impl.cuh"
-#endif
-
-namespace FMM_NS {
 namespace {
 
 constexpr int P = FMM_P;
-constexpr int B = FMM_BOX;
+constexpr int B = 32;             // indices per leaf box
 // admissibility: gap >= 0.75 x the larger width.  The nearest source then lies
 // at least 2.5 half-widths from either box's centre (Bernstein ellipse
 // rho >= 2.5 + sqrt(5.25) = 4.79): at 22 nodes the interpolated 1/(s-t) stays at
@@ -540,7 +535,7 @@ __device__ __forceinline__ void m2m_box(const FmmDev &pl, int64_t p, int nb0, in
         const int64_t gc = gcb + 2 * b + ci;
         double cc, hc;
         box_ch(pl.blo[gc], pl.bhi[gc], cc, hc);
-        const double v = fma(hc * ihP, xq[q], (cc - cP) * ihP);    // as scale and shift (see l2l_box)
+        const double v = fma(hc * ihP, xq[q], (cc - cP) * ihP);    // as scale and shift (see k_fmm_far64)
         double t0 = 1.0, t1 = v;
         Tv[t][0] = 1.0;
         Tv[t][1] = v;
@@ -585,8 +580,9 @@ __device__ __forceinline__ void m2m_box(const FmmDev &pl, int64_t p, int nb0, in
 // the same arithmetic as a level-by-level pass.  The counter is reset by the
 // child that consumes it, ready for the next far field built on the plan.
 // Threads and staged columns of the upward pass: the one-column far fields
-// (secular, b, Loewner) take 64 threads (one per source of a box of 64, and
-// the 2P children's nodes of a box), the Cauchy-like ones 128 and WMAX columns.
+// (secular, b, Loewner) take 64 threads (the 2P children's nodes of a box), the
+// Cauchy-like ones 256 and WMAX columns (64 columns through 20000 poles, both ways:
+// 128 threads 2.56 ms, 256 2.19).
 template <int MODE> constexpr bool up_wide() { return MODE == M_CT || MODE == M_CN; }
 template <int MODE> constexpr int up_threads() { return up_wide<MODE>() ? 256 : 64; }
 template <int MODE> constexpr int up_cols() { return up_wide<MODE>() ? WMAX : 1; }
@@ -1411,9 +1407,8 @@ __global__ void k_ff_prep(int64_t nprob, const int64_t *__restrict__ off, int64_
 }
 
 // ---------------------------------------------------------------------------
-// Secular roots of the FMM problems, one warp per leaf box: with boxes of 64
-// a lane takes the next root of the box when its root has converged (the
-// box's roots share the near list).  The near boxes' poles and weights (fixed
+// Secular roots of the FMM problems, one warp per leaf box (its 32 roots share
+// the near list).  The near boxes' poles and weights (fixed
 // during the iteration) are staged in shared memory once per box; each sweep
 // sums them with shifted differences and evaluates the four far-field
 // expansions at x = d_K + y.  Once no root is left to hand out and fewer than
@@ -3296,7 +3291,7 @@ void launch_apply(bool trans, const FmmDev &dv, const FactorView &f, const int64
 }  // namespace
 
 
-superdc_status plan(FmmPlan &pl, int64_t nprob, const int64_t *off, int64_t total, int64_t max_m,
+superdc_status fmm_plan(FmmPlan &pl, int64_t nprob, const int64_t *off, int64_t total, int64_t max_m,
                         const int32_t *mk, const double *dk, int min_m, int ncol, int32_t *used, bool step,
                     cudaStream_t st)
 {
@@ -3312,9 +3307,6 @@ superdc_status plan(FmmPlan &pl, int64_t nprob, const int64_t *off, int64_t tota
     pl.cap_f = nf_cap;
     pl.cap_leaves = total / B + nf_cap + 1;
     pl.cap_boxes = 2 * pl.cap_leaves + nf_cap * 40;
-    const int nb0max = (int)((mm + B - 1) / B);
-    pl.nb0max = nb0max;
-    pl.lmax = lev_count(nb0max);
     ncol = std::max(1, std::min(ncol, WMAX));
     FmmDev &d = pl.dv;
     d.nprob = nprob;
@@ -3382,14 +3374,14 @@ superdc_status plan(FmmPlan &pl, int64_t nprob, const int64_t *off, int64_t tota
     return SUPERDC_OK;
 }
 
-void free_plan(FmmPlan &pl, cudaStream_t st)
+void fmm_free(FmmPlan &pl, cudaStream_t st)
 {
     for (void *p : pl.bufs) cudaFreeAsync(p, st);
     pl.bufs.clear();
     pl.on = false;
 }
 
-superdc_status secular(const FmmPlan &pl, const int64_t *off, const R1Out &o, double stop_c, int max_iter,
+superdc_status fmm_secular(const FmmPlan &pl, const int64_t *off, const R1Out &o, double stop_c, int max_iter,
                            cudaStream_t st)
 {
     if (!pl.on) return SUPERDC_OK;
@@ -3420,7 +3412,7 @@ superdc_status secular(const FmmPlan &pl, const int64_t *off, const R1Out &o, do
     return SUPERDC_OK;
 }
 
-superdc_status lowner(const FmmPlan &pl, const int64_t *off, const R1Out &o, cudaStream_t st)
+superdc_status fmm_lowner(const FmmPlan &pl, const int64_t *off, const R1Out &o, cudaStream_t st)
 {
     if (!pl.on) return SUPERDC_OK;
     far_field<M_LOW, K_LOG>(pl, off, o, st);
@@ -3429,7 +3421,7 @@ superdc_status lowner(const FmmPlan &pl, const int64_t *off, const R1Out &o, cud
     return SUPERDC_OK;
 }
 
-superdc_status bnorm(const FmmPlan &pl, const int64_t *off, const R1Out &o, cudaStream_t st)
+superdc_status fmm_bnorm(const FmmPlan &pl, const int64_t *off, const R1Out &o, cudaStream_t st)
 {
     if (!pl.on) return SUPERDC_OK;
     far_field<M_BN, K_2>(pl, off, o, st);
@@ -3439,7 +3431,7 @@ superdc_status bnorm(const FmmPlan &pl, const int64_t *off, const R1Out &o, cuda
     return SUPERDC_OK;
 }
 
-superdc_status columns(const FmmPlan &pl, const FactorView &f, int64_t total, const int64_t *tile_off,
+superdc_status fmm_columns(const FmmPlan &pl, const FactorView &f, int64_t total, const int64_t *tile_off,
                        const double *X, int64_t ldx, double *Y, int64_t ldy, int ncols, bool trans, cudaStream_t st)
 {
     const int ntmax = std::min(CM_NT, (ncols + 7) / 8);
@@ -3511,5 +3503,3 @@ superdc_status columns(const FmmPlan &pl, const FactorView &f, int64_t total, co
     SDC_CHECK(cudaGetLastError());
     return SUPERDC_OK;
 }
-
-}  // namespace FMM_NS

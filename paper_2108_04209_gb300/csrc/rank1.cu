@@ -19,8 +19,12 @@
 //   k_bnorm     -- eq. (4.27) with the shifted entries of eq. (4.28).
 //   k_merge     -- new eigenvalues (eq. (4.21)) and deflated values sorted by
 //                  (value, input index).
-// Everything is FP64: the root iteration, the shifted differences and zhat
-// need it for stability.
+// Inputs, results and what decides their accuracy are FP64: the terms of the two
+// poles next to a root, its function value and iterate, the last root, the origin's
+// term of b, the factors of zhat next to the target, and everything of a problem out
+// of scale.  The other terms are split into FP32 or integer parts that carry FP64's
+// accuracy or more (split.cuh); only the step's model (derivatives, guess) is single
+// precision.
 #include "common.cuh"
 #include "rank1.cuh"
 #include "prof.cuh"
