@@ -535,7 +535,7 @@ __device__ __forceinline__ void m2m_box(const FmmDev &pl, int64_t p, int nb0, in
         const int64_t gc = gcb + 2 * b + ci;
         double cc, hc;
         box_ch(pl.blo[gc], pl.bhi[gc], cc, hc);
-        const double v = fma(hc * ihP, xq[q], (cc - cP) * ihP);    // as scale and shift (see k_fmm_far64)
+        const double v = fma(hc * ihP, xq[q], (cc - cP) * ihP);    // as scale and shift (see far64)
         double t0 = 1.0, t1 = v;
         Tv[t][0] = 1.0;
         Tv[t][1] = v;
@@ -972,195 +972,6 @@ __device__ __forceinline__ double far_split(const FmmDev &pl, int64_t gl, double
     return low_eval(cf, u);
 }
 
-template <int KER>
-__global__ void __launch_bounds__(FAR_NW * 32) k_fmm_far(FmmDev pl, const int64_t *__restrict__ off, R1Out o)
-{
-    __shared__ double Tx[P * P], xq[P], Mt[LOWN * LOWN];
-    __shared__ float Tf[(KER == K_SEC) ? P * P : 1];
-    __shared__ ff_logtab lt[(KER == K_LOG) ? 128 : 1];
-    __shared__ ff_f4 sp[FAR_NW][P];
-    __shared__ ff_f2 sw[FAR_NW][P];
-    __shared__ int list[FAR_NW][32 * FAR_TAKE];
-    __shared__ double sF[FAR_NW][P + 2];
-    __shared__ float fL[FAR_NW][P], fR[FAR_NW][P];
-    const unsigned FULL = 0xffffffffu;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, q = min(lane, P - 1);
-    cheb_tables(xq, Tx);
-    mono_table(Mt);
-    if (KER == K_LOG)
-        for (int i = threadIdx.x; i < 128; i += blockDim.x) {
-            const float c = ff_logc(i);
-            const double v = -log((double)c);
-            lt[i] = {c, (float)v, (float)(v - (double)(float)v)};
-        }
-    __syncthreads();
-    if (KER == K_SEC)
-        for (int i = threadIdx.x; i < P * P; i += blockDim.x) Tf[i] = (float)Tx[i];
-    __syncthreads();
-    const int64_t nleaf = pl.leaf_base[pl.nprob];
-    for (int64_t gl = (int64_t)blockIdx.x * FAR_NW + warp; gl < nleaf; gl += (int64_t)gridDim.x * FAR_NW) {
-        const int64_t p = sdc_upper_index(pl.leaf_base, pl.nprob, gl);
-        if (pl.fslot[p] < 0 || pl.ffbad[p]) continue;        // out of scale: k_fmm_far64
-        const int64_t b0 = off[p], g0 = pl.box_base[p];
-        const int m = o.mk[p], nb0 = (m + B - 1) / B, L = lev_count(nb0);
-        const int Tb = (int)(gl - pl.leaf_base[p]);
-        const FfScale fs = ff_scale(o.dk[b0], o.dk[b0 + m - 1], o.wsum[p]);
-        double cT, hT;
-        box_ch(pl.blo[g0 + Tb], pl.bhi[g0 + Tb], cT, hT);
-        const ff_f4 x = ff_point(cT, hT * xq[q], fs), xc = ff_pole(cT, fs);
-        FfAcc AL = {}, AR = {}, AC = {};          // AC: K_LOG, the sum at the centre
-        // lane l: the interaction list of the leaf's ancestor on level l
-        int A = 0, npn = 0, sec = 0, lb = 0;
-        int64_t pst = 0;
-        unsigned long long mask = 0;
-        if (lane < L - 1 && pl.nnear[g0 + Tb] >= 0) {
-            A = Tb >> lane;
-            lb = lev_base(nb0, lane);
-            const int64_t gP = g0 + lev_base(nb0, lane + 1) + (A >> 1);
-            npn = pl.nnear[gP];
-            pst = pl.nstart[gP];
-            mask = pl.amask[g0 + lb + A];
-        }
-        int npair = 0;
-        while (__any_sync(FULL, mask != 0 || 64 * (sec + 1) < 2 * npn)) {
-            if (mask == 0 && 64 * (sec + 1) < 2 * npn) {
-                sec++;
-                mask = adm_mask(pl, g0 + lb, lev_nb(nb0, lane), A, pst, npn, sec, false);     // coarse problems are out of scale
-            }
-            const int cnt = min(FAR_TAKE, __popcll(mask));
-            int pos = cnt;
-            for (int s = 1; s < 32; s <<= 1) {
-                const int v = __shfl_up_sync(FULL, pos, s);
-                if (lane >= s) pos += v;
-            }
-            const int total = __shfl_sync(FULL, pos, 31);
-            pos -= cnt;
-            __syncwarp();
-            for (int i = 0; i < cnt; i++) {
-                const int c = __ffsll((long long)mask) - 1;
-                mask &= mask - 1;
-                const int S = SDC_IDX(2 * pl.near[pst + ((64 * sec + c) >> 1)] + (c & 1), lev_nb(nb0, lane), o.status);
-                list[warp][pos + i] = ((lb + S) << 1) | (S < A ? 1 : 0);
-            }
-            __syncwarp();
-            npair += total;
-            ff_f4 v = {};
-            ff_f2 w = {};
-            if (total > 0) {
-                const int64_t t = (g0 + (list[warp][0] >> 1)) * P + q;
-                v = pl.npos[t];
-                w = pl.nwt[t];
-            }
-            for (int i = 0; i < total; i++) {
-                const int e = list[warp][i];
-                const bool left = e & 1;
-                __syncwarp();
-                if (lane < P) { sp[warp][lane] = v; sw[warp][lane] = w; }
-                __syncwarp();
-                const ff_f4 vq = v;
-                const ff_f2 wq = w;
-                if (i + 1 < total) {                         // the next pair's nodes, ahead of their use
-                    const int64_t t = (g0 + (list[warp][i + 1] >> 1)) * P + q;
-                    v = pl.npos[t];
-                    w = pl.nwt[t];
-                }
-                FfAcc S = (KER == K_SEC && !left) ? AR : AL;
-                // unrolled as a whole: two nodes at a time held a small launch back (90 steps of n =
-                // 131072: 12.4 -> 11.2 ms for zhat)
-#pragma unroll
-                for (int j = 0; j < P; j++) {
-                    float t, tp, tq2;
-                    if (KER == K_2) ff_term2(sp[warp][j], sw[warp][j], x, t, tp);
-                    else ff_term(sp[warp][j], sw[warp][j], x, t, tp, tq2);
-                    ff_addto(S, t, tp);
-                    if ((j & 7) == 7) ff_norm(S);
-                }
-                if (KER == K_SEC) ff_close3(S); else ff_close(S);
-                if (KER == K_SEC && !left) AR = S; else AL = S;
-                if (KER == K_LOG) {
-                    // node q of the source against the centre; the box's weights sum
-                    // to zero, so one exponent per box drops out
-                    float t, tl2, y, yl;
-                    ff_diff(vq, xc, t, tl2);
-                    if (t < 0.0f) { t = -t; tl2 = -tl2; }
-                    const int e0 = __shfl_sync(FULL, ff_fexp(t), 0);
-                    ff_log(t, tl2, e0, lt, y, yl);
-                    float pr, pe;
-                    ff_two_mul(wq.x, y, pr, pe);
-                    pe = ff_fma(wq.y, y, ff_fma(wq.x, yl, pe));
-                    if (lane < P) ff_addto(AC, pr, pe);
-                    ff_close(AC);
-                }
-            }
-        }
-        // the leaf's coefficients
-        double *cf = pl.coef + gl * NFIELD * P;
-        const double c1 = ff_pow2(fs.kk + fs.kw);
-        const double fn = (lane == 0) ? 1.0 / P : 2.0 / P;
-        auto series = [&](double F) {              // coefficient lane of the series with node values F
-            __syncwarp();
-            if (lane < P) sF[warp][lane] = F;
-            __syncwarp();
-            double a = 0.0;
-            for (int j = 0; j < P; j++) a = fma(sF[warp][j], Tx[j * P + q], a);
-            return a * fn;
-        };
-        if (KER == K_SEC) {
-            // psi + phi in FP64; psi and the two derivatives in single precision,
-            // scaled like the near sums (ff_collect)
-            const double a = series(((double)AL.s + ((double)AL.sl + (double)AL.c) + ((double)AR.s + ((double)AR.sl + (double)AR.c))) * c1);
-            if (lane < P) { fL[warp][lane] = AL.s; fR[warp][lane] = AR.s; }
-            __syncwarp();
-            float l = 0.0f, r = 0.0f;
-            for (int j = 0; j < P; j++) {
-                l = fmaf(fL[warp][j], Tf[j * P + q], l);
-                r = fmaf(fR[warp][j], Tf[j * P + q], r);
-            }
-            l *= (float)fn;
-            r *= (float)fn;
-            __syncwarp();
-            if (lane < P) { fL[warp][lane] = l; fR[warp][lane] = r; }
-            __syncwarp();
-            const float ih = (float)(1.0 / (hT * ff_pow2(fs.kk)));
-            float dl = 0.0f, dr = 0.0f;
-            for (int n = q + 1; n < P; n += 2) {
-                dl = fmaf((float)(2 * n), fL[warp][n], dl);
-                dr = fmaf((float)(2 * n), fR[warp][n], dr);
-            }
-            if (q == 0) { dl *= 0.5f; dr *= 0.5f; }
-            if (lane < P) {
-                float *ff = (float *)(cf + P);
-                ff[lane] = l;
-                ff[P + lane] = dl * ih;
-                ff[2 * P + lane] = dr * ih;
-            }
-            store_series(a, ff_pow2(-(fs.kk + fs.kw)), Mt, sF[warp], cf);
-        } else if (KER == K_2) {
-            store_series(series((double)AL.s + (double)AL.sl), 1.0, Mt, sF[warp], cf);
-        } else {
-            // F' -> antiderivative G = sum B_k T_k (k = 1..P; T_P vanishes at the
-            // nodes but not at 0), F(u) = F(centre) + h (G(u) - G(0))
-            const double a = series(-((double)AL.s + (double)AL.sl) * ff_pow2(fs.kk));
-            double c = (double)AC.s + (double)AC.sl;
-            if (lane >= P) c = 0.0;
-            for (int s = 16; s > 0; s >>= 1) c += __shfl_xor_sync(FULL, c, s);
-            __syncwarp();
-            if (lane < P + 2) sF[warp][lane] = (lane < P) ? a : 0.0;
-            __syncwarp();
-            double bk = 0.0;                       // lane k holds B_k
-            if (lane == 1) bk = sF[warp][0] - 0.5 * sF[warp][2];
-            else if (lane >= 2 && lane <= P) bk = (sF[warp][lane - 1] - sF[warp][lane + 1]) * (0.5 / lane);
-            double g0s = (lane >= 2 && lane <= P && !(lane & 1)) ? ((lane & 2) ? -bk : bk) : 0.0;   // T_k(0)
-            for (int s = 16; s > 0; s >>= 1) g0s += __shfl_xor_sync(FULL, g0s, s);
-            const double a2 = (lane == 0) ? c - hT * g0s : hT * bk;
-            store_series(a2, 1.0, Mt, sF[warp], cf);
-        }
-        if (pl.flops && lane == 0 && npair)
-            atomicAdd(pl.flops, (unsigned long long)npair * P * (P * (KER == K_SEC ? 7 : 5) + (KER == K_LOG ? 3 : 0)) +
-                                    2 * P * P);
-    }
-}
-
 // ---------------------------------------------------------------------------
 // Far fields of the problems out of the split arithmetic's scale, in FP64 (poles
 // closer than its positions resolve): series of P coefficients per field and leaf
@@ -1168,7 +979,7 @@ __global__ void __launch_bounds__(FAR_NW * 32) k_fmm_far(FmmDev pl, const int64_
 // lists of itself and of every ancestor at its own nodes, the boxes below it their
 // own lists, plus the parent's series at their nodes; the series of the current
 // path stay in shared memory.  About 7 + 3.5 levels / 2^sub box pairs per leaf, as by
-// translation level by level but in one launch (summing every ancestor's list at
+// translation level by level but in one launch (none for the one-column sums; summing every ancestor's list at
 // the leaf: 3.5 per level).  Fields: K_SEC the sums w/(s-t) to the left and right,
 // then w/(s-t)^2; K_2 w/(s-t)^2; K_LOG w log|s-t| as its derivative at the nodes,
 // integrated in coefficient space, plus the sum itself at the box's centre; K_1 and
@@ -1187,9 +998,8 @@ template <int KER> constexpr int far_fields() { return KER == K_SEC ? 4 : far_co
 template <int KER> constexpr int far_threads() { return far_cols<KER>() ? 256 : 128; }
 
 template <int KER>
-__global__ void __launch_bounds__(far_threads<KER>())
-k_fmm_far64(FmmDev pl, const int32_t *__restrict__ mk, const int32_t *__restrict__ only, int nw, int sub,
-            double *__restrict__ coef, int nfield, int32_t *word)
+__device__ __noinline__ void far64(const FmmDev &pl, const int32_t *__restrict__ mk, const int32_t *__restrict__ only,
+                                   int nw, int sub, double *__restrict__ coef, int nfield, int32_t *word)
 {
     constexpr bool COLS = far_cols<KER>();
     constexpr int NF = far_fields<KER>(), NT = far_threads<KER>(), PARTS = NT / P, PAIRS = COLS ? 1 : 32;
@@ -1202,7 +1012,7 @@ k_fmm_far64(FmmDev pl, const int32_t *__restrict__ mk, const int32_t *__restrict
     __shared__ double red[COLS ? 1 : NF][COLS ? 1 : PARTS][P];
     __shared__ int s_list[32], s_nlist;
     __shared__ double s_ctr[4];
-    if (only[pl.nprob] == 0) return;                     // no problem out of scale
+    __syncthreads();
     cheb_tables(xq, Tx);
     // columns f0 .. f0 + nf - 1 of the nw (blockIdx.y: halves)
     const int f0 = COLS ? (int)((int64_t)nw * blockIdx.y / gridDim.y) : 0;
@@ -1373,6 +1183,207 @@ k_fmm_far64(FmmDev pl, const int32_t *__restrict__ mk, const int32_t *__restrict
                            (int64_t)(2 << top) * 4 * P * P * nf);
         }
     }
+}
+
+// the columns' kernel (the one-column sums': at the end of k_fmm_far)
+template <int KER>
+__global__ void __launch_bounds__(far_threads<KER>())
+k_fmm_far64(FmmDev pl, const int32_t *__restrict__ mk, const int32_t *__restrict__ only, int nw, int sub,
+            double *__restrict__ coef, int nfield, int32_t *word)
+{
+    if (only[pl.nprob] == 0) return;                     // no problem out of scale
+    far64<KER>(pl, mk, only, nw, sub, coef, nfield, word);
+}
+
+template <int KER>
+__global__ void __launch_bounds__(FAR_NW * 32, 5) k_fmm_far(FmmDev pl, const int64_t *__restrict__ off, R1Out o, int sub)
+{
+    __shared__ double Tx[P * P], xq[P], Mt[LOWN * LOWN];
+    __shared__ float Tf[(KER == K_SEC) ? P * P : 1];
+    __shared__ ff_logtab lt[(KER == K_LOG) ? 128 : 1];
+    __shared__ ff_f4 sp[FAR_NW][P];
+    __shared__ ff_f2 sw[FAR_NW][P];
+    __shared__ int list[FAR_NW][32 * FAR_TAKE];
+    __shared__ double sF[FAR_NW][P + 2];
+    __shared__ float fL[FAR_NW][P], fR[FAR_NW][P];
+    const unsigned FULL = 0xffffffffu;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, q = min(lane, P - 1);
+    cheb_tables(xq, Tx);
+    mono_table(Mt);
+    if (KER == K_LOG)
+        for (int i = threadIdx.x; i < 128; i += blockDim.x) {
+            const float c = ff_logc(i);
+            const double v = -log((double)c);
+            lt[i] = {c, (float)v, (float)(v - (double)(float)v)};
+        }
+    __syncthreads();
+    if (KER == K_SEC)
+        for (int i = threadIdx.x; i < P * P; i += blockDim.x) Tf[i] = (float)Tx[i];
+    __syncthreads();
+    const int64_t nleaf = pl.leaf_base[pl.nprob];
+    for (int64_t gl = (int64_t)blockIdx.x * FAR_NW + warp; gl < nleaf; gl += (int64_t)gridDim.x * FAR_NW) {
+        const int64_t p = sdc_upper_index(pl.leaf_base, pl.nprob, gl);
+        if (pl.fslot[p] < 0 || pl.ffbad[p]) continue;        // out of scale: far64
+        const int64_t b0 = off[p], g0 = pl.box_base[p];
+        const int m = o.mk[p], nb0 = (m + B - 1) / B, L = lev_count(nb0);
+        const int Tb = (int)(gl - pl.leaf_base[p]);
+        const FfScale fs = ff_scale(o.dk[b0], o.dk[b0 + m - 1], o.wsum[p]);
+        double cT, hT;
+        box_ch(pl.blo[g0 + Tb], pl.bhi[g0 + Tb], cT, hT);
+        const ff_f4 x = ff_point(cT, hT * xq[q], fs), xc = ff_pole(cT, fs);
+        FfAcc AL = {}, AR = {}, AC = {};          // AC: K_LOG, the sum at the centre
+        // lane l: the interaction list of the leaf's ancestor on level l
+        int A = 0, npn = 0, sec = 0, lb = 0;
+        int64_t pst = 0;
+        unsigned long long mask = 0;
+        if (lane < L - 1 && pl.nnear[g0 + Tb] >= 0) {
+            A = Tb >> lane;
+            lb = lev_base(nb0, lane);
+            const int64_t gP = g0 + lev_base(nb0, lane + 1) + (A >> 1);
+            npn = pl.nnear[gP];
+            pst = pl.nstart[gP];
+            mask = pl.amask[g0 + lb + A];
+        }
+        int npair = 0;
+        while (__any_sync(FULL, mask != 0 || 64 * (sec + 1) < 2 * npn)) {
+            if (mask == 0 && 64 * (sec + 1) < 2 * npn) {
+                sec++;
+                mask = adm_mask(pl, g0 + lb, lev_nb(nb0, lane), A, pst, npn, sec, false);     // coarse problems are out of scale
+            }
+            const int cnt = min(FAR_TAKE, __popcll(mask));
+            int pos = cnt;
+            for (int s = 1; s < 32; s <<= 1) {
+                const int v = __shfl_up_sync(FULL, pos, s);
+                if (lane >= s) pos += v;
+            }
+            const int total = __shfl_sync(FULL, pos, 31);
+            pos -= cnt;
+            __syncwarp();
+            for (int i = 0; i < cnt; i++) {
+                const int c = __ffsll((long long)mask) - 1;
+                mask &= mask - 1;
+                const int S = SDC_IDX(2 * pl.near[pst + ((64 * sec + c) >> 1)] + (c & 1), lev_nb(nb0, lane), o.status);
+                list[warp][pos + i] = ((lb + S) << 1) | (S < A ? 1 : 0);
+            }
+            __syncwarp();
+            npair += total;
+            ff_f4 v = {};
+            ff_f2 w = {};
+            if (total > 0) {
+                const int64_t t = (g0 + (list[warp][0] >> 1)) * P + q;
+                v = pl.npos[t];
+                w = pl.nwt[t];
+            }
+            for (int i = 0; i < total; i++) {
+                const int e = list[warp][i];
+                const bool left = e & 1;
+                __syncwarp();
+                if (lane < P) { sp[warp][lane] = v; sw[warp][lane] = w; }
+                __syncwarp();
+                const ff_f4 vq = v;
+                const ff_f2 wq = w;
+                if (i + 1 < total) {                         // the next pair's nodes, ahead of their use
+                    const int64_t t = (g0 + (list[warp][i + 1] >> 1)) * P + q;
+                    v = pl.npos[t];
+                    w = pl.nwt[t];
+                }
+                FfAcc S = (KER == K_SEC && !left) ? AR : AL;
+                // unrolled as a whole, with registers for five CTAs per SM: two nodes at a time wait
+                // for their loads (zhat of 4096 problems 1.53 -> 1.41 ms, of the 90 steps of n = 131072
+                // 10.6 -> 9.6)
+#pragma unroll
+                for (int j = 0; j < P; j++) {
+                    float t, tp, tq2;
+                    if (KER == K_2) ff_term2(sp[warp][j], sw[warp][j], x, t, tp);
+                    else ff_term(sp[warp][j], sw[warp][j], x, t, tp, tq2);
+                    ff_addto(S, t, tp);
+                    if ((j & 7) == 7) ff_norm(S);
+                }
+                if (KER == K_SEC) ff_close3(S); else ff_close(S);
+                if (KER == K_SEC && !left) AR = S; else AL = S;
+                if (KER == K_LOG) {
+                    // node q of the source against the centre; the box's weights sum
+                    // to zero, so one exponent per box drops out
+                    float t, tl2, y, yl;
+                    ff_diff(vq, xc, t, tl2);
+                    if (t < 0.0f) { t = -t; tl2 = -tl2; }
+                    const int e0 = __shfl_sync(FULL, ff_fexp(t), 0);
+                    ff_log(t, tl2, e0, lt, y, yl);
+                    float pr, pe;
+                    ff_two_mul(wq.x, y, pr, pe);
+                    pe = ff_fma(wq.y, y, ff_fma(wq.x, yl, pe));
+                    if (lane < P) ff_addto(AC, pr, pe);
+                    ff_close(AC);
+                }
+            }
+        }
+        // the leaf's coefficients
+        double *cf = pl.coef + gl * NFIELD * P;
+        const double c1 = ff_pow2(fs.kk + fs.kw);
+        const double fn = (lane == 0) ? 1.0 / P : 2.0 / P;
+        auto series = [&](double F) {              // coefficient lane of the series with node values F
+            __syncwarp();
+            if (lane < P) sF[warp][lane] = F;
+            __syncwarp();
+            double a = 0.0;
+            for (int j = 0; j < P; j++) a = fma(sF[warp][j], Tx[j * P + q], a);
+            return a * fn;
+        };
+        if (KER == K_SEC) {
+            // psi + phi in FP64; psi and the two derivatives in single precision,
+            // scaled like the near sums (ff_collect)
+            const double a = series(((double)AL.s + ((double)AL.sl + (double)AL.c) + ((double)AR.s + ((double)AR.sl + (double)AR.c))) * c1);
+            if (lane < P) { fL[warp][lane] = AL.s; fR[warp][lane] = AR.s; }
+            __syncwarp();
+            float l = 0.0f, r = 0.0f;
+            for (int j = 0; j < P; j++) {
+                l = fmaf(fL[warp][j], Tf[j * P + q], l);
+                r = fmaf(fR[warp][j], Tf[j * P + q], r);
+            }
+            l *= (float)fn;
+            r *= (float)fn;
+            __syncwarp();
+            if (lane < P) { fL[warp][lane] = l; fR[warp][lane] = r; }
+            __syncwarp();
+            const float ih = (float)(1.0 / (hT * ff_pow2(fs.kk)));
+            float dl = 0.0f, dr = 0.0f;
+            for (int n = q + 1; n < P; n += 2) {
+                dl = fmaf((float)(2 * n), fL[warp][n], dl);
+                dr = fmaf((float)(2 * n), fR[warp][n], dr);
+            }
+            if (q == 0) { dl *= 0.5f; dr *= 0.5f; }
+            if (lane < P) {
+                float *ff = (float *)(cf + P);
+                ff[lane] = l;
+                ff[P + lane] = dl * ih;
+                ff[2 * P + lane] = dr * ih;
+            }
+            store_series(a, ff_pow2(-(fs.kk + fs.kw)), Mt, sF[warp], cf);
+        } else if (KER == K_2) {
+            store_series(series((double)AL.s + (double)AL.sl), 1.0, Mt, sF[warp], cf);
+        } else {
+            // F' -> antiderivative G = sum B_k T_k (k = 1..P; T_P vanishes at the
+            // nodes but not at 0), F(u) = F(centre) + h (G(u) - G(0))
+            const double a = series(-((double)AL.s + (double)AL.sl) * ff_pow2(fs.kk));
+            double c = (double)AC.s + (double)AC.sl;
+            if (lane >= P) c = 0.0;
+            for (int s = 16; s > 0; s >>= 1) c += __shfl_xor_sync(FULL, c, s);
+            __syncwarp();
+            if (lane < P + 2) sF[warp][lane] = (lane < P) ? a : 0.0;
+            __syncwarp();
+            double bk = 0.0;                       // lane k holds B_k
+            if (lane == 1) bk = sF[warp][0] - 0.5 * sF[warp][2];
+            else if (lane >= 2 && lane <= P) bk = (sF[warp][lane - 1] - sF[warp][lane + 1]) * (0.5 / lane);
+            double g0s = (lane >= 2 && lane <= P && !(lane & 1)) ? ((lane & 2) ? -bk : bk) : 0.0;   // T_k(0)
+            for (int s = 16; s > 0; s >>= 1) g0s += __shfl_xor_sync(FULL, g0s, s);
+            const double a2 = (lane == 0) ? c - hT * g0s : hT * bk;
+            store_series(a2, 1.0, Mt, sF[warp], cf);
+        }
+        if (pl.flops && lane == 0 && npair)
+            atomicAdd(pl.flops, (unsigned long long)npair * P * (P * (KER == K_SEC ? 7 : 5) + (KER == K_LOG ? 3 : 0)) +
+                                    2 * P * P);
+    }
+    if (pl.ffbad[pl.nprob]) far64<KER>(pl, o.mk, pl.ffbad, 1, sub, pl.coef, NFIELD, o.status);
 }
 
 // Split parts of the kept poles and weights of the FMM problems (split.cuh);
@@ -3036,7 +3047,7 @@ k_cm_apply(FmmDev pl, FactorView f, const int64_t *__restrict__ tile_off, CmDev 
 // What the tiles leave out, at most NC columns per launch: the deflated slots
 // (identity part of the factor) and, in FP64, the problems out of the positions'
 // scale: a warp per leaf box (32 targets; without a tree every box is near), near
-// sources staged, far field from the box's series (k_fmm_far64, figures
+// sources staged, far field from the box's series (far64, figures
 // there).  The inner loop runs all NC columns.
 template <bool TRANS, int NC>
 __global__ void __launch_bounds__(128)
@@ -3230,20 +3241,25 @@ SrcArgs src_from_r1(const int64_t *off, const R1Out &o)
     return a;
 }
 
-// Far fields of the problems with only[p] != 0.  Subtrees of 8 leaf boxes where that
-// leaves four to an SM (their lists differ in length), of 4 where it leaves one, the
-// columns in two halves where there are few.  GB300, applications of 19 columns to
-// 124000 rows, of 64 to 20000, poles graded: 8 boxes 36.3 and 13.8 ms, 4 boxes 29.9 and
-// 9.0, 2 boxes 30 and 10.7
+// Levels of far64's subtrees: of 8 leaf boxes where that leaves four subtrees to an SM
+// (their lists differ in length), of 4 where it leaves one; the columns' in two halves
+// where there are few.  GB300, applications of 19 columns to 124000 rows, of 64 to
+// 20000, poles graded: 8 boxes 36.3 and 13.8 ms, 4 boxes 29.9 and 9.0, 2 boxes 30 and 10.7
+int far64_sub(const FmmPlan &pl)
+{
+    const int64_t nsm = sdc_num_sms();
+    return (pl.cap_leaves >> 3) >= 4 * nsm ? 3 : (pl.cap_leaves >> 2) >= nsm ? 2 : 1;
+}
+
+// far fields of the columns of the problems with only[p] != 0
 template <int KER>
 void launch_far64(const FmmPlan &pl, const int32_t *mk, const int32_t *only, int nw, double *coef, int nfield,
                   int32_t *word, cudaStream_t st)
 {
-    const int64_t nsm = sdc_num_sms();
-    const int sub = (pl.cap_leaves >> 3) >= 4 * nsm ? 3 : (pl.cap_leaves >> 2) >= nsm ? 2 : 1;
+    const int sub = far64_sub(pl);
     const int64_t units = (pl.cap_leaves >> sub) + 1;
     const unsigned g = (unsigned)std::min<int64_t>(units, resident_grid<k_fmm_far64<KER>>(far_threads<KER>()));
-    const dim3 grid(g, far_cols<KER>() && nw > 8 && units < 2 * nsm ? 2 : 1);
+    const dim3 grid(g, nw > 8 && units < 2 * (int64_t)sdc_num_sms() ? 2 : 1);
     PROF_LAUNCH("fmm_far", st, k_fmm_far64<KER><<<grid, far_threads<KER>(), 0, st>>>(pl.dv, mk, only, nw, sub, coef, nfield, word));
 }
 
@@ -3257,10 +3273,10 @@ superdc_status far_field(const FmmPlan &pl, const int64_t *off, const R1Out &o, 
     const unsigned gu = (unsigned)std::min<int64_t>((pl.cap_leaves + 3) / 4, resident_grid<k_fmm_up1<MODE>>(128));
     PROF_LAUNCH("fmm_up", st, k_fmm_up1<MODE><<<gu, 128, 0, st>>>(dv, a));
     PROF_LAUNCH("fmm_up", st, k_fmm_up<MODE><<<up_grid<MODE>(), up_threads<MODE>(), 0, st>>>(dv, a));
-    const int64_t want = (pl.cap_leaves + FAR_NW - 1) / FAR_NW;
+    const int sub = far64_sub(pl);               // (a CTA per subtree of far64, should one be out of scale)
+    const int64_t want = std::max((pl.cap_leaves + FAR_NW - 1) / FAR_NW, (pl.cap_leaves >> sub) + 1);
     const unsigned g = (unsigned)std::min<int64_t>(want, resident_grid<k_fmm_far<KER>>(FAR_NW * 32));
-    PROF_LAUNCH("fmm_far", st, k_fmm_far<KER><<<g, FAR_NW * 32, 0, st>>>(dv, off, o));
-    launch_far64<KER>(pl, o.mk, dv.ffbad, 1, dv.coef, NFIELD, o.status, st);
+    PROF_LAUNCH("fmm_far", st, k_fmm_far<KER><<<g, FAR_NW * 32, 0, st>>>(dv, off, o, sub));
     return SUPERDC_OK;
 }
 
