@@ -1387,14 +1387,14 @@ __global__ void __launch_bounds__(FAR_NW * 32, 5) k_fmm_far(FmmDev pl, const int
 }
 
 // Split parts of the kept poles and weights of the FMM problems (split.cuh);
-// pl.ffbad says which problems' scale and gaps do not allow them
+// pl.ffbad says which problems' scale, gaps or stopping test do not allow them
 struct FfDev {
     const ff_f4 *d;
     const ff_f2 *w;
 };
 
 __global__ void k_ff_prep(int64_t nprob, const int64_t *__restrict__ off, int64_t total,
-                          const int32_t *__restrict__ fslot, R1Out o, ff_f4 *__restrict__ fd,
+                          const int32_t *__restrict__ fslot, R1Out o, double stop_c, ff_f4 *__restrict__ fd,
                           ff_f2 *__restrict__ fw, int32_t *__restrict__ bad)
 {
     for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < total;
@@ -1406,7 +1406,7 @@ __global__ void k_ff_prep(int64_t nprob, const int64_t *__restrict__ off, int64_
         const int m = o.mk[p], j = (int)(x - b0);
         if (j >= m) continue;
         const FfScale s = ff_scale(o.dk[b0], o.dk[b0 + m - 1], o.wsum[p]);
-        if (!s.ok || o.unshifted || (j + 1 < m && !ff_gap_ok(o.dk[x], o.dk[x + 1], s.kk))) {
+        if (!s.ok || o.unshifted || stop_c < SPLIT_STOP || (j + 1 < m && !ff_gap_ok(o.dk[x], o.dk[x + 1], s.kk))) {
             bad[p] = 1;
             bad[nprob] = 1;
             continue;
@@ -3410,7 +3410,7 @@ superdc_status fmm_secular(const FmmPlan &pl, const int64_t *off, const R1Out &o
     SDC_CHECK(cudaMemsetAsync(pl.dv.ffbad, 0, (size_t)(pl.dv.nprob + 1) * sizeof(int32_t), st));
     const unsigned gp = (unsigned)std::max<int64_t>(1, std::min<int64_t>((pl.total + 255) / 256,
                                                                          (int64_t)sdc_num_sms() * 8));
-    PROF_LAUNCH("fmm_secular", st, k_ff_prep<<<gp, 256, 0, st>>>(pl.dv.nprob, off, pl.total, pl.dv.fslot, o, fd, fw,
+    PROF_LAUNCH("fmm_secular", st, k_ff_prep<<<gp, 256, 0, st>>>(pl.dv.nprob, off, pl.total, pl.dv.fslot, o, stop_c, fd, fw,
                                                                  pl.dv.ffbad));
     const FfDev ff = {fd, fw};
     far_field<M_SEC, K_SEC>(pl, off, o, st);

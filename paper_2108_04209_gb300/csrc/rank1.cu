@@ -501,10 +501,11 @@ k_secular(const int64_t *__restrict__ off, const int4 *__restrict__ units,
         const double *dk = o.dk + b0, *zk = o.zk + b0;
         const double W = o.wsum[p];
         const double tol = stop_c * (double)m * SDC_EPS;
-        // split FP32 sweeps where the problem's scale allows; its last root (right
-        // of every pole, outside the fixed-point range) then runs on its own
+        // split FP32 sweeps where the problem's scale and the stopping test allow; its
+        // last root (right of every pole, outside the fixed-point range) then runs on
+        // its own
         const FfScale fs = ff_scale(dk[0], dk[m - 1], W);
-        bool okt = fs.ok && !o.unshifted && m >= 2;
+        bool okt = fs.ok && !o.unshifted && m >= 2 && stop_c >= SPLIT_STOP;
         for (int j = threadIdx.x; okt && j + 1 < m; j += NW * 32) okt = ff_gap_ok(dk[j], dk[j + 1], fs.kk);
         const bool ok = __syncthreads_and(okt);
         auto last_root = [&]() {
