@@ -58,16 +58,6 @@ __global__ void k_prep(int64_t nprob, const int64_t *__restrict__ off, int64_t t
     }
 }
 
-// 1 / t rounded to nearest (Markstein, 1990: a reciprocal within an ulp, corrected
-// by its residual)
-__device__ __forceinline__ double rcp_rn(double t)
-{
-    const int e = (__double2hiint(t) >> 20) & 0x7FF;
-    if (e < 31 || e > 2015) return 1.0 / t;
-    const double r = rcp_nr2(t);
-    return fma(r, fma(-t, r, 1.0), r);
-}
-
 // Per kept root k, columns [c0, c0 + nc): u_k and g_k from the four sums P, R,
 // Gamma, Delta of every column, each added up in the order of the sources.  (One
 // factor per pair, s_kl = sum_c (ybar_kc alpha_lc - y_kc beta_lc), takes half of

@@ -14,5 +14,6 @@ int fmm_default_min_m() { return 512; }
 // 0.98, of 2048 1.00 / 0.82; the applications (1 to 64 columns) cross between 1024
 // and 2048 as well.  Above the line: 64 problems of 768 1.63 / 1.11, of 1024 2.20
 // / 1.24, functions of a factor of 32768 rows to 64 columns 4 ms slower with 1536.  An eigendecomposition of n = 512 (leaf 32, rank 4)
-// 6.4 -> 5.4 ms.
+// 6.4 -> 5.4 ms.  Steps called directly keep 512 at any number of rows: which problems
+// took the tree is one of their results (superdc_rank1_out.fmm).
 int fmm_few_rows_min_m() { return 1536; }

@@ -3086,7 +3086,6 @@ k_cm_rest(FmmDev pl, FactorView f, int64_t total, const int64_t *__restrict__ ti
         const int64_t gx = tree ? pl.box_base[p] + Tb : 0;
         const int nnr = tree ? pl.nnear[gx] : -1;
         const int nn = near_len(nnr, nb0);
-        const int64_t nrow = f.off[p + 1] - b0;
         const int r = min(Tb * B + lane, tend - 1);
         const double a0 = TRANS ? dorg[r] : dk[r], a1 = TRANS ? eta[r] : 0.0;
         double acc[NC];
@@ -3106,7 +3105,7 @@ k_cm_rest(FmmDev pl, FactorView f, int64_t total, const int64_t *__restrict__ ti
             __syncwarp();
             if (lane < cnt) {
                 const int j = j0 + lane;
-                const int64_t row = b0 + SDC_IDX(TRANS ? f.src[b0 + j] : f.pinv[b0 + j], nrow, f.status);
+                const int64_t row = b0 + SDC_IDX(TRANS ? f.src[b0 + j] : f.pinv[b0 + j], f.off[p + 1] - b0, f.status);
                 sd[warp][lane] = TRANS ? dk[j] : dorg[j];
                 se[warp][lane] = TRANS ? 0.0 : eta[j];
                 sf[warp][lane] = TRANS ? f.vhat[b0 + j] : f.bnorm[b0 + j];
@@ -3124,13 +3123,13 @@ k_cm_rest(FmmDev pl, FactorView f, int64_t total, const int64_t *__restrict__ ti
         }
         if (!TRANS) {                                    // the last eigenvalue, outside the tree
             const double w = f.bnorm[b0 + m - 1] * rcp_nr2((a0 - dorg[m - 1]) - eta[m - 1]);
-            const int64_t row = b0 + SDC_IDX(f.pinv[b0 + m - 1], nrow, f.status);
+            const int64_t row = b0 + SDC_IDX(f.pinv[b0 + m - 1], f.off[p + 1] - b0, f.status);
 #pragma unroll
             for (int q = 0; q < NC; q++)
                 if (q < nc) acc[q] = fma(w, X[row + (int64_t)(col0 + q) * ldx], acc[q]);
         }
         if (Tb * B + lane < tend) {
-            const int64_t row = b0 + SDC_IDX(TRANS ? f.pinv[b0 + r] : f.src[b0 + r], nrow, f.status);
+            const int64_t row = b0 + SDC_IDX(TRANS ? f.pinv[b0 + r] : f.src[b0 + r], f.off[p + 1] - b0, f.status);
             const double sc = TRANS ? f.bnorm[b0 + r] : f.vhat[b0 + r];
 #pragma unroll
             for (int q = 0; q < NC; q++)

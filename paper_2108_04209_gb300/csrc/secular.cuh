@@ -66,6 +66,16 @@ __device__ __forceinline__ double rcp_any(double t)
     return (e > 30 && e < 2016) ? rcp_nr2(t) : 1.0 / t;
 }
 
+// 1 / t rounded to nearest (Markstein, 1990: a reciprocal within an ulp, corrected
+// by its residual)
+__device__ __forceinline__ double rcp_rn(double t)
+{
+    const int e = (__double2hiint(t) >> 20) & 0x7FF;
+    if (e < 31 || e > 2015) return 1.0 / t;
+    const double r = rcp_nr2(t);
+    return fma(r, fma(-t, r, 1.0), r);
+}
+
 // q^(-1/2) to about 2^-22 for a normal q > 0: the FP32 approximate reciprocal
 // square root of the leading mantissa bits (scaled into [1, 4) to make the
 // exponent even), the exponent halved by integer arithmetic; no conversion
