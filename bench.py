@@ -678,8 +678,9 @@ def main():
                          "fp64_pipe_pct_ncu": (prof or {}).get("fp64_pipe_pct"),
                          "peak_source": peak_src,
                          "algorithmic": rl.get(dom, {}).get("algorithmic"),
-                         "note": "FP64-accurate terms computed by split FP32 and integer arithmetic, counted as the "
-                                 "FP64 operations that they stand for: the fraction of the FP64 peak exceeds 1",
+                         "note": "terms computed by split FP32 and integer arithmetic (function values and iterates to "
+                                 "FP64's accuracy, derivatives and part of the series in single precision), counted as "
+                                 "the FP64 operations that they stand for: the fraction of the FP64 peak exceeds 1",
                          "other": {k: {"achieved": v["achieved"], "frac": v["achieved"] / peak, "ms": v["ms"]}
                                    for k, v in rl.items() if k != dom}},
             "whole_step": {"flops": step_flops, "achieved_tflops": step_flops / (tmax / args.steps * 1e-3) / 1e12,

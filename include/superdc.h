@@ -49,7 +49,8 @@ typedef enum {
 
 typedef struct {
     double  tau;          /* deflation tolerance of Remark 4.1 (absolute; strict '<' tests) */
-    double  stop_c;       /* constant c of the stopping test eq. (4.12): |f| < c m (1+|psi|+|phi|) eps */
+    double  stop_c;       /* constant c of the stopping test eq. (4.12): |f| < c m (1+|psi|+|phi|) eps;
+                             below 0.1 the sweeps run in FP64 (slower) */
     int32_t max_iter;     /* iteration cap of the secular solver (the paper is silent; default 50) */
     int32_t tile_roots;   /* secular schedule: roots per work unit (32..4096, multiple of 32);
                              other values: chosen from the batch size */
@@ -189,7 +190,13 @@ superdc_status superdc_secular_batched_host(int64_t nprob, const int64_t *offset
  * X, Y total x ncols column-major (ld ldx, ldy >= total), problem p owning rows
  * [offsets[p], offsets[p+1]).  X is read only; X and Y must not overlap.
  * opts (may be NULL: defaults): only fmm_min_m is used (problems whose kept
- * size reaches it use the triangular FMM for the Cauchy-like sums). */
+ * size reaches it use the triangular FMM for the Cauchy-like sums).
+ * Accuracy is in norm: an entry of Y is off by a few 2^-53 of the problem's
+ * largest kept entry of the column (times the norm of its row of Qhat), whatever
+ * the sizes of the terms that it is the sum of; a column whose entries differ by
+ * many orders of magnitude is best split by size where each part matters.  Rows of
+ * deflated slots pass through exactly.  A problem with a non-finite kept entry is
+ * summed in FP64, column by column. */
 superdc_status superdc_rank1_apply(int64_t nprob, const int64_t *offsets, int64_t total,
                                    const superdc_rank1_out *fwd, int32_t trans, int64_t ncols,
                                    const double *X, int64_t ldx, double *Y, int64_t ldy,
@@ -392,7 +399,8 @@ void superdc_eigfact_free(superdc_eigfact *f);
 /* Y = Q X (trans = 0) or Y = Q^T X (trans = 1), Algorithm 4 applied at the
  * root.  X, Y: DEVICE, n x ncols column-major with leading dimensions
  * ldx, ldy >= n; X and Y must not overlap.  Work buffers come from the
- * stream-ordered allocator. */
+ * stream-ordered allocator.  Accuracy is in norm, per column (see
+ * superdc_rank1_apply). */
 superdc_status superdc_apply_Q(const superdc_eigfact *f, int32_t trans, int64_t ncols,
                                const double *X, int64_t ldx, double *Y, int64_t ldy,
                                cudaStream_t stream);

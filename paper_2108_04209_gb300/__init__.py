@@ -222,7 +222,8 @@ class EigFactor:
         self.lmax, self.rank, self.n = lm.value, r.value, n.value
 
     def apply_Q(self, X, trans=False):
-        """Y = Q X (trans False) or Q^T X; X: float64 CUDA tensor n or n x k."""
+        """Y = Q X (trans False) or Q^T X; X: float64 CUDA tensor n or n x k.  Accurate
+        in norm, column by column."""
         vec = X.dim() == 1
         Xc = X.reshape(self.n, -1)
         Xf = Xc.t().contiguous().t() if not Xc.t().is_contiguous() else Xc    # column-major view
@@ -353,7 +354,8 @@ def _apply_rank1_T(offsets, out, X):
 
 def apply_rank1(offsets, out, X, trans=True, opts=None):
     """Qhat^T X (trans) or Qhat X for the factors of a secular_batched result
-    (opts: only fmm_min_m is used; None = defaults)."""
+    (opts: only fmm_min_m is used; None = defaults).  Accurate relative to each
+    problem's largest kept entry of a column."""
     total = int(offsets[-1].item())
     ncols = X.shape[1]
     Xf = X.t().contiguous().t()
