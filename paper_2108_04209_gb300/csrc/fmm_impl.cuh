@@ -2244,10 +2244,15 @@ struct CmDev {
     int32_t *eb;                 // per box: exponent of its node weights over the columns' scales
     double *lastp;               // per (tile of 64, column of the pass): partial sums for the last eigenvalue
     double *coef;                // per leaf box and column: far field's series of the problems out of scale
+    int cs;                      // their columns per leaf box
 };
 
+// Positions and factors of the sources; which problems are out of scale; the scale of
+// every column over its problem's kept rows (a deflated row passes through unchanged,
+// whatever its size).  A problem with a non-finite entry takes the FP64 loops: the
+// digits of one column share the boxes' scales with the others.
 template <bool TRANS>
-__global__ void k_cm_prep(FactorView f, int64_t total, CmDev c)
+__global__ void k_cm_prep(FactorView f, int64_t total, const double *__restrict__ X, int64_t ldx, int ncols, CmDev c)
 {
     for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < total;
          x += (int64_t)gridDim.x * blockDim.x) {
@@ -2273,15 +2278,6 @@ __global__ void k_cm_prep(FactorView f, int64_t total, CmDev c)
         c.fac[x] = {t.a, t.b, t.c, 0.0f};
         c.pos[x] = (TRANS || j == m - 1) ? ff_pole(dk[j], s) : ff_point(dK, f.eta[x], s);
     }
-}
-
-// Scale of every column over its problem's kept rows (a deflated row passes through
-// unchanged, whatever its size).  A problem with a non-finite entry takes the FP64
-// loops: the digits of one column share the boxes' scales with the others.
-template <bool TRANS>
-__global__ void k_cm_colmax(FactorView f, int64_t total, const double *__restrict__ X, int64_t ldx, int ncols,
-                            CmDev c)
-{
     for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < total * ncols;
          t += (int64_t)gridDim.x * blockDim.x) {
         const int64_t x = t % total;
@@ -3095,7 +3091,7 @@ k_cm_rest(FmmDev pl, FactorView f, int64_t total, const int64_t *__restrict__ ti
             double cT, hT;
             box_ch(pl.blo[gx], pl.bhi[gx], cT, hT);
             const double v = ((a0 + a1) - cT) * rcp_any(hT);
-            const double *cf = c.coef + (pl.leaf_base[p] + Tb) * CM_BC * P;
+            const double *cf = c.coef + (pl.leaf_base[p] + Tb) * c.cs * P;
 #pragma unroll
             for (int q = 0; q < NC; q++)
                 if (q < nc) acc[q] = clenshaw(cf + q * P, v);
@@ -3465,17 +3461,19 @@ superdc_status fmm_columns(const FmmPlan &pl, const FactorView &f, int64_t total
         SDC_CHECK(sc.get(&c.wf0, (size_t)pl.cap_boxes * ntmax * CM_D * 32));
         SDC_CHECK(sc.get(&c.wf1, (size_t)pl.cap_boxes * ntmax * CM_D * 32));
         SDC_CHECK(sc.get(&c.eb, (size_t)pl.cap_boxes));
-        SDC_CHECK(sc.get(&c.coef, (size_t)pl.cap_leaves * CM_BC * P));
+        // the digits are read for the last time before the FP64 loops write their series:
+        // cs columns of P doubles in the digits' place of a box
+        c.coef = (double *)c.wf0;
+        c.cs = CM_D * 32 / P * ntmax;
+        static_assert(CM_D * 32 / P >= 8 && sizeof(uint2) == sizeof(double), "a tile's series fit its digits");
     }
     SDC_CHECK(cudaMemsetAsync(c.bad, 0, nflag * sizeof(int32_t), st));
     auto gr = [&](int64_t n) {
         return (unsigned)std::max<int64_t>(1, std::min<int64_t>((n + 255) / 256, (int64_t)sdc_num_sms() * 8));
     };
     const int64_t rows = chunks * 16;
-    if (trans) PROF_LAUNCH("cauchy", st, k_cm_prep<true><<<gr(total), 256, 0, st>>>(f, total, c));
-    else PROF_LAUNCH("cauchy", st, k_cm_prep<false><<<gr(total), 256, 0, st>>>(f, total, c));
-    if (trans) PROF_LAUNCH("cauchy", st, k_cm_colmax<true><<<gr(total * ncols), 256, 0, st>>>(f, total, X, ldx, ncols, c));
-    else PROF_LAUNCH("cauchy", st, k_cm_colmax<false><<<gr(total * ncols), 256, 0, st>>>(f, total, X, ldx, ncols, c));
+    if (trans) PROF_LAUNCH("cauchy", st, k_cm_prep<true><<<gr(total * ncols), 256, 0, st>>>(f, total, X, ldx, ncols, c));
+    else PROF_LAUNCH("cauchy", st, k_cm_prep<false><<<gr(total * ncols), 256, 0, st>>>(f, total, X, ldx, ncols, c));
     FmmDev dv = pl.dv;
     if (!pl.on) dv = FmmDev{};
     int32_t *word = nullptr;                             // of the index guards (checked build)
@@ -3508,8 +3506,8 @@ superdc_status fmm_columns(const FmmPlan &pl, const FactorView &f, int64_t total
 #endif
             if (trans) PROF_LAUNCH("fmm_up", st, k_fmm_up<M_CT><<<up_grid<M_CT>(), up_threads<M_CT>(), 0, st>>>(dv, a));
             else PROF_LAUNCH("fmm_up", st, k_fmm_up<M_CN><<<up_grid<M_CN>(), up_threads<M_CN>(), 0, st>>>(dv, a));
-            if (trans) launch_far64<K_1>(pl, f.mk, c.bad, nc, c.coef, CM_BC, word, st);
-            else launch_far64<K_1N>(pl, f.mk, c.bad, nc, c.coef, CM_BC, word, st);
+            if (trans) launch_far64<K_1>(pl, f.mk, c.bad, nc, c.coef, c.cs, word, st);
+            else launch_far64<K_1N>(pl, f.mk, c.bad, nc, c.coef, c.cs, word, st);
         }
         auto fn = nc <= 2 ? launch_rest<2> : nc <= 4 ? launch_rest<4> : nc <= 8 ? launch_rest<8> : nc <= 12 ? launch_rest<12>
                 : nc <= 16 ? launch_rest<16> : nc <= 20 ? launch_rest<20> : nc <= 24 ? launch_rest<24> : launch_rest<CM_BC>;
