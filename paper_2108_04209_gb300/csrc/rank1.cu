@@ -37,6 +37,9 @@
 namespace {
 
 constexpr int SEC_CHUNK = 1024;   // poles staged per shared-memory chunk (24 bytes each)
+constexpr int LONG_M = 512;       // more poles than this: split sweeps with three-float totals (ff_close3); the
+                                  // blocks of fewer leave less error than the terms.  Chosen per launch by what
+                                  // the direct kernels can meet: per problem it costs what it saves
 constexpr int DEFL_BIG = 128;     // problems larger than this deflate with more than one warp
 
 
@@ -469,8 +472,10 @@ __global__ void k_units(int64_t nprob, const int32_t *__restrict__ mk, const int
 // applies the same update, so the replicated root state stays identical.
 // Both keep the live roots of a warp inside a short window, so the psi/phi
 // split keeps its three warp-uniform regions.
-template <int NW, bool SPLIT>
-__global__ void __launch_bounds__(NW * 32)
+// (Registers for five CTAs per SM: left to itself the compiler takes 72 without SPLIT,
+// 2048 problems of 100 to 500: 4.26 ms a step, with 94 4.07.)
+template <int NW, bool SPLIT, bool LONG>
+__global__ void __launch_bounds__(NW * 32, 5)
 k_secular(const int64_t *__restrict__ off, const int4 *__restrict__ units,
           const int *__restrict__ nunits, int *__restrict__ counter,
           R1Out o, double stop_c, int max_iter)
@@ -568,7 +573,7 @@ k_secular(const int64_t *__restrict__ off, const int4 *__restrict__ units,
                 const int j0 = SPLIT ? (int)(((int64_t)cn * warp) / NW) : 0;
                 const int j1 = SPLIT ? (int)(((int64_t)cn * (warp + 1)) / NW) : cn;
                 if (any) {
-                    if (ok)      ff_sweep(fd, fw, j0, j1, c0, kk, kwlo, kwhi, x, S);
+                    if (ok)      ff_sweep<LONG>(fd, fw, j0, j1, c0, kk, kwlo, kwhi, x, S);
                     else if (p0) sweep<false>(sd, sw, j0, j1, c0, kk, kwlo, kwhi, R.dK, R.y, A);
                     else         sweep<true>(sd, sw, j0, j1, c0, kk, kwlo, kwhi, R.dK, R.y, A);
                 }
@@ -991,12 +996,11 @@ superdc_status r1_run(const R1Args &a_in, cudaStream_t st)
     secular_schedule(a.rows >= 0 ? a.rows : a.total, a.sched, a.tile_roots, slots, &split, &ubig);
     PROF_LAUNCH("units", st, k_units<<<1, 1024, ksm, st>>>(a.nprob, a.o.mk, fslot, ubig, split ? 1 : 0, units,
                                                            ucount, ucount + 1));
-    if (split)
-        PROF_LAUNCH("secular", st, (k_secular<4, true><<<(unsigned)slots, 128, 0, st>>>(
-                                       a.off, units, ucount, ucount + 1, a.o, a.stop_c, a.max_iter)));
-    else
-        PROF_LAUNCH("secular", st, (k_secular<4, false><<<(unsigned)slots, 128, 0, st>>>(
-                                       a.off, units, ucount, ucount + 1, a.o, a.stop_c, a.max_iter)));
+    const bool lng = a.fmm_min_m <= 0 || a.fmm_min_m > LONG_M + 1;      // else the tree takes the larger ones
+    const auto k_sec = split ? (lng ? k_secular<4, true, true> : k_secular<4, true, false>)
+                             : (lng ? k_secular<4, false, true> : k_secular<4, false, false>);
+    PROF_LAUNCH("secular", st, k_sec<<<(unsigned)slots, 128, 0, st>>>(a.off, units, ucount, ucount + 1, a.o, a.stop_c,
+                                                                      a.max_iter));
     superdc_status fs = fmm_secular(fp, a.off, a.o, a.stop_c, a.max_iter, st);
     unsigned long long *tq = nullptr;          // tile queues of the direct Loewner and b kernels
     SDC_CHECK(sc.get(&tq, 2));
@@ -1131,12 +1135,8 @@ extern "C" superdc_status superdc_secular_batched_noalloc(int64_t nprob, const i
     int ubig;
     secular_schedule(a.total, a.sched, a.tile_roots, slots, &split, &ubig);
     k_units<<<1, 1024, ksm, st>>>(a.nprob, a.o.mk, nullptr, ubig, split ? 1 : 0, units, ucount, ucount + 1);
-    if (split)
-        k_secular<4, true><<<(unsigned)slots, 128, 0, st>>>(a.off, units, ucount, ucount + 1, a.o, a.stop_c,
-                                                             a.max_iter);
-    else
-        k_secular<4, false><<<(unsigned)slots, 128, 0, st>>>(a.off, units, ucount, ucount + 1, a.o, a.stop_c,
-                                                              a.max_iter);
+    const auto k_sec = split ? k_secular<4, true, true> : k_secular<4, false, true>;
+    k_sec<<<(unsigned)slots, 128, 0, st>>>(a.off, units, ucount, ucount + 1, a.o, a.stop_c, a.max_iter);
     const auto k_low = dsplit ? k_lowner<32, 8> : k_lowner<128, 1>;
     const auto k_b = dsplit ? k_bnorm<32, 8> : k_bnorm<128, 1>;
     const int dthreads = dsplit ? 256 : 128;

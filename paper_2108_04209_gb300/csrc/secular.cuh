@@ -388,9 +388,6 @@ struct Root {
         const int kf = kk + kw;
         const bool right = K != k;
         const double D = d1 - d0, ay = fabs(y), g = D - ay;
-        // a gap at the end of the exponent range (a weight whose square is subnormal) has
-        // no reciprocal: the guess stands
-        if (phase != 0 && fexp(ay) < 31) return true;
         const double wn = right ? w1 : w0, wf = right ? w0 : w1;
         const double rn = rcp_nr2(ay), rf = rcp_nr2(g);
         const double c1 = ff_pow2(kf);
@@ -401,6 +398,9 @@ struct Root {
         const bool fit = abs(kf) < 50 && fexp(ay) + kk > 973 && fexp(wn) - kw > 923 && fexp(wf) - kw > 923 &&
                          ef - kf < 1073 && er - kf < 1073;
         if (!fit) {
+            // a gap at the end of the exponent range (a weight whose square is subnormal)
+            // has no reciprocal: the guess stands
+            if (phase != 0 && fexp(ay) < 31) return true;
             const double c2 = ff_pow2(kf + kk), an = wn * rn, af = wf * rf;
             Acc A;
             A.psi = fma((double)S.psi, c1, right ? -af : -an);
