@@ -472,10 +472,12 @@ __global__ void k_units(int64_t nprob, const int32_t *__restrict__ mk, const int
 // applies the same update, so the replicated root state stays identical.
 // Both keep the live roots of a warp inside a short window, so the psi/phi
 // split keeps its three warp-uniform regions.
-// (Registers for five CTAs per SM: left to itself the compiler takes 72 without SPLIT,
-// 2048 problems of 100 to 500: 4.26 ms a step, with 94 4.07.)
+// (Without SPLIT, registers for five CTAs per SM: left to itself the compiler takes 72,
+// 2048 problems of 100 to 500: 4.26 ms a step, with 96 4.07.  With SPLIT it is left to
+// itself, 96 too: one batch of 16 problems 307 us, 309 with the bound, 299 with all the
+// registers it wants, but then 2600 problems take 0.62 ms in this kernel instead of 0.48.)
 template <int NW, bool SPLIT, bool LONG>
-__global__ void __launch_bounds__(NW * 32, 5)
+__global__ void __launch_bounds__(NW * 32, SPLIT ? 0 : 5)
 k_secular(const int64_t *__restrict__ off, const int4 *__restrict__ units,
           const int *__restrict__ nunits, int *__restrict__ counter,
           R1Out o, double stop_c, int max_iter)
